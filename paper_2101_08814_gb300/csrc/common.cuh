@@ -157,7 +157,6 @@ struct rascal_ctx {
     float* mlp_params;   // FP32 master parameters
     float* mlp_m;        // Adam moments
     float* mlp_v;
-    float* mlp_grad;
     float* mlp_scale;    // [F] output scales
     void* mlp_w2t;       // BF16 operand tiles for the tensor-core inference
     void* mlp_w3t;

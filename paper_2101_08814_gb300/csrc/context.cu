@@ -453,7 +453,6 @@ extern "C" void rascal_destroy(rascal_ctx* ctx) {
     cudaFree(ctx->mlp_params);
     cudaFree(ctx->mlp_m);
     cudaFree(ctx->mlp_v);
-    cudaFree(ctx->mlp_grad);
     cudaFree(ctx->mlp_scale);
     cudaFree(ctx->mlp_w2t);
     cudaFree(ctx->mlp_w3t);
