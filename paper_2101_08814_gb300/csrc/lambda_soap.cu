@@ -7,9 +7,9 @@
 // removes the others), and only l1 <= l2: T(l2, l1) is the transpose of T(l1, l2).
 //
 // Host: Racah's closed form for the CG coefficients in FP64, the unitary U per l, the real tables per (l1, l2), kept
-// as their (at most two) non-zero m1 terms per (mu, m2), cached per lambda in the context. Device: one CTA per centre; per pair the two coefficient blocks are staged in
-// shared memory, then per chunk of mu the half-contractions X[q1][m2] = sum_m1 R c_{q1 l1 m1} and the output tiles
-// T[q1][q2] = sum_m2 X[q1][m2] c_{q2 l2 m2}, written with streaming 16-byte stores. Bound: HBM (the output).
+// as their (at most two) non-zero m1 terms per (mu, m2), cached per lambda in the context. Device: one CTA per centre
+// with its coefficients in shared memory; per pair the half-contractions X[q1][m2] = sum_m1 R c_{q1 l1 m1} and the
+// output tiles T[q1][q2] = sum_m2 X[q1][m2] c_{q2 l2 m2}. Bound: HBM (the output).
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -17,15 +17,17 @@
 #include <vector>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 
 namespace rascal {
 
 struct LsoapTable {
     int lambda = -1;
     int n_pairs = 0;
-    int4* d_hdr = nullptr;   // per pair: l1, l2, offset of its entries in d_R, 0
+    int4* d_hdr = nullptr;   // per pair: first slots of l1 and l2 in a padded row, offset of its entries in d_R,
+                             // 2 l2 + 1 | ceil(65536 / (2 l2 + 1 rounded up to 4)) << 6
     float4* d_R = nullptr;   // per pair [2 lambda + 1][2 l2 + 1]: the (at most two) non-zero m1 terms of R[mu][.][m2]
-                             // as {value0, value1, m1_0 * Q, m1_1 * Q} (offsets as integer bits; value 0 pads)
+                             // as {value0, value1, m1_0, m1_1} (indices as integer bits; value 0 pads)
 };
 
 static double fact(int n) {
@@ -105,105 +107,163 @@ static void lsoap_pairs(int l_max, int lam, std::vector<int2>& p) {
             if (std::abs(l1 - l2) <= lam && lam <= l1 + l2 && ((l1 + l2 + lam) & 1) == 0) p.push_back(make_int2(l1, l2));
 }
 
-// One CTA per centre. The centre's coefficients are staged once, transposed to cT[lm][q]; per pair and chunk of mu
-// values the half-contractions X[u][q1][m2] = sum_m1 R c_{q1 l1 m1} go to one of two buffers, one block barrier,
-// then 2 x 4 output tiles per thread (one 16-byte load of cT serves four outputs), stored with streaming 16-byte
-// writes. The alternating X buffers let the next chunk's X start while other threads still store this one.
-constexpr int kLsoapXFloats = 6144;  // shared-memory budget of one X buffer (24 KB)
+// One CTA per centre. Rows and columns of the output go in groups of four: with Q a multiple of 4 (VEC) group g holds
+// q = 4 g .. 4 g + 3, so that a thread's four columns are adjacent and leave as one streaming 16-byte store; otherwise it
+// holds g, g + QT, g + 2 QT, g + 3 QT (QT = ceil(Q / 4)), so that the scalar stores of neighbouring lanes are adjacent.
+// The centre's coefficients are staged once as C[g][v][slot], every l block of a row padded with zeros to a multiple of 4
+// slots (exp_lp), so that both contractions read 16-byte pieces along m; a group's 16 bytes of slack make neighbouring
+// groups' rows differ by an odd number of 16-byte words (conflict-free).
+// Per pair (l1, l2) the row groups of all mu (tau = mu QT + g) are made in chunks: the half-contractions
+// X[tau][v][m2] = sum_m1 R c_{q1 l1 m1} of a chunk go to one of two buffers (pads zero; row pitch PX, a compile-time
+// constant, so that the loads of a tile's rows need no address arithmetic), one block barrier, then 8 x 4 output tiles
+// per thread (two row groups), summed over m2 four at a time: 12 16-byte shared loads and 64 paired FMAs (even and odd m2
+// in the two halves of an accumulator, added at the end) for 128 products.
+// Bound: HBM (the output). 9 001 centres, Q = 48, l_max 9, lambda 1: 1 017 us with 2 x 4 tiles that loaded one value of X
+// per two products (issue-bound, 83 % issue-active); 718 us with 4 x 4 tiles (shared-memory loads 74 % of their rate);
+// 637 us = 3.8 TB/s in this form. Four CTAs of 128 threads per SM hide the barriers better than two of 256
+// (692 against 844 us with runtime pitches).
+constexpr int kLsoapThreads = 128, kLsoapCtas = 4;
+constexpr int kLsoapGroups = 36;  // row groups per chunk: X takes 11.5 KB (PX = 20) or 20.7 KB (PX = 36) per buffer
 
-__global__ void __launch_bounds__(256) k_lambda_soap(int64_t n, const float* __restrict__ c, int Q, int n_lm, int kmax,
-                                                     int lam, int mchunk, int n_pairs, const int4* __restrict__ hdr,
-                                                     const float4* __restrict__ R, float* __restrict__ out) {
+template <bool VEC, int PX>
+__global__ void __launch_bounds__(kLsoapThreads, kLsoapCtas) k_lambda_soap(const float* __restrict__ c, int Q, int l_max, int lam,
+                                                                           int chunk, unsigned qt_inv, int n_pairs,
+                                                                           const int4* __restrict__ hdr,
+                                                                           const float4* __restrict__ R,
+                                                                           float* __restrict__ out) {
     extern __shared__ __align__(16) float sm[];
-    const int i = blockIdx.x;
-    if (i >= n) return;
-    float* cT = sm;                              // [n_lm][Q]
-    float* const sX0 = cT + (size_t)n_lm * Q;
-    float* const sX1 = sX0 + (size_t)mchunk * Q * kmax;
-    const float* ci = c + (int64_t)i * Q * n_lm;
-    const int M = 2 * lam + 1;
-    const int64_t QQ = (int64_t)Q * Q;
-    const bool vec = (Q & 3) == 0;
-    {
-        const int lm = threadIdx.x % n_lm, r0 = threadIdx.x / n_lm, rs = blockDim.x / n_lm;
-        if (threadIdx.x < n_lm * rs)
-            for (int q = r0; q < Q; q += rs) cT[lm * Q + q] = ci[q * n_lm + lm];
-    }
-    // output tiling (fixed for the kernel): each thread owns one 4-column group and a stride of row pairs
-    const int nq2 = Q >> 2, nq1 = Q >> 1;
-    const int t_q2 = vec ? threadIdx.x % nq2 : 0, t_r = vec ? threadIdx.x / nq2 : 0;
-    const int r_step = vec ? blockDim.x / nq2 : 1;
-    const bool t_on = vec && threadIdx.x < nq2 * r_step;
-    int buf = 0;
+    const int64_t i = blockIdx.x;
+    const int n_lm = (l_max + 1) * (l_max + 1), pitch = exp_ly(l_max), gs = 4 * pitch + 4, QT = (Q + 3) >> 2;
+    const int tid = threadIdx.x, groups = (2 * lam + 1) * QT;
+    float* C = sm;                           // [QT][gs]
+    float* sX = C + QT * gs;                 // two buffers [chunk][4][PX]
+    const float* ci = c + i * Q * n_lm;
+    for (int e = tid; e < QT * gs / 4; e += kLsoapThreads) reinterpret_cast<float4*>(C)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto div_qt = [&](int x) { return QT == 1 ? x : (int)__umulhi((unsigned)x, qt_inv); };  // x / QT, exact for x < 65536
     __syncthreads();
-    for (int p = 0; p < n_pairs; ++p) {
-        const int4 h = hdr[p];
-        const int l1 = h.x, l2 = h.y, d2 = 2 * l2 + 1;
-        const float4* Rp = R + h.z;
-        const float* A = cT + l1 * l1 * Q;  // A[m1][q]
-        const float* B = cT + l2 * l2 * Q;  // B[m2][q]
-        const int b_c = threadIdx.x % d2, b_r = threadIdx.x / d2, b_s = blockDim.x / d2;
-        const bool b_on = threadIdx.x < d2 * b_s;
-        for (int mu0 = 0; mu0 < M; mu0 += mchunk, buf ^= 1) {
-            const int mc = min(mchunk, M - mu0);
-            float* sX = buf ? sX1 : sX0;
-            if (b_on) {
-                // rows rr = u Q + q1 of X over the whole chunk, so that all mc * Q rows share the threads evenly
-                int u = 0, q1 = b_r;
-                while (q1 >= Q) {
-                    q1 -= Q;
-                    ++u;
-                }
-                for (int rr = b_r; rr < mc * Q; rr += b_s) {
-                    const float4 e = __ldg(Rp + (size_t)(mu0 + u) * d2 + b_c);  // the two non-zero m1 of this (mu, m2)
-                    const float x = fmaf(e.x, A[__float_as_int(e.z) + q1], e.y * A[__float_as_int(e.w) + q1]);
-                    sX[(size_t)rr * d2 + b_c] = x;
-                    q1 += b_s;
-                    while (q1 >= Q) {
-                        q1 -= Q;
-                        ++u;
+    {
+        const int warp = tid >> 5, lane = tid & 31;
+        for (int lm = lane; lm < n_lm; lm += 32) {  // lanes over lm: coalesced, the slot worked out once
+            const int l = (int)sqrtf((float)lm);
+            float* slot = C + exp_lp(l) + lm - l * l;
+#pragma unroll 4
+            for (int q = warp; q < Q; q += kLsoapThreads / 32) {
+                const int v = VEC ? q & 3 : div_qt(q), g = VEC ? q >> 2 : q - v * QT;
+                slot[g * gs + v * pitch] = __ldg(ci + q * n_lm + lm);
+            }
+        }
+    }
+    // output tiling (fixed for the kernel): each thread owns one column group and a stride of row groups
+    const int t_r = div_qt(tid), t_c = tid - t_r * QT, r_step = div_qt(kLsoapThreads);
+    const bool t_on = t_r < r_step;
+    const int64_t pair_floats = (int64_t)(2 * lam + 1) * Q * Q;
+    float* op = out + i * n_pairs * pair_floats + (VEC ? 4 * t_c : t_c);
+    const int x_floats = chunk * 4 * PX;
+    int cur = 0;  // offset of the X buffer in use
+    int4 h = __ldg(hdr);
+    __syncthreads();
+    for (int p = 0; p < n_pairs; ++p, op += pair_floats) {
+        const int d2 = h.w & 63, dp = (d2 + 3) & ~3, inv = h.w >> 6;  // inv = ceil(65536 / dp)
+        const int b_r = (tid * inv) >> 16, b_c = tid - b_r * dp, b_s = (kLsoapThreads * inv) >> 16;
+        const float4* Rp = R + h.z + b_c;
+        const float* A = C + h.x;
+        const float* Bt = C + h.y + t_c * gs;
+        h = __ldg(hdr + min(p + 1, n_pairs - 1));
+        for (int g0 = 0; g0 < groups; g0 += chunk, cur = x_floats - cur) {
+            const int ng = min(chunk, groups - g0);
+            float* X = sX + cur;
+            if (b_r < b_s) {
+#pragma unroll 2
+                for (int r = b_r; r < ng; r += b_s) {
+                    const int u = div_qt(g0 + r);
+                    float w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                    if (b_c < d2) {
+                        const float4 e = __ldg(Rp + u * d2);  // the two non-zero m1 of this (mu, m2)
+                        const float* ag = A + (g0 + r - u * QT) * gs;
+                        const float* a0 = ag + __float_as_int(e.z);
+                        const float* a1 = ag + __float_as_int(e.w);
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) w[v] = fmaf(e.x, a0[v * pitch], e.y * a1[v * pitch]);
                     }
+                    float* x = X + r * 4 * PX + b_c;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) x[v * PX] = w[v];
                 }
             }
             __syncthreads();
-            float* o = out + (((int64_t)i * n_pairs + p) * M + mu0) * QQ;
-            if (vec) {
-                if (t_on) {
-                    // row pairs over the whole chunk: row 2 rp of [mc Q][..] is (u, q1) = (2 rp / Q, 2 rp % Q), and both
-                    // X and the output of consecutive mu are contiguous, so no division is needed
-                    for (int rp = t_r; rp < mc * nq1; rp += r_step) {
-                        {
-                            const int q2 = 4 * t_q2;
-                            const float* x0 = sX + (size_t)(2 * rp) * d2;
-                            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-                            for (int m2 = 0; m2 < d2; ++m2) {
-                                const float4 bv = *reinterpret_cast<const float4*>(B + m2 * Q + q2);
-                                const float xa = x0[m2], xb = x0[d2 + m2];
-                                a.x = fmaf(xa, bv.x, a.x);
-                                a.y = fmaf(xa, bv.y, a.y);
-                                a.z = fmaf(xa, bv.z, a.z);
-                                a.w = fmaf(xa, bv.w, a.w);
-                                b.x = fmaf(xb, bv.x, b.x);
-                                b.y = fmaf(xb, bv.y, b.y);
-                                b.z = fmaf(xb, bv.z, b.z);
-                                b.w = fmaf(xb, bv.w, b.w);
-                            }
-                            float* ou = o + (int64_t)(2 * rp) * Q + q2;
-                            __stcs(reinterpret_cast<float4*>(ou), a);
-                            __stcs(reinterpret_cast<float4*>(ou + Q), b);
+            if (!t_on) continue;
+            const int half = (ng + 1) >> 1;  // a thread's two row groups: r and r + half, if there is one
+#pragma unroll 1
+            for (int r = t_r; r < half; r += r_step) {
+                uint64_t acc[8][4];
+                const bool two = r + half < ng;
+                const float* x0 = X + r * 4 * PX;
+                const float* x1 = two ? x0 + half * 4 * PX : x0;
+                const float *b0 = Bt, *b1 = Bt + pitch, *b2 = b1 + pitch, *b3 = b2 + pitch;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[u][v] = 0ull;
+#pragma unroll 1
+                for (int m = 0; m < dp; m += 4) {
+                    ulonglong2 b[4];
+                    b[0] = *reinterpret_cast<const ulonglong2*>(b0);
+                    b[1] = *reinterpret_cast<const ulonglong2*>(b1);
+                    b[2] = *reinterpret_cast<const ulonglong2*>(b2);
+                    b[3] = *reinterpret_cast<const ulonglong2*>(b3);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>((u < 4 ? x0 : x1) + (u & 3) * PX);
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            acc[u][v] = f2_fma(x.x, b[v].x, acc[u][v]);
+                            acc[u][v] = f2_fma(x.y, b[v].y, acc[u][v]);
                         }
                     }
+                    b0 += 4;
+                    b1 += 4;
+                    b2 += 4;
+                    b3 += 4;
+                    x0 += 4;
+                    x1 += 4;
                 }
-            } else {
-                for (int e = threadIdx.x; e < mc * Q * Q; e += blockDim.x) {
-                    const int u = e / (Q * Q), r = e % (Q * Q), q1 = r / Q, q2 = r % Q;
-                    float t = 0.0f;
-                    for (int m2 = 0; m2 < d2; ++m2) t = fmaf(sX[((size_t)u * Q + q1) * d2 + m2], B[m2 * Q + q2], t);
-                    o[u * QQ + r] = t;
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    if (k == 1 && !two) break;
+                    const int tau = g0 + r + k * half, mu = div_qt(tau), g = tau - mu * QT;
+                    float* o = op + (mu * Q + (VEC ? 4 * g : g)) * Q;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (!VEC && g + QT * u >= Q) break;
+                        float w[4];
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            float lo, hi;
+                            f2_unpack(acc[4 * k + u][v], lo, hi);
+                            w[v] = lo + hi;
+                        }
+                        if (VEC) {
+                            __stcs(reinterpret_cast<float4*>(o), make_float4(w[0], w[1], w[2], w[3]));
+                        } else {
+#pragma unroll
+                            for (int v = 0; v < 4; ++v)
+                                if (t_c + QT * v < Q) __stcs(o + QT * v, w[v]);
+                        }
+                        o += VEC ? Q : QT * Q;
+                    }
                 }
             }
         }
     }
+}
+
+// row pitch of X: 20 holds the widest pair up to l_max 9 (2 l_max + 1 <= 20), 36 every other; an odd number of 16-byte words
+static int lsoap_px(int l_max) { return l_max <= 9 ? 20 : 36; }
+
+static auto lsoap_kernel(int Q, int l_max) {
+    const bool vec = Q % 4 == 0;
+    return lsoap_px(l_max) == 20 ? (vec ? k_lambda_soap<true, 20> : k_lambda_soap<false, 20>)
+                                 : (vec ? k_lambda_soap<true, 36> : k_lambda_soap<false, 36>);
 }
 
 int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const float4** R) {
@@ -215,12 +275,12 @@ int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const 
         std::vector<int4> h(P.size());
         std::vector<float4> all;
         std::vector<float> one;
-        const int Q = ctx->Q;
         for (size_t k = 0; k < P.size(); ++k) {
             const int l1 = P[k].x, l2 = P[k].y, d1 = 2 * l1 + 1, d2 = 2 * l2 + 1;
             if (!real_table(l1, l2, lam, one))
                 return set_error(RASCAL_E_UNSUPPORTED, "coupling (%d, %d) -> %d is not real", l1, l2, lam);
-            h[k] = make_int4(l1, l2, (int)all.size(), 0);
+            const int dp = (d2 + 3) / 4 * 4;
+            h[k] = make_int4(exp_lp(l1), exp_lp(l2), (int)all.size(), d2 | ((65536 + dp - 1) / dp) << 6);
             for (int u = 0; u < 2 * lam + 1; ++u)
                 for (int m2 = 0; m2 < d2; ++m2) {
                     float v[2] = {0.0f, 0.0f};
@@ -232,17 +292,19 @@ int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const 
                             return set_error(RASCAL_E_UNSUPPORTED, "coupling (%d, %d) -> %d has more than two terms",
                                              l1, l2, lam);
                         v[nz] = r;
-                        o[nz++] = m1 * Q;
+                        o[nz++] = m1;
                     }
                     float f[2];
-                    std::memcpy(f, o, sizeof(f));  // offsets travel as integer bits
+                    std::memcpy(f, o, sizeof(f));  // indices travel as integer bits
                     all.push_back(make_float4(v[0], v[1], f[0], f[1]));
                 }
         }
         LsoapTable* t = new LsoapTable();
         t->lambda = lam;
         t->n_pairs = (int)P.size();
-        cudaError_t e = cudaMalloc(&t->d_hdr, sizeof(int4) * std::max<size_t>(1, h.size()));
+        cudaError_t e = cudaFuncSetAttribute(lsoap_kernel(ctx->Q, ctx->l_max), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             227 * 1024);
+        if (e == cudaSuccess) e = cudaMalloc(&t->d_hdr, sizeof(int4) * std::max<size_t>(1, h.size()));
         if (e == cudaSuccess) e = cudaMalloc(&t->d_R, sizeof(float4) * std::max<size_t>(1, all.size()));
         if (e == cudaSuccess && !h.empty())
             e = cudaMemcpy(t->d_hdr, h.data(), sizeof(int4) * h.size(), cudaMemcpyHostToDevice);
@@ -312,18 +374,19 @@ extern "C" int rascal_lambda_soap(rascal_ctx* ctx, int64_t n_centres, const floa
     if (!d_coeffs || !d_out) return set_error(RASCAL_E_ARG, "NULL device pointer");
     if ((reinterpret_cast<uintptr_t>(d_out) & 15) != 0) return set_error(RASCAL_E_ARG, "d_out must be 16-byte aligned");
     if (n_centres > 0x7fffffffLL) return set_error(RASCAL_E_ARG, "too many centres for one launch");
+    // the coefficients and one row of half-contractions per q, twice, have to fit a CTA's shared memory
     const int kmax = 2 * ctx->l_max + 1;
-    const int mchunk = std::max(1, std::min(2 * lambda + 1, kLsoapXFloats / (ctx->Q * kmax)));
-    const size_t smem = sizeof(float) * ((size_t)ctx->n_lm * ctx->Q + (size_t)2 * mchunk * ctx->Q * kmax);
-    static bool attr = false;
-    if (!attr) {
-        RASCAL_CUDA(cudaFuncSetAttribute(k_lambda_soap, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        attr = true;
-    }
-    if (smem > 227 * 1024)
+    if (sizeof(float) * ((size_t)ctx->n_lm * ctx->Q + (size_t)2 * ctx->Q * kmax) > 227 * 1024)
         return set_error(RASCAL_E_UNSUPPORTED, "n_species * n_max * (l_max + 1)^2 too large for the equivariant kernel");
-    k_lambda_soap<<<(unsigned)n_centres, 256, smem, ctx->stream>>>(n_centres, d_coeffs, ctx->Q, ctx->n_lm, kmax, lambda,
-                                                                    mchunk, np, hdr, R, d_out);
+    // row groups of X per chunk: the widest bases leave room for fewer than kLsoapGroups (never below 6: every shape
+    // that passes the check above fits so)
+    const int px = lsoap_px(ctx->l_max), QT = (ctx->Q + 3) / 4;
+    const size_t c_floats = (size_t)QT * (4 * exp_ly(ctx->l_max) + 4);
+    int chunk = std::min((2 * lambda + 1) * QT, kLsoapGroups);
+    while (chunk > 6 && sizeof(float) * (c_floats + (size_t)2 * 4 * chunk * px) > 227 * 1024) --chunk;
+    const size_t smem = sizeof(float) * (c_floats + (size_t)2 * 4 * chunk * px);
+    lsoap_kernel(ctx->Q, ctx->l_max)<<<(unsigned)n_centres, kLsoapThreads, smem, ctx->stream>>>(
+        d_coeffs, ctx->Q, ctx->l_max, lambda, chunk, (unsigned)((0x100000000ull + QT - 1) / QT), np, hdr, R, d_out);
     RASCAL_LAUNCH_CHECK("k_lambda_soap");
     return RASCAL_OK;
 }

@@ -4,8 +4,11 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
+from oracle import lambda_soap as ols  # noqa: E402
 from oracle import mlp as omlp  # noqa: E402
+from oracle import soap as osoap  # noqa: E402
 from synth import mlp_initial_params  # noqa: E402
+from tests.gpu_common import block_rel_err  # noqa: E402
 
 H = 64
 
@@ -49,3 +52,21 @@ def test_training_step_tiles(rg, n_max, l_max, batch):
     order = torch.arange(batch - 1, -1, -1, dtype=torch.int64, device="cuda")
     first = calc.mlp_train(torch.tensor(t, device="cuda"), torch.tensor(y, device="cuda"), order, batch=batch, steps=1)
     assert abs(first.item() - loss_ref) <= 1e-5 * loss_ref
+
+
+# Q = 1, 5, 7, 18 (scalar stores), 36, 256 (16-byte stores); one row group per thread and several, a pair split into
+# chunks of rows with a remainder, the widest basis the kernel takes (its smallest chunk), the top rank. FP32 products
+# of FP32 inputs summed over at most 31 terms, twice: 2e-6 of a block's largest entry, as for the tiny cell.
+@pytest.mark.parametrize("n_max,S,l_max,lam", [(1, 1, 0, 0), (1, 1, 15, 3), (5, 1, 3, 1), (7, 1, 4, 8), (9, 2, 6, 3),
+                                               (12, 3, 5, 2), (16, 16, 12, 1)])
+def test_equivariant_tiles(rg, n_max, S, l_max, lam):
+    import torch
+
+    species = list(range(1, S + 1))
+    calc = rg.SoapCalculator(5.0, 0.5, n_max, l_max, species, spline_intervals=64)
+    h = osoap.Hypers(5.0, 0.5, n_max, l_max, species)
+    n = 2 if S == 16 else 5
+    c = np.random.default_rng(23).standard_normal((n, S, n_max, (l_max + 1) ** 2)).astype(np.float32)
+    T = calc.lambda_soap(torch.tensor(c, device="cuda"), lam)
+    ref = ols.equivariants(c, h, lam)
+    assert block_rel_err(T.cpu().numpy(), ref, 2) <= 2e-6
