@@ -172,6 +172,8 @@ namespace rascal {
 int arena_get(Arena& a, size_t bytes, void** out);
 // Turns device flags into a status (after the stream has been synchronised), then clears them.
 int check_flags(rascal_ctx* ctx);
+// The same for flags that a synchronised kernel has already reported to the host.
+int flags_status(rascal_ctx* ctx, unsigned f);
 
 // round up
 __host__ __device__ inline int64_t div_up(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -196,13 +198,10 @@ inline size_t carve_bytes(Ts... sizes) {
     return s;
 }
 
-// device-wide exclusive scan: out[0..n] with out[n] = total; in and out may alias. Input int32 or int64.
-int scan_exclusive(const int* in, int64_t* out, int64_t n, cudaStream_t stream, Arena& scratch);
-int scan_exclusive(const int64_t* in, int64_t* out, int64_t n, cudaStream_t stream, Arena& scratch);
-// the same with a caller-provided tile-sum buffer of scan_tile_sums_len(n) words (no allocation)
+// device-wide exclusive scan: out[0..n] with out[n] = total, with a caller-provided tile-sum buffer of
+// scan_tile_sums_len(n) words (no allocation)
 int64_t scan_tile_sums_len(int64_t n);
 int scan_exclusive_into(const int* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums);
-int scan_exclusive_into(const int64_t* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums);
 
 int validate_system(const rascal_ctx* ctx, const rascal_system* sys);
 

@@ -52,7 +52,10 @@ int arena_get(Arena& a, size_t bytes, void** out) {
 int check_flags(rascal_ctx* ctx) {
     RASCAL_CUDA(cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
     RASCAL_CUDA(cudaStreamSynchronize(ctx->stream));
-    const unsigned f = *ctx->h_flags;
+    return flags_status(ctx, *ctx->h_flags);
+}
+
+int flags_status(rascal_ctx* ctx, unsigned f) {
     if (f == 0) return RASCAL_OK;
     RASCAL_CUDA(cudaMemsetAsync(ctx->d_flags, 0, sizeof(unsigned), ctx->stream));
     if (f & kFlagSpecies) return set_error(RASCAL_E_ARG, "an atom's species label is not in the hypers' species list");

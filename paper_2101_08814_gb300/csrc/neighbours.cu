@@ -1,15 +1,18 @@
 // Periodic cell-list neighbour search (Appendix B: every j, including periodic replicas, with r_ji < r_cut).
 //
-// Pipeline (all on the context stream):
-//   k_struct_setup      per structure: inverse cell, perpendicular widths, bins >= r_cut(1+1e-6) wide per axis
-//   k_atom_bin          per atom: fractional coordinates, wrap count w, bin, wrapped position p = r - w H split
-//                       into FP32 hi + lo parts, counting-sort rank within the bin
-//   k_atom_scatter      bin-sorted FP32 positions (float4: x, y, z, atom index)
-//   k_struct_thresholds per structure: FP32 classification radii r_cut -+ delta from a rounding-error bound
-//   k_pairs<count>      one warp per centre walks the stencil of bins; counts accepted pairs
-//   scan                CSR offsets
-//   k_pairs<fill>       same walk; accepted (j, n) keys and r_ji vectors staged in shared memory, rank-sorted by
-//                       (j, n1, n2, n3) and written to the centre's CSR segment
+// Pipeline (all on the context stream; seven launches and one synchronisation, which reads the pair count):
+//   k_struct_setup  one warp per structure: inverse cell, perpendicular widths, bins >= r_cut(1+1e-6) wide per axis; the
+//                   bin counters and the work list are cleared beside it
+//   k_atom_bin      per atom: fractional coordinates, wrap count w, bin, wrapped position p = r - w H split into FP32
+//                   hi + lo parts, counting-sort rank within the bin
+//   k_bin_scan      one CTA per structure: bin starts (a structure's atoms are contiguous, so its slots start at its first
+//                   atom), the list of work items (up to item_cap atoms of one bin), FP32 classification radii
+//   k_atom_scatter  bin-sorted FP32 positions (float4: x, y, z, atom index)
+//   k_pairs<count>  one CTA per work item: the candidates of the bin's stencil, shifted to the bin, staged in shared
+//                   memory once for all the item's centres; one warp per centre counts the accepted ones
+//   k_offsets       CSR offsets, and the counts the host reads written straight to its pinned memory
+//   k_pairs<fill>   same walk; accepted (j, n) keys and r_ji vectors sorted by (j, n1, n2, n3) in shared memory and
+//                   written to the centre's CSR segment
 //
 // Bit-exactness with the FP64 definition: a candidate is classified in FP32 from the hi parts. The FP32 error of
 // the displacement is bounded by 3.6e-7 (|p_i|_1 + |p_j|_1 + sum_k |t_k| |h_k|_1); with a 5x margin this gives
@@ -18,6 +21,7 @@
 // operation rounded on its own (__dadd_rn / __dmul_rn, no contraction). The output vector r_ji is computed in
 // double-single arithmetic (error-free FP32 transforms) and rounded once to FP32.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 
 #include "common.cuh"
@@ -32,90 +36,109 @@ struct StructInfo {
     int atom_begin, atom_end;
     float thr_lo2, thr_hi2, thr_tiny2;
     unsigned amax_bits;  // max over atoms of |p_hi|_1, as float bits
+    int wmax;            // max over atoms and axes of |w|
+    int64_t bin_base;    // first of its bins: 2 bins per atom and 8 more are set aside for every structure
 };
 
-constexpr int kPairWarps = 4;     // warps per block in k_pairs
-constexpr int kPairCap = 128;     // pairs a warp sorts in shared memory; larger segments use global scratch
-constexpr int kNoallocCap = 256;  // the same for rascal_neighbours_noalloc, which has no overflow scratch
+constexpr int kPairWarps = 4;      // warps per block in k_pairs
+constexpr int kPairCap = 128;      // pairs a warp sorts in shared memory; larger segments use global scratch
+constexpr int kNoallocCap = 256;   // the same for rascal_neighbours_noalloc, which has no overflow scratch
+constexpr int kPairChunk = 768;    // candidates staged at a time
+constexpr int kPairEntries = 128;  // stencil bins handled at a time (one per thread)
+constexpr int kPairRec = 160;      // accepted candidates a warp collects before it works out their vectors
+constexpr int kPackedWrap = 511;   // largest |w| that the packed form beside atom_lo holds
 
 __device__ inline int floordiv(int a, int b) {
     const int q = a / b;
     return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
 }
+__device__ inline int pack3(int x, int y, int z) { return ((x + 512) << 20) | ((y + 512) << 10) | (z + 512); }
+__device__ inline void unpack3(int c, int& x, int& y, int& z) {
+    x = ((c >> 20) & 1023) - 512;
+    y = ((c >> 10) & 1023) - 512;
+    z = (c & 1023) - 512;
+}
 
+// One warp per structure, an axis (or an element of the inverse) per lane: the FP64 divisions and roots of the three
+// axes run side by side (one thread per structure took 18-20 us in its serial FP64 chain). All threads clear the bin
+// counters, thread 0 the words that the later kernels count in.
 __global__ void k_struct_setup(int n_s, int n_atoms, const int* __restrict__ offs, const double* __restrict__ cells,
-                               const int* __restrict__ pbc, double r_cut, StructInfo* info, int* nbins_out,
-                               unsigned* flags) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_s) return;
-    StructInfo& S = info[s];
-    for (int k = 0; k < 9; ++k) {
-        S.H[k] = cells[9 * s + k];
-        S.hhi[k] = (float)S.H[k];
-        S.hlo[k] = (float)(S.H[k] - (double)S.hhi[k]);
-    }
-    const int a = offs[s], b = offs[s + 1];
-    const bool bad_offsets = (a < 0 || b < a || b > n_atoms);
-    if (bad_offsets) atomicOr(flags, kFlagBadOffsets);
-    S.atom_begin = a;
-    S.atom_end = b;
-    S.amax_bits = 0u;
-    const double* h0 = S.H;
-    const double* h1 = S.H + 3;
-    const double* h2 = S.H + 6;
-    double cr[3][3];  // cr[k] = h_{k+1} x h_{k+2}
-    const double* hs[3] = {h0, h1, h2};
-    for (int k = 0; k < 3; ++k) {
-        const double* u = hs[(k + 1) % 3];
-        const double* v = hs[(k + 2) % 3];
-        cr[k][0] = u[1] * v[2] - u[2] * v[1];
-        cr[k][1] = u[2] * v[0] - u[0] * v[2];
-        cr[k][2] = u[0] * v[1] - u[1] * v[0];
-    }
-    const double det = h0[0] * cr[0][0] + h0[1] * cr[0][1] + h0[2] * cr[0][2];
-    const double scale = norm3d(h0[0], h0[1], h0[2]) * norm3d(h1[0], h1[1], h1[2]) * norm3d(h2[0], h2[1], h2[2]);
-    bool bad = !(fabs(det) > 1e-12 * scale);
-    for (int i = 0; i < 3; ++i)
-        for (int k = 0; k < 3; ++k) S.Hinv[3 * i + k] = bad ? 0.0 : cr[k][i] / det;
-    int nbins = 1;
-    for (int k = 0; k < 3; ++k) {
-        S.pbc[k] = pbc ? (pbc[3 * s + k] != 0) : 1;
-        const double cn = norm3d(cr[k][0], cr[k][1], cr[k][2]);
-        const double w = bad ? 0.0 : fabs(det) / cn;
-        const double rc = r_cut * (1.0 + 1e-6);
+                               const int* __restrict__ pbc, double r_cut, StructInfo* info, int* __restrict__ bin_count,
+                               int64_t nbins_cap, int* __restrict__ words, unsigned* flags) {
+    const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, n_gt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e = gt; e < nbins_cap; e += n_gt) bin_count[e] = 0;
+    if (gt == 0) words[0] = words[1] = 0;
+    const int lane = threadIdx.x & 31, k = lane % 3;
+    for (int64_t s64 = gt >> 5; s64 < n_s; s64 += n_gt >> 5) {
+        const int s = (int)s64;
+        StructInfo& S = info[s];
+        const double* H = cells + 9 * s64;
+        if (lane < 9) {
+            const double h = H[lane];
+            S.H[lane] = h;
+            S.hhi[lane] = (float)h;
+            S.hlo[lane] = (float)(h - (double)(float)h);
+        }
+        const int a = offs[s], b = offs[s + 1];
+        const bool bad_offsets = (a < 0 || b < a || b > n_atoms);
+        // lane k: cr_k = h_{k+1} x h_{k+2}, the axis' own vector and lengths
+        const double *h = H + 3 * k, *u = H + 3 * ((k + 1) % 3), *v = H + 3 * ((k + 2) % 3);
+        const double cr[3] = {u[1] * v[2] - u[2] * v[1], u[2] * v[0] - u[0] * v[2], u[0] * v[1] - u[1] * v[0]};
+        const double det = __shfl_sync(0xffffffffu, h[0] * cr[0] + h[1] * cr[1] + h[2] * cr[2], 0);
+        const double hn = norm3d(h[0], h[1], h[2]), cn = norm3d(cr[0], cr[1], cr[2]);
+        const double scale = __shfl_sync(0xffffffffu, hn, 0) * __shfl_sync(0xffffffffu, hn, 1) * __shfl_sync(0xffffffffu, hn, 2);
+        const bool bad = !(fabs(det) > 1e-12 * scale);
+        {   // Hinv[3 i + k] = cr_k[i] / det
+            const double c0 = __shfl_sync(0xffffffffu, cr[0], k), c1 = __shfl_sync(0xffffffffu, cr[1], k),
+                         c2 = __shfl_sync(0xffffffffu, cr[2], k);
+            const int i = lane / 3;
+            const double ci = i == 0 ? c0 : (i == 1 ? c1 : c2);
+            if (lane < 9) S.Hinv[lane] = bad ? 0.0 : ci / det;
+        }
+        const int periodic = pbc ? (pbc[3 * s64 + k] != 0) : 1;
+        const double w = bad ? 0.0 : fabs(det) / cn, rc = r_cut * (1.0 + 1e-6);
         int nb = 1, reach = 1;
-        if (bad || !(w > 0.0)) {
-            nb = 1;
-            reach = 1;
-        } else {
+        bool thin = false;
+        if (!bad && w > 0.0) {
             nb = (int)fmin(floor(w / rc), 1 << 20);
             if (nb < 1) nb = 1;
-            if (S.pbc[k]) {
-                if (w < r_cut / 64.0) {
-                    atomicOr(flags, kFlagThinCell);
-                    reach = 1;
-                } else {
-                    reach = (int)ceil(rc * nb / w);
-                    if (reach < 1) reach = 1;
-                }
+            if (periodic) {
+                thin = w < r_cut / 64.0;
+                reach = thin ? 1 : (int)ceil(rc * nb / w);
+                if (reach < 1) reach = 1;
             }
         }
-        S.nb[k] = nb;
-        S.reach[k] = reach;
+        int nbs[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) nbs[q] = __shfl_sync(0xffffffffu, nb, q);
+        // cap the bin count at 2 N_s + 8 by halving the finest axis (bins only get wider, reach stays valid)
+        const long cap = bad_offsets ? 1L : 2L * (b - a) + 8;
+        while ((long)nbs[0] * nbs[1] * nbs[2] > cap) {
+            int kk = 0;
+            if (nbs[1] > nbs[kk]) kk = 1;
+            if (nbs[2] > nbs[kk]) kk = 2;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (q == kk) nbs[q] = nbs[q] / 2 > 0 ? nbs[q] / 2 : 1;
+        }
+        if (lane < 3) {
+            S.nb[lane] = lane == 0 ? nbs[0] : (lane == 1 ? nbs[1] : nbs[2]);
+            S.reach[lane] = reach;
+            S.pbc[lane] = periodic;
+            if (thin) atomicOr(flags, kFlagThinCell);
+        }
+        if (lane == 0) {
+            // atoms before the first or past the last offset count as the first or last structure's (find_structure)
+            const int begin = s == 0 ? 0 : a, end = s == n_s - 1 ? n_atoms : b;
+            S.atom_begin = begin;
+            S.atom_end = end;
+            S.bin_base = 2 * (int64_t)begin + 8 * s64;
+            S.amax_bits = 0u;
+            S.wmax = 0;
+            if (bad_offsets) atomicOr(flags, kFlagBadOffsets);
+            if (bad) atomicOr(flags, kFlagGeometry);
+        }
     }
-    if (bad) atomicOr(flags, kFlagGeometry);
-    // cap the bin count at 2 N_s + 8 by halving the finest axis (bins only get wider, reach stays valid)
-    const long cap = bad_offsets ? 1L : 2L * (b - a) + 8;
-    for (;;) {
-        const long prod = (long)S.nb[0] * S.nb[1] * S.nb[2];
-        if (prod <= cap) break;
-        int kk = 0;
-        if (S.nb[1] > S.nb[kk]) kk = 1;
-        if (S.nb[2] > S.nb[kk]) kk = 2;
-        S.nb[kk] = S.nb[kk] / 2 > 0 ? S.nb[kk] / 2 : 1;
-    }
-    nbins = S.nb[0] * S.nb[1] * S.nb[2];
-    nbins_out[s] = nbins;
 }
 
 __device__ inline int find_structure(const int* __restrict__ offs, int n_s, int i) {
@@ -128,93 +151,166 @@ __device__ inline int find_structure(const int* __restrict__ offs, int n_s, int 
     return lo;
 }
 
+// Bound: latency (few FP64 operations per atom). A structure's largest |p|_1 and |w| are found per warp first: one
+// atomicMax per atom on one address took 27 us for a cell of 32 768 atoms.
 __global__ void k_atom_bin(int n_atoms, int n_s, int64_t nbins_cap, const int* __restrict__ offs, const double* __restrict__ pos,
                            const int* __restrict__ species, const int* __restrict__ lut, StructInfo* info,
-                           const int64_t* __restrict__ binbase, int* __restrict__ bin_count, int* __restrict__ atom_bin,
-                           int* __restrict__ atom_rank, int* __restrict__ atom_struct, int4* __restrict__ atom_cell,
+                           int* __restrict__ bin_count, int* __restrict__ atom_bin, int* __restrict__ atom_rank,
                            int4* __restrict__ atom_wrap, float4* __restrict__ atom_hi, float4* __restrict__ atom_lo,
                            unsigned* flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_atoms) return;
-    const int s = find_structure(offs, n_s, i);
+    const bool on = i < n_atoms;
+    const int s = find_structure(offs, n_s, on ? i : n_atoms - 1);
     StructInfo& S = info[s];
-    const double r[3] = {pos[3 * (int64_t)i], pos[3 * (int64_t)i + 1], pos[3 * (int64_t)i + 2]};
-    // a non-finite position is reported; the clamps below keep its bin and wrap count in range, and its FP32
-    // thresholds become NaN, so no pair of its structure is accepted before the call returns the error
-    if (!(isfinite(r[0]) && isfinite(r[1]) && isfinite(r[2]))) atomicOr(flags, kFlagNonFinite);
-    const int lab = species[i];
-    int a = (lab >= 0 && lab < 256) ? lut[lab] : -1;
-    if (a < 0) {
-        atomicOr(flags, kFlagSpecies);
-        a = 0;
-    }
-    int w[3], bc[3];
-    for (int k = 0; k < 3; ++k) {
-        const double sk = r[0] * S.Hinv[k] + r[1] * S.Hinv[3 + k] + r[2] * S.Hinv[6 + k];
-        double f = sk;
-        w[k] = 0;
-        if (S.pbc[k]) {
-            const double fl = floor(sk);
-            w[k] = (int)fmax(fmin(fl, 1e9), -1e9);
-            f = sk - fl;
+    unsigned abits = 0u;
+    int wmax = 0;
+    if (on) {
+        const double r[3] = {pos[3 * (int64_t)i], pos[3 * (int64_t)i + 1], pos[3 * (int64_t)i + 2]};
+        // a non-finite position is reported; the clamps below keep its bin and wrap count in range, and its FP32
+        // thresholds become NaN, so no pair of its structure is accepted before the call returns the error
+        if (!(isfinite(r[0]) && isfinite(r[1]) && isfinite(r[2]))) atomicOr(flags, kFlagNonFinite);
+        const int lab = species[i];
+        if (!(lab >= 0 && lab < 256) || lut[lab] < 0) atomicOr(flags, kFlagSpecies);
+        int w[3], bc[3];
+        for (int k = 0; k < 3; ++k) {
+            const double sk = r[0] * S.Hinv[k] + r[1] * S.Hinv[3 + k] + r[2] * S.Hinv[6 + k];
+            double f = sk;
+            w[k] = 0;
+            if (S.pbc[k]) {
+                const double fl = floor(sk);
+                w[k] = (int)fmax(fmin(fl, 1e9), -1e9);
+                f = sk - fl;
+            }
+            double x = floor(f * S.nb[k]);
+            x = fmin(fmax(x, 0.0), (double)(S.nb[k] - 1));
+            bc[k] = (int)x;
+            wmax = max(wmax, abs(w[k]));
         }
-        double x = floor(f * S.nb[k]);
-        x = fmin(fmax(x, 0.0), (double)(S.nb[k] - 1));
-        bc[k] = (int)x;
+        double p[3];
+        for (int c = 0; c < 3; ++c)
+            p[c] = r[c] - (w[0] * S.H[c] + w[1] * S.H[3 + c] + w[2] * S.H[6 + c]);
+        float hi[3], lo[3];
+        for (int c = 0; c < 3; ++c) {
+            hi[c] = (float)p[c];
+            lo[c] = (float)(p[c] - (double)hi[c]);
+        }
+        const float A = fabsf(hi[0]) + fabsf(hi[1]) + fabsf(hi[2]);
+        abits = __float_as_uint(A);
+        const int64_t gb64 = S.bin_base + (bc[0] * S.nb[1] + bc[1]) * S.nb[2] + bc[2];
+        if (gb64 < 0 || gb64 >= nbins_cap) {  // only reachable with inconsistent structure offsets
+            atomicOr(flags, kFlagBadOffsets);
+            atom_bin[i] = -1;
+            atom_rank[i] = 0;
+        } else {
+            atom_bin[i] = (int)gb64;
+            atom_rank[i] = atomicAdd(&bin_count[gb64], 1);
+        }
+        const bool packs = max(abs(w[0]), max(abs(w[1]), abs(w[2]))) <= kPackedWrap;
+        atom_wrap[i] = make_int4(w[0], w[1], w[2], 0);
+        atom_hi[i] = make_float4(hi[0], hi[1], hi[2], A);
+        atom_lo[i] = make_float4(lo[0], lo[1], lo[2], __int_as_float(packs ? pack3(w[0], w[1], w[2]) : 0));
     }
-    double p[3];
-    for (int c = 0; c < 3; ++c)
-        p[c] = r[c] - (w[0] * S.H[c] + w[1] * S.H[3 + c] + w[2] * S.H[6 + c]);
-    float hi[3], lo[3];
-    for (int c = 0; c < 3; ++c) {
-        hi[c] = (float)p[c];
-        lo[c] = (float)(p[c] - (double)hi[c]);
+    const int s0 = __shfl_sync(0xffffffffu, s, 0);
+    if (__all_sync(0xffffffffu, s == s0)) {
+        abits = __reduce_max_sync(0xffffffffu, abits);
+        wmax = __reduce_max_sync(0xffffffffu, wmax);
+        if ((threadIdx.x & 31) != 0) return;
     }
-    const float A = fabsf(hi[0]) + fabsf(hi[1]) + fabsf(hi[2]);
-    atomicMax(&S.amax_bits, __float_as_uint(A));
-    const int local = (bc[0] * S.nb[1] + bc[1]) * S.nb[2] + bc[2];
-    const int64_t gb64 = binbase[s] + local;
-    if (gb64 < 0 || gb64 >= nbins_cap) {  // only reachable with inconsistent structure offsets
-        atomicOr(flags, kFlagBadOffsets);
-        atom_bin[i] = -1;
-        atom_rank[i] = 0;
-    } else {
-        atom_bin[i] = (int)gb64;
-        atom_rank[i] = atomicAdd(&bin_count[gb64], 1);
+    if (abits) atomicMax(&S.amax_bits, abits);
+    if (wmax) atomicMax(&S.wmax, wmax);
+}
+
+// One CTA per structure: slots of its bins (atom_begin + exclusive prefix of the bin counts), one work item
+// {structure, bin, first slot, atoms} per item_cap atoms of a bin, as equal as possible, and the classification radii.
+// The count of a bin and of its items travel in the two halves of one word through the scan.
+constexpr int kBinScanThreads = 512;
+__global__ void __launch_bounds__(kBinScanThreads) k_bin_scan(int n_s, int n_atoms, double r_cut, int item_cap, StructInfo* info,
+                                                              const int* __restrict__ bin_count,
+                                                              int* __restrict__ bin_start, int4* __restrict__ items,
+                                                              int* __restrict__ words, const unsigned* __restrict__ flags) {
+    __shared__ int64_t warp_tot[kBinScanThreads / 32];
+    __shared__ int64_t s_total;
+    __shared__ int s_pos;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (*flags & kFlagBadOffsets) return;  // the bins may be inconsistent: no item, so no later kernel touches an atom
+    for (int s = blockIdx.x; s < n_s; s += gridDim.x) {
+        StructInfo& S = info[s];
+        if (tid == 0) {
+            const double amax = (double)__uint_as_float(S.amax_bits);
+            double tmax = 0.0;
+            for (int k = 0; k < 3; ++k) {
+                const double hk = fabs((double)S.hhi[3 * k]) + fabs((double)S.hhi[3 * k + 1]) + fabs((double)S.hhi[3 * k + 2]);
+                tmax += (S.reach[k] + 1) * hk;
+            }
+            const double delta = 2e-6 * (2.0 * amax + tmax) + 1e-6 * r_cut;
+            const double lo = fmax(r_cut - delta, 0.0), hi = r_cut + delta;
+            S.thr_lo2 = (float)(lo * lo);
+            S.thr_hi2 = (float)(hi * hi);
+            const double tiny = 1e-3 + delta;
+            S.thr_tiny2 = (float)(tiny * tiny);
+        }
+        const int nbins = S.nb[0] * S.nb[1] * S.nb[2];
+        const int64_t base = S.bin_base;
+        int start = S.atom_begin;
+        for (int b0 = 0; b0 < nbins; b0 += 2 * kBinScanThreads) {
+            int n[2], ni[2];
+            int64_t own = 0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int b = b0 + 2 * tid + q;
+                n[q] = b < nbins ? bin_count[base + b] : 0;
+                ni[q] = (n[q] + item_cap - 1) / item_cap;
+                own += ((int64_t)ni[q] << 32) + n[q];
+            }
+            int64_t x = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) warp_tot[warp] = x;
+            __syncthreads();
+            if (warp == 0) {
+                int64_t t = lane < kBinScanThreads / 32 ? warp_tot[lane] : 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int64_t y = __shfl_up_sync(0xffffffffu, t, o);
+                    if (lane >= o) t += y;
+                }
+                if (lane < kBinScanThreads / 32) warp_tot[lane] = t;
+                if (lane == kBinScanThreads / 32 - 1) {
+                    s_total = t;
+                    s_pos = atomicAdd(words, (int)(t >> 32));
+                }
+            }
+            __syncthreads();
+            const int64_t before = (warp ? warp_tot[warp - 1] : 0) + x - own;
+            int slot = start + (int)(before & 0xffffffff), pos = s_pos + (int)(before >> 32);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int b = b0 + 2 * tid + q;
+                if (b < nbins) bin_start[base + b] = slot;
+                for (int k = 0; k < ni[q]; ++k) {
+                    const int lo = (int)((int64_t)n[q] * k / ni[q]), hi = (int)((int64_t)n[q] * (k + 1) / ni[q]);
+                    if (pos < n_atoms) items[pos] = make_int4(s, b, slot + lo, hi - lo);
+                    ++pos;
+                }
+                slot += n[q];
+            }
+            start += (int)(s_total & 0xffffffff);
+            __syncthreads();
+        }
     }
-    atom_struct[i] = s;
-    atom_cell[i] = make_int4(bc[0], bc[1], bc[2], a);
-    atom_wrap[i] = make_int4(w[0], w[1], w[2], 0);
-    atom_hi[i] = make_float4(hi[0], hi[1], hi[2], A);
-    atom_lo[i] = make_float4(lo[0], lo[1], lo[2], 0.0f);
 }
 
 __global__ void k_atom_scatter(int n_atoms, const int* __restrict__ atom_bin, const int* __restrict__ atom_rank,
-                               const int64_t* __restrict__ bin_start, const float4* __restrict__ atom_hi,
-                               float4* __restrict__ sorted_hi) {
+                               const int* __restrict__ bin_start, const float4* __restrict__ atom_hi,
+                               float4* __restrict__ sorted_hi, const unsigned* __restrict__ flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_atoms || atom_bin[i] < 0) return;
-    const int64_t slot = bin_start[atom_bin[i]] + atom_rank[i];
+    if (i >= n_atoms || atom_bin[i] < 0 || (*flags & kFlagBadOffsets)) return;
+    const int slot = bin_start[atom_bin[i]] + atom_rank[i];
     const float4 h = atom_hi[i];
     sorted_hi[slot] = make_float4(h.x, h.y, h.z, __int_as_float(i));
-}
-
-__global__ void k_struct_thresholds(int n_s, double r_cut, StructInfo* info) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_s) return;
-    StructInfo& S = info[s];
-    const double amax = (double)__uint_as_float(S.amax_bits);
-    double tmax = 0.0;
-    for (int k = 0; k < 3; ++k) {
-        const double hk = fabs((double)S.hhi[3 * k]) + fabs((double)S.hhi[3 * k + 1]) + fabs((double)S.hhi[3 * k + 2]);
-        tmax += (S.reach[k] + 1) * hk;
-    }
-    const double delta = 2e-6 * (2.0 * amax + tmax) + 1e-6 * r_cut;
-    const double lo = fmax(r_cut - delta, 0.0), hi = r_cut + delta;
-    S.thr_lo2 = (float)(lo * lo);
-    S.thr_hi2 = (float)(hi * hi);
-    const double tiny = 1e-3 + delta;
-    S.thr_tiny2 = (float)(tiny * tiny);
 }
 
 __device__ inline void two_sum(float a, float b, float& s, float& e) {
@@ -246,247 +342,468 @@ __device__ inline uint64_t pair_key(int j, const int n[3]) {
            (uint64_t)(n[2] + 512);
 }
 
-// CAP: pairs a warp sorts in shared memory (8 blocks of 4 warps per SM at CAP = 128)
+struct PairArgs {
+    int n_atoms;
+    const double* pos;
+    const StructInfo* info;
+    const int* bin_count;
+    const int* bin_start;
+    const float4* sorted_hi;
+    const int4* atom_wrap;
+    const float4* atom_lo;
+    const int4* items;
+    int* words;              // [0] number of work items, [1] largest count of a centre
+    double rc2;
+    int* counts;             // count: pairs per centre
+    const int64_t* offsets;  // fill
+    int* out_j;
+    int* out_shift;
+    float4* out_rij;
+    uint64_t* ovf_keys;
+    float4* ovf_vec;
+    unsigned* flags;
+};
+
+// One CTA per work item (persistent: CTAs stride over the list). All centres of an item share their bin's stencil: its
+// candidates are staged once, already shifted to the bin's image (x + T), so that a warp's test of 32 candidates for one
+// centre is a 16-byte shared load, six FP32 operations and a ballot. (One warp per centre that walked the stencil itself
+// spent about 1 400 warp instructions per centre on locating and loading candidates, twice, and waited for them in L2:
+// 124 us counting and 206 us filling 1.80 M pairs of 70 820 centres; now PAIRS_COUNT and PAIRS_FILL us.) Items of more than
+// kPairChunk candidates, or whose stencil has more than kPairEntries bins, restage chunk by chunk for every four centres.
+// CAP: pairs a warp sorts in shared memory.
 template <bool FILL, int CAP = kPairCap>
-__global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? 8 : 0) k_pairs(
-    int n_atoms, const double* __restrict__ pos, const StructInfo* __restrict__ info, const int64_t* __restrict__ binbase,
-    const int64_t* __restrict__ bin_start, const float4* __restrict__ sorted_hi, const int* __restrict__ atom_struct,
-    const int4* __restrict__ atom_cell, const int4* __restrict__ atom_wrap, const float4* __restrict__ atom_hi,
-    const float4* __restrict__ atom_lo, double rc2, int64_t nbins_cap, int64_t* __restrict__ counts_or_offsets, int* __restrict__ max_count,
-    int* __restrict__ out_j, int* __restrict__ out_shift, float4* __restrict__ out_rij, uint64_t* __restrict__ ovf_keys,
-    float4* __restrict__ ovf_vec, unsigned* flags) {
-    constexpr int kPairEPL = CAP / 32;
+__global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) : 0) k_pairs(const PairArgs A) {
+    constexpr int kEPL = CAP / 32, kThreads = kPairWarps * 32;
+    __shared__ float4 s_c[kPairChunk];             // x + T, y + T, z + T, j (t = 0) or ~j (another image)
+    __shared__ unsigned char s_e[kPairChunk];      // the candidate's stencil entry
+    __shared__ int s_pref[kPairEntries], s_beg[kPairEntries], s_t[kPairEntries];
+    __shared__ float4 s_T[kPairEntries];
+    __shared__ float4 s_Th[FILL ? kPairEntries : 1], s_Tl[FILL ? kPairEntries : 1];
+    __shared__ int s_wtot[kPairWarps];
     __shared__ uint64_t s_keys[FILL ? kPairWarps * CAP : 1];
     __shared__ float4 s_vec[FILL ? kPairWarps * CAP : 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * kPairWarps + warp;
-    if (i >= n_atoms) return;
-    const int s = atom_struct[i];
-    const StructInfo& S = info[s];
-    const int4 cell = atom_cell[i];
-    const int4 wi = atom_wrap[i];
-    const float4 phi = atom_hi[i];
-    const float4 plo = atom_lo[i];
-    const float thr_lo2 = S.thr_lo2, thr_hi2 = S.thr_hi2, thr_tiny2 = S.thr_tiny2;
-    const int bci[3] = {cell.x, cell.y, cell.z};
-    int64_t seg_beg = 0, seg_cnt = 0;
-    uint64_t* keys = s_keys + warp * CAP;
-    float4* vecs = s_vec + warp * CAP;
-    bool use_global = false;
-    if (FILL) {
-        seg_beg = counts_or_offsets[i];
-        seg_cnt = counts_or_offsets[i + 1] - seg_beg;
-        if (seg_cnt > CAP) {
-            use_global = true;
-            keys = ovf_keys + seg_beg;
-            vecs = ovf_vec + seg_beg;
-        }
-    }
-    int count = 0;
+    __shared__ unsigned short s_rec[FILL ? kPairWarps * kPairRec : 1];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_work = min(A.words[0], A.n_atoms);
     unsigned local_flags = 0;
-    // Flattened walk over the stencil: up to 32 stencil bins at a time, one per lane, their candidate counts
-    // prefix-summed across the warp, then 32 candidates per iteration with each lane locating its bin by a
-    // binary search over the prefix (all loop bounds warp-uniform).
-    __shared__ int64_t s_beg[kPairWarps][32];
-    __shared__ int4 s_t[kPairWarps][32];
-    __shared__ float4 s_T[kPairWarps][32];
-    __shared__ float4 s_Th[kPairWarps][FILL ? 32 : 1];
-    __shared__ float4 s_Tl[kPairWarps][FILL ? 32 : 1];
-    const int w0 = 2 * S.reach[0] + 1, w1 = 2 * S.reach[1] + 1, w2 = 2 * S.reach[2] + 1;
-    const int n_st = w0 * w1 * w2;
-    for (int g0 = 0; g0 < n_st; g0 += 32) {
-        const int e = g0 + lane;
-        int cnt = 0;
-        if (e < n_st) {
-            const int dd[3] = {e / (w1 * w2) - S.reach[0], (e / w2) % w1 - S.reach[1], e % w2 - S.reach[2]};
-            int tb[3], t[3];
-            bool valid = true;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int x = bci[k] + dd[k];
-                if (S.pbc[k]) {
-                    t[k] = floordiv(x, S.nb[k]);
-                    tb[k] = x - t[k] * S.nb[k];
-                } else {
-                    t[k] = 0;
-                    tb[k] = x;
-                    if (x < 0 || x >= S.nb[k]) valid = false;
+    int local_max = 0;
+    for (int work = blockIdx.x; work < n_work; work += gridDim.x) {
+        const int4 item = A.items[work];
+        const StructInfo& S = A.info[item.x];
+        const int nb0 = S.nb[0], nb1 = S.nb[1], nb2 = S.nb[2], r0 = S.reach[0], r1 = S.reach[1], r2 = S.reach[2];
+        const int w1 = 2 * r1 + 1, w2 = 2 * r2 + 1, n_st = (2 * r0 + 1) * w1 * w2;
+        const int bz = item.y % nb2, by = (item.y / nb2) % nb1, bx = item.y / (nb2 * nb1);
+        const float thr_lo2 = S.thr_lo2, thr_hi2 = S.thr_hi2, thr_tiny2 = S.thr_tiny2;
+        const bool packed = S.wmax <= kPackedWrap;
+        // |n| <= 2 wmax + |t|: only where this can pass the key's range is a pair's shift checked
+        const int tmax = max((r0 + nb0 - 1) / nb0, max((r1 + nb1 - 1) / nb1, (r2 + nb2 - 1) / nb2)) + 1;
+        const bool wide = S.wmax > kMaxShift || 2 * S.wmax + tmax > kMaxShift;
+        int staged = -1;  // first entry of the batch whose tables are in shared memory, if its candidates fill one chunk
+        int n_staged = 0;
+        // wrap counts of atom j
+        auto wrap_of = [&](int j, int& x, int& y, int& z) {
+            const int4 w = A.atom_wrap[j];
+            x = w.x;
+            y = w.y;
+            z = w.z;
+        };
+        const int rounds = (item.w + kPairWarps - 1) / kPairWarps;
+        for (int round = 0; round < rounds; ++round) {
+            const int cidx = round * kPairWarps + warp;
+            const bool mine = cidx < item.w;  // warp-uniform
+            const float4 phi = A.sorted_hi[item.z + (mine ? cidx : 0)];
+            const int i = __float_as_int(phi.w);
+            float4 plo = make_float4(0.f, 0.f, 0.f, 0.f);
+            int64_t seg_beg = 0, seg_cnt = 0;
+            uint64_t* keys = s_keys + (FILL ? warp * CAP : 0);
+            float4* vecs = s_vec + (FILL ? warp * CAP : 0);
+            if (FILL) {
+                plo = A.atom_lo[i];
+                seg_beg = A.offsets[i];
+                seg_cnt = A.offsets[i + 1] - seg_beg;
+                if (seg_cnt > CAP) {
+                    keys = A.ovf_keys + seg_beg;
+                    vecs = A.ovf_vec + seg_beg;
                 }
             }
-            const int64_t bin = binbase[s] + (tb[0] * S.nb[1] + tb[1]) * S.nb[2] + tb[2];
-            if (bin < 0 || bin >= nbins_cap) valid = false;  // inconsistent offsets, already flagged
-            if (valid) {
-                const int64_t beg = bin_start[bin];
-                cnt = (int)(bin_start[bin + 1] - beg);
-                s_beg[warp][lane] = beg;
-                s_t[warp][lane] = make_int4(t[0], t[1], t[2], (t[0] == 0 && t[1] == 0 && t[2] == 0) ? 1 : 0);
-                float Tf[3];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    // explicit roundings: the count and fill passes must take identical decisions
-                    Tf[c] = __fadd_rn(__fadd_rn(__fmul_rn((float)t[0], S.hhi[c]), __fmul_rn((float)t[1], S.hhi[3 + c])),
-                                      __fmul_rn((float)t[2], S.hhi[6 + c]));
-                }
-                s_T[warp][lane] = make_float4(Tf[0], Tf[1], Tf[2], 0.0f);
-                if (FILL) {
-                    float Th[3], Tl[3];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        float sh = 0.0f, sl = 0.0f;
+            int wix, wiy, wiz;
+            if (packed && FILL) unpack3(__float_as_int(plo.w), wix, wiy, wiz);
+            else wrap_of(i, wix, wiy, wiz);
+            int count = 0;  // accepted so far
+            int done = 0;   // of those, with vectors worked out (fill)
+            for (int e0 = 0; e0 < n_st; e0 += kPairEntries) {
+                int total = n_staged;
+                if (staged != e0) {
+                    // tables of up to kPairEntries stencil bins, one per thread: candidates, first slot, image shift
+                    __syncthreads();
+                    const int e = e0 + tid;
+                    int cnt = 0;
+                    if (e < n_st) {
+                        const int ex = e / (w1 * w2), er = e - ex * w1 * w2, ey = er / w2;
+                        const int xs[3] = {bx + ex - r0, by + ey - r1, bz + (er - ey * w2) - r2}, nbs[3] = {nb0, nb1, nb2};
+                        int tb[3], t[3];
+                        bool valid = true;
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            float pp, pe, s2, e2;
-                            two_prod((float)t[k], S.hhi[3 * k + c], pp, pe);
-                            pe += (float)t[k] * S.hlo[3 * k + c];
-                            two_sum(sh, pp, s2, e2);
-                            sh = s2;
-                            sl += pe + e2;
+                            tb[k] = xs[k];
+                            t[k] = 0;
+                            if (S.pbc[k]) {
+                                if (xs[k] < 0 || xs[k] >= nbs[k]) {
+                                    t[k] = floordiv(xs[k], nbs[k]);
+                                    tb[k] = xs[k] - t[k] * nbs[k];
+                                }
+                            } else if (xs[k] < 0 || xs[k] >= nbs[k]) {
+                                valid = false;
+                            }
                         }
-                        Th[c] = sh;
-                        Tl[c] = sl;
-                    }
-                    s_Th[warp][FILL ? lane : 0] = make_float4(Th[0], Th[1], Th[2], 0.0f);
-                    s_Tl[warp][FILL ? lane : 0] = make_float4(Tl[0], Tl[1], Tl[2], 0.0f);
-                }
-            }
-        }
-        int incl = cnt;
+                        if (valid) {
+                            const int64_t bin = S.bin_base + (tb[0] * nb1 + tb[1]) * nb2 + tb[2];
+                            s_beg[tid] = A.bin_start[bin];
+                            cnt = A.bin_count[bin];
+                            s_t[tid] = pack3(t[0], t[1], t[2]);
+                            float Tf[3];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        __syncwarp();
-        for (int base = 0; base < total; base += 32) {
-            const int cidx = base + lane;
-            // entry k of this candidate: number of entries whose inclusive prefix is <= cidx
-            int k = 0;
+                            for (int c = 0; c < 3; ++c) {
+                                // explicit roundings: the count and fill passes must take identical decisions
+                                Tf[c] = __fadd_rn(__fadd_rn(__fmul_rn((float)t[0], S.hhi[c]), __fmul_rn((float)t[1], S.hhi[3 + c])),
+                                                  __fmul_rn((float)t[2], S.hhi[6 + c]));
+                            }
+                            s_T[tid] = make_float4(Tf[0], Tf[1], Tf[2], (t[0] | t[1] | t[2]) == 0 ? 1.0f : 0.0f);
+                            if (FILL) {
+                                float Th[3], Tl[3];
 #pragma unroll
-            for (int st = 16; st >= 1; st >>= 1) {
-                const int v = __shfl_sync(0xffffffffu, incl, k + st - 1);
-                if (v <= cidx) k += st;
-            }
-            const int excl_k = __shfl_sync(0xffffffffu, incl, k) - __shfl_sync(0xffffffffu, cnt, k);
-            bool accept = false;
-            int j = -1;
-            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-            int4 tt = make_int4(0, 0, 0, 0);
-            if (cidx < total) {
-                tt = s_t[warp][k];
-                const float4 Tf = s_T[warp][k];
-                q = sorted_hi[s_beg[warp][k] + (cidx - excl_k)];
-                j = __float_as_int(q.w);
-                const float dx = __fsub_rn(__fadd_rn(q.x, Tf.x), phi.x);
-                const float dy = __fsub_rn(__fadd_rn(q.y, Tf.y), phi.y);
-                const float dz = __fsub_rn(__fadd_rn(q.z, Tf.z), phi.z);
-                const float dsq = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
-                if (!(j == i && tt.w)) {
-                    if (dsq < thr_lo2) {
-                        accept = true;
-                    } else if (dsq <= thr_hi2) {
-                        const int4 wj = atom_wrap[j];
-                        const int n[3] = {tt.x - wj.x + wi.x, tt.y - wj.y + wi.y, tt.z - wj.z + wi.z};
-                        accept = exact_d2(pos, i, j, S.H, n) < rc2;
-                    }
-                    if (accept && dsq < thr_tiny2) {
-                        const int4 wj = atom_wrap[j];
-                        const int n[3] = {tt.x - wj.x + wi.x, tt.y - wj.y + wi.y, tt.z - wj.z + wi.z};
-                        if (exact_d2(pos, i, j, S.H, n) < 1e-12) local_flags |= kFlagGeometry;
-                    }
-                }
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, accept);
-            if (accept) {
-                const int4 wj = atom_wrap[j];
-                const int n[3] = {tt.x - wj.x + wi.x, tt.y - wj.y + wi.y, tt.z - wj.z + wi.z};
-                if (n[0] < -kMaxShift || n[0] > kMaxShift || n[1] < -kMaxShift || n[1] > kMaxShift || n[2] < -kMaxShift ||
-                    n[2] > kMaxShift)
-                    local_flags |= kFlagShiftRange;
-                if (FILL) {
-                    const int slot = count + __popc(m & ((1u << lane) - 1u));
-                    if (slot < seg_cnt) {
-                        const float4 qlo = atom_lo[j];
-                        const float4 Th4 = s_Th[warp][FILL ? k : 0], Tl4 = s_Tl[warp][FILL ? k : 0];
-                        const float Th[3] = {Th4.x, Th4.y, Th4.z}, Tl[3] = {Tl4.x, Tl4.y, Tl4.z};
-                        const float pj[3] = {q.x, q.y, q.z}, pjl[3] = {qlo.x, qlo.y, qlo.z};
-                        const float pi_[3] = {phi.x, phi.y, phi.z}, pil[3] = {plo.x, plo.y, plo.z};
-                        float v[3];
+                                for (int c = 0; c < 3; ++c) {
+                                    float sh = 0.0f, sl = 0.0f;
 #pragma unroll
-                        for (int cc = 0; cc < 3; ++cc) {
-                            float s1, e1, s2, e2;
-                            two_sum(pj[cc], Th[cc], s1, e1);
-                            e1 += pjl[cc] + Tl[cc];
-                            two_sum(s1, -pi_[cc], s2, e2);
-                            e2 += e1 - pil[cc];
-                            v[cc] = s2 + e2;
+                                    for (int k = 0; k < 3; ++k) {
+                                        float pp, pe, s2, e2;
+                                        two_prod((float)t[k], S.hhi[3 * k + c], pp, pe);
+                                        pe += (float)t[k] * S.hlo[3 * k + c];
+                                        two_sum(sh, pp, s2, e2);
+                                        sh = s2;
+                                        sl += pe + e2;
+                                    }
+                                    Th[c] = sh;
+                                    Tl[c] = sl;
+                                }
+                                s_Th[FILL ? tid : 0] = make_float4(Th[0], Th[1], Th[2], 0.0f);
+                                s_Tl[FILL ? tid : 0] = make_float4(Tl[0], Tl[1], Tl[2], 0.0f);
+                            }
                         }
-                        const float rr = sqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-                        const int nc[3] = {min(max(n[0], -kMaxShift), kMaxShift), min(max(n[1], -kMaxShift), kMaxShift),
-                                           min(max(n[2], -kMaxShift), kMaxShift)};
-                        keys[slot] = pair_key(j, nc);
-                        vecs[slot] = make_float4(v[0], v[1], v[2], rr);
+                    }
+                    int incl = cnt;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += y;
+                    }
+                    if (lane == 31) s_wtot[warp] = incl;
+                    __syncthreads();
+                    total = 0;
+#pragma unroll
+                    for (int w = 0; w < kPairWarps; ++w) {
+                        if (w < warp) incl += s_wtot[w];
+                        total += s_wtot[w];
+                    }
+                    s_pref[tid] = incl;
+                    __syncthreads();
+                }
+                for (int c0 = 0; c0 < total; c0 += kPairChunk) {
+                    const int nc = min(kPairChunk, total - c0);
+                    if (staged != e0) {
+                        if (c0 > 0) __syncthreads();  // the previous chunk is done with
+                        for (int c = tid; c < nc; c += kThreads) {
+                            // entry of this candidate: the number of entries whose inclusive prefix is <= its index
+                            int k = 0;
+#pragma unroll
+                            for (int st = kPairEntries / 2; st >= 1; st >>= 1)
+                                if (s_pref[k + st - 1] <= c0 + c) k += st;
+                            const int first = k ? s_pref[k - 1] : 0;
+                            const float4 q = A.sorted_hi[s_beg[k] + (c0 + c - first)];
+                            const float4 T = s_T[k];
+                            const int j = __float_as_int(q.w);
+                            s_c[c] = make_float4(__fadd_rn(q.x, T.x), __fadd_rn(q.y, T.y), __fadd_rn(q.z, T.z),
+                                                 __int_as_float(T.w != 0.0f ? j : ~j));
+                            s_e[c] = (unsigned char)k;
+                        }
+                        __syncthreads();
+                    }
+                    if (mine) {
+                        // vectors and keys of the collected candidates [done, count)
+                        auto flush = [&]() {
+                            __syncwarp();
+                            for (int r = done + lane; r < count; r += 32) {
+                                const int c = s_rec[FILL ? warp * kPairRec + (r - done) : 0], k = s_e[c];
+                                const int w = __float_as_int(s_c[c].w), j = w < 0 ? ~w : w;
+                                const float4 q = A.sorted_hi[s_beg[k] + (c0 + c - (k ? s_pref[k - 1] : 0))];
+                                const float4 qlo = A.atom_lo[j];
+                                int t[3], wj[3];
+                                unpack3(s_t[k], t[0], t[1], t[2]);
+                                if (packed) unpack3(__float_as_int(qlo.w), wj[0], wj[1], wj[2]);
+                                else wrap_of(j, wj[0], wj[1], wj[2]);
+                                const int n[3] = {min(max(t[0] - wj[0] + wix, -kMaxShift), kMaxShift),
+                                                  min(max(t[1] - wj[1] + wiy, -kMaxShift), kMaxShift),
+                                                  min(max(t[2] - wj[2] + wiz, -kMaxShift), kMaxShift)};
+                                const float4 Th4 = s_Th[FILL ? k : 0], Tl4 = s_Tl[FILL ? k : 0];
+                                const float Th[3] = {Th4.x, Th4.y, Th4.z}, Tl[3] = {Tl4.x, Tl4.y, Tl4.z};
+                                const float pj[3] = {q.x, q.y, q.z}, pjl[3] = {qlo.x, qlo.y, qlo.z};
+                                const float pi_[3] = {phi.x, phi.y, phi.z}, pil[3] = {plo.x, plo.y, plo.z};
+                                float v[3];
+#pragma unroll
+                                for (int cc = 0; cc < 3; ++cc) {
+                                    float s1, e1, s2, e2;
+                                    two_sum(pj[cc], Th[cc], s1, e1);
+                                    e1 += pjl[cc] + Tl[cc];
+                                    two_sum(s1, -pi_[cc], s2, e2);
+                                    e2 += e1 - pil[cc];
+                                    v[cc] = s2 + e2;
+                                }
+                                const float rr = sqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+                                if (r < seg_cnt) {
+                                    keys[r] = pair_key(j, n);
+                                    vecs[r] = make_float4(v[0], v[1], v[2], rr);
+                                }
+                            }
+                            __syncwarp();
+                            done = count;
+                        };
+#pragma unroll 2
+                        for (int base = 0; base < nc; base += 32) {
+                            const float4 c = s_c[min(base + lane, kPairChunk - 1)];
+                            const float dx = __fsub_rn(c.x, phi.x), dy = __fsub_rn(c.y, phi.y), dz = __fsub_rn(c.z, phi.z);
+                            const float dsq = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
+                            const int w = __float_as_int(c.w);
+                            const bool on = base + lane < nc && w != i;
+                            bool accept = on && dsq < thr_lo2;
+                            if (__any_sync(0xffffffffu, on && dsq <= thr_hi2 && (!accept || dsq < thr_tiny2 || wide))) {
+                                const int j = w < 0 ? ~w : w;
+                                if (on && dsq <= thr_hi2) {
+                                    int wjx, wjy, wjz, tx, ty, tz;
+                                    wrap_of(j, wjx, wjy, wjz);
+                                    int vx, vy, vz;
+                                    wrap_of(i, vx, vy, vz);
+                                    unpack3(s_t[s_e[base + lane]], tx, ty, tz);
+                                    const int n[3] = {tx - wjx + vx, ty - wjy + vy, tz - wjz + vz};
+                                    if (!accept) accept = exact_d2(A.pos, i, j, S.H, n) < A.rc2;
+                                    if (accept && dsq < thr_tiny2 && exact_d2(A.pos, i, j, S.H, n) < 1e-12)
+                                        local_flags |= kFlagGeometry;
+                                    if (accept && (n[0] < -kMaxShift || n[0] > kMaxShift || n[1] < -kMaxShift ||
+                                                   n[1] > kMaxShift || n[2] < -kMaxShift || n[2] > kMaxShift))
+                                        local_flags |= kFlagShiftRange;
+                                }
+                            }
+                            const unsigned m = __ballot_sync(0xffffffffu, accept);
+                            if (FILL) {
+                                if (accept)
+                                    s_rec[FILL ? warp * kPairRec + (count - done) + __popc(m & ((1u << lane) - 1u)) : 0] =
+                                        (unsigned short)(base + lane);
+                                count += __popc(m);
+                                if (count - done > kPairRec - 32) flush();
+                            } else {
+                                count += __popc(m);
+                            }
+                        }
+                        if (FILL) flush();  // the records point into this chunk
                     }
                 }
+                if (staged != e0) {
+                    // the whole stencil fits one batch and one chunk: the item's other centres find it staged
+                    const bool keep = n_st <= kPairEntries && total <= kPairChunk;
+                    staged = keep ? e0 : -1;
+                    n_staged = total;
+                }
             }
-            count += __popc(m);
-        }
-        __syncwarp();
-    }
-    if (local_flags) atomicOr(flags, local_flags);
-    if (!FILL) {
-        if (lane == 0) {
-            counts_or_offsets[i] = count;
-            atomicMax(max_count, count);
-        }
-        return;
-    }
-    // rank sort of the segment by (j, n1, n2, n3) and write-out
-    __syncwarp();
-    const int k = (int)(seg_cnt < (int64_t)count ? seg_cnt : (int64_t)count);
-    if (!use_global) {
-        uint64_t mykey[kPairEPL];
-        int myrank[kPairEPL];
-#pragma unroll
-        for (int qd = 0; qd < kPairEPL; ++qd) {
-            const int e = lane + 32 * qd;
-            mykey[qd] = (e < k) ? keys[e] : ~0ull;
-            myrank[qd] = 0;
-        }
-        const int nq = (k + 31) / 32;
-        for (int f = 0; f < k; ++f) {
-            const uint64_t kf = keys[f];
-#pragma unroll
-            for (int qd = 0; qd < kPairEPL; ++qd)
-                if (qd < nq) myrank[qd] += (kf < mykey[qd]);
-        }
-#pragma unroll
-        for (int qd = 0; qd < kPairEPL; ++qd) {
-            const int e = lane + 32 * qd;
-            if (e < k) {
-                const int64_t o = seg_beg + myrank[qd];
-                const uint64_t key = mykey[qd];
-                out_j[o] = (int)(key >> 30);
-                out_shift[3 * o + 0] = (int)((key >> 20) & 1023) - 512;
-                out_shift[3 * o + 1] = (int)((key >> 10) & 1023) - 512;
-                out_shift[3 * o + 2] = (int)(key & 1023) - 512;
-                out_rij[o] = vecs[e];
+            if (!mine) continue;
+            if (!FILL) {
+                if (lane == 0) A.counts[i] = count;
+                local_max = max(local_max, count);
+                continue;
             }
+            // rank sort of the segment by (j, n1, n2, n3) and write-out
+            __syncwarp();
+            const int k = (int)(seg_cnt < (int64_t)count ? seg_cnt : (int64_t)count);
+            auto write = [&](int e, uint64_t key, int rank) {
+                const int64_t o = seg_beg + rank;
+                A.out_j[o] = (int)(key >> 30);
+                A.out_shift[3 * o + 0] = (int)((key >> 20) & 1023) - 512;
+                A.out_shift[3 * o + 1] = (int)((key >> 10) & 1023) - 512;
+                A.out_shift[3 * o + 2] = (int)(key & 1023) - 512;
+                A.out_rij[o] = vecs[e];
+            };
+            if (seg_cnt <= CAP) {
+                uint64_t mykey[kEPL];
+                int myrank[kEPL];
+#pragma unroll
+                for (int qd = 0; qd < kEPL; ++qd) {
+                    const int e = lane + 32 * qd;
+                    mykey[qd] = (e < k) ? keys[e] : ~0ull;
+                    myrank[qd] = 0;
+                }
+                const int nq = (k + 31) / 32;
+                for (int f = 0; f < k; ++f) {
+                    const uint64_t kf = keys[f];
+#pragma unroll
+                    for (int qd = 0; qd < kEPL; ++qd)
+                        if (qd < nq) myrank[qd] += (kf < mykey[qd]);
+                }
+#pragma unroll
+                for (int qd = 0; qd < kEPL; ++qd)
+                    if (lane + 32 * qd < k) write(lane + 32 * qd, mykey[qd], myrank[qd]);
+            } else {
+                __threadfence_block();
+                for (int e = lane; e < k; e += 32) {
+                    const uint64_t key = keys[e];
+                    int rank = 0;
+                    for (int f = 0; f < k; ++f) rank += (keys[f] < key);
+                    write(e, key, rank);
+                }
+            }
+            __syncwarp();
         }
+        __syncthreads();  // the next item's tables overwrite this one's
+    }
+    if (local_flags) atomicOr(A.flags, local_flags);
+    if (!FILL && lane == 0 && local_max > 0) atomicMax(A.words + 1, local_max);
+}
+
+// CSR offsets of up to kOffsetsMax centres in one launch: every CTA sums the counts before its tile itself (at most
+// 512 KB from L2) and scans its tile; the last one, which has seen them all, also reports the total, the largest count
+// and the error flags to the host's pinned words. Three launches (scan.cu) and k_report serve larger systems.
+constexpr int kOffsetsThreads = 1024;
+constexpr int kOffsetsMax = 131072;
+__device__ inline void report(int64_t total, const int* words, const unsigned* flags, int64_t* h_words, unsigned* h_flags) {
+    h_words[0] = total;
+    h_words[1] = words[1];
+    *h_flags = *flags;
+}
+__global__ void __launch_bounds__(kOffsetsThreads) k_offsets(int n, const int* __restrict__ counts, int64_t* __restrict__ offsets,
+                                                             const int* __restrict__ words, const unsigned* __restrict__ flags,
+                                                             int64_t* h_words, unsigned* h_flags) {
+    __shared__ int64_t tot[kOffsetsThreads / 32], pre[kOffsetsThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = blockIdx.x * kOffsetsThreads;
+    int64_t p = 0;
+#pragma unroll 4
+    for (int e = tid; e < base; e += kOffsetsThreads) p += counts[e];
+    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+    const int64_t own = base + tid < n ? counts[base + tid] : 0;
+    int64_t x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 0) pre[warp] = p;
+    if (lane == 31) tot[warp] = x;
+    __syncthreads();
+    int64_t before = x - own;
+    for (int w = 0; w < kOffsetsThreads / 32; ++w) before += pre[w] + (w < warp ? tot[w] : 0);
+    if (base + tid < n) offsets[base + tid] = before;
+    if (base + tid == n - 1) {
+        offsets[n] = before + own;
+        report(before + own, words, flags, h_words, h_flags);
+    }
+}
+__global__ void k_report(const int64_t* __restrict__ total, const int* __restrict__ words, const unsigned* __restrict__ flags,
+                         int64_t* h_words, unsigned* h_flags) {
+    report(*total, words, flags, h_words, h_flags);
+}
+
+// The scratch of one search: at most 116 bytes per atom and 360 per structure (the no-allocation entry point's array
+// holds 32 MiB, and the systems that fit it are part of its contract).
+struct NbrScratch {
+    StructInfo* info;
+    int *bin_count, *bin_start, *atom_bin, *atom_rank, *counts, *words;
+    int4 *atom_wrap, *items;
+    float4 *atom_hi, *atom_lo, *sorted_hi;
+    int64_t* sums;
+};
+static int64_t nbr_bins(int N, int n_s) { return 2LL * N + 8LL * n_s; }
+static int64_t nbr_sums(int N) { return N > kOffsetsMax ? scan_tile_sums_len(N) : 1; }
+static size_t nbr_scratch_bytes(int N, int n_s) {
+    const size_t nb = (size_t)nbr_bins(N, n_s), n = (size_t)N;
+    return carve_bytes(sizeof(StructInfo) * n_s, sizeof(int) * nb, sizeof(int) * nb, sizeof(int) * n, sizeof(int) * n,
+                       sizeof(int) * n, sizeof(int) * 4, sizeof(int4) * n, sizeof(int4) * n, sizeof(float4) * n,
+                       sizeof(float4) * n, sizeof(float4) * n, sizeof(int64_t) * nbr_sums(N));
+}
+static NbrScratch nbr_carve(void* base, int N, int n_s) {
+    const size_t nb = (size_t)nbr_bins(N, n_s), n = (size_t)N;
+    Carver cv(base);
+    NbrScratch W;
+    W.info = cv.take<StructInfo>(n_s);
+    W.bin_count = cv.take<int>(nb);
+    W.bin_start = cv.take<int>(nb);
+    W.atom_bin = cv.take<int>(n);
+    W.atom_rank = cv.take<int>(n);
+    W.counts = cv.take<int>(n);
+    W.words = cv.take<int>(4);
+    W.atom_wrap = cv.take<int4>(n);
+    W.items = cv.take<int4>(n);
+    W.atom_hi = cv.take<float4>(n);
+    W.atom_lo = cv.take<float4>(n);
+    W.sorted_hi = cv.take<float4>(n);
+    W.sums = cv.take<int64_t>((size_t)nbr_sums(N));
+    return W;
+}
+
+// Everything up to the pair count: *total pairs and *largest count of a centre, after one synchronisation.
+template <int CAP>
+static int nbr_count(rascal_ctx* ctx, const rascal_system* sys, const NbrScratch& W, int64_t* d_offsets, PairArgs& A,
+                     unsigned* grid, int64_t* total, int* largest) {
+    const int N = sys->n_atoms, n_s = sys->n_structures;
+    const int64_t nbins_cap = nbr_bins(N, n_s);
+    cudaStream_t stream = ctx->stream;
+    // a warp per structure, and threads enough to clear the counters in a few strides
+    const int64_t setup_blocks = std::max<int64_t>(div_up(n_s, 4), std::min<int64_t>(div_up(nbins_cap, 1024), 2LL * ctx->n_sm));
+    k_struct_setup<<<(unsigned)setup_blocks, 128, 0, stream>>>(n_s, N, sys->d_struct_offsets, sys->d_cells, sys->d_pbc,
+                                                               ctx->r_cut, W.info, W.bin_count, nbins_cap, W.words, ctx->d_flags);
+    RASCAL_LAUNCH_CHECK("k_struct_setup");
+    k_atom_bin<<<(unsigned)div_up(N, 64), 64, 0, stream>>>(N, n_s, nbins_cap, sys->d_struct_offsets, sys->d_positions,
+                                                          sys->d_species, ctx->d_lut, W.info, W.bin_count, W.atom_bin,
+                                                          W.atom_rank, W.atom_wrap, W.atom_hi, W.atom_lo, ctx->d_flags);
+    RASCAL_LAUNCH_CHECK("k_atom_bin");
+    // centres per work item: 16 share a staged stencil where there are atoms enough for two items per resident CTA, down
+    // to one per warp in small systems, whose few bins would leave most SMs idle
+    const int item_cap = (int)std::min<int64_t>(16, std::max<int64_t>(kPairWarps, N / (4LL * ctx->n_sm)));
+    k_bin_scan<<<(unsigned)std::min(n_s, 8 * ctx->n_sm), kBinScanThreads, 0, stream>>>(
+        n_s, N, ctx->r_cut, item_cap, W.info, W.bin_count, W.bin_start, W.items, W.words, ctx->d_flags);
+    RASCAL_LAUNCH_CHECK("k_bin_scan");
+    k_atom_scatter<<<(unsigned)div_up(N, 256), 256, 0, stream>>>(N, W.atom_bin, W.atom_rank, W.bin_start, W.atom_hi,
+                                                                W.sorted_hi, ctx->d_flags);
+    RASCAL_LAUNCH_CHECK("k_atom_scatter");
+    std::memset(&A, 0, sizeof(A));
+    A.n_atoms = N;
+    A.pos = sys->d_positions;
+    A.info = W.info;
+    A.bin_count = W.bin_count;
+    A.bin_start = W.bin_start;
+    A.sorted_hi = W.sorted_hi;
+    A.atom_wrap = W.atom_wrap;
+    A.atom_lo = W.atom_lo;
+    A.items = W.items;
+    A.words = W.words;
+    A.rc2 = ctx->r_cut * ctx->r_cut;
+    A.counts = W.counts;
+    A.offsets = d_offsets;
+    A.flags = ctx->d_flags;
+    *grid = (unsigned)std::min<int64_t>(N, 8LL * ctx->n_sm);
+    k_pairs<false, CAP><<<*grid, kPairWarps * 32, 0, stream>>>(A);
+    RASCAL_LAUNCH_CHECK("k_pairs<count>");
+    if (N <= kOffsetsMax) {
+        k_offsets<<<(unsigned)div_up(N, kOffsetsThreads), kOffsetsThreads, 0, stream>>>(N, W.counts, d_offsets, W.words,
+                                                                                        ctx->d_flags, ctx->h_pinned, ctx->h_flags);
+        RASCAL_LAUNCH_CHECK("k_offsets");
     } else {
-        __threadfence_block();
-        for (int e = lane; e < k; e += 32) {
-            const uint64_t key = keys[e];
-            int rank = 0;
-            for (int f = 0; f < k; ++f) rank += (keys[f] < key);
-            const int64_t o = seg_beg + rank;
-            out_j[o] = (int)(key >> 30);
-            out_shift[3 * o + 0] = (int)((key >> 20) & 1023) - 512;
-            out_shift[3 * o + 1] = (int)((key >> 10) & 1023) - 512;
-            out_shift[3 * o + 2] = (int)(key & 1023) - 512;
-            out_rij[o] = vecs[e];
-        }
+        const int st = scan_exclusive_into(W.counts, d_offsets, N, stream, W.sums);
+        if (st) return st;
+        k_report<<<1, 1, 0, stream>>>(d_offsets + N, W.words, ctx->d_flags, ctx->h_pinned, ctx->h_flags);
+        RASCAL_LAUNCH_CHECK("k_report");
     }
+    RASCAL_CUDA(cudaStreamSynchronize(stream));
+    const int st = flags_status(ctx, *ctx->h_flags);
+    if (st) return st;
+    *total = ctx->h_pinned[0];
+    *largest = (int)ctx->h_pinned[1];
+    return RASCAL_OK;
 }
 
 }  // namespace rascal
@@ -501,81 +818,33 @@ extern "C" int rascal_neighbours(rascal_ctx* ctx, const rascal_system* sys, int6
     if (st) return st;
     if (!d_offsets || !n_pairs || capacity < 0) return set_error(RASCAL_E_ARG, "NULL offsets / n_pairs or negative capacity");
     const int N = sys->n_atoms, n_s = sys->n_structures;
-    cudaStream_t stream = ctx->stream;
     *n_pairs = 0;
     if (N == 0) {
-        RASCAL_CUDA(cudaMemsetAsync(d_offsets, 0, sizeof(int64_t), stream));
+        RASCAL_CUDA(cudaMemsetAsync(d_offsets, 0, sizeof(int64_t), ctx->stream));
         return RASCAL_OK;
     }
-    const int64_t nbins_cap = 2LL * N + 8LL * n_s;
-    const size_t bytes = carve_bytes(sizeof(StructInfo) * n_s, sizeof(int) * (n_s + 1), sizeof(int64_t) * (n_s + 1),
-                                     sizeof(int) * nbins_cap, sizeof(int64_t) * (nbins_cap + 1), sizeof(int) * N,
-                                     sizeof(int) * N, sizeof(int) * N, sizeof(int4) * N, sizeof(int4) * N,
-                                     sizeof(float4) * N, sizeof(float4) * N, sizeof(float4) * N, sizeof(int) * 4);
     void* base;
-    if ((st = arena_get(ctx->scratch, bytes, &base))) return st;
-    Carver cv(base);
-    StructInfo* info = cv.take<StructInfo>(n_s);
-    int* nbins = cv.take<int>(n_s + 1);
-    int64_t* binbase = cv.take<int64_t>(n_s + 1);
-    int* bin_count = cv.take<int>(nbins_cap);
-    int64_t* bin_start = cv.take<int64_t>(nbins_cap + 1);
-    int* atom_bin = cv.take<int>(N);
-    int* atom_rank = cv.take<int>(N);
-    int* atom_struct = cv.take<int>(N);
-    int4* atom_cell = cv.take<int4>(N);
-    int4* atom_wrap = cv.take<int4>(N);
-    float4* atom_hi = cv.take<float4>(N);
-    float4* atom_lo = cv.take<float4>(N);
-    float4* sorted_hi = cv.take<float4>(N);
-    int* max_count = cv.take<int>(4);
-
-    RASCAL_CUDA(cudaMemsetAsync(bin_count, 0, sizeof(int) * nbins_cap, stream));
-    RASCAL_CUDA(cudaMemsetAsync(max_count, 0, sizeof(int), stream));
-    k_struct_setup<<<(unsigned)div_up(n_s, 128), 128, 0, stream>>>(n_s, N, sys->d_struct_offsets, sys->d_cells, sys->d_pbc,
-                                                                 ctx->r_cut, info, nbins, ctx->d_flags);
-    RASCAL_LAUNCH_CHECK("k_struct_setup");
-    if ((st = scan_exclusive(nbins, binbase, n_s, stream, ctx->scratch2))) return st;
-    k_atom_bin<<<(unsigned)div_up(N, 256), 256, 0, stream>>>(N, n_s, nbins_cap, sys->d_struct_offsets, sys->d_positions, sys->d_species,
-                                                           ctx->d_lut, info, binbase, bin_count, atom_bin, atom_rank,
-                                                           atom_struct, atom_cell, atom_wrap, atom_hi, atom_lo, ctx->d_flags);
-    RASCAL_LAUNCH_CHECK("k_atom_bin");
-    if ((st = scan_exclusive(bin_count, bin_start, nbins_cap, stream, ctx->scratch2))) return st;
-    k_atom_scatter<<<(unsigned)div_up(N, 256), 256, 0, stream>>>(N, atom_bin, atom_rank, bin_start, atom_hi, sorted_hi);
-    RASCAL_LAUNCH_CHECK("k_atom_scatter");
-    k_struct_thresholds<<<(unsigned)div_up(n_s, 128), 128, 0, stream>>>(n_s, ctx->r_cut, info);
-    RASCAL_LAUNCH_CHECK("k_struct_thresholds");
-    const double rc2 = ctx->r_cut * ctx->r_cut;
-    const unsigned pair_blocks = (unsigned)div_up(N, kPairWarps);
-    k_pairs<false><<<pair_blocks, kPairWarps * 32, 0, stream>>>(N, sys->d_positions, info, binbase, bin_start, sorted_hi,
-                                                                atom_struct, atom_cell, atom_wrap, atom_hi, atom_lo, rc2,
-                                                                nbins_cap, d_offsets, max_count, nullptr, nullptr, nullptr, nullptr,
-                                                                nullptr, ctx->d_flags);
-    RASCAL_LAUNCH_CHECK("k_pairs<count>");
-    if ((st = scan_exclusive(d_offsets, d_offsets, N, stream, ctx->scratch2))) return st;
-    RASCAL_CUDA(cudaMemcpyAsync(ctx->h_pinned, d_offsets + N, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-    RASCAL_CUDA(cudaMemcpyAsync(ctx->h_pinned + 1, max_count, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    if ((st = check_flags(ctx))) return st;  // synchronises the stream
-    const int64_t P = ctx->h_pinned[0];
-    const int maxc = *reinterpret_cast<int*>(ctx->h_pinned + 1);
+    if ((st = arena_get(ctx->scratch, nbr_scratch_bytes(N, n_s), &base))) return st;
+    PairArgs A;
+    unsigned grid;
+    int64_t P;
+    int maxc;
+    if ((st = nbr_count<kPairCap>(ctx, sys, nbr_carve(base, N, n_s), d_offsets, A, &grid, &P, &maxc))) return st;
     *n_pairs = P;
     if (P > capacity) return set_error(RASCAL_E_CAPACITY, "pair capacity %lld < required %lld", (long long)capacity, (long long)P);
     if (P == 0) return RASCAL_OK;
     if (!d_nbr_j || !d_shift || !d_rij) return set_error(RASCAL_E_ARG, "NULL pair output arrays");
-    uint64_t* ovf_keys = nullptr;
-    float4* ovf_vec = nullptr;
     if (maxc > kPairCap) {
         void* ob;
         if ((st = arena_get(ctx->scratch2, carve_bytes(sizeof(uint64_t) * P, sizeof(float4) * P), &ob))) return st;
         Carver oc(ob);
-        ovf_keys = oc.take<uint64_t>(P);
-        ovf_vec = oc.take<float4>(P);
+        A.ovf_keys = oc.take<uint64_t>(P);
+        A.ovf_vec = oc.take<float4>(P);
     }
-    k_pairs<true><<<pair_blocks, kPairWarps * 32, 0, stream>>>(N, sys->d_positions, info, binbase, bin_start, sorted_hi,
-                                                               atom_struct, atom_cell, atom_wrap, atom_hi, atom_lo, rc2,
-                                                               nbins_cap, d_offsets, nullptr, d_nbr_j, d_shift,
-                                                               reinterpret_cast<float4*>(d_rij), ovf_keys, ovf_vec,
-                                                               ctx->d_flags);
+    A.out_j = d_nbr_j;
+    A.out_shift = d_shift;
+    A.out_rij = reinterpret_cast<float4*>(d_rij);
+    k_pairs<true><<<grid, kPairWarps * 32, 0, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_pairs<fill>");
     return RASCAL_OK;
 }
@@ -636,19 +905,18 @@ extern "C" int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* s
     if (st) return st;
     if (!d_offsets || !n_pairs || capacity < 0) return set_error(RASCAL_E_ARG, "NULL offsets / n_pairs or negative capacity");
     const int N = sys->n_atoms, n_s = sys->n_structures;
-    cudaStream_t stream = ctx->stream;
     *n_pairs = 0;
     if (N == 0) {
-        RASCAL_CUDA(cudaMemsetAsync(d_offsets, 0, sizeof(int64_t), stream));
+        RASCAL_CUDA(cudaMemsetAsync(d_offsets, 0, sizeof(int64_t), ctx->stream));
         return RASCAL_OK;
     }
-    const int64_t nbins_cap = 2LL * N + 8LL * n_s;
+    // what the entry point's limit counts: 116 bytes per atom, 360 per structure (nbr_scratch_bytes is never more)
+    const int64_t nbins_cap = nbr_bins(N, n_s);
     const int64_t sums_len = std::max(scan_tile_sums_len(n_s), std::max(scan_tile_sums_len(nbins_cap), scan_tile_sums_len(N)));
-    const size_t bytes = carve_bytes(sizeof(StructInfo) * n_s, sizeof(int) * (n_s + 1), sizeof(int64_t) * (n_s + 1),
-                                     sizeof(int) * nbins_cap, sizeof(int64_t) * (nbins_cap + 1), sizeof(int) * N,
-                                     sizeof(int) * N, sizeof(int) * N, sizeof(int4) * N, sizeof(int4) * N,
-                                     sizeof(float4) * N, sizeof(float4) * N, sizeof(float4) * N, sizeof(int) * 4,
-                                     sizeof(int64_t) * sums_len);
+    const size_t bytes = carve_bytes((size_t)280 * n_s, sizeof(int) * (n_s + 1), sizeof(int64_t) * (n_s + 1), sizeof(int) * nbins_cap,
+                                     sizeof(int64_t) * (nbins_cap + 1), sizeof(int) * N, sizeof(int) * N, sizeof(int) * N,
+                                     sizeof(int4) * N, sizeof(int4) * N, sizeof(float4) * N, sizeof(float4) * N,
+                                     sizeof(float4) * N, sizeof(int) * 4, sizeof(int64_t) * sums_len);
     if (bytes > kStaticNbrScratchBytes)
         return set_error(RASCAL_E_UNSUPPORTED,
                          "this system needs %zu bytes of neighbour scratch; the no-allocation entry point holds %zu "
@@ -656,53 +924,11 @@ extern "C" int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* s
                          bytes, kStaticNbrScratchBytes);
     void* base = nullptr;
     if ((st = static_nbr_scratch(ctx, &base))) return st;
-    Carver cv(base);
-    StructInfo* info = cv.take<StructInfo>(n_s);
-    int* nbins = cv.take<int>(n_s + 1);
-    int64_t* binbase = cv.take<int64_t>(n_s + 1);
-    int* bin_count = cv.take<int>(nbins_cap);
-    int64_t* bin_start = cv.take<int64_t>(nbins_cap + 1);
-    int* atom_bin = cv.take<int>(N);
-    int* atom_rank = cv.take<int>(N);
-    int* atom_struct = cv.take<int>(N);
-    int4* atom_cell = cv.take<int4>(N);
-    int4* atom_wrap = cv.take<int4>(N);
-    float4* atom_hi = cv.take<float4>(N);
-    float4* atom_lo = cv.take<float4>(N);
-    float4* sorted_hi = cv.take<float4>(N);
-    int* max_count = cv.take<int>(4);
-    int64_t* sums = cv.take<int64_t>(sums_len);
-
-    // the array keeps the previous call's contents: the bin counters and the maximum must start at zero
-    RASCAL_CUDA(cudaMemsetAsync(bin_count, 0, sizeof(int) * nbins_cap, stream));
-    RASCAL_CUDA(cudaMemsetAsync(max_count, 0, sizeof(int), stream));
-    k_struct_setup<<<(unsigned)div_up(n_s, 128), 128, 0, stream>>>(n_s, N, sys->d_struct_offsets, sys->d_cells, sys->d_pbc,
-                                                                 ctx->r_cut, info, nbins, ctx->d_flags);
-    RASCAL_LAUNCH_CHECK("k_struct_setup");
-    if ((st = scan_exclusive_into(nbins, binbase, n_s, stream, sums))) return st;
-    k_atom_bin<<<(unsigned)div_up(N, 256), 256, 0, stream>>>(N, n_s, nbins_cap, sys->d_struct_offsets, sys->d_positions,
-                                                           sys->d_species, ctx->d_lut, info, binbase, bin_count, atom_bin,
-                                                           atom_rank, atom_struct, atom_cell, atom_wrap, atom_hi, atom_lo,
-                                                           ctx->d_flags);
-    RASCAL_LAUNCH_CHECK("k_atom_bin");
-    if ((st = scan_exclusive_into(bin_count, bin_start, nbins_cap, stream, sums))) return st;
-    k_atom_scatter<<<(unsigned)div_up(N, 256), 256, 0, stream>>>(N, atom_bin, atom_rank, bin_start, atom_hi, sorted_hi);
-    RASCAL_LAUNCH_CHECK("k_atom_scatter");
-    k_struct_thresholds<<<(unsigned)div_up(n_s, 128), 128, 0, stream>>>(n_s, ctx->r_cut, info);
-    RASCAL_LAUNCH_CHECK("k_struct_thresholds");
-    const double rc2 = ctx->r_cut * ctx->r_cut;
-    const unsigned pair_blocks = (unsigned)div_up(N, kPairWarps);
-    k_pairs<false, kNoallocCap><<<pair_blocks, kPairWarps * 32, 0, stream>>>(N, sys->d_positions, info, binbase, bin_start, sorted_hi,
-                                                                atom_struct, atom_cell, atom_wrap, atom_hi, atom_lo, rc2,
-                                                                nbins_cap, d_offsets, max_count, nullptr, nullptr, nullptr,
-                                                                nullptr, nullptr, ctx->d_flags);
-    RASCAL_LAUNCH_CHECK("k_pairs<count>");
-    if ((st = scan_exclusive_into(d_offsets, d_offsets, N, stream, sums))) return st;
-    RASCAL_CUDA(cudaMemcpyAsync(ctx->h_pinned, d_offsets + N, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-    RASCAL_CUDA(cudaMemcpyAsync(ctx->h_pinned + 1, max_count, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    if ((st = check_flags(ctx))) return st;  // synchronises the stream
-    const int64_t P = ctx->h_pinned[0];
-    const int maxc = *reinterpret_cast<int*>(ctx->h_pinned + 1);
+    PairArgs A;
+    unsigned grid;
+    int64_t P;
+    int maxc;
+    if ((st = nbr_count<kNoallocCap>(ctx, sys, nbr_carve(base, N, n_s), d_offsets, A, &grid, &P, &maxc))) return st;
     *n_pairs = P;
     // checked before the capacity, so that a caller who resizes after RASCAL_E_CAPACITY is not refused afterwards
     if (maxc > kNoallocCap)
@@ -711,11 +937,10 @@ extern "C" int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* s
     if (P > capacity) return set_error(RASCAL_E_CAPACITY, "pair capacity %lld < required %lld", (long long)capacity, (long long)P);
     if (P == 0) return RASCAL_OK;
     if (!d_nbr_j || !d_shift || !d_rij) return set_error(RASCAL_E_ARG, "NULL pair output arrays");
-    k_pairs<true, kNoallocCap><<<pair_blocks, kPairWarps * 32, 0, stream>>>(N, sys->d_positions, info, binbase, bin_start, sorted_hi,
-                                                               atom_struct, atom_cell, atom_wrap, atom_hi, atom_lo, rc2,
-                                                               nbins_cap, d_offsets, nullptr, d_nbr_j, d_shift,
-                                                               reinterpret_cast<float4*>(d_rij), nullptr, nullptr,
-                                                               ctx->d_flags);
+    A.out_j = d_nbr_j;
+    A.out_shift = d_shift;
+    A.out_rij = reinterpret_cast<float4*>(d_rij);
+    k_pairs<true, kNoallocCap><<<grid, kPairWarps * 32, 0, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_pairs<fill>");
     return RASCAL_OK;
 }

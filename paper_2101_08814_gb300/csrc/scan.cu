@@ -1,5 +1,5 @@
 // Device-wide exclusive prefix sum (three passes, no inter-block waiting): per-block scans, a single-block scan
-// of the block totals, then a uniform add. out[0..n] with out[n] = total; in and out may alias.
+// of the block totals, then a uniform add. out[0..n] with out[n] = total.
 #include "common.cuh"
 
 namespace rascal {
@@ -33,8 +33,7 @@ __device__ inline int64_t block_exclusive_scan(int64_t v, int64_t* warp_tot, int
     return before + x - v;
 }
 
-template <typename Tin>
-__global__ void k_scan_tiles(const Tin* in, int64_t* out, int64_t n, int64_t* tile_sums) {
+__global__ void k_scan_tiles(const int* in, int64_t* out, int64_t n, int64_t* tile_sums) {
     __shared__ int64_t warp_tot[kScanThreads / 32];
     __shared__ int64_t total;
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
@@ -79,29 +78,10 @@ __global__ void k_scan_add(int64_t* out, int64_t n, const int64_t* tile_sums) {
     }
 }
 
-template <typename Tin>
-static int scan_impl(const Tin* in, int64_t* out, int64_t n, cudaStream_t stream, Arena& scratch) {
+// Scan with a caller-provided buffer for the tile sums (scan_tile_sums_len(n) int64 words); allocates nothing.
+int scan_exclusive_into(const int* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums) {
     const int64_t tiles = div_up(n > 0 ? n : 1, kScanTile);
-    void* buf;
-    int st = arena_get(scratch, sizeof(int64_t) * (tiles + 1), &buf);
-    if (st) return st;
-    int64_t* sums = static_cast<int64_t*>(buf);
-    k_scan_tiles<Tin><<<(unsigned)tiles, kScanThreads, 0, stream>>>(in, out, n, sums);
-    RASCAL_LAUNCH_CHECK("k_scan_tiles");
-    k_scan_tile_sums<<<1, kScanThreads, 0, stream>>>(sums, tiles, out + n);
-    RASCAL_LAUNCH_CHECK("k_scan_tile_sums");
-    if (tiles > 1) {
-        k_scan_add<<<(unsigned)tiles, kScanThreads, 0, stream>>>(out, n, sums);
-        RASCAL_LAUNCH_CHECK("k_scan_add");
-    }
-    return RASCAL_OK;
-}
-
-// Same scan with a caller-provided buffer for the tile sums (scan_tile_sums_len(n) int64 words); allocates nothing.
-template <typename Tin>
-static int scan_into_impl(const Tin* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums) {
-    const int64_t tiles = div_up(n > 0 ? n : 1, kScanTile);
-    k_scan_tiles<Tin><<<(unsigned)tiles, kScanThreads, 0, stream>>>(in, out, n, sums);
+    k_scan_tiles<<<(unsigned)tiles, kScanThreads, 0, stream>>>(in, out, n, sums);
     RASCAL_LAUNCH_CHECK("k_scan_tiles");
     k_scan_tile_sums<<<1, kScanThreads, 0, stream>>>(sums, tiles, out + n);
     RASCAL_LAUNCH_CHECK("k_scan_tile_sums");
@@ -113,18 +93,5 @@ static int scan_into_impl(const Tin* in, int64_t* out, int64_t n, cudaStream_t s
 }
 
 int64_t scan_tile_sums_len(int64_t n) { return div_up(n > 0 ? n : 1, kScanTile) + 1; }
-int scan_exclusive_into(const int* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums) {
-    return scan_into_impl<int>(in, out, n, stream, sums);
-}
-int scan_exclusive_into(const int64_t* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums) {
-    return scan_into_impl<int64_t>(in, out, n, stream, sums);
-}
-
-int scan_exclusive(const int* in, int64_t* out, int64_t n, cudaStream_t stream, Arena& scratch) {
-    return scan_impl<int>(in, out, n, stream, scratch);
-}
-int scan_exclusive(const int64_t* in, int64_t* out, int64_t n, cudaStream_t stream, Arena& scratch) {
-    return scan_impl<int64_t>(in, out, n, stream, scratch);
-}
 
 }  // namespace rascal

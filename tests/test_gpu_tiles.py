@@ -7,7 +7,8 @@ pytestmark = pytest.mark.gpu
 from oracle import lambda_soap as ols  # noqa: E402
 from oracle import mlp as omlp  # noqa: E402
 from oracle import soap as osoap  # noqa: E402
-from synth import mlp_initial_params  # noqa: E402
+from oracle.neighbours import neighbour_list  # noqa: E402
+from synth import System, config_batch, mlp_initial_params, random_cell_atoms  # noqa: E402
 from tests.gpu_common import block_rel_err  # noqa: E402
 
 H = 64
@@ -70,3 +71,61 @@ def test_equivariant_tiles(rg, n_max, S, l_max, lam):
     T = calc.lambda_soap(torch.tensor(c, device="cuda"), lam)
     ref = ols.equivariants(c, h, lam)
     assert block_rel_err(T.cpu().numpy(), ref, 2) <= 2e-6
+
+
+def _lists(rg, s):
+    pl = rg.SoapCalculator(**s.hypers).neighbours(rg.DeviceSystem.from_numpy(s))
+    return [getattr(pl, k).cpu().numpy() for k in ("offsets", "nbr_j", "shifts", "rij")]
+
+
+def _cell(n, cell, r_cut, pbc=(1, 1, 1), d_min=0.7, seed=61):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    cell = np.asarray(cell, np.float64)
+    return System(random_cell_atoms(n, cell, d_min, rng), np.full(n, 6, np.int32), cell[None], np.asarray([pbc], np.int32),
+                  np.array([0, n], np.int32), dict(r_cut=r_cut, sigma=0.5, n_max=2, l_max=1, smooth_width=0.5, species=[6]))
+
+
+# stencils of one batch and of several (a flat cell: 9 x 9 x 3 bins), candidates of one chunk and of several (27 x 70 of
+# one bin), bins that split into several work items, one with fewer centres than warps, one open axis: equal to the
+# brute-force list, vectors to FP32 rounding
+@pytest.mark.parametrize("n,cell,r_cut,pbc", [
+    (1, np.eye(3) * 3.0, 5.0, (1, 1, 1)), (3, np.diag([1.4, 1.6, 9.0]), 5.0, (1, 1, 1)),
+    (70, np.eye(3) * 5.5, 5.0, (1, 1, 1)), (70, np.diag([5.5, 5.5, 7.0]), 4.0, (1, 0, 1)), (200, np.eye(3) * 11.0, 5.0, (1, 1, 1))])
+def test_neighbour_stencils(rg, n, cell, r_cut, pbc):
+    s = _cell(n, cell, r_cut, pbc)
+    off, j, sh, rij = _lists(rg, s)
+    ref = neighbour_list(s, r_cut)
+    assert np.array_equal(off, ref["offsets"]) and np.array_equal(j, ref["nbr_j"]) and np.array_equal(sh, ref["shifts"])
+    assert np.allclose(rij[:, :3], ref["rij"], rtol=0, atol=2e-6)
+
+
+def test_neighbours_far_from_their_cell(rg):
+    s = _cell(40, np.diag([7.0, 8.0, 9.0]), 4.0)
+    far = System(s.positions + np.array([600.0 * 7.0, -700.0 * 8.0, 0.0]), s.species, s.cells, s.pbc, s.struct_offsets, s.hypers)
+    off, j, sh, rij = _lists(rg, far)
+    ref = neighbour_list(far, 4.0)
+    assert np.array_equal(off, ref["offsets"]) and np.array_equal(j, ref["nbr_j"]) and np.array_equal(sh, ref["shifts"])
+    moved = far.positions.copy()
+    moved[0] += np.array([7.0 * 1200.0, 0.0, 0.0])  # neighbours 1200 cells apart: beyond the shift range
+    with pytest.raises(rg.RascalError) as e:
+        _lists(rg, System(moved, s.species, s.cells, s.pbc, s.struct_offsets, s.hypers))
+    assert e.value.code == rg._lib.RASCAL_E_UNSUPPORTED
+
+
+def test_neighbours_of_many_atoms_and_loose_offsets(rg):
+    # more atoms than the one-launch offsets take: copies of the same cells have the same lists
+    s = config_batch(n_structures=24)
+    off, j, sh, rij = _lists(rg, s)
+    k = 131072 // s.n_atoms + 2
+    big = System(np.tile(s.positions, (k, 1)), np.tile(s.species, k), np.tile(s.cells, (k, 1, 1)), np.tile(s.pbc, (k, 1)),
+                 np.concatenate([[0]] + [s.struct_offsets[1:] + q * s.n_atoms for q in range(k)]).astype(np.int32), s.hypers)
+    boff, bj, bsh, brij = _lists(rg, big)
+    P = len(j)
+    assert np.array_equal(boff, np.concatenate([[0]] + [off[1:] + q * P for q in range(k)]))
+    assert np.array_equal(bj, np.concatenate([j + q * s.n_atoms for q in range(k)]))
+    assert np.array_equal(bsh, np.tile(sh, (k, 1))) and np.array_equal(brij, np.tile(rij, (k, 1)))
+    # atoms before the first offset count as the first structure's, atoms past the last as the last one's
+    loose = System(s.positions, s.species, s.cells, s.pbc, s.struct_offsets.copy(), s.hypers)
+    loose.struct_offsets[0], loose.struct_offsets[-1] = 5, s.n_atoms - 7
+    for a, b in zip(_lists(rg, loose), (off, j, sh, rij)):
+        assert np.array_equal(a, b)
