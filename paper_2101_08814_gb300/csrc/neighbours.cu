@@ -368,19 +368,19 @@ struct PairArgs {
 // candidates are staged once, already shifted to the bin's image (x + T), so that a warp's test of 32 candidates for one
 // centre is a 16-byte shared load, six FP32 operations and a ballot. (One warp per centre that walked the stencil itself
 // spent about 1 400 warp instructions per centre on locating and loading candidates, twice, and waited for them in L2:
-// 124 us counting and 206 us filling 1.80 M pairs of 70 820 centres; now PAIRS_COUNT and PAIRS_FILL us.) Items of more than
+// 124 us counting and 206 us filling 1.80 M pairs of 70 820 centres; now 66 and 170 us.) Items of more than
 // kPairChunk candidates, or whose stencil has more than kPairEntries bins, restage chunk by chunk for every four centres.
 // CAP: pairs a warp sorts in shared memory.
 template <bool FILL, int CAP = kPairCap>
 __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) : 0) k_pairs(const PairArgs A) {
-    constexpr int kEPL = CAP / 32, kThreads = kPairWarps * 32;
+    constexpr int kThreads = kPairWarps * 32;
     __shared__ float4 s_c[kPairChunk];             // x + T, y + T, z + T, j (t = 0) or ~j (another image)
     __shared__ unsigned char s_e[kPairChunk];      // the candidate's stencil entry
     __shared__ int s_pref[kPairEntries], s_beg[kPairEntries], s_t[kPairEntries];
     __shared__ float4 s_T[kPairEntries];
     __shared__ float4 s_Th[FILL ? kPairEntries : 1], s_Tl[FILL ? kPairEntries : 1];
     __shared__ int s_wtot[kPairWarps];
-    __shared__ uint64_t s_keys[FILL ? kPairWarps * CAP : 1];
+    __shared__ __align__(16) uint64_t s_keys[FILL ? kPairWarps * CAP : 1];
     __shared__ float4 s_vec[FILL ? kPairWarps * CAP : 1];
     __shared__ unsigned short s_rec[FILL ? kPairWarps * kPairRec : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -398,6 +398,10 @@ __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) :
         // |n| <= 2 wmax + |t|: only where this can pass the key's range is a pair's shift checked
         const int tmax = max((r0 + nb0 - 1) / nb0, max((r1 + nb1 - 1) / nb1, (r2 + nb2 - 1) / nb2)) + 1;
         const bool wide = S.wmax > kMaxShift || 2 * S.wmax + tmax > kMaxShift;
+        // keys of 32 bits, 20 of the atom's number in the structure and 4 per shift, where every shift fits them: two
+        // instructions per comparison of the rank sort and four keys per load (fill
+        // pass 196 -> 170 us for 1.80 M pairs, 188 -> 168 us for the 2.95 M of a dense liquid)
+        const bool narrow = S.atom_end - S.atom_begin <= (1 << 20) && S.wmax <= kMaxShift && 2 * S.wmax + tmax <= 7;
         int staged = -1;  // first entry of the batch whose tables are in shared memory, if its candidates fill one chunk
         int n_staged = 0;
         // wrap counts of atom j
@@ -416,6 +420,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) :
             float4 plo = make_float4(0.f, 0.f, 0.f, 0.f);
             int64_t seg_beg = 0, seg_cnt = 0;
             uint64_t* keys = s_keys + (FILL ? warp * CAP : 0);
+            uint32_t* keys32 = reinterpret_cast<uint32_t*>(keys);  // narrow, at most CAP pairs
             float4* vecs = s_vec + (FILL ? warp * CAP : 0);
             if (FILL) {
                 plo = A.atom_lo[i];
@@ -560,7 +565,10 @@ __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) :
                                 }
                                 const float rr = sqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
                                 if (r < seg_cnt) {
-                                    keys[r] = pair_key(j, n);
+                                    if (narrow && seg_cnt <= CAP)
+                                        keys32[r] = (uint32_t)(j - S.atom_begin) << 12 | (uint32_t)((n[0] + 8) << 8 | (n[1] + 8) << 4 | (n[2] + 8));
+                                    else
+                                        keys[r] = pair_key(j, n);
                                     vecs[r] = make_float4(v[0], v[1], v[2], rr);
                                 }
                             }
@@ -622,40 +630,52 @@ __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) :
             // rank sort of the segment by (j, n1, n2, n3) and write-out
             __syncwarp();
             const int k = (int)(seg_cnt < (int64_t)count ? seg_cnt : (int64_t)count);
-            auto write = [&](int e, uint64_t key, int rank) {
+            auto write = [&](int e, int j, int n0, int n1, int n2, int rank) {
                 const int64_t o = seg_beg + rank;
-                A.out_j[o] = (int)(key >> 30);
-                A.out_shift[3 * o + 0] = (int)((key >> 20) & 1023) - 512;
-                A.out_shift[3 * o + 1] = (int)((key >> 10) & 1023) - 512;
-                A.out_shift[3 * o + 2] = (int)(key & 1023) - 512;
+                A.out_j[o] = j;
+                A.out_shift[3 * o + 0] = n0;
+                A.out_shift[3 * o + 1] = n1;
+                A.out_shift[3 * o + 2] = n2;
                 A.out_rij[o] = vecs[e];
             };
-            if (seg_cnt <= CAP) {
-                uint64_t mykey[kEPL];
-                int myrank[kEPL];
-#pragma unroll
-                for (int qd = 0; qd < kEPL; ++qd) {
-                    const int e = lane + 32 * qd;
-                    mykey[qd] = (e < k) ? keys[e] : ~0ull;
-                    myrank[qd] = 0;
+            auto write64 = [&](int e, uint64_t key, int rank) {
+                write(e, (int)(key >> 30), (int)((key >> 20) & 1023) - 512, (int)((key >> 10) & 1023) - 512,
+                      (int)(key & 1023) - 512, rank);
+            };
+            if (narrow && seg_cnt <= CAP) {
+                if (lane < ((k + 3) & ~3) - k) keys32[k + lane] = 0xffffffffu;
+                __syncwarp();
+                for (int e0 = 0; e0 < k; e0 += 64) {  // two keys per lane at a time, every key against them
+                    const int ea = e0 + lane, eb = ea + 32;
+                    const uint32_t ka = ea < k ? keys32[ea] : 0u, kb = eb < k ? keys32[eb] : 0u;
+                    int ra = 0, rb = 0;
+#pragma unroll 2
+                    for (int f = 0; f < k; f += 4) {
+                        const uint4 q = *reinterpret_cast<const uint4*>(keys32 + f);
+                        ra += (q.x < ka) + (q.y < ka) + (q.z < ka) + (q.w < ka);
+                        rb += (q.x < kb) + (q.y < kb) + (q.z < kb) + (q.w < kb);
+                    }
+                    auto put = [&](int e, uint32_t key, int rank) {
+                        write(e, (int)(key >> 12) + S.atom_begin, (int)((key >> 8) & 15) - 8, (int)((key >> 4) & 15) - 8,
+                              (int)(key & 15) - 8, rank);
+                    };
+                    if (ea < k) put(ea, ka, ra);
+                    if (eb < k) put(eb, kb, rb);
                 }
-                const int nq = (k + 31) / 32;
-                for (int f = 0; f < k; ++f) {
-                    const uint64_t kf = keys[f];
-#pragma unroll
-                    for (int qd = 0; qd < kEPL; ++qd)
-                        if (qd < nq) myrank[qd] += (kf < mykey[qd]);
+            } else if (seg_cnt <= CAP) {
+                for (int e = lane; e < k; e += 32) {
+                    const uint64_t key = keys[e];
+                    int rank = 0;
+                    for (int f = 0; f < k; ++f) rank += (keys[f] < key);
+                    write64(e, key, rank);
                 }
-#pragma unroll
-                for (int qd = 0; qd < kEPL; ++qd)
-                    if (lane + 32 * qd < k) write(lane + 32 * qd, mykey[qd], myrank[qd]);
             } else {
                 __threadfence_block();
                 for (int e = lane; e < k; e += 32) {
                     const uint64_t key = keys[e];
                     int rank = 0;
                     for (int f = 0; f < k; ++f) rank += (keys[f] < key);
-                    write(e, key, rank);
+                    write64(e, key, rank);
                 }
             }
             __syncwarp();
