@@ -850,6 +850,7 @@ static ExpArgs make_args(rascal_ctx* ctx, const rascal_system* sys, const int64_
     A.l_max = ctx->l_max;
     A.S = ctx->n_species;
     A.n_lm = ctx->n_lm;
+    A.Q = ctx->Q;  // compared by exp_shape_of also where no Gram follows
     A.F = ctx->F;
     A.F_pad = P.F_pad;
     A.n_pad = P.n_pad;
