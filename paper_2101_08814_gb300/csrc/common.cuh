@@ -152,6 +152,8 @@ struct rascal_ctx {
     int* d_fmap;    // [F_pad] table column (l*n_max + n) of a padded radial slot, -1 for padding
     int* d_pstasks; // power-spectrum tasks, see power_spectrum.cu
     int n_pstasks;
+    unsigned* d_psitems;  // Gram items of power_spectrum.cu: warp tiles, then thread tiles PACKED and FULL, each by falling l
+    int n_psitems[3];     // of each kind per l
 
     // MLP surrogate of the radial integrals (mlp.cu); mlp_params == NULL until parameters are set
     float* mlp_params;   // FP32 master parameters
@@ -219,6 +221,9 @@ int expansion_setup(rascal_ctx* ctx);
 int power_spectrum_setup(rascal_ctx* ctx);
 // BF16 / TF32x3 power spectrum of given coefficients [n][Q][n_lm] by the fused kernel's tensor-core Gram
 int power_spectrum_tc(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps);
+// FP32, BF16 or TF32x3 power spectrum of given coefficients by the kernel of power_spectrum.cu; RASCAL_E_UNSUPPORTED
+// (without a message) where a centre does not fit its shared memory
+int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps);
 int gradients_setup(rascal_ctx* ctx);
 // caches the device address of the no-allocation neighbour scratch for ctx->device (neighbours.cu)
 int nbr_static_prepare(rascal_ctx* ctx);

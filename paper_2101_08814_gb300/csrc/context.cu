@@ -453,6 +453,7 @@ extern "C" void rascal_destroy(rascal_ctx* ctx) {
     cudaFree(ctx->d_tasks);
     cudaFree(ctx->d_fmap);
     cudaFree(ctx->d_pstasks);
+    cudaFree(ctx->d_psitems);
     cudaFree(ctx->mlp_params);
     cudaFree(ctx->mlp_m);
     cudaFree(ctx->mlp_v);

@@ -129,3 +129,34 @@ def test_neighbours_of_many_atoms_and_loose_offsets(rg):
     loose.struct_offsets[0], loose.struct_offsets[-1] = 5, s.n_atoms - 7
     for a, b in zip(_lists(rg, loose), (off, j, sh, rij)):
         assert np.array_equal(a, b)
+
+
+# Q = 1 and 7 (one block of rows, partly empty), 16, 17, 24, 35, 48, 60 and 128 (32-row blocks with and without a lone
+# 16-row block after them, several items left of the diagonal), and Q = 256, whose FULL l blocks do not fit the staging
+# area. The bars are those of the other power-spectrum tests: 1e-5 per (centre, l) block in FP32 and TF32x3; BF16 inputs
+# 2^-7 of a block's largest entry and 5e-3 of its norm.
+@pytest.mark.parametrize("n_max,S,l_max", [(1, 1, 0), (7, 1, 3), (8, 2, 6), (17, 1, 2), (12, 2, 9), (7, 5, 5), (12, 4, 9),
+                                           (15, 4, 4), (16, 8, 12), (16, 16, 1)])
+def test_power_spectrum_items(rg, n_max, S, l_max):
+    import torch
+
+    species = list(range(1, S + 1))
+    calc = rg.SoapCalculator(5.0, 0.5, n_max, l_max, species, spline_intervals=64)
+    h = osoap.Hypers(5.0, 0.5, n_max, l_max, species)
+    rng = np.random.default_rng(29)
+    c = rng.standard_normal((4, S, n_max, (l_max + 1) ** 2)).astype(np.float32)
+    c[-1] = 0.0
+    c_dev = torch.tensor(c, device="cuda")
+    for layout in ("packed", "full"):
+        ref = osoap.power_spectrum(c.astype(np.float64), h, layout).reshape(4, l_max + 1, -1)
+        for precision in ("fp32", "tf32x3", "bf16"):
+            if precision != "fp32" and (h.q > 128 or (precision == "tf32x3" and h.q > 96)):
+                continue  # refused by the library
+            p = calc.power_spectrum(c_dev, precision=precision, layout=layout).cpu().numpy().reshape(ref.shape)
+            assert np.all(p[-1] == 0.0)
+            if precision == "bf16":
+                assert block_rel_err(p, ref, 2) <= 2.0 ** -7
+                fro = np.sqrt(np.sum((p - ref) ** 2, axis=-1) / np.maximum(np.sum(ref ** 2, axis=-1), 1e-300))
+                assert np.max(fro) <= 5e-3
+            else:
+                assert block_rel_err(p, ref, 2) <= 1e-5, (layout, precision)
