@@ -81,10 +81,9 @@ struct GradArgs {
     const float* weights;   // [S][Fp] or NULL
     const float* wsym;      // weights only: k_l (W_l + W_l^T) per species and l, dense [S][L1][Q][Qw] (Qw = ceil4(Q))
     int Qw, Lp_adj, n_adj_tasks;
-    int w_tiled;            // per-centre dE/dp: tiled adjoint with one dense l block staged in shared memory
-    int w_off;              // bytes from the pair area to that block
+    int w_lg, w_rows;       // per-centre dE/dp: packed l blocks staged at once (0: the per-element adjoint), rows of a warp
+    int w_off;              // bytes from the pair area (k_gradients: from the start of shared memory) to those blocks
     int aux_off;            // bytes from the pair area to the small tables (past both the pair area and C)
-    int adj_pref[kMaxLMax + 2];  // prefix counts of the adjoint tile tasks per l
     float* forces;          // FP32 accumulation, converted to the FP64 output afterwards
     double* virial;
     unsigned* flags;
@@ -110,6 +109,12 @@ __device__ inline void cutoff_and_slope(float r, float r_cut, float w, float& f,
 }
 
 constexpr int kGradThreads = 256;
+// Floats of a species' H in k_gradients: (l, m >= 0) x n rounded up to even x two signs, an odd number of 16-byte words, so that
+// lanes of neighbouring species read different banks; float2 of a pair's radial values: an odd number of 16-byte words as well.
+__host__ __device__ constexpr int grad_h_pitch(int l_max, int n_max) {
+    return ((l_max + 1) * (l_max + 2) / 2 * ((n_max + 1) & ~1) * 2 / 4 | 1) * 4;
+}
+__host__ __device__ constexpr int grad_g_pitch(int F_pad) { return (F_pad / 2 | 1) * 2; }
 
 // Dense symmetric adjoint weights: Ws[a][l][k][q] = k_l (W_l + W_l^T)[k][q] from the packed upper-triangular
 // weight rows (entry (q1 <= q2) at q1 (2Q - q1 - 1) / 2 + q2), zero in the padding columns q >= Q.
@@ -134,7 +139,466 @@ __global__ void k_wsym(int S, int L1, int Q, int Qw, int ps_norm, const float* _
     }
 }
 
+// Hyper shape of a gradient kernel: compile-time constants for the instantiated shapes (kExpShapes), the launch arguments
+// otherwise.
+template <int SHAPE>
+struct GradShape {
+    int Nmax, Lmax, Q, Nlm, Npad, Fpad, F, Qw, LpAdj, AdjTasks;
+    __device__ __forceinline__ explicit GradShape(const GradArgs& A) {
+        constexpr ExpShape C = kExpShapes[SHAPE];
+        Nmax = SHAPE ? C.n_max : A.n_max;
+        Lmax = SHAPE ? C.l_max : A.l_max;
+        Q = SHAPE ? C.n_max * C.S : A.Q;
+        Nlm = SHAPE ? (C.l_max + 1) * (C.l_max + 1) : A.n_lm;
+        Npad = SHAPE ? exp_npad(C.n_max) : A.n_pad;
+        Fpad = SHAPE ? (C.l_max + 1) * exp_npad(C.n_max) : A.F_pad;
+        F = SHAPE ? (C.l_max + 1) * C.n_max : A.F;
+        Qw = SHAPE ? (C.n_max * C.S + 3) / 4 * 4 : A.Qw;
+        LpAdj = SHAPE ? exp_lp(C.l_max + 1) : A.Lp_adj;
+        AdjTasks = SHAPE ? (C.n_max * C.S + 3) / 4 * (exp_lp(C.l_max + 1) / 4) : A.n_adj_tasks;
+    }
+};
+
+// Rows of chat_l for l in [l0, l1) from staged packed symmetric blocks (pitch Wp, odd: lanes of different l read different
+// banks): a warp takes R rows q, its lanes the 4-column tiles of the padded rows of C. Whether k lies before, in or past the
+// rows, and with it where W[q][k] sits in the packed block, is the same for the whole warp.
+template <int R, class Shape, class Put>
+__device__ __forceinline__ void adjoint_rows(const Shape& K, const float* s_C, const float* s_W, int Wp, int l0, int l1, int ps_norm,
+                                             Put put) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, Q = K.Q, Lq = K.LpAdj;
+    for (int q0 = R * warp; q0 < Q; q0 += R * nwarps) {
+        for (int t = exp_lp(l0) / 4 + lane; t < exp_lp(l1) / 4; t += 32) {
+            int l = l0;
+            while (exp_lp(l + 1) <= 4 * t) ++l;
+            const float* W = s_W + (l - l0) * Wp;
+            const float* C = s_C + 4 * t;
+            uint64_t a[R][2];
+#pragma unroll
+            for (int u = 0; u < R; ++u) a[u][0] = a[u][1] = 0ull;
+            auto step = [&](int k, auto&& w) {
+                const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(C + k * Lq);
+#pragma unroll
+                for (int u = 0; u < R; ++u) {
+                    const float v = w(u);
+                    const uint64_t vv = f2_pack(v, v);
+                    a[u][0] = f2_fma(vv, c.x, a[u][0]);
+                    a[u][1] = f2_fma(vv, c.y, a[u][1]);
+                }
+            };
+            // the packed entry (lo <= hi) sits at lo (2Q - lo - 1) / 2 + hi
+            const float* wr[R];  // rows q0 + u (the last row again for those past it, which are not written)
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const int q = min(q0 + u, Q - 1);
+                wr[u] = W + (q * (2 * Q - q - 1)) / 2;
+            }
+            const float* wk = W + q0;
+            const int last = Q - 1 - q0;
+#pragma unroll 2
+            for (int k = 0; k < q0; ++k) {
+                step(k, [&](int u) { return wk[min(u, last)]; });
+                wk += Q - k - 1;
+            }
+            for (int k = q0; k < min(q0 + R, Q); ++k)
+                step(k, [&](int u) {
+                    const int q = min(q0 + u, Q - 1), lo = min(q, k), hi = max(q, k);
+                    const float v = W[(lo * (2 * Q - lo - 1)) / 2 + hi];
+                    return q == k ? 2.0f * v : v;  // W + W^T
+                });
+#pragma unroll 2
+            for (int k = q0 + R; k < Q; ++k) step(k, [&](int u) { return wr[u][k]; });
+            const float kl = ps_norm ? rsqrtf((float)(2 * l + 1)) : 1.0f;
+            const int s0 = 4 * t - exp_lp(l);
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                if (q0 + u >= Q) break;
+                float v[4];
+                f2_unpack(a[u][0], v[0], v[1]);
+                f2_unpack(a[u][1], v[2], v[3]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (s0 + e <= 2 * l) put(q0 + u, l, s0 + e, kl * v[e]);
+            }
+        }
+    }
+}
+
+// chat = k_l (W + W^T) C of centre i from its coefficients (staged at s_C) and its weights; put(q, l, s, v) takes
+// chat[q][l, m = s - l]. W: what the weights may be, kLinear (a species' dense blocks), kPerCentre (dE/dp; s_W: room for
+// w_lg packed l blocks, or none) or kPerElement (dE/dp read from global memory). s_C holds nothing else yet; a barrier
+// follows before s_C and s_W may be reused.
+// Per-centre dE/dp: with each l block expanded to a dense matrix in turn, two barriers and 12 to 60 tile tasks per l, the
+// adjoint was 640 us of the kernel's 818 on 8 960 centres (n_max 12, l_max 9, 4 species); all packed blocks staged at once
+// and read as they are, 240 of 557 (0.42 GB of dE/dp: 63 us).
+enum { kLinear = 1, kPerCentre = 2, kPerElement = 4 };
+template <int SHAPE, int W, class Put>
+__device__ __forceinline__ void adjoint(const GradArgs& A, const GradShape<SHAPE>& K, int i, int a_i, float* s_C, float* s_W, Put put) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int L1 = K.Lmax + 1, Q = K.Q, n_lm = K.Nlm, Qpk = Q * (Q + 1) / 2, QN = Q * n_lm;
+    const float* Gp = A.grad_ps ? A.grad_ps + (int64_t)i * A.Fp : (a_i >= 0 ? A.weights + (int64_t)a_i * A.Fp : nullptr);
+    const float* c = A.coeffs + (int64_t)i * QN;
+    // prefix counts of the adjoint tile tasks per l: ceil(Q / 4) ceil((2l' + 1) / 4) summed over l' < l
+    auto adj_pref = [&](int l) { return (Q + 3) / 4 * (exp_lp(l) / 4); };
+    // one 4 x 4 register tile of chat_l = Ws_l C_l (rows 4 qt.., columns 4 st.. of the l block), Ws_l dense and
+    // symmetric with row pitch Qw in global memory (the linear model)
+    auto adjoint_tile = [&](const float* Wl, const float* Cl, int Lq, int l, int qt, int st) {
+        // paired FMAs (fma.rn.f32x2): each product rounded exactly as fmaf rounds it
+        uint64_t ap[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) ap[u][0] = ap[u][1] = 0ull;
+        for (int k = 0; k < Q; ++k) {
+            const float4 w4 = __ldg(reinterpret_cast<const float4*>(Wl + k * K.Qw));
+            const float4 c4 = *reinterpret_cast<const float4*>(Cl + k * Lq);
+            const float ww[4] = {w4.x, w4.y, w4.z, w4.w};
+            const uint64_t c01 = f2_pack(c4.x, c4.y), c23 = f2_pack(c4.z, c4.w);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint64_t wu = f2_pack(ww[u], ww[u]);
+                ap[u][0] = f2_fma(wu, c01, ap[u][0]);
+                ap[u][1] = f2_fma(wu, c23, ap[u][1]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = 4 * qt + u;
+            if (q >= Q) break;
+            float v[4];
+            f2_unpack(ap[u][0], v[0], v[1]);
+            f2_unpack(ap[u][1], v[2], v[3]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int sx = 4 * st + e;
+                if (sx <= 2 * l) put(q, l, sx, v[e]);
+            }
+        }
+    };
+    const bool linear = (W & kLinear) && A.wsym;
+    if (linear || ((W & kPerCentre) && A.w_lg)) {
+        // adjoint as 4 x 4 register tiles of chat_l = Ws_l C_l: C staged with every l block padded to a multiple of
+        // 4 columns (zeros), so that tiles load float4 rows of C and of the dense symmetric weights
+        const int Lq = K.LpAdj;
+        // the padding columns of the l blocks (ceil4(2l + 1) - (2l + 1) of them: three for even l, one for odd l)
+        // read as zero; they are disjoint from the copied columns, so the barrier after the copies covers both
+        const int n_padc = 4 * (L1 >> 1) + 3 * (L1 & 1);
+        for (int e = tid; e < Q * n_padc; e += blockDim.x) {
+            const int q = e / n_padc, r = e - q * n_padc;
+            const bool odd = (r & 3) == 3;
+            const int l = 2 * (r >> 2) + (odd ? 1 : 0);
+            s_C[q * Lq + exp_lp(l) + 2 * l + 1 + (odd ? 0 : (r & 3))] = 0.0f;
+        }
+        // lanes over lm, warps over rows
+        for (int lm = lane; lm < n_lm; lm += 32) {
+            const int l = (int)sqrtf((float)lm);  // l with l^2 <= lm < (l + 1)^2
+            const int col = exp_lp(l) + (lm - l * l);
+            for (int q = warp; q < Q; q += nwarps) cp_async4(s_C + q * Lq + col, c + q * n_lm + lm);
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        const int QT = (Q + 3) >> 2;
+        if (linear) {  // linear model: the species' dense blocks, shared by all centres, from global memory (L2)
+            const float* Wsa = A.wsym + (int64_t)(a_i < 0 ? 0 : a_i) * L1 * Q * K.Qw;
+            for (int t = tid; t < K.AdjTasks && a_i >= 0; t += blockDim.x) {
+                int l = 0;
+                while (adj_pref(l + 1) <= t) ++l;
+                const int r = t - adj_pref(l);
+                const int st = r / QT, qt = r - st * QT;
+                adjoint_tile(Wsa + (int64_t)l * Q * K.Qw + 4 * qt, s_C + exp_lp(l) + 4 * st, Lq, l, qt, st);
+            }
+            if (a_i < 0)
+                for (int e = tid; e < QN; e += blockDim.x) {
+                    const int q = e / n_lm, lm = e - q * n_lm, l = (int)sqrtf((float)lm);
+                    put(q, l, lm - l * l, 0.0f);
+                }
+        } else if constexpr ((W & kPerCentre) != 0) {  // this centre's dE/dp: groups of w_lg packed l blocks staged in shared memory
+            const int Wp = Qpk | 1;
+            for (int l0 = 0; l0 < L1; l0 += A.w_lg) {
+                const int l1 = min(L1, l0 + A.w_lg);
+                if (l0) __syncthreads();
+                for (int l = l0; l < l1; ++l)
+                    for (int e = tid; e < Qpk; e += blockDim.x) cp_async4(s_W + (l - l0) * Wp + e, Gp + (int64_t)l * Qpk + e);
+                cp_async_wait_all();
+                __syncthreads();
+                if (A.w_rows == 6)
+                    adjoint_rows<6>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
+                else
+                    adjoint_rows<4>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
+            }
+        }
+        return;
+    }
+    if (W == kLinear) return;
+    for (int e = tid; e < QN; e += blockDim.x) cp_async4(s_C + e, c + e);
+    cp_async_wait_all();
+    __syncthreads();
+    // adjoint chat[q][lm] = k_l sum_k (W + W^T)[q][k] C[k][lm]; the packed entry (q1 <= q2) sits at
+    // q1 (2Q - q1 - 1) / 2 + q2, and (W + W^T) doubles the diagonal
+    for (int e = tid; e < QN; e += blockDim.x) {
+        const int q = e / n_lm, lm = e - q * n_lm;
+        const int l = (int)sqrtf((float)lm);
+        float acc = 0.0f;
+        if (Gp) {
+            const float* W = Gp + (int64_t)l * Qpk;
+            const float* Cc = s_C + lm;
+            int idx = q;  // entry (k, q), k < q
+            for (int k = 0; k < q; ++k) {
+                acc = fmaf(__ldg(W + idx), Cc[k * n_lm], acc);
+                idx += Q - k - 1;
+            }
+            const int ro = (q * (2 * Q - q - 1)) / 2;  // entries (q, k), k >= q
+            acc = fmaf(2.0f * __ldg(W + ro + q), Cc[q * n_lm], acc);
+            for (int k = q + 1; k < Q; ++k) acc = fmaf(__ldg(W + ro + k), Cc[k * n_lm], acc);
+        }
+        put(q, l, lm - l * l, (A.ps_norm ? rsqrtf((float)(2 * l + 1)) : 1.0f) * acc);
+    }
+}
+
 // One CTA per centre i:
+//   1. chat = k_l (W + W^T) C (adjoint), kept as H[a][(l, m >= 0)][n / 2][m, -m][n % 2];
+//   2. per chunk of 32 of the centre's pairs (two CTA barriers per chunk):
+//      radial values (f I, (f I)') per pair into shared memory (a warp takes two pairs at a time, lanes over (l, n));
+//      the m chains: a warp takes an m, its lanes the chunk's pairs. Going up in l it has Y_lm, Y_l-m and their gradients in
+//      registers and forms u = sum_n chat (f I)' and v = sum_n chat f I for both signs of m from two 16-byte loads per two
+//      n (the pair's radial values, the species' H), so that Y is never stored and a value of chat serves 32 pairs;
+//      it leaves its share of s = sum_lm Y u and w = sum_lm dY/du v per pair in shared memory;
+//      the last warp adds the shares of the m up, one pair per lane: dE/dr_ji, the force scatter, F_i and the virial, and
+//      stages the next chunk's records (r_ji, the neighbour's species, j, f_cut, f_cut') beside the others' work.
+// Bound: of 1 383 us on 32 768 centres with 90 pairs (n_max 10, l_max 8, 3 species), the chains take 520 (shared-memory
+// wavefronts: four of radial values and two of chat per eight products of a lane), the spline rows 390 (4.2 GB from L2) and
+// the adjoint 180. With a warp per pair, lanes over lm and Y in shared memory (two loads per two products) the kernel
+// took 2 328 us; 81 -> 58 us on 4 096 centres with 34 pairs (8, 6, 2). Two m per task, halves of n to a warp: 1 430 us.
+// Three CTAs per SM instead of four: 1 510 us.
+template <int SHAPE, int W>
+__global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradients(const GradArgs A) {
+    const GradShape<SHAPE> K(A);
+    constexpr int chunk = 32, nwarps = kGradThreads / 32;
+    const int L1 = K.Lmax + 1, n2 = (K.Nmax + 1) & ~1;             // n in pairs
+    const int Hl = 2 * n2, Hs = grad_h_pitch(K.Lmax, K.Nmax);      // floats of an (l, m) and of a species in H
+    const int NP = n2 / 2;                                         // pairs of n
+    const int Gp = grad_g_pitch(K.Fpad);                           // float2 of a pair's radial values
+    extern __shared__ __align__(16) float sm[];
+    float* s_H = sm;                                               // [S][Hs]
+    // per-pair records, two buffers that alternate between chunks
+    float4* s_vec = reinterpret_cast<float4*>(s_H + A.S * Hs);     // [2][chunk]
+    float4* s_part = s_vec + 2 * chunk;                            // [nwarps][chunk] shares of (s, w)
+    float* s_fc = reinterpret_cast<float*>(s_part + nwarps * chunk);  // [2][chunk]
+    float* s_dfc = s_fc + 2 * chunk;
+    int* s_spc = reinterpret_cast<int*>(s_dfc + 2 * chunk);
+    int* s_j = s_spc + 2 * chunk;
+    // the coefficients are needed only by the adjoint, before the pair loop: they share the area of the radial values
+    float* s_C = reinterpret_cast<float*>(s_j + 2 * chunk);
+    float2* s_GD = reinterpret_cast<float2*>(s_C);                 // [chunk][Gp]
+    __shared__ float s_acc[12][32];  // per lane of the last warp: sums of F_i and of the virial
+    __shared__ int s_sid;
+
+    const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp == nwarps - 1) {  // the centre's structure, for the virial and the energy
+        const int sid = warp_find_structure(A.offs, A.n_s, i, lane);
+        if (lane == 0) s_sid = sid;
+    }
+    const int lab_i = A.species[i];
+    const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
+    // what the adjoint leaves out (m = 0 has no partner, an odd n_max a last n) reads as zero; its first barrier follows
+    for (int e = tid; e < A.S * Hs / 4; e += kGradThreads) reinterpret_cast<float4*>(s_H)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    adjoint<SHAPE, W>(A, K, i, a_i, s_C, reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sm) + A.w_off),
+                   [&](int q, int l, int s, float v) {
+                                         const int a = q / K.Nmax, n = q - a * K.Nmax, m = s - l;
+                                         s_H[a * Hs + (l * (l + 1) / 2 + abs(m)) * Hl + 4 * (n >> 1) + (n & 1) + (m < 0 ? 2 : 0)] = v;
+                                     });
+    const int64_t seg_beg = A.offsets[i];
+    const int seg_len = (int)(A.offsets[i + 1] - seg_beg);
+    const bool last = warp == nwarps - 1;
+    auto stage = [&](int pos, int b) {  // last warp: the records of the chunk at pos into buffer b
+        if (pos + lane >= seg_len) return;
+        const float4 v = __ldg(A.rij + seg_beg + pos + lane);
+        const int j = __ldg(A.nbr_j + seg_beg + pos + lane);
+        const int lab = A.species[j];
+        int a = (lab >= 0 && lab < 256) ? A.lut[lab] : -1;
+        if (!(v.w > 1e-6f)) a = -1;
+        const int o = b * chunk + lane;
+        s_vec[o] = v;
+        s_spc[o] = a;
+        s_j[o] = j;
+        cutoff_and_slope(v.w, A.r_cut, A.width, s_fc[o], s_dfc[o]);
+    };
+    auto finish = [&](int pos, int b) {  // last warp: dE/dr_ji of the chunk at pos, one pair per lane
+        const int o = b * chunk + lane;
+        if (pos + lane >= seg_len || s_spc[o] < 0) return;
+        float S = 0.0f, Wx = 0.0f, Wy = 0.0f, Wz = 0.0f;
+        for (int w = 0; w < min(nwarps, L1); ++w) {
+            const float4 t = s_part[w * chunk + lane];
+            S += t.x;
+            Wx += t.y;
+            Wy += t.z;
+            Wz += t.w;
+        }
+        const float4 v = s_vec[o];
+        const float inv_r = 1.0f / v.w;
+        const float ux = v.x * inv_r, uy = v.y * inv_r, uz = v.z * inv_r;
+        const float wu = Wx * ux + Wy * uy + Wz * uz;
+        const float g[3] = {S * ux + (Wx - wu * ux) * inv_r, S * uy + (Wy - wu * uy) * inv_r, S * uz + (Wz - wu * uz) * inv_r};
+        const int j = s_j[o];
+        const float d[3] = {v.x, v.y, v.z};
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            if (j != i) {
+                atomicAdd(&A.forces[3 * (int64_t)j + x], -g[x]);
+                s_acc[x][lane] += g[x];
+            }
+#pragma unroll
+            for (int y = 0; y < 3; ++y) s_acc[3 + 3 * x + y][lane] = fmaf(g[x], d[y], s_acc[3 + 3 * x + y][lane]);
+        }
+    };
+    if (last) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) s_acc[k][lane] = 0.0f;
+        stage(0, 0);
+    }
+    int b = 0;
+    for (int pos = 0; pos < seg_len; pos += chunk, b ^= 1) {
+        const int nc = min(chunk, seg_len - pos), bo = b * chunk;
+        // the chunk's records are staged; the adjoint is done with the coefficients, the chains with the radial values
+        __syncthreads();
+        auto put = [](float2* gd, int f, float g, float dg) {  // slot f = l n_pad + n of a pair: even and odd n side by side
+            float* o = reinterpret_cast<float*>(gd) + 4 * (f >> 1) + (f & 1);
+            o[0] = g;
+            o[2] = dg;
+        };
+        if (pos == 0 && K.Npad != K.Nmax)  // the padding slots are read as zero and written only here
+            for (int e = tid; e < chunk * L1 * (K.Npad - K.Nmax); e += kGradThreads) {
+                const int q = K.Npad - K.Nmax, n = e % q, l = e / q % L1;
+                put(s_GD + e / q / L1 * Gp, l * K.Npad + K.Nmax + n, 0.0f, 0.0f);
+            }
+        // radial values and slopes: a warp takes two pairs at a time, lanes over (l, n)
+        for (int p = 2 * warp; p < nc; p += 2 * nwarps) {
+            const bool two = p + 1 < nc;
+            const int ob = bo + p, oc = ob + (two ? 1 : 0);
+            const float f0 = s_fc[ob], d0 = s_dfc[ob], f1 = s_fc[oc], d1 = s_dfc[oc];
+            float2* gd = s_GD + p * Gp;
+            auto slot = [&](int c) { return c + c / K.Nmax * (K.Npad - K.Nmax); };  // column l n_max + n -> l n_pad + n
+            if (A.pre_G) {
+                const float* pg = A.pre_G + (seg_beg + pos + p) * K.F;
+                const float* pd = A.pre_D + (seg_beg + pos + p) * K.F;
+                const int64_t o1 = two ? K.F : 0;
+#pragma unroll 4
+                for (int c = lane; c < K.F; c += 32) {
+                    const float g0 = __ldg(pg + c), e0 = __ldg(pd + c), g1 = __ldg(pg + o1 + c), e1 = __ldg(pd + o1 + c);
+                    const int f = slot(c);
+                    put(gd, f, f0 * g0, d0 * g0 + f0 * e0);
+                    if (two) put(gd + Gp, f, f1 * g1, d1 * g1 + f1 * e1);
+                }
+            } else {
+                auto row = [&](int o, float& u) {
+                    const float x = s_vec[o].w * A.inv_delta;
+                    const int k = min(max((int)x, 0), A.M - 1);
+                    u = x - (float)k;
+                    return A.table + k * K.F;
+                };
+                auto value = [&](const float4& cf, float u, float f, float df, float2* o, int fp) {
+                    const float g = fmaf(u, fmaf(u, fmaf(u, cf.w, cf.z), cf.y), cf.x);
+                    const float dg = fmaf(u, fmaf(u, 3.0f * cf.w, 2.0f * cf.z), cf.y) * A.inv_delta;
+                    put(o, fp, f * g, df * g + f * dg);
+                };
+                float u0, u1;
+                const float4 *t0 = row(ob, u0), *t1 = row(oc, u1);
+#pragma unroll 4
+                for (int c = lane; c < K.F; c += 32) {
+                    const float4 c0 = __ldg(t0 + c), c1 = __ldg(t1 + c);
+                    const int f = slot(c);
+                    value(c0, u0, f0, d0, gd, f);
+                    if (two) value(c1, u1, f1, d1, gd + Gp, f);
+                }
+            }
+        }
+        if (last && pos > 0) finish(pos - chunk, b ^ 1);  // its shares stand until the barrier below
+        __syncthreads();
+        // m chains, lanes over the chunk's pairs
+        if (lane < nc && warp < L1) {
+            float S = 0.0f, Wx = 0.0f, Wy = 0.0f, Wz = 0.0f;
+            const float4 v = s_vec[bo + lane];
+            const float inv_r = v.w > 1e-6f ? 1.0f / v.w : 0.0f;
+            const float x = v.x * inv_r, y = v.y * inv_r, z = v.z * inv_r;
+            const float* Ha = s_H + max(s_spc[bo + lane], 0) * Hs;
+            const float2* gp = s_GD + lane * Gp;
+            // warp w takes m = w, 2 nwarps - 1 - w, ...: long chains with short ones
+#pragma unroll 1
+            for (int k = 0; k * nwarps < L1; ++k) {
+                const int m = k * nwarps + ((k & 1) ? nwarps - 1 - warp : warp);
+                if (m >= L1) continue;
+                float q = c_ylm_K[m], q2 = 0.0f, dq = 0.0f, d2 = 0.0f;  // Y_lm / C_m along l, its z derivative
+                float sa = 0.0f, sb = 0.0f, wa = 0.0f, wb = 0.0f, wc = 0.0f, wd = 0.0f;  // sums of q u+-, q v+-, q' v+-
+#pragma unroll 2
+                for (int l = m; l < L1; ++l) {
+                    const ulonglong2* h = reinterpret_cast<const ulonglong2*>(Ha + (l * (l + 1) / 2 + m) * Hl);
+                    const ulonglong2* gr = reinterpret_cast<const ulonglong2*>(gp + l * K.Npad);
+                    uint64_t vp = 0ull, up = 0ull, vn = 0ull, un = 0ull;  // even and odd n
+#pragma unroll
+                    for (int n = 0; n < NP; ++n) {
+                        const ulonglong2 g = gr[n], c = h[n];  // (f I, (f I)') and (chat_m, chat_-m) of two n
+                        vp = f2_fma(c.x, g.x, vp);
+                        up = f2_fma(c.x, g.y, up);
+                        vn = f2_fma(c.y, g.x, vn);
+                        un = f2_fma(c.y, g.y, un);
+                    }
+                    auto sum = [](uint64_t t) {
+                        float e, o;
+                        f2_unpack(t, e, o);
+                        return e + o;
+                    };
+                    const float v0 = sum(vp), v1 = sum(vn);
+                    sa = fmaf(q, sum(up), sa);
+                    sb = fmaf(q, sum(un), sb);
+                    wa = fmaf(q, v0, wa);
+                    wb = fmaf(q, v1, wb);
+                    wc = fmaf(dq, v0, wc);
+                    wd = fmaf(dq, v1, wd);
+                    if (l + 1 == L1) break;
+                    const float Al = c_ylm_A[(l + 1) * 16 + m], Bl = c_ylm_B[(l + 1) * 16 + m];
+                    const float qn = Al * (z * q - Bl * q2), dn = Al * (q + z * dq - Bl * d2);
+                    q2 = q;
+                    d2 = dq;
+                    q = qn;
+                    dq = dn;
+                }
+                float cm = 1.0f, sn = 0.0f, cp = 0.0f, sp = 0.0f;  // (x + iy)^m and (x + iy)^(m - 1)
+#pragma unroll 1
+                for (int e = 0; e < m; ++e) {
+                    cp = cm;
+                    sp = sn;
+                    cm = cp * x - sp * y;
+                    sn = cp * y + sp * x;
+                }
+                // Y_lm = q C_m, Y_l-m = q S_m; d/dx = q m (C_m-1, S_m-1), d/dy = q m (-S_m-1, C_m-1), d/dz = q' (C_m, S_m)
+                const float fm = (float)m;
+                S += sa * cm + sb * sn;
+                Wx += fm * (wa * cp + wb * sp);
+                Wy += fm * (wb * cp - wa * sp);
+                Wz += wc * cm + wd * sn;
+            }
+            s_part[warp * chunk + lane] = make_float4(S, Wx, Wy, Wz);
+        }
+        if (last && pos + chunk < seg_len) stage(pos + chunk, b ^ 1);  // its last readers finished before the barrier above
+    }
+    __syncthreads();
+    if (last && seg_len > 0) finish((seg_len - 1) / chunk * chunk, b ^ 1);
+    // F_i and the virial from the last warp's lanes
+    if (!last) return;
+    float t = 0.0f;  // of component `lane`
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        float v = s_acc[k][lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == k) t = v;
+    }
+    if (lane < 3) {
+        if (t != 0.0f) atomicAdd(&A.forces[3 * (int64_t)i + lane], t);
+    } else if (lane < 12) {
+        atomicAdd(&A.virial[9 * (int64_t)s_sid + (lane - 3)], (double)t);
+    }
+}
+
+// The same for bases whose H and radial values do not fit shared memory beside the coefficients: Y and a few pairs' radial
+// values staged per chunk. One CTA per centre i:
 //   1. chat = k_l (W + W^T) C from the centre's coefficients (shared memory) and its weight block (global, L1);
 //   2. per chunk of the centre's pairs (two CTA barriers per chunk):
 //      radial values (f I, (f I)') per pair (one warp per pair, lanes over (l, n));
@@ -144,20 +608,10 @@ __global__ void k_wsym(int S, int L1, int Q, int Qw, int ps_norm, const float* _
 //      contraction s = sum_lm Y sum_n chat (f I)', w = sum_lm dY/du sum_n chat f I, then dE/dr_ji, the force
 //      scatter and the virial (one warp per pair, lanes over lm, warp-shuffle reduction; F_i and the virial summed
 //      per lane, FP64 across the warps at the end).
-template <int SHAPE = 0>
-__global__ void __launch_bounds__(kGradThreads, 5) k_gradients(const GradArgs A) {
-    // hyper shape: compile-time constants for the instantiated shapes (kExpShapes), the launch arguments otherwise
-    constexpr ExpShape Cs = kExpShapes[SHAPE];
-    const int kNmax = SHAPE ? Cs.n_max : A.n_max, kLmax = SHAPE ? Cs.l_max : A.l_max;
-    const int kQ = SHAPE ? Cs.n_max * Cs.S : A.Q, kNlm = SHAPE ? (Cs.l_max + 1) * (Cs.l_max + 1) : A.n_lm;
-    const int kNpad = SHAPE ? exp_npad(Cs.n_max) : A.n_pad, kFpad = SHAPE ? (Cs.l_max + 1) * exp_npad(Cs.n_max) : A.F_pad;
-    // with n_max a multiple of 4 the padded radial slot f = l n_pad + n is the table column l n_max + n itself
-    constexpr bool kFmapId = SHAPE != 0 && Cs.n_max % 4 == 0;
-    const int kF = SHAPE ? (Cs.l_max + 1) * Cs.n_max : A.F, kQw = SHAPE ? (Cs.n_max * Cs.S + 3) / 4 * 4 : A.Qw;
-    const int kLpAdj = SHAPE ? exp_lp(Cs.l_max + 1) : A.Lp_adj;
-    const int kAdjTasks = SHAPE ? (Cs.n_max * Cs.S + 3) / 4 * (exp_lp(Cs.l_max + 1) / 4) : A.n_adj_tasks;
-    // prefix counts of the adjoint tile tasks per l: ceil(Q / 4) ceil((2l' + 1) / 4) summed over l' < l
-    auto adj_pref = [&](int l) { return SHAPE ? (kQ + 3) / 4 * (exp_lp(l) / 4) : A.adj_pref[l]; };
+static __global__ void __launch_bounds__(kGradThreads, 5) k_gradients_wide(const GradArgs A) {
+    const GradShape<0> K(A);
+    const int kNmax = A.n_max, kLmax = A.l_max, kQ = A.Q, kNlm = A.n_lm, kNpad = A.n_pad, kFpad = A.F_pad, kF = A.F;
+    constexpr bool kFmapId = false;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int chunk = A.chunk;
     const int QN = kQ * kNlm;
@@ -193,130 +647,7 @@ __global__ void __launch_bounds__(kGradThreads, 5) k_gradients(const GradArgs A)
         for (int t = tid; t < kFpad; t += blockDim.x) s_fmap[t] = A.fmap[t];
     const int lab_i = A.species[i];
     const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
-    const float* Gp = A.grad_ps ? A.grad_ps + (int64_t)i * A.Fp : (a_i >= 0 ? A.weights + (int64_t)a_i * A.Fp : nullptr);
-    const float* c = A.coeffs + (int64_t)i * QN;
-    const int Q = kQ, n_lm = kNlm, Qpk = Q * (Q + 1) / 2;
-    // one 4 x 4 register tile of chat_l = Ws_l C_l (rows 4 qt.., columns 4 st.. of the l block), Ws_l dense and
-    // symmetric with row pitch Qw (in global memory for the linear model, in shared memory for a per-centre dE/dp)
-    auto adjoint_tile = [&](const float* Wl, const float* Cl, int Lq, int l, int qt, int st, bool w_global) {
-        // paired FMAs (fma.rn.f32x2): each product rounded exactly as fmaf rounds it
-        uint64_t ap[4][2];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ap[u][0] = ap[u][1] = 0ull;
-        for (int k = 0; k < kQ; ++k) {
-            const float4 w4 = w_global ? __ldg(reinterpret_cast<const float4*>(Wl + k * kQw))
-                                       : *reinterpret_cast<const float4*>(Wl + k * kQw);
-            const float4 c4 = *reinterpret_cast<const float4*>(Cl + k * Lq);
-            const float ww[4] = {w4.x, w4.y, w4.z, w4.w};
-            const uint64_t c01 = f2_pack(c4.x, c4.y), c23 = f2_pack(c4.z, c4.w);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint64_t wu = f2_pack(ww[u], ww[u]);
-                ap[u][0] = f2_fma(wu, c01, ap[u][0]);
-                ap[u][1] = f2_fma(wu, c23, ap[u][1]);
-            }
-        }
-        float acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            f2_unpack(ap[u][0], acc[u][0], acc[u][1]);
-            f2_unpack(ap[u][1], acc[u][2], acc[u][3]);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int q = 4 * qt + u;
-            if (q >= kQ) break;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int sx = 4 * st + v;
-                if (sx <= 2 * l) s_H[q * kNlm + l * l + sx] = acc[u][v];
-            }
-        }
-    };
-    if (A.wsym || A.w_tiled) {
-        // adjoint as 4 x 4 register tiles of chat_l = Ws_l C_l: C staged with every l block padded to a multiple of
-        // 4 columns (zeros), so that tiles load float4 rows of C and of the dense symmetric weights
-        const int Lq = kLpAdj;
-        // the padding columns of the l blocks (ceil4(2l + 1) - (2l + 1) of them: three for even l, one for odd l)
-        // read as zero; they are disjoint from the copied columns, so the barrier after the copies covers both
-        const int n_padc = 4 * (L1 >> 1) + 3 * (L1 & 1);
-        for (int e = tid; e < Q * n_padc; e += blockDim.x) {
-            const int q = e / n_padc, r = e - q * n_padc;
-            const bool odd = (r & 3) == 3;
-            const int l = 2 * (r >> 2) + (odd ? 1 : 0);
-            s_C[q * Lq + exp_lp(l) + 2 * l + 1 + (odd ? 0 : (r & 3))] = 0.0f;
-        }
-        // lanes over lm, warps over rows; no barrier separates these copies from the prologue, so l is computed
-        // here (once per lm) rather than read from s_lofm, which other warps are still writing
-        for (int lm = lane; lm < n_lm; lm += 32) {
-            const int l = (int)sqrtf((float)lm);  // l with l^2 <= lm < (l + 1)^2
-            const int col = exp_lp(l) + (lm - l * l);
-            for (int q = warp; q < Q; q += nwarps) cp_async4(s_C + q * Lq + col, c + q * n_lm + lm);
-        }
-        cp_async_wait_all();
-        __syncthreads();
-        const int QT = (Q + 3) >> 2;
-        if (A.wsym) {  // linear model: the species' dense blocks, shared by all centres, from global memory (L2)
-            const float* Wsa = A.wsym + (int64_t)(a_i < 0 ? 0 : a_i) * L1 * Q * kQw;
-            for (int t = tid; t < kAdjTasks && a_i >= 0; t += blockDim.x) {
-                int l = 0;
-                while (adj_pref(l + 1) <= t) ++l;
-                const int r = t - adj_pref(l);
-                const int st = r / QT, qt = r - st * QT;
-                adjoint_tile(Wsa + (int64_t)l * Q * kQw + 4 * qt, s_C + exp_lp(l) + 4 * st, Lq, l, qt, st, true);
-            }
-            if (a_i < 0)
-                for (int e = tid; e < QN; e += blockDim.x) s_H[e] = 0.0f;
-        } else {  // this centre's dE/dp: one l block at a time, expanded to k_l (W_l + W_l^T) in shared memory
-            float* s_W = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(s_vec) + A.w_off);  // [Q][Qw]
-            for (int l = 0; l < L1; ++l) {
-                const float kl = A.ps_norm ? rsqrtf((float)(2 * l + 1)) : 1.0f;
-                const float* Wp = Gp + (int64_t)l * Qpk;
-                for (int e = tid; e < Q * kQw; e += blockDim.x) {
-                    const int k = e / kQw, q = e - k * kQw;
-                    float v = 0.0f;
-                    if (q < Q) {  // the packed entry (lo <= hi) sits at lo (2Q - lo - 1) / 2 + hi
-                        const int lo = min(q, k), hi = max(q, k);
-                        v = __ldg(Wp + (lo * (2 * Q - lo - 1)) / 2 + hi);
-                        if (q == k) v *= 2.0f;
-                        v *= kl;
-                    }
-                    s_W[e] = v;
-                }
-                __syncthreads();
-                const int ntl = QT * ((2 * l + 1 + 3) / 4);
-                for (int t = tid; t < ntl; t += blockDim.x) {
-                    const int st = t / QT, qt = t - st * QT;
-                    adjoint_tile(s_W + 4 * qt, s_C + exp_lp(l) + 4 * st, Lq, l, qt, st, false);
-                }
-                __syncthreads();
-            }
-        }
-    } else {
-    for (int e = tid; e < QN; e += blockDim.x) cp_async4(s_C + e, c + e);
-    cp_async_wait_all();
-    __syncthreads();
-    // adjoint chat[q][lm] = k_l sum_k (W + W^T)[q][k] C[k][lm]; the packed entry (q1 <= q2) sits at
-    // q1 (2Q - q1 - 1) / 2 + q2, and (W + W^T) doubles the diagonal
-    for (int e = tid; e < QN; e += blockDim.x) {
-        const int q = e / n_lm, lm = e - q * n_lm;
-        const int l = s_lofm[lm];
-        float acc = 0.0f;
-        if (Gp) {
-            const float* W = Gp + (int64_t)l * Qpk;
-            const float* Cc = s_C + lm;
-            int idx = q;  // entry (k, q), k < q
-            for (int k = 0; k < q; ++k) {
-                acc = fmaf(__ldg(W + idx), Cc[k * n_lm], acc);
-                idx += Q - k - 1;
-            }
-            const int ro = (q * (2 * Q - q - 1)) / 2;  // entries (q, k), k >= q
-            acc = fmaf(2.0f * __ldg(W + ro + q), Cc[q * n_lm], acc);
-            for (int k = q + 1; k < Q; ++k) acc = fmaf(__ldg(W + ro + k), Cc[k * n_lm], acc);
-        }
-        s_H[e] = (A.ps_norm ? rsqrtf((float)(2 * l + 1)) : 1.0f) * acc;
-    }
-    }
+    adjoint<0, kLinear | kPerElement>(A, K, i, a_i, s_C, nullptr, [&](int q, int l, int s, float v) { s_H[q * kNlm + l * l + s] = v; });
     // per-lane sums of F_i (lanes 0..2) and of the virial (lanes 3..11, row-major): FP32 within a warp, FP64 across
     // the warps (GB300's FP64 rate is a small fraction of its FP32 rate)
     float racc = 0.0f;
@@ -440,16 +771,16 @@ __global__ void __launch_bounds__(kGradThreads, 5) k_gradients(const GradArgs A)
         for (int p = warp; p < nc; p += nwarps) {
             const int a = s_spc[bo + p];
             if (a < 0) continue;  // warp-uniform
-            const float* H = s_H + a * kNmax * n_lm;
+            const float* H = s_H + a * kNmax * kNlm;
             const float2* gd = s_GD + p * kFpad;
             const float4* Yrow = s_Yv + p * Yp;
             float S = 0.0f, Wx = 0.0f, Wy = 0.0f, Wz = 0.0f;
-            for (int lm = lane; lm < n_lm; lm += 32) {
+            for (int lm = lane; lm < kNlm; lm += 32) {
                 const float2* g = gd + s_lofm[lm] * kNpad;
                 const float* h = H + lm;
                 float uu = 0.0f, vv = 0.0f;
                 for (int n = 0; n < kNmax; ++n) {
-                    const float hv = h[n * n_lm];
+                    const float hv = h[n * kNlm];
                     const float2 x = g[n];
                     vv = fmaf(hv, x.x, vv);
                     uu = fmaf(hv, x.y, uu);
@@ -518,26 +849,40 @@ static size_t grad_aux_off(const rascal_ctx* ctx, int chunk, bool tiled) {
     return align_up(records + std::max(yg, sizeof(float) * QL4), 16);
 }
 
-// bytes from the pair area to the dense weight block of the per-centre tiled adjoint (behind the small tables)
-static size_t grad_w_off(const rascal_ctx* ctx, int chunk) {
-    return align_up(grad_aux_off(ctx, chunk, true) + sizeof(int) * (ctx->n_lm + ctx->plan.F_pad), 16);
-}
-
-static size_t grad_smem(const rascal_ctx* ctx, int chunk, bool tiled, bool w_block = false) {
+static size_t grad_smem(const rascal_ctx* ctx, int chunk, bool tiled) {
     const ExpPlan& P = ctx->plan;
     const size_t QN4 = ((size_t)ctx->Q * ctx->n_lm + 3) / 4 * 4;
-    if (w_block)
-        return sizeof(float) * QN4 + grad_w_off(ctx, chunk) + sizeof(float) * ctx->Q * ((ctx->Q + 3) / 4 * 4) + 64;
     return sizeof(float) * QN4 + grad_aux_off(ctx, chunk, tiled) + sizeof(int) * (ctx->n_lm + P.F_pad) + 64;
 }
 
+// bytes of k_gradients' shared memory before the area that the coefficients (with the dense weight block of a per-centre
+// dE/dp behind them) and then the radial values use, and in all
+static size_t grad_c_off(const rascal_ctx* ctx) {
+    return sizeof(float) * ctx->n_species * grad_h_pitch(ctx->l_max, ctx->n_max) + 32 * (2 * 16 + kGradThreads / 32 * 16 + 2 * 16);
+}
+static size_t grad_c_bytes(const rascal_ctx* ctx, bool tiled) {
+    return align_up(sizeof(float) * ctx->Q * (tiled ? ctx->plan.Lp : ctx->n_lm), 16);
+}
+static size_t grad_w_bytes(const rascal_ctx* ctx, int w_lg) { return sizeof(float) * w_lg * ((ctx->Q * (ctx->Q + 1) / 2) | 1); }
+static size_t grad_chain_smem(const rascal_ctx* ctx, bool tiled, int w_lg) {
+    const size_t c = grad_c_bytes(ctx, tiled) + grad_w_bytes(ctx, w_lg);
+    return grad_c_off(ctx) + std::max(c, sizeof(float2) * 32 * grad_g_pitch(ctx->plan.F_pad));
+}
+
+using GradKernel = void (*)(GradArgs);
+static const GradKernel kGradLinear[] = {k_gradients<0, kLinear>, k_gradients<1, kLinear>, k_gradients<2, kLinear>,
+                                         k_gradients<3, kLinear>, k_gradients<4, kLinear>};
+static const GradKernel kGradPerCentre[] = {k_gradients<0, kPerCentre>, k_gradients<1, kPerCentre>, k_gradients<2, kPerCentre>,
+                                            k_gradients<3, kPerCentre>, k_gradients<4, kPerCentre>};
+static_assert(kNumExpShapes == 5, "an instance per shape");
+
 int gradients_setup(rascal_ctx* ctx) {
     RASCAL_CUDA(upload_ylm_constants(ctx->stream));
-    RASCAL_CUDA(cudaFuncSetAttribute(k_gradients<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    RASCAL_CUDA(cudaFuncSetAttribute(k_gradients<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    RASCAL_CUDA(cudaFuncSetAttribute(k_gradients<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    RASCAL_CUDA(cudaFuncSetAttribute(k_gradients<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    RASCAL_CUDA(cudaFuncSetAttribute(k_gradients<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    RASCAL_CUDA(cudaFuncSetAttribute(k_gradients_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    for (int k = 0; k < kNumExpShapes; ++k) {
+        RASCAL_CUDA(cudaFuncSetAttribute(kGradLinear[k], cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        RASCAL_CUDA(cudaFuncSetAttribute(kGradPerCentre[k], cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    }
     return RASCAL_OK;
 }
 
@@ -588,7 +933,7 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
     RASCAL_CUDA(cudaMemsetAsync(f32, 0, sizeof(float) * 3 * sys->n_atoms, ctx->stream));
     if (!d_offsets || !d_nbr_j || !d_rij || !d_coeffs) return set_error(RASCAL_E_ARG, "NULL device pointer");
     const ExpPlan& P = ctx->plan;
-    GradArgs A;
+    GradArgs A = {};
     A.offsets = d_offsets;
     A.nbr_j = d_nbr_j;
     A.rij = reinterpret_cast<const float4*>(d_rij);
@@ -629,42 +974,42 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
         k_wsym<<<blocks, 256, 0, ctx->stream>>>(ctx->n_species, L1, ctx->Q, A.Qw, ctx->ps_norm, d_weights, A.Fp, ws);
         RASCAL_LAUNCH_CHECK("k_wsym");
         A.wsym = ws;
-        const int QT = (ctx->Q + 3) / 4;
-        A.adj_pref[0] = 0;
-        for (int l = 0; l < L1; ++l) A.adj_pref[l + 1] = A.adj_pref[l] + QT * ((2 * l + 1 + 3) / 4);
-        for (int l = L1; l < kMaxLMax + 1; ++l) A.adj_pref[l + 1] = A.adj_pref[l];
-        A.n_adj_tasks = A.adj_pref[L1];
+        A.n_adj_tasks = (ctx->Q + 3) / 4 * (P.Lp / 4);
     }
-    // the largest chunk (<= 32: one warp stages a chunk, a pair per lane) that keeps five CTAs per SM (48 registers); a
-    // per-centre dE/dp takes the tiled adjoint with one dense l block in shared memory when four CTAs per SM keep a
-    // chunk of at least 8 pairs, else the per-element adjoint
-    int chunk = 32;
-    bool w_tiled = false;
-    if (!d_weights) {
-        while (chunk > 8 && grad_smem(ctx, chunk, true, true) > 54 * 1024) --chunk;
-        w_tiled = grad_smem(ctx, chunk, true, true) <= 54 * 1024;
-        if (!w_tiled) chunk = 32;
+    size_t smem = 0;
+    // a per-centre dE/dp: all its l blocks staged at once where two CTAs per SM still fit, else as many as fit
+    A.w_lg = d_weights ? 0 : L1;
+    while (A.w_lg > 1 && grad_chain_smem(ctx, true, A.w_lg) > 112 * 1024) --A.w_lg;
+    if (A.w_lg && grad_chain_smem(ctx, true, A.w_lg) > 220 * 1024) A.w_lg = 0;
+    smem = grad_chain_smem(ctx, A.wsym || A.w_lg, A.w_lg);
+    const bool chains = smem <= 220 * 1024;  // all but the widest bases (about n_species n_max (l_max + 1)^2 > 24 500)
+    {  // rows of a warp: the fewest rounds x (loads of a step)
+        const int w = kGradThreads / 32;
+        auto cost = [&](int r) { return (ctx->Q + r * w - 1) / (r * w) * (r + 4); };
+        A.w_rows = cost(6) < cost(4) ? 6 : 4;
     }
-    const bool tiled = A.wsym != nullptr || w_tiled;
-    if (!w_tiled)
+    if (chains) {
+        A.chunk = 32;
+        A.w_off = (int)(grad_c_off(ctx) + grad_c_bytes(ctx, true));
+        A.aux_off = 0;
+        if (A.w_lg) A.Lp_adj = P.Lp;
+    } else {
+        // the largest chunk (<= 32: one warp stages a chunk, a pair per lane) that keeps five CTAs per SM (48 registers)
+        const bool tiled = A.wsym != nullptr;
+        int chunk = 32;
         while (chunk > 1 && grad_smem(ctx, chunk, tiled) > 44 * 1024) --chunk;
-    // the radial and contraction phases deal the chunk's pairs to the 8 warps: a chunk one or two pairs past a
-    // multiple of 8 is rounded down, so that no nearly empty last round remains (rounding down only shrinks the
-    // shared memory below)
-    constexpr int kW = kGradThreads / 32;
-    if (chunk > kW && chunk % kW <= 2) chunk -= chunk % kW;
-    // every shared-memory offset and the size come from this final chunk
-    A.chunk = chunk;
-    A.w_tiled = w_tiled ? 1 : 0;
-    A.w_off = 0;
-    if (w_tiled) {
-        A.Qw = Qw;
-        A.Lp_adj = P.Lp;
-        A.w_off = (int)grad_w_off(ctx, chunk);
+        // the radial and contraction phases deal the chunk's pairs to the 8 warps: a chunk one or two pairs past a
+        // multiple of 8 is rounded down, so that no nearly empty last round remains (rounding down only shrinks the
+        // shared memory below)
+        constexpr int kW = kGradThreads / 32;
+        if (chunk > kW && chunk % kW <= 2) chunk -= chunk % kW;
+        // every shared-memory offset and the size come from this final chunk
+        A.chunk = chunk;
+        A.w_lg = 0;
+        A.aux_off = (int)grad_aux_off(ctx, chunk, tiled);
+        smem = grad_smem(ctx, chunk, tiled);
+        if (smem > 220 * 1024) return set_error(RASCAL_E_UNSUPPORTED, "hypers too large for the gradient kernel");
     }
-    A.aux_off = (int)grad_aux_off(ctx, chunk, tiled);
-    const size_t smem = grad_smem(ctx, chunk, tiled, w_tiled);
-    if (smem > 220 * 1024) return set_error(RASCAL_E_UNSUPPORTED, "hypers too large for the gradient kernel");
     if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, true, &A.pre_G, &A.pre_D))) return st;
     // a compiled instance for the hyper shape when the plan's sizes match it (kExpShapes), else the generic kernel
     int shape = 0;
@@ -675,14 +1020,10 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
             ctx->n_lm == (c.l_max + 1) * (c.l_max + 1) && ctx->F == (c.l_max + 1) * c.n_max && (!A.wsym || A.Qw == (ctx->Q + 3) / 4 * 4))
             shape = k;
     }
-    static_assert(kNumExpShapes == 5, "one launch case per shaped instance");
-    switch (shape) {
-        case 1: k_gradients<1><<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A); break;
-        case 2: k_gradients<2><<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A); break;
-        case 3: k_gradients<3><<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A); break;
-        case 4: k_gradients<4><<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A); break;
-        default: k_gradients<0><<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A); break;
-    }
+    if (chains)
+        (d_weights ? kGradLinear : kGradPerCentre)[shape]<<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A);
+    else
+        k_gradients_wide<<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_gradients");
     const int64_t n3 = 3 * (int64_t)sys->n_atoms;
     k_forces_f64<<<(unsigned)std::min<int64_t>((n3 + 255) / 256, 8192), 256, 0, ctx->stream>>>(n3, f32, d_forces);

@@ -160,3 +160,61 @@ def test_power_spectrum_items(rg, n_max, S, l_max):
                 assert np.max(fro) <= 5e-3
             else:
                 assert block_rel_err(p, ref, 2) <= 1e-5, (layout, precision)
+
+
+# Centres with 0, 1, 32, 33 and 65 neighbours (no chunk of 32 pairs, a single pair, full chunks, chunks with one left), odd
+# and even n_max, l_max 0 and 15, one warp's rows of four and of six, packed blocks that do not all fit at once, compiled
+# shapes, and the widest basis, whose tables do not fit and which takes the other kernel. Against sums in 64 bits over the
+# pairs' explicit feature gradients; the bound is the longest chain of roundings that a product passes (rows, columns,
+# l, and the pairs of an atom) times the sum of the products' magnitudes.
+@pytest.mark.parametrize("n_max,l_max,S", [(1, 0, 1), (3, 1, 2), (5, 15, 1), (8, 6, 2), (10, 8, 3), (12, 9, 4), (11, 7, 5),
+                                           (16, 12, 8), (12, 15, 8)])
+def test_gradient_chunks(rg, n_max, l_max, S):
+    import torch
+
+    species = list(range(1, S + 1))
+    calc = rg.SoapCalculator(6.0, 0.5, n_max, l_max, species, spline_intervals=64)
+    rng = np.random.default_rng(43)
+    sizes = (1, 2, 33, 34, 66)
+    pos = np.concatenate([random_cell_atoms(n, np.eye(3) * (1.0 + 0.9 * n ** (1 / 3)), 0.4, rng) * 0.6 for n in sizes])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    N, Q, L1, M = int(off[-1]), S * n_max, l_max + 1, (l_max + 1) ** 2
+    s = System(pos, rng.integers(1, S + 1, N).astype(np.int32), np.tile(np.eye(3) * 40.0, (5, 1, 1)), np.zeros((5, 3), np.int32),
+               off, {})
+    ds = rg.DeviceSystem.from_numpy(s)
+    pairs = calc.neighbours(ds)
+    po = pairs.offsets.cpu().numpy()
+    assert sorted(set(np.diff(po))) == [0, 1, 32, 33, 65]
+    i, j = np.repeat(np.arange(N), np.diff(po)), pairs.nbr_j.cpu().numpy()
+    c = rng.standard_normal((N, Q, M)).astype(np.float32)
+    w = rng.standard_normal((S, L1 * Q * (Q + 1) // 2)).astype(np.float32)
+    g = rng.standard_normal((N, w.shape[1])).astype(np.float32) if N * w.shape[1] < 2e7 else w[s.species - 1]
+    d = torch.cat([calc.debug_pair_gradients(r).double() for r in pairs.rij.split(256)]).cuda()  # [P, 3, n_max, M]
+    ti, tj = torch.tensor(i, device="cuda"), torch.tensor(j, device="cuda").long()
+    lo, hi = np.triu_indices(Q)
+    sid = torch.tensor(np.searchsorted(off, i, side="right") - 1, device="cuda")
+    rij = pairs.rij[:, :3].double()
+    eps = 2.0 ** -24 * (Q + 2 * n_max + 8 * L1 + 32 + 130)
+    cd = torch.tensor(c, device="cuda").double()
+    for weights in (True, False):
+        wi = torch.tensor(w[s.species - 1] if weights else g, device="cuda").double().view(N, L1, -1)
+        pair = torch.zeros(len(i), 3, device="cuda", dtype=torch.float64)
+        size = torch.zeros(len(i), device="cuda", dtype=torch.float64)
+        own = torch.tensor((s.species - 1)[j], device="cuda")
+        for l in range(L1):
+            W = torch.zeros(N, Q, Q, device="cuda", dtype=torch.float64)
+            W[:, lo, hi] = wi[:, l]
+            W = W + W.transpose(1, 2)
+            sl = slice(l * l, (l + 1) ** 2)
+            rows = lambda A, C: ((A @ C) / np.sqrt(2 * l + 1)).view(N, S, n_max, -1)[ti, own]  # noqa: E731
+            chat, mag = rows(W, cd[:, :, sl]), rows(W.abs(), cd[:, :, sl].abs())
+            pair += torch.einsum("pnm,pxnm->px", chat, d[..., sl])
+            size += (mag.norm(dim=2) * d[..., sl].norm(dim=(1, 3))).sum(dim=1)
+        f = torch.zeros(N, 3, device="cuda", dtype=torch.float64).index_add(0, ti, pair).index_add(0, tj, -pair)
+        f_size = torch.zeros(N, device="cuda", dtype=torch.float64).index_add(0, ti, size).index_add(0, tj, size)
+        v = torch.zeros(5, 3, 3, device="cuda", dtype=torch.float64).index_add(0, sid, pair[:, :, None] * rij[:, None, :])
+        v_size = torch.zeros(5, device="cuda", dtype=torch.float64).index_add(0, sid, size * rij.norm(dim=1))
+        kw = dict(weights=torch.tensor(w, device="cuda")) if weights else dict(grad_ps=torch.tensor(g, device="cuda"))
+        fg, vg = calc.gradients(ds, pairs, torch.tensor(c, device="cuda"), **kw)
+        assert bool(((fg - f).abs().amax(dim=1) <= eps * f_size).all()), (weights, float(((fg - f).abs().amax(1) / (eps * f_size)).nan_to_num().max()))
+        assert bool(((vg - v).abs().amax(dim=(1, 2)) <= eps * v_size).all())
