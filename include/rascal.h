@@ -248,6 +248,13 @@ int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
                      const float* d_rij, const float* d_coeffs, const float* d_grad_ps, const float* d_weights,
                      double* d_forces, double* d_virial);
 
+/* The linear model from the coefficients alone: forces and virial as rascal_gradients with d_weights, and the energies
+ * of rascal_linear_energy as half the product of dE_i/dc_i and c_i (E_i is quadratic in c_i), without a power spectrum.
+ *   d_energy [n_structures] float64: overwritten with sum_i w_{a_i} . p_i */
+int rascal_linear_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets, const int* d_nbr_j,
+                            const float* d_rij, const float* d_coeffs, const float* d_weights, double* d_energy,
+                            double* d_forces, double* d_virial);
+
 /* Sparse GPR energy model (Eq. sparse-gp) with the polynomial kernel k(M_I, A_i) = (M^_I . p^_i)^zeta, one model
  * per centre species: E_i = sum over the sparse points I of the centre's species of x_I k(M_I, A_i). With
  * normalize = 1 both vectors are unit-normalised (p^ = p/|p|; a centre with p = 0 keeps p^ = 0), else used as given.

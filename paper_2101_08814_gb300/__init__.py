@@ -253,6 +253,22 @@ class SoapCalculator:
                                                _ptr(forces), _ptr(virial)))
         return forces, virial
 
+    def linear_gradients(self, system: DeviceSystem, pairs: PairList, coeffs, weights):
+        """Energy, forces and virial of the linear model from the coefficients, without their power spectrum."""
+        import torch
+
+        self._bind_stream()
+        _need(coeffs, system.n_atoms * self.coeffs_per_centre, "coeffs")
+        _need(weights, self.n_species * self.n_features("packed"), "weights")
+        energy = torch.empty(system.n_structures, dtype=torch.float64, device=self.device)
+        forces = torch.empty((system.n_atoms, 3), dtype=torch.float64, device=self.device)
+        virial = torch.empty((system.n_structures, 3, 3), dtype=torch.float64, device=self.device)
+        sys_c = system.c_struct()
+        _lib.check(_lib.lib().rascal_linear_gradients(self._ctx, C.byref(sys_c), _ptr(pairs.offsets), _ptr(pairs.nbr_j),
+                                                      _ptr(pairs.rij), _ptr(coeffs), _ptr(weights), _ptr(energy),
+                                                      _ptr(forces), _ptr(virial)))
+        return energy, forces, virial
+
     def debug_pair_gradients(self, rij):
         """d/dr_ji of each pair's term f_cut I^o_nl Y_lm: [P, 3, n_max, (l_max+1)^2] float32 (a test hook)."""
         import torch

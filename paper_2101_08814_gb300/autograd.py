@@ -42,9 +42,8 @@ class LinearSoapEnergy:
 
     def __call__(self, system: DeviceSystem, forces=True):
         pairs = self.calc.neighbours(system)
-        coeffs, ps = self.calc.soap(system, pairs, layout="packed")
-        energy = self.calc.linear_energy(system, ps, self.weights)
-        if not forces:
-            return energy, None, None
-        f, v = self.calc.gradients(system, pairs, coeffs, weights=self.weights)
-        return energy, f, v
+        if forces:  # the adjoint of the forces has the energy too: no power spectrum
+            coeffs = self.calc.spherical_expansion(system, pairs)
+            return self.calc.linear_gradients(system, pairs, coeffs, self.weights)
+        _, ps = self.calc.soap(system, pairs, layout="packed")
+        return self.calc.linear_energy(system, ps, self.weights), None, None

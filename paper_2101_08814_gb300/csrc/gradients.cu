@@ -86,6 +86,7 @@ struct GradArgs {
     int aux_off;            // bytes from the pair area to the small tables (past both the pair area and C)
     float* forces;          // FP32 accumulation, converted to the FP64 output afterwards
     double* virial;
+    double* energy;         // linear model: per-structure energies, or NULL
     unsigned* flags;
     int N, n_s, n_max, l_max, S, Q, n_lm, F, F_pad, n_pad, Lp, M, chunk, ps_norm;
     int64_t Fp;
@@ -226,17 +227,19 @@ __device__ __forceinline__ void adjoint_rows(const Shape& K, const float* s_C, c
 // chat = k_l (W + W^T) C of centre i from its coefficients (staged at s_C) and its weights; put(q, l, s, v) takes
 // chat[q][l, m = s - l]. W: what the weights may be, kLinear (a species' dense blocks), kPerCentre (dE/dp; s_W: room for
 // w_lg packed l blocks, or none) or kPerElement (dE/dp read from global memory). s_C holds nothing else yet; a barrier
-// follows before s_C and s_W may be reused.
+// follows before s_C and s_W may be reused. Returns this thread's share of chat . c (linear: twice E_i = w . p_i, which is
+// quadratic in c).
 // Per-centre dE/dp: with each l block expanded to a dense matrix in turn, two barriers and 12 to 60 tile tasks per l, the
 // adjoint was 640 us of the kernel's 818 on 8 960 centres (n_max 12, l_max 9, 4 species); all packed blocks staged at once
 // and read as they are, 240 of 557 (0.42 GB of dE/dp: 63 us).
 enum { kLinear = 1, kPerCentre = 2, kPerElement = 4 };
 template <int SHAPE, int W, class Put>
-__device__ __forceinline__ void adjoint(const GradArgs& A, const GradShape<SHAPE>& K, int i, int a_i, float* s_C, float* s_W, Put put) {
+__device__ __forceinline__ float adjoint(const GradArgs& A, const GradShape<SHAPE>& K, int i, int a_i, float* s_C, float* s_W, Put put) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int L1 = K.Lmax + 1, Q = K.Q, n_lm = K.Nlm, Qpk = Q * (Q + 1) / 2, QN = Q * n_lm;
     const float* Gp = A.grad_ps ? A.grad_ps + (int64_t)i * A.Fp : (a_i >= 0 ? A.weights + (int64_t)a_i * A.Fp : nullptr);
     const float* c = A.coeffs + (int64_t)i * QN;
+    float dot = 0.0f;
     // prefix counts of the adjoint tile tasks per l: ceil(Q / 4) ceil((2l' + 1) / 4) summed over l' < l
     auto adj_pref = [&](int l) { return (Q + 3) / 4 * (exp_lp(l) / 4); };
     // one 4 x 4 register tile of chat_l = Ws_l C_l (rows 4 qt.., columns 4 st.. of the l block), Ws_l dense and
@@ -265,6 +268,8 @@ __device__ __forceinline__ void adjoint(const GradArgs& A, const GradShape<SHAPE
             float v[4];
             f2_unpack(ap[u][0], v[0], v[1]);
             f2_unpack(ap[u][1], v[2], v[3]);
+            const float4 own = *reinterpret_cast<const float4*>(Cl + q * Lq);  // zero in the padding columns
+            dot = fmaf(v[0], own.x, fmaf(v[1], own.y, fmaf(v[2], own.z, fmaf(v[3], own.w, dot))));
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int sx = 4 * st + e;
@@ -324,9 +329,9 @@ __device__ __forceinline__ void adjoint(const GradArgs& A, const GradShape<SHAPE
                     adjoint_rows<4>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
             }
         }
-        return;
+        return dot;
     }
-    if (W == kLinear) return;
+    if (W == kLinear) return dot;
     for (int e = tid; e < QN; e += blockDim.x) cp_async4(s_C + e, c + e);
     cp_async_wait_all();
     __syncthreads();
@@ -350,10 +355,24 @@ __device__ __forceinline__ void adjoint(const GradArgs& A, const GradShape<SHAPE
         }
         put(q, l, lm - l * l, (A.ps_norm ? rsqrtf((float)(2 * l + 1)) : 1.0f) * acc);
     }
+    return dot;
+}
+
+// E_i = chat . c / 2: FP32 per thread and warp (s_e, a value per warp), FP64 across the warps (read by a warp after a barrier)
+// and one atomic per centre.
+__device__ __forceinline__ void warp_energy(float dot, float* s_e) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = dot;
+}
+__device__ __forceinline__ void add_energy(const float* s_e, double* energy) {
+    double e = 0.0;
+    for (int w = 0; w < kGradThreads / 32; ++w) e += (double)s_e[w];
+    atomicAdd(energy, 0.5 * e);
 }
 
 // One CTA per centre i:
-//   1. chat = k_l (W + W^T) C (adjoint), kept as H[a][(l, m >= 0)][n / 2][m, -m][n % 2];
+//   1. chat = k_l (W + W^T) C (adjoint; with it the linear model's energy), kept as H[a][(l, m >= 0)][n / 2][m, -m][n % 2];
 //   2. per chunk of 32 of the centre's pairs (two CTA barriers per chunk):
 //      radial values (f I, (f I)') per pair into shared memory (a warp takes two pairs at a time, lanes over (l, n));
 //      the m chains: a warp takes an m, its lanes the chunk's pairs. Going up in l it has Y_lm, Y_l-m and their gradients in
@@ -387,6 +406,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     // the coefficients are needed only by the adjoint, before the pair loop: they share the area of the radial values
     float* s_C = reinterpret_cast<float*>(s_j + 2 * chunk);
     float2* s_GD = reinterpret_cast<float2*>(s_C);                 // [chunk][Gp]
+    __shared__ float s_e[nwarps];
     __shared__ float s_acc[12][32];  // per lane of the last warp: sums of F_i and of the virial
     __shared__ int s_sid;
 
@@ -399,11 +419,12 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
     // what the adjoint leaves out (m = 0 has no partner, an odd n_max a last n) reads as zero; its first barrier follows
     for (int e = tid; e < A.S * Hs / 4; e += kGradThreads) reinterpret_cast<float4*>(s_H)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    adjoint<SHAPE, W>(A, K, i, a_i, s_C, reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sm) + A.w_off),
+    const float dot = adjoint<SHAPE, W>(A, K, i, a_i, s_C, reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sm) + A.w_off),
                    [&](int q, int l, int s, float v) {
                                          const int a = q / K.Nmax, n = q - a * K.Nmax, m = s - l;
                                          s_H[a * Hs + (l * (l + 1) / 2 + abs(m)) * Hl + 4 * (n >> 1) + (n & 1) + (m < 0 ? 2 : 0)] = v;
                                      });
+    if (W == kLinear && A.energy) warp_energy(dot, s_e);
     const int64_t seg_beg = A.offsets[i];
     const int seg_len = (int)(A.offsets[i + 1] - seg_beg);
     const bool last = warp == nwarps - 1;
@@ -582,6 +603,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     if (last && seg_len > 0) finish((seg_len - 1) / chunk * chunk, b ^ 1);
     // F_i and the virial from the last warp's lanes
     if (!last) return;
+    if (W == kLinear && A.energy && lane == 0) add_energy(s_e, &A.energy[s_sid]);
     float t = 0.0f;  // of component `lane`
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
@@ -633,6 +655,7 @@ static __global__ void __launch_bounds__(kGradThreads, 5) k_gradients_wide(const
     int* s_lofm = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(s_vec) + A.aux_off);  // [n_lm] l of lm
     int* s_fmap = s_lofm + kNlm;                            // [F_pad]
     __shared__ double red[kGradThreads / 32][12];
+    __shared__ float s_e[kGradThreads / 32];
     __shared__ int s_sid;
 
     const int i = blockIdx.x;
@@ -647,7 +670,8 @@ static __global__ void __launch_bounds__(kGradThreads, 5) k_gradients_wide(const
         for (int t = tid; t < kFpad; t += blockDim.x) s_fmap[t] = A.fmap[t];
     const int lab_i = A.species[i];
     const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
-    adjoint<0, kLinear | kPerElement>(A, K, i, a_i, s_C, nullptr, [&](int q, int l, int s, float v) { s_H[q * kNlm + l * l + s] = v; });
+    const float dot = adjoint<0, kLinear | kPerElement>(A, K, i, a_i, s_C, nullptr, [&](int q, int l, int s, float v) { s_H[q * kNlm + l * l + s] = v; });
+    if (A.energy) warp_energy(dot, s_e);
     // per-lane sums of F_i (lanes 0..2) and of the virial (lanes 3..11, row-major): FP32 within a warp, FP64 across
     // the warps (GB300's FP64 rate is a small fraction of its FP32 rate)
     float racc = 0.0f;
@@ -829,6 +853,8 @@ static __global__ void __launch_bounds__(kGradThreads, 5) k_gradients_wide(const
         } else {
             atomicAdd(&A.virial[9 * (int64_t)s_sid + (tid - 3)], s);
         }
+    } else if (tid == 32 && A.energy) {
+        add_energy(s_e, &A.energy[s_sid]);
     }
 }
 
@@ -907,9 +933,9 @@ extern "C" int rascal_linear_energy(rascal_ctx* ctx, const rascal_system* sys, c
     return RASCAL_OK;
 }
 
-extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets, const int* d_nbr_j,
-                                const float* d_rij, const float* d_coeffs, const float* d_grad_ps, const float* d_weights,
-                                double* d_forces, double* d_virial) {
+static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets, const int* d_nbr_j,
+                     const float* d_rij, const float* d_coeffs, const float* d_grad_ps, const float* d_weights,
+                     double* d_energy, double* d_forces, double* d_virial) {
     clear_error();
     if (!ctx) return set_error(RASCAL_E_ARG, "NULL context");
     int st = validate_system(ctx, sys);
@@ -919,6 +945,7 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
         return set_error(RASCAL_E_ARG, "exactly one of grad_ps and weights must be given");
     RASCAL_CUDA(cudaMemsetAsync(d_forces, 0, sizeof(double) * 3 * sys->n_atoms, ctx->stream));
     RASCAL_CUDA(cudaMemsetAsync(d_virial, 0, sizeof(double) * 9 * sys->n_structures, ctx->stream));
+    if (d_energy) RASCAL_CUDA(cudaMemsetAsync(d_energy, 0, sizeof(double) * sys->n_structures, ctx->stream));
     if (sys->n_atoms == 0) return RASCAL_OK;
     const int L1 = ctx->l_max + 1;
     const int Qw = (ctx->Q + 3) / 4 * 4;
@@ -947,6 +974,7 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
     A.weights = d_weights;
     A.forces = f32;
     A.virial = d_virial;
+    A.energy = d_energy;
     A.flags = ctx->d_flags;
     A.N = sys->n_atoms;
     A.n_s = sys->n_structures;
@@ -1029,6 +1057,22 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
     k_forces_f64<<<(unsigned)std::min<int64_t>((n3 + 255) / 256, 8192), 256, 0, ctx->stream>>>(n3, f32, d_forces);
     RASCAL_LAUNCH_CHECK("k_forces_f64");
     return RASCAL_OK;
+}
+
+extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets, const int* d_nbr_j,
+                                const float* d_rij, const float* d_coeffs, const float* d_grad_ps, const float* d_weights,
+                                double* d_forces, double* d_virial) {
+    return gradients(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs, d_grad_ps, d_weights, nullptr, d_forces, d_virial);
+}
+
+extern "C" int rascal_linear_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets,
+                                       const int* d_nbr_j, const float* d_rij, const float* d_coeffs, const float* d_weights,
+                                       double* d_energy, double* d_forces, double* d_virial) {
+    if (!d_energy) {
+        clear_error();
+        return set_error(RASCAL_E_ARG, "NULL energy");
+    }
+    return gradients(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs, nullptr, d_weights, d_energy, d_forces, d_virial);
 }
 
 namespace rascal {

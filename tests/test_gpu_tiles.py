@@ -218,3 +218,15 @@ def test_gradient_chunks(rg, n_max, l_max, S):
         fg, vg = calc.gradients(ds, pairs, torch.tensor(c, device="cuda"), **kw)
         assert bool(((fg - f).abs().amax(dim=1) <= eps * f_size).all()), (weights, float(((fg - f).abs().amax(1) / (eps * f_size)).nan_to_num().max()))
         assert bool(((vg - v).abs().amax(dim=(1, 2)) <= eps * v_size).all())
+        if not weights:
+            continue
+        # the energies from the coefficients: half of chat . c, at most rows, columns and 130 atoms of roundings
+        e, fe, ve = calc.linear_gradients(ds, pairs, torch.tensor(c, device="cuda"), kw["weights"])
+        p = calc.power_spectrum(torch.tensor(c, device="cuda")).double()
+        pa = calc.power_spectrum(torch.tensor(np.abs(c), device="cuda")).double()
+        at = torch.tensor(np.repeat(np.arange(5), sizes), device="cuda")
+        wa = torch.tensor(w[s.species - 1], device="cuda").double()
+        ref = torch.zeros(5, device="cuda", dtype=torch.float64).index_add(0, at, (p * wa).sum(1))
+        e_size = torch.zeros(5, device="cuda", dtype=torch.float64).index_add(0, at, (pa * wa.abs()).sum(1))
+        assert bool(((e - ref).abs() <= eps * e_size).all())
+        assert bool(((fe - f).abs().amax(dim=1) <= eps * f_size).all()) and bool(((ve - v).abs().amax(dim=(1, 2)) <= eps * v_size).all())
