@@ -110,12 +110,30 @@ __device__ inline void cutoff_and_slope(float r, float r_cut, float w, float& f,
 }
 
 constexpr int kGradThreads = 256;
+
+// Y_lm = q_lm(z) C_m, Y_l-m = q_lm(z) S_m down in m at fixed l, from Legendre's equation differentiated m times:
+// q_lm = x z q_{l,m+1} + y (1 - z^2) q_{l,m+2} and dq_lm/dz = w q_{l,m+1} with (x, y, w) = c_ylm_down[l][m], q_ll = c_ylm_K[l].
+// In FP32 the errors are 0.6 (l = 8) to 0.5 (l = 12) times those of the recurrence up in l, 0.2 times near the poles.
+static __constant__ float4 c_ylm_down[16 * 16];
+
+static cudaError_t upload_ylm_down(cudaStream_t stream) {
+    float4 t[256] = {};
+    for (int l = 1; l < 16; ++l)
+        for (int m = 0; m < l; ++m) {
+            const double s = m ? 1.0 : sqrt(0.5), p = (double)(l - m) * (l + m + 1);
+            t[l * 16 + m] = make_float4((float)(2.0 * (m + 1) * s / sqrt(p)), (float)(-s * sqrt((l + m + 2.0) * (l - m - 1.0) / p)),
+                                        (float)(s * sqrt(p)), 0.0f);
+        }
+    return cudaMemcpyToSymbolAsync(c_ylm_down, t, sizeof(t), 0, cudaMemcpyHostToDevice, stream);
+}
+
 // Floats of a species' H in k_gradients: (l, m >= 0) x n rounded up to even x two signs, an odd number of 16-byte words, so that
-// lanes of neighbouring species read different banks; float2 of a pair's radial values: an odd number of 16-byte words as well.
+// lanes of neighbouring species read different banks; floats of a pair's radial values and slopes: an odd number of 8-byte
+// words (F_pad is a multiple of 4).
 __host__ __device__ constexpr int grad_h_pitch(int l_max, int n_max) {
     return ((l_max + 1) * (l_max + 2) / 2 * ((n_max + 1) & ~1) * 2 / 4 | 1) * 4;
 }
-__host__ __device__ constexpr int grad_g_pitch(int F_pad) { return (F_pad / 2 | 1) * 2; }
+__host__ __device__ constexpr int grad_g_pitch(int F_pad) { return 2 * F_pad + 2; }
 
 // Dense symmetric adjoint weights: Ws[a][l][k][q] = k_l (W_l + W_l^T)[k][q] from the packed upper-triangular
 // weight rows (entry (q1 <= q2) at q1 (2Q - q1 - 1) / 2 + q2), zero in the padding columns q >= Q.
@@ -375,17 +393,17 @@ __device__ __forceinline__ void add_energy(const float* s_e, double* energy) {
 //   1. chat = k_l (W + W^T) C (adjoint; with it the linear model's energy), kept as H[a][(l, m >= 0)][n / 2][m, -m][n % 2];
 //   2. per chunk of 32 of the centre's pairs (two CTA barriers per chunk):
 //      radial values (f I, (f I)') per pair into shared memory (a warp takes two pairs at a time, lanes over (l, n));
-//      the m chains: a warp takes an m, its lanes the chunk's pairs. Going up in l it has Y_lm, Y_l-m and their gradients in
-//      registers and forms u = sum_n chat (f I)' and v = sum_n chat f I for both signs of m from two 16-byte loads per two
-//      n (the pair's radial values, the species' H), so that Y is never stored and a value of chat serves 32 pairs;
-//      it leaves its share of s = sum_lm Y u and w = sum_lm dY/du v per pair in shared memory;
-//      the last warp adds the shares of the m up, one pair per lane: dE/dr_ji, the force scatter, F_i and the virial, and
+//      the contraction: a warp takes an l (and a block of n), its lanes the chunk's pairs. The pair's radial values of that l
+//      stay in registers; going down in m it forms u = sum_n chat (f I)' and v = sum_n chat f I for both signs of m from one
+//      16-byte load of H per two n and eight products, has q_lm and its slope from a recurrence, and sums over m by Horner's
+//      rule in x + iy, so that Y is never stored; it leaves its share of s = sum_lm Y u and w = sum_lm dY/du v per pair;
+//      the last warp adds the shares up, one pair per lane: dE/dr_ji, the force scatter, F_i and the virial, and
 //      stages the next chunk's records (r_ji, the neighbour's species, j, f_cut, f_cut') beside the others' work.
-// Bound: of 1 383 us on 32 768 centres with 90 pairs (n_max 10, l_max 8, 3 species), the chains take 520 (shared-memory
-// wavefronts: four of radial values and two of chat per eight products of a lane), the spline rows 390 (4.2 GB from L2) and
-// the adjoint 180. With a warp per pair, lanes over lm and Y in shared memory (two loads per two products) the kernel
-// took 2 328 us; 81 -> 58 us on 4 096 centres with 34 pairs (8, 6, 2). Two m per task, halves of n to a warp: 1 430 us.
-// Three CTAs per SM instead of four: 1 510 us.
+// Bound: latency at four CTAs of 256 threads per SM between the phases' barriers (issue slots 55 %, shared memory 70 %). Of
+// 1 390 us on 32 768 centres with 90 pairs (n_max 10, l_max 8, 3 species), the contraction takes 500, the radial values 420
+// (4.2 GB from L2) and the adjoint 180. With a warp per pair, lanes over lm and Y in shared memory (two loads per two
+// products) the kernel took 2 328 us; with a warp per m, up in l, radial values loaded for every m, 1 422; with half of n_max
+// 10 per task 1 526; with three CTAs per SM 1 510. 4 096 centres with 34 pairs (8, 6, 2): 81 -> 63 us.
 template <int SHAPE, int W>
 __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradients(const GradArgs A) {
     const GradShape<SHAPE> K(A);
@@ -393,7 +411,10 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     const int L1 = K.Lmax + 1, n2 = (K.Nmax + 1) & ~1;             // n in pairs
     const int Hl = 2 * n2, Hs = grad_h_pitch(K.Lmax, K.Nmax);      // floats of an (l, m) and of a species in H
     const int NP = n2 / 2;                                         // pairs of n
-    const int Gp = grad_g_pitch(K.Fpad);                           // float2 of a pair's radial values
+    // pairs of n of a task (its radial values stay in registers: all of n_max up to 10, else half), and tasks of an l
+    constexpr int kN = kExpShapes[SHAPE].n_max, NB = SHAPE == 0 ? 4 : (kN <= 10 ? (kN + 1) / 2 : (kN + 3) / 4);
+    const int NK = (NP + NB - 1) / NB;
+    const int Gp = grad_g_pitch(K.Fpad);                           // floats of a pair's radial values
     extern __shared__ __align__(16) float sm[];
     float* s_H = sm;                                               // [S][Hs]
     // per-pair records, two buffers that alternate between chunks
@@ -405,7 +426,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     int* s_j = s_spc + 2 * chunk;
     // the coefficients are needed only by the adjoint, before the pair loop: they share the area of the radial values
     float* s_C = reinterpret_cast<float*>(s_j + 2 * chunk);
-    float2* s_GD = reinterpret_cast<float2*>(s_C);                 // [chunk][Gp]
+    float* s_G = s_C;                                              // [chunk][Gp]: f I, then (f I)'
     __shared__ float s_e[nwarps];
     __shared__ float s_acc[12][32];  // per lane of the last warp: sums of F_i and of the virial
     __shared__ int s_sid;
@@ -419,11 +440,11 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
     // what the adjoint leaves out (m = 0 has no partner, an odd n_max a last n) reads as zero; its first barrier follows
     for (int e = tid; e < A.S * Hs / 4; e += kGradThreads) reinterpret_cast<float4*>(s_H)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float dot = adjoint<SHAPE, W>(A, K, i, a_i, s_C, reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sm) + A.w_off),
-                   [&](int q, int l, int s, float v) {
-                                         const int a = q / K.Nmax, n = q - a * K.Nmax, m = s - l;
-                                         s_H[a * Hs + (l * (l + 1) / 2 + abs(m)) * Hl + 4 * (n >> 1) + (n & 1) + (m < 0 ? 2 : 0)] = v;
-                                     });
+    float* s_W = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sm) + A.w_off);
+    const float dot = adjoint<SHAPE, W>(A, K, i, a_i, s_C, s_W, [&](int q, int l, int s, float v) {
+        const int a = q / K.Nmax, n = q - a * K.Nmax, m = s - l;
+        s_H[a * Hs + (l * (l + 1) / 2 + abs(m)) * Hl + 4 * (n >> 1) + (n & 1) + (m < 0 ? 2 : 0)] = v;
+    });
     if (W == kLinear && A.energy) warp_energy(dot, s_e);
     const int64_t seg_beg = A.offsets[i];
     const int seg_len = (int)(A.offsets[i + 1] - seg_beg);
@@ -445,7 +466,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
         const int o = b * chunk + lane;
         if (pos + lane >= seg_len || s_spc[o] < 0) return;
         float S = 0.0f, Wx = 0.0f, Wy = 0.0f, Wz = 0.0f;
-        for (int w = 0; w < min(nwarps, L1); ++w) {
+        for (int w = 0; w < nwarps; ++w) {
             const float4 t = s_part[w * chunk + lane];
             S += t.x;
             Wx += t.y;
@@ -479,22 +500,21 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
         const int nc = min(chunk, seg_len - pos), bo = b * chunk;
         // the chunk's records are staged; the adjoint is done with the coefficients, the chains with the radial values
         __syncthreads();
-        auto put = [](float2* gd, int f, float g, float dg) {  // slot f = l n_pad + n of a pair: even and odd n side by side
-            float* o = reinterpret_cast<float*>(gd) + 4 * (f >> 1) + (f & 1);
-            o[0] = g;
-            o[2] = dg;
+        auto put = [&](float* gd, int f, float g, float dg) {  // slot f = l n_pad + n of a pair
+            gd[f] = g;
+            gd[K.Fpad + f] = dg;
         };
         if (pos == 0 && K.Npad != K.Nmax)  // the padding slots are read as zero and written only here
             for (int e = tid; e < chunk * L1 * (K.Npad - K.Nmax); e += kGradThreads) {
                 const int q = K.Npad - K.Nmax, n = e % q, l = e / q % L1;
-                put(s_GD + e / q / L1 * Gp, l * K.Npad + K.Nmax + n, 0.0f, 0.0f);
+                put(s_G + e / q / L1 * Gp, l * K.Npad + K.Nmax + n, 0.0f, 0.0f);
             }
         // radial values and slopes: a warp takes two pairs at a time, lanes over (l, n)
         for (int p = 2 * warp; p < nc; p += 2 * nwarps) {
             const bool two = p + 1 < nc;
             const int ob = bo + p, oc = ob + (two ? 1 : 0);
             const float f0 = s_fc[ob], d0 = s_dfc[ob], f1 = s_fc[oc], d1 = s_dfc[oc];
-            float2* gd = s_GD + p * Gp;
+            float* gd = s_G + p * Gp;
             auto slot = [&](int c) { return c + c / K.Nmax * (K.Npad - K.Nmax); };  // column l n_max + n -> l n_pad + n
             if (A.pre_G) {
                 const float* pg = A.pre_G + (seg_beg + pos + p) * K.F;
@@ -514,10 +534,11 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
                     u = x - (float)k;
                     return A.table + k * K.F;
                 };
-                auto value = [&](const float4& cf, float u, float f, float df, float2* o, int fp) {
-                    const float g = fmaf(u, fmaf(u, fmaf(u, cf.w, cf.z), cf.y), cf.x);
-                    const float dg = fmaf(u, fmaf(u, 3.0f * cf.w, 2.0f * cf.z), cf.y) * A.inv_delta;
-                    put(o, fp, f * g, df * g + f * dg);
+                auto value = [&](const float4& cf, float u, float f, float df, float* o, int fp) {
+                    // value and slope of the cubic by Horner's scheme twice
+                    const float b1 = fmaf(u, cf.w, cf.z), b0 = fmaf(u, b1, cf.y), g = fmaf(u, b0, cf.x);
+                    const float dg = fmaf(u, fmaf(u, cf.w, b1), b0);
+                    put(o, fp, f * g, fmaf(df, g, f * A.inv_delta * dg));
                 };
                 float u0, u1;
                 const float4 *t0 = row(ob, u0), *t1 = row(oc, u1);
@@ -532,33 +553,48 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
         }
         if (last && pos > 0) finish(pos - chunk, b ^ 1);  // its shares stand until the barrier below
         __syncthreads();
-        // m chains, lanes over the chunk's pairs
-        if (lane < nc && warp < L1) {
+        // contraction, lanes over the chunk's pairs; a warp's tasks: t = w, 2 nwarps - 1 - w, ...: large l with small ones
+        if (lane < nc) {
             float S = 0.0f, Wx = 0.0f, Wy = 0.0f, Wz = 0.0f;
             const float4 v = s_vec[bo + lane];
             const float inv_r = v.w > 1e-6f ? 1.0f / v.w : 0.0f;
-            const float x = v.x * inv_r, y = v.y * inv_r, z = v.z * inv_r;
+            const float x = v.x * inv_r, y = v.y * inv_r, z = v.z * inv_r, xy2 = x * x + y * y;
             const float* Ha = s_H + max(s_spc[bo + lane], 0) * Hs;
-            const float2* gp = s_GD + lane * Gp;
-            // warp w takes m = w, 2 nwarps - 1 - w, ...: long chains with short ones
+            const float* gp = s_G + lane * Gp;
+            const int tasks = L1 * NK;
 #pragma unroll 1
-            for (int k = 0; k * nwarps < L1; ++k) {
-                const int m = k * nwarps + ((k & 1) ? nwarps - 1 - warp : warp);
-                if (m >= L1) continue;
-                float q = c_ylm_K[m], q2 = 0.0f, dq = 0.0f, d2 = 0.0f;  // Y_lm / C_m along l, its z derivative
-                float sa = 0.0f, sb = 0.0f, wa = 0.0f, wb = 0.0f, wc = 0.0f, wd = 0.0f;  // sums of q u+-, q v+-, q' v+-
-#pragma unroll 2
-                for (int l = m; l < L1; ++l) {
-                    const ulonglong2* h = reinterpret_cast<const ulonglong2*>(Ha + (l * (l + 1) / 2 + m) * Hl);
-                    const ulonglong2* gr = reinterpret_cast<const ulonglong2*>(gp + l * K.Npad);
+            for (int k = 0; k * nwarps < tasks; ++k) {
+                const int t = k * nwarps + ((k & 1) ? nwarps - 1 - warp : warp);
+                if (t >= tasks) continue;
+                const int l = K.Lmax - t / NK, n0 = t % NK * NB;  // pairs of n from n0
+                uint64_t g[NB], d[NB];
+#pragma unroll
+                for (int n = 0; n < NB; ++n) {
+                    if (NP % NB && n0 + n >= NP) break;
+                    g[n] = *reinterpret_cast<const uint64_t*>(gp + l * K.Npad + 2 * (n0 + n));
+                    d[n] = *reinterpret_cast<const uint64_t*>(gp + K.Fpad + l * K.Npad + 2 * (n0 + n));
+                }
+                // down in m: q = Y_lm / C_m, dq its z derivative; sums over m of (q u_m - i q u_-m) w^m, the same with v
+                // and dq, and of m (q v_m - i q v_-m) w^(m - 1), w = x + iy, by Horner's rule
+                float q = c_ylm_K[l], q1 = 0.0f, dq = 0.0f;
+                float sr = 0.0f, si = 0.0f, zr = 0.0f, zi = 0.0f, tr = 0.0f, ti = 0.0f;
+                auto horner = [&](float& re, float& im, float a, float b) {
+                    const float r = fmaf(re, x, fmaf(-im, y, a));
+                    im = fmaf(re, y, fmaf(im, x, -b));
+                    re = r;
+                };
+                const ulonglong2* h = reinterpret_cast<const ulonglong2*>(Ha + (l * (l + 1) / 2 + l) * Hl) + n0;
+#pragma unroll 1
+                for (int m = l;; --m, h -= NP) {
                     uint64_t vp = 0ull, up = 0ull, vn = 0ull, un = 0ull;  // even and odd n
 #pragma unroll
-                    for (int n = 0; n < NP; ++n) {
-                        const ulonglong2 g = gr[n], c = h[n];  // (f I, (f I)') and (chat_m, chat_-m) of two n
-                        vp = f2_fma(c.x, g.x, vp);
-                        up = f2_fma(c.x, g.y, up);
-                        vn = f2_fma(c.y, g.x, vn);
-                        un = f2_fma(c.y, g.y, un);
+                    for (int n = 0; n < NB; ++n) {
+                        if (NP % NB && n0 + n >= NP) break;
+                        const ulonglong2 c = h[n];  // (chat_m, chat_-m) of two n
+                        vp = f2_fma(c.x, g[n], vp);
+                        up = f2_fma(c.x, d[n], up);
+                        vn = f2_fma(c.y, g[n], vn);
+                        un = f2_fma(c.y, d[n], un);
                     }
                     auto sum = [](uint64_t t) {
                         float e, o;
@@ -566,34 +602,21 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
                         return e + o;
                     };
                     const float v0 = sum(vp), v1 = sum(vn);
-                    sa = fmaf(q, sum(up), sa);
-                    sb = fmaf(q, sum(un), sb);
-                    wa = fmaf(q, v0, wa);
-                    wb = fmaf(q, v1, wb);
-                    wc = fmaf(dq, v0, wc);
-                    wd = fmaf(dq, v1, wd);
-                    if (l + 1 == L1) break;
-                    const float Al = c_ylm_A[(l + 1) * 16 + m], Bl = c_ylm_B[(l + 1) * 16 + m];
-                    const float qn = Al * (z * q - Bl * q2), dn = Al * (q + z * dq - Bl * d2);
-                    q2 = q;
-                    d2 = dq;
+                    horner(sr, si, q * sum(up), q * sum(un));
+                    horner(zr, zi, dq * v0, dq * v1);
+                    if (m == 0) break;
+                    const float mq = (float)m * q;
+                    horner(tr, ti, mq * v0, mq * v1);
+                    const float4 f = c_ylm_down[l * 16 + m - 1];
+                    const float qn = fmaf(f.x * z, q, f.y * (xy2 * q1));
+                    dq = f.z * q;
+                    q1 = q;
                     q = qn;
-                    dq = dn;
                 }
-                float cm = 1.0f, sn = 0.0f, cp = 0.0f, sp = 0.0f;  // (x + iy)^m and (x + iy)^(m - 1)
-#pragma unroll 1
-                for (int e = 0; e < m; ++e) {
-                    cp = cm;
-                    sp = sn;
-                    cm = cp * x - sp * y;
-                    sn = cp * y + sp * x;
-                }
-                // Y_lm = q C_m, Y_l-m = q S_m; d/dx = q m (C_m-1, S_m-1), d/dy = q m (-S_m-1, C_m-1), d/dz = q' (C_m, S_m)
-                const float fm = (float)m;
-                S += sa * cm + sb * sn;
-                Wx += fm * (wa * cp + wb * sp);
-                Wy += fm * (wb * cp - wa * sp);
-                Wz += wc * cm + wd * sn;
+                S += sr;  // Y_lm = q C_m, Y_l-m = q S_m with w^m = C_m + i S_m
+                Wx += tr;
+                Wy -= ti;
+                Wz += zr;
             }
             s_part[warp * chunk + lane] = make_float4(S, Wx, Wy, Wz);
         }
@@ -670,7 +693,8 @@ static __global__ void __launch_bounds__(kGradThreads, 5) k_gradients_wide(const
         for (int t = tid; t < kFpad; t += blockDim.x) s_fmap[t] = A.fmap[t];
     const int lab_i = A.species[i];
     const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
-    const float dot = adjoint<0, kLinear | kPerElement>(A, K, i, a_i, s_C, nullptr, [&](int q, int l, int s, float v) { s_H[q * kNlm + l * l + s] = v; });
+    const float dot = adjoint<0, kLinear | kPerElement>(
+        A, K, i, a_i, s_C, nullptr, [&](int q, int l, int s, float v) { s_H[q * kNlm + l * l + s] = v; });
     if (A.energy) warp_energy(dot, s_e);
     // per-lane sums of F_i (lanes 0..2) and of the virial (lanes 3..11, row-major): FP32 within a warp, FP64 across
     // the warps (GB300's FP64 rate is a small fraction of its FP32 rate)
@@ -892,7 +916,7 @@ static size_t grad_c_bytes(const rascal_ctx* ctx, bool tiled) {
 static size_t grad_w_bytes(const rascal_ctx* ctx, int w_lg) { return sizeof(float) * w_lg * ((ctx->Q * (ctx->Q + 1) / 2) | 1); }
 static size_t grad_chain_smem(const rascal_ctx* ctx, bool tiled, int w_lg) {
     const size_t c = grad_c_bytes(ctx, tiled) + grad_w_bytes(ctx, w_lg);
-    return grad_c_off(ctx) + std::max(c, sizeof(float2) * 32 * grad_g_pitch(ctx->plan.F_pad));
+    return grad_c_off(ctx) + std::max(c, sizeof(float) * 32 * grad_g_pitch(ctx->plan.F_pad));
 }
 
 using GradKernel = void (*)(GradArgs);
@@ -904,6 +928,7 @@ static_assert(kNumExpShapes == 5, "an instance per shape");
 
 int gradients_setup(rascal_ctx* ctx) {
     RASCAL_CUDA(upload_ylm_constants(ctx->stream));
+    RASCAL_CUDA(upload_ylm_down(ctx->stream));
     RASCAL_CUDA(cudaFuncSetAttribute(k_gradients_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     for (int k = 0; k < kNumExpShapes; ++k) {
         RASCAL_CUDA(cudaFuncSetAttribute(kGradLinear[k], cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
