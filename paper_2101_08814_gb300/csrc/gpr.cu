@@ -9,16 +9,15 @@
 //
 // Both contractions are dense GEMMs between the centres of one species and that species' sparse points, so the
 // centres are first bucketed by species (k_gpr_count, k_gpr_scatter: a stable counting sort on the device).
-//   k_gpr_kernel: D[128 centres][<= 512 sparse points] = p_rows . M^T over the features, A rows gathered from the
-//     feature matrix by cp.async (16-byte copies, zero-filled past the end), B = M^ rows (TF32-rounded at model
-//     creation); 5-stage shared-memory pipeline (kGprStages), one thread issues the MMAs, completion per stage on mbarriers.
+//   k_gpr_kernel: D[128 centres][128, 256 or 512 sparse points] = p_rows . M^T over the features, A rows gathered from the
+//     feature matrix by cp.async (16-byte copies, zero-filled past the end), B = M^ rows (TF32-rounded at model creation).
 //     Epilogue (TMEM -> registers): the row norms (accumulated from the staged A tiles), k^zeta, E partials and the
 //     per-(centre, point) factor W = x zeta k^(zeta-1), stored for the gradient GEMM.
 //   k_gpr_finish: per structure, E_i summed over the passes, FP64 structure energies, zeta E_i / |p_i|^2 (the
 //     normalisation's share of the chain rule; 0 without normalisation).
 //   k_gpr_grad: D[128 centres][256 features] = W . M^ over the active set, epilogue dE/dp = D / |p| - zeta E p / |p|^2.
-// Operand tiles in shared memory are K-major with 64 bytes of K per row and stage, in the 64-byte swizzled layout
-// (8-row atoms of 512 bytes): TMA writes it for the dense operands (the sparse points, W), the gathered feature
+// Operand tiles in shared memory are K-major with 128 bytes of K per row and stage (64 in 512-point tiles), in the 128-byte
+// (64-byte) swizzled layout (8-row atoms): TMA writes it for the dense operands (the sparse points, W), the gathered feature
 // rows are copied into it by cp.async.
 #include <algorithm>
 #include <cmath>
@@ -39,24 +38,25 @@ struct rascal_gpr {
     int n_pad[rascal::kMaxSpecies];         // rounded up to 16
     int64_t row_off[rascal::kMaxSpecies];   // first row of a species in M and x
     int64_t t_off[rascal::kMaxSpecies];     // first element of a species' block [Fn][n_pad] in MT
-    int n_pad_max, passes_max;
+    int n_pad_max;
     int64_t rows;
     float* d_M;   // [rows][Fk]   M^ rows, TF32-rounded, zero-padded
     float* d_MT;  // per species [Fn][n_pad]: M^ transposed (K-major operand of the gradient GEMM)
     float* d_x;   // [rows] x_I (0 in the padding)
-    CUtensorMap tmM;                          // TMA maps of d_M and of each species' block of d_MT
+    CUtensorMap tmM, tmM32;                   // TMA maps of d_M (16 and 32 columns a box) and of each species' block of d_MT
     CUtensorMap tmMT[rascal::kMaxSpecies];
 };
 
 namespace rascal {
 
 constexpr int kGprThreads = 256;
-constexpr int kGprStages = 5;               // kernel GEMM pipeline depth (40 KB per stage)
-constexpr int kGprStages2 = 4;              // gradient GEMM (24 KB per stage, two CTAs per SM)
-constexpr int kGprKB = 16;                   // K elements (TF32) per stage: 64 bytes per operand row
-constexpr int kGprATile = 128 * 64;          // bytes of one A stage
-constexpr int kGprB1 = 512 * 64;             // B stage of the kernel GEMM (up to 512 sparse points)
-constexpr int kGprB2 = 256 * 64;             // B stage of the gradient GEMM (256 features)
+constexpr int kGprThreads2 = kGprThreads + 64;  // gradient GEMM: eight epilogue warps, the MMAs' and the loads'
+// kernel GEMM pipeline depth for tiles of 128 (16 KB per stage), 256 (24 KB) and 512 sparse points (40 KB)
+constexpr int gpr_stages(int cols) { return cols == 128 ? 6 : (cols == 256 ? 4 : 5); }
+constexpr int gpr_kb(int cols) { return cols == 512 ? 16 : 32; }  // K elements (TF32) per stage
+constexpr int kGprStages2 = 2;              // gradient GEMM (48 KB per stage, two CTAs per SM)
+constexpr int kGprFT = 256;                  // features of a tile of the gradient GEMM
+constexpr int kGprB2 = kGprFT * 128;         // its B stage
 
 struct GprArgs {
     int N, S;
@@ -72,13 +72,13 @@ struct GprArgs {
     int64_t row_off[kMaxSpecies];
     int64_t t_off[kMaxSpecies];
     int n_pad_max, passes_max;
-    float* e_part;        // [passes_max][N] energy partials per 512-point pass
+    float* e_part;        // [passes_max][N] energy partials per pass over the sparse points
     float* inv;           // [N] 1/|p_i| (1 without normalisation or for p_i = 0)
     float* W;             // [N sorted][n_pad_max] x zeta k^(zeta-1) (NULL: energies only)
     const float* c2;      // [N] zeta E_i / |p_i|^2
     float* grad;          // [N][F]
     unsigned* flags;
-    CUtensorMap tmM;                   // M^ rows [rows][Fk], boxes 16 B x 64 rows
+    CUtensorMap tmM, tmM32;            // M^ rows [rows][Fk], boxes of 256 rows x 16 or 128 rows x 32 columns
     CUtensorMap tmW;                   // W [N sorted][n_pad_max]
     CUtensorMap tmMT[kMaxSpecies];     // per species M^T [Fn][n_pad]
 };
@@ -117,42 +117,69 @@ __device__ inline void gpr_drain_tma(uint64_t* full, int stages, int64_t from, i
     for (int64_t i = from; i < to; ++i) mbar_wait_bounded(&full[i % stages], (uint32_t)((i / stages) & 1));
 }
 
-// ------------------------------------------------------------------------------------------ kernel GEMM
-// Warp-specialised pipeline: warps 0-3 gather A (feature rows of the tile's centres) by cp.async into the 64-byte
-// swizzled layout and, once their own copies of a stage have landed, arrive on its `full` barrier; warp 4 loads B (the
-// species' sparse points) by TMA onto the same barrier and issues the MMAs, which release the stage through `empty`.
-// The row norms are accumulated by the A threads from their own chunks and reduced per tile.
-constexpr int kGprProducers = 128;  // A-copy threads (warps 0-3)
-constexpr int kGprLag = 3;          // k-blocks a producer keeps in flight before it waits for its oldest
+// stage, phase parity and whether the stage was used before of the k-block number g of a CTA, stepped without divisions
+template <int STAGES>
+struct GprRing {
+    int stage;
+    uint32_t phase;
+    bool used;
+    __device__ __forceinline__ explicit GprRing(int64_t g)
+        : stage((int)(g % STAGES)), phase((uint32_t)((g / STAGES) & 1)), used(g >= STAGES) {}
+    __device__ __forceinline__ void next() {
+        if (++stage == STAGES) {
+            stage = 0;
+            phase ^= 1u;
+            used = true;
+        }
+    }
+};
 
-template <bool VEC16>
-__global__ void __launch_bounds__(kGprThreads, 1) k_gpr_kernel(const __grid_constant__ GprArgs A) {
+// ------------------------------------------------------------------------------------------ kernel GEMM
+// Warp-specialised pipeline over the stages (empty -> copies landed -> full -> empty): warps 0-3 gather A (feature rows of the
+// tile's centres) by cp.async into the swizzled layout, which arrives on `landed`; warps 4-7 take the row norms from the
+// landed tile and, in turns, make it visible to the tensor core and arrive on `full`; one thread of warp 9 loads B (the
+// species' sparse points) by TMA onto `full`; one of warp 8 issues the MMAs, which release the stage with the norm warps.
+// Bound: the issue of the four MMAs of a k-block and the hand-overs around it (0.49 us per 32 features of a 128 x 128 tile,
+// whatever the load on memory). 8 960 centres, 11 760 features, 256 points for each of 4 species: 502 us with 72 tiles of 256
+// points, one thread issuing MMAs and loads, 16 features a stage; 376 with 144 tiles of 128 points; 271 with 32 features a
+// stage; 181 with the loads and the norms in warps of their own (0.42 GB of features: 63 us).
+constexpr int kGprProducers = 128;  // A-copy threads (warps 0-3)
+constexpr int kGprThreads1 = 2 * kGprProducers + 64;
+
+template <bool VEC16, int COLS>
+__global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_constant__ GprArgs A) {
+    constexpr int kKB = gpr_kb(COLS), kRow = 4 * kKB;  // features and bytes of an operand row in a stage
+    constexpr int kGprStages = gpr_stages(COLS), kGprB1 = COLS * kRow, kGprATile = 128 * kRow;
+    constexpr int kParts = kKB / 16;
+    constexpr int kMmaWarp = 2 * kGprProducers / 32;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem;                                        // [stages][8 KB]
-    unsigned char* sB = sA + kGprStages * kGprATile;                 // [stages][32 KB]
-    float* s_x = reinterpret_cast<float*>(sB + kGprStages * kGprB1);  // [512]
-    float* s_inv = s_x + 512;                                        // [128]
+    unsigned char* sB = sA + kGprStages * kGprATile;                 // [stages][COLS * 64 bytes]
+    float* s_x = reinterpret_cast<float*>(sB + kGprStages * kGprB1);  // [COLS]
+    float* s_inv = s_x + COLS;                                       // [128]
     float* s_E = s_inv + 128;                                        // [2][128]; [4][128] norm partials before
     int* s_atom = reinterpret_cast<int*>(s_E + 512);                 // [128]
     int* s_off = s_atom + 128;                                       // [S + 1]
     int* s_per = s_off + kMaxSpecies + 1;                            // [S] passes per species
-    uint64_t* bars = reinterpret_cast<uint64_t*>(s_per + kMaxSpecies + 1);  // [stages] empty, [stages] full, done
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * kGprStages + 1);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(s_per + kMaxSpecies + 1);  // [stages] empty, full, landed; done
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 3 * kGprStages + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint64_t* empty = bars;
     uint64_t* full = bars + kGprStages;
-    uint64_t* done = bars + 2 * kGprStages;
+    uint64_t* landed = bars + 2 * kGprStages;
+    uint64_t* done = bars + 3 * kGprStages;
 
     for (int s = tid; s <= A.S; s += blockDim.x) s_off[s] = A.off[s];
-    for (int s = tid; s < A.S; s += blockDim.x) s_per[s] = (A.n_pad[s] + 511) / 512;
+    for (int s = tid; s < A.S; s += blockDim.x) s_per[s] = (A.n_pad[s] + COLS - 1) / COLS;
     if (warp == 0) {
-        tmem_alloc(s_tmem, 512);
+        tmem_alloc(s_tmem, COLS);
         tmem_relinquish();
     }
     if (tid == 0) {
         for (int i = 0; i < kGprStages; ++i) {
-            mbar_init(&empty[i], 1);
-            mbar_init(&full[i], kGprProducers + 1);
+            mbar_init(&empty[i], 1 + kGprProducers / 32);  // the MMAs and the norm warps
+            mbar_init(&full[i], 2);                         // a norm warp and the B load
+            mbar_init(&landed[i], kGprProducers);
         }
         mbar_init(done, 1);
         fence_mbar_init();
@@ -163,8 +190,7 @@ __global__ void __launch_bounds__(kGprThreads, 1) k_gpr_kernel(const __grid_cons
     const uint32_t taddr = *s_tmem;
     const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
     int64_t g = 0;          // k-blocks of this CTA so far (stage = g % stages, use = g / stages)
-    int64_t g_tma = 0;      // warp 4: k-blocks whose B load was issued
-    int64_t g_full = 0;     // warp 4: k-blocks whose stage it has seen full
+    int64_t g_tma = 0;      // last warp: k-blocks whose B load was issued
     uint32_t done_phase = 0;
     bool ok = true;
 
@@ -172,129 +198,145 @@ __global__ void __launch_bounds__(kGprThreads, 1) k_gpr_kernel(const __grid_cons
         int s, row0, pass;
         if (!gpr_tile(s_off, A.S, s_per, t, s, row0, pass)) break;
         const int n_rows = min(128, s_off[s + 1] - row0);
-        const int col0 = pass * 512;
-        const int ncols = min(512, A.n_pad[s] - col0);
-        const int nk = (int)(A.Fk / kGprKB);
+        const int col0 = pass * COLS;
+        const int ncols = min(COLS, A.n_pad[s] - col0);
+        const int nk = (int)((A.Fk + kKB - 1) / kKB);
         if (tid < 128) s_atom[tid] = tid < n_rows ? A.perm[row0 + tid] : -1;
-        for (int c = tid; c < 512; c += blockDim.x) s_x[c] = c < ncols ? A.x[A.row_off[s] + col0 + c] : 0.0f;
+        for (int c = tid; c < COLS; c += blockDim.x) s_x[c] = c < ncols ? A.x[A.row_off[s] + col0 + c] : 0.0f;
         __syncthreads();
 
-        if (warp < 4) {
-            // ---- A producers: rows r0 + 32 j (j < 4), 16-byte chunk c
-            const int r0 = tid >> 2, c = tid & 3;
-            const uint32_t d0 = sw64_off(r0, c);  // row r0 + 32 j lands 2048 j bytes further
-            const float* pa[4];
-            int64_t lim[4];
+        if (warp < kMmaWarp) {
+            // ---- A rows r0 + kStep j (j < kRows), 16-byte chunks c and c + 4, by one producer and one norm thread
+            constexpr int kStep = kGprProducers / 4, kRows = 128 / kStep;
+            const int r0 = (tid % kGprProducers) >> 2, c = tid & 3;
+            // row r0 + kStep j lands kStep kRow j bytes further, its chunk c + 4 64 bytes across
+            const uint32_t d0 = kKB == 16 ? sw64_off(r0, c) : sw128_off(r0, c);
+            auto at = [&](int t) { return (d0 ^ (uint32_t)(t % kParts * 64)) + kStep * kRow * (t / kParts); };
+            GprRing<kGprStages> ring(g);
+            if (warp < kGprProducers / 32) {
+                const float* pa[kRows];
+                int64_t lim[kRows];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int atom = s_atom[r0 + 32 * j];
-                pa[j] = atom >= 0 ? A.p + (int64_t)atom * A.F : A.p;
-                lim[j] = atom >= 0 ? A.F : 0;
-            }
-            float nrm[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            auto land = [&](int kb) {  // this thread's chunks of k-block kb are in shared memory: norms, arrive
-                const unsigned char* a = sA + (int)((g + kb) % kGprStages) * kGprATile + d0;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float4 v = *reinterpret_cast<const float4*>(a + 2048 * j);
-                    nrm[j] = fmaf(v.x, v.x, nrm[j]);
-                    nrm[j] = fmaf(v.y, v.y, nrm[j]);
-                    nrm[j] = fmaf(v.z, v.z, nrm[j]);
-                    nrm[j] = fmaf(v.w, v.w, nrm[j]);
+                for (int j = 0; j < kRows; ++j) {
+                    const int atom = s_atom[r0 + kStep * j];
+                    pa[j] = atom >= 0 ? A.p + (int64_t)atom * A.F : A.p;
+                    lim[j] = atom >= 0 ? A.F : 0;
                 }
-                mbar_arrive(&full[(g + kb) % kGprStages]);
-            };
-            int landed = 0;
-            for (int kb = 0; kb < nk && ok; ++kb) {
-                const int64_t gi = g + kb;
-                const int stage = (int)(gi % kGprStages);
-                if (gi >= kGprStages &&
-                    !mbar_wait_bounded(&empty[stage], (uint32_t)(((gi - kGprStages) / kGprStages) & 1))) {
-                    ok = false;
-                    break;
-                }
-                const int64_t k0 = (int64_t)kb * kGprKB;
-                unsigned char* a = sA + stage * kGprATile + d0;
-                if (VEC16) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool in = k0 + 4 * c < lim[j];
-                        cp_async16_zfill(a + 2048 * j, in ? pa[j] + k0 + 4 * c : A.p, in ? 16u : 0u);
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const bool in = k0 + 4 * c + e < lim[j];
-                            cp_async4_zfill(a + 2048 * j + 4 * e, in ? pa[j] + k0 + 4 * c + e : A.p, in ? 4u : 0u);
-                        }
-                }
-                cp_async_commit();
-                if (kb >= kGprLag) {
-                    cp_async_wait_group<kGprLag>();
-                    fence_proxy_async_smem();
-                    land(landed++);
-                }
-            }
-            cp_async_wait_group<0>();
-            fence_proxy_async_smem();
-            while (ok && landed < nk) land(landed++);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s_E[c * 128 + r0 + 32 * j] = nrm[j];  // partials [chunk][row]
-        } else if (warp == 4) {
-          if (lane == 0) {
-            // ---- B loads and MMAs
-            const int n0 = min(256, ncols), n1 = ncols - n0;
-            const int nq = (ncols + 63) / 64;
-            const int brow = (int)(A.row_off[s] + col0);
-            const uint32_t id0 = instr_desc(2u, 128u, (uint32_t)n0);
-            const uint32_t id1 = instr_desc(2u, 128u, (uint32_t)max(n1, 16));
-            auto load_b = [&](int kb) {
-                const int stage = (int)((g + kb) % kGprStages);
-                unsigned char* b = sB + stage * kGprB1;
-                mbar_expect_tx(&full[stage], (uint32_t)(nq * 4096));
-                for (int qq = 0; qq < nq; ++qq)
-                    tma_load_2d(b + qq * 4096, &A.tmM, kb * kGprKB, brow + 64 * qq, &full[stage]);
-                ++g_tma;
-            };
-            for (int i = 0; i < kGprStages - 1 && i < nk; ++i) load_b(i);
-            for (int kb = 0; kb < nk; ++kb) {
-                const int64_t gi = g + kb;
-                const int stage = (int)(gi % kGprStages);
-                if (!mbar_wait_bounded(&full[stage], (uint32_t)((gi / kGprStages) & 1))) {
-                    ok = false;
-                    break;
-                }
-                ++g_full;
-                tc_fence_after();
-                const uint32_t a0 = a_base + stage * kGprATile, b0 = b_base + stage * kGprB1;
-#pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    const uint64_t da = smem_desc_sw64(a0 + kk * 32, 512);
-                    mma_tf32_ss(taddr, da, smem_desc_sw64(b0 + kk * 32, 512), id0, (kb | kk) != 0);
-                    if (n1 > 0) mma_tf32_ss(taddr + 256, da, smem_desc_sw64(b0 + 16384 + kk * 32, 512), id1, (kb | kk) != 0);
-                }
-                mma_commit(&empty[stage]);
-                const int nxt = kb + kGprStages - 1;
-                if (nxt < nk) {
-                    if (gi >= 1 && !mbar_wait_bounded(&empty[(gi - 1) % kGprStages], (uint32_t)(((gi - 1) / kGprStages) & 1))) {
+                for (int kb = 0; kb < nk; ++kb, ring.next()) {
+                    bool free = true;
+                    if (ring.used && lane == 0) free = mbar_wait_spin(&empty[ring.stage], ring.phase ^ 1u);
+                    if (!__shfl_sync(0xffffffffu, free, 0)) {
                         ok = false;
                         break;
                     }
-                    load_b(nxt);
+                    const int64_t k0 = (int64_t)kb * kKB + 4 * c;
+                    unsigned char* a = sA + ring.stage * kGprATile;
+#pragma unroll
+                    for (int t = 0; t < kRows * kParts; ++t) {
+                        const int j = t / kParts;
+                        const int64_t f = k0 + t % kParts * 16;
+                        unsigned char* o = a + at(t);
+                        if (VEC16) {
+                            const bool in = f < lim[j];
+                            cp_async16_zfill(o, in ? pa[j] + f : A.p, in ? 16u : 0u);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const bool in = f + e < lim[j];
+                                cp_async4_zfill(o + 4 * e, in ? pa[j] + f + e : A.p, in ? 4u : 0u);
+                            }
+                        }
+                    }
+                    cp_async_arrive(&landed[ring.stage]);
+                }
+                cp_async_wait_all();
+            } else {
+                float nrm[kRows] = {};
+                for (int kb = 0; kb < nk; ++kb, ring.next()) {
+                    bool here = true;
+                    if (lane == 0) here = mbar_wait_spin(&landed[ring.stage], ring.phase);
+                    if (!__shfl_sync(0xffffffffu, here, 0)) {
+                        ok = false;
+                        break;
+                    }
+                    // the norm warps take turns to make the tile visible to the tensor core
+                    if (((g + kb) & 3) == (warp & 3)) {
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&full[ring.stage]);
+                    }
+                    const unsigned char* a = sA + ring.stage * kGprATile;
+#pragma unroll
+                    for (int t = 0; t < kRows * kParts; ++t) {
+                        const int j = t / kParts;
+                        const float4 v = *reinterpret_cast<const float4*>(a + at(t));
+                        nrm[j] = fmaf(v.x, v.x, nrm[j]);
+                        nrm[j] = fmaf(v.y, v.y, nrm[j]);
+                        nrm[j] = fmaf(v.z, v.z, nrm[j]);
+                        nrm[j] = fmaf(v.w, v.w, nrm[j]);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&empty[ring.stage]);
+                }
+#pragma unroll
+                for (int j = 0; j < kRows; ++j) s_E[c * 128 + r0 + kStep * j] = nrm[j];  // partials [chunk][row]
+            }
+        } else if (warp == kMmaWarp) {
+            if (lane == 0) {  // ---- MMAs
+                const int n0 = min(256, ncols), n1 = ncols - n0;
+                const uint32_t id0 = instr_desc(2u, 128u, (uint32_t)n0);
+                const uint32_t id1 = instr_desc(2u, 128u, (uint32_t)max(n1, 16));
+                auto desc = [&](uint32_t at) { return kKB == 16 ? smem_desc_sw64(at, 512) : smem_desc_sw128(at, 1024); };
+                const uint64_t da0 = desc(a_base), db0 = desc(b_base);  // the address is the descriptor's low field, in 16 bytes
+                GprRing<kGprStages> use(g);
+                for (int kb = 0; kb < nk; ++kb, use.next()) {
+                    if (!mbar_wait_spin(&full[use.stage], use.phase)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t da = da0 + (uint32_t)(use.stage * (kGprATile >> 4)), db = db0 + (uint32_t)(use.stage * (kGprB1 >> 4));
+                    const int nkk = (int)min((int64_t)kKB, A.Fk - (int64_t)kb * kKB) / 8;
+#pragma unroll
+                    for (int kk = 0; kk < kKB / 8; ++kk) {
+                        if (kk >= nkk) break;
+                        mma_tf32_ss(taddr, da + 2 * kk, db + 2 * kk, id0, (kb | kk) != 0);
+                        if (COLS > 256 && n1 > 0)
+                            mma_tf32_ss(taddr + 256, da + 2 * kk, db + (256 * kRow >> 4) + 2 * kk, id1, (kb | kk) != 0);
+                    }
+                    mma_commit(&empty[use.stage]);
+                }
+                mma_commit(done);
+            }
+            __syncwarp();  // the other lanes wait here, not in a spin beside lane 0
+        } else {
+            if (lane == 0) {  // ---- B loads: a TMA issue takes as long as an MMA's, so another warp than the MMAs'
+                constexpr int kBoxRows = kKB == 16 ? 256 : 128;
+                const int nq = (ncols + kBoxRows - 1) / kBoxRows;
+                const int brow = (int)(A.row_off[s] + col0);
+                GprRing<kGprStages> ring(g);
+                for (int kb = 0; kb < nk; ++kb, ring.next()) {
+                    if (ring.used && !mbar_wait_spin(&empty[ring.stage], ring.phase ^ 1u)) {
+                        ok = false;
+                        break;
+                    }
+                    unsigned char* b = sB + ring.stage * kGprB1;
+                    mbar_expect_tx(&full[ring.stage], (uint32_t)(nq * kBoxRows * kRow));
+                    for (int qq = 0; qq < nq; ++qq)
+                        tma_load_2d(b + qq * kBoxRows * kRow, kKB == 16 ? &A.tmM : &A.tmM32, kb * kKB, brow + kBoxRows * qq,
+                                    &full[ring.stage]);
+                    ++g_tma;
                 }
             }
-            mma_commit(done);
-          }
-          __syncwarp();  // the other lanes of the MMA warp wait here, not in a spin beside lane 0
+            __syncwarp();
         }
         g += nk;
         const bool fin = mbar_wait_bounded(done, done_phase);
         done_phase ^= 1u;
         ok = __syncthreads_and(ok && fin) != 0;
         if (!ok) {
-            if (warp == 4 && lane == 0) gpr_drain_tma(full, kGprStages, g_full, g_tma);
+            if (warp == kMmaWarp + 1 && lane == 0)
+                gpr_drain_tma(full, kGprStages, g_tma > kGprStages ? g_tma - kGprStages : 0, g_tma);
             gpr_fail(A, done, done_phase ^ 1u);
             break;
         }
@@ -308,12 +350,12 @@ __global__ void __launch_bounds__(kGprThreads, 1) k_gpr_kernel(const __grid_cons
         tc_fence_after();
         // epilogue: warp -> lane quadrant (rows) and column half
         const int q = warp & 3, h = warp >> 2, row = 32 * q + lane;
+        const bool valid = row < n_rows;
         const float iv = s_inv[row];
         float e = 0.0f;
-        const int c_end = min(ncols, 256 * h + 256);
+        const int c_end = min(ncols, COLS / 2 * (h + 1));
         float* wrow = A.W ? A.W + (int64_t)(row0 + row) * A.n_pad_max + col0 : nullptr;
-        const bool valid = row < n_rows;
-        for (int cc = 256 * h; cc < c_end; cc += 16) {
+        for (int cc = COLS / 2 * h; h < 2 && cc < c_end; cc += 16) {
             float v[16];
             tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)cc, v);
             float w[16];
@@ -332,7 +374,7 @@ __global__ void __launch_bounds__(kGprThreads, 1) k_gpr_kernel(const __grid_cons
             }
         }
         __syncthreads();  // the norm partials in s_E are read; the energies may reuse it
-        s_E[h * 128 + row] = e;
+        if (h < 2) s_E[h * 128 + row] = e;
         tc_fence_before();
         __syncthreads();
         if (tid < 128 && s_atom[tid] >= 0) A.e_part[(int64_t)pass * A.N + s_atom[tid]] = s_E[tid] + s_E[128 + tid];
@@ -341,19 +383,26 @@ __global__ void __launch_bounds__(kGprThreads, 1) k_gpr_kernel(const __grid_cons
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(taddr, 512);
+        tmem_dealloc(taddr, COLS);
     }
 }
 
 // ---------------------------------------------------------------------------------------- gradient GEMM
-// Both operands by TMA: A = W rows [chunk][128 rows][16 B], B = the species' M^T rows [chunk][256 rows][16 B]; one
-// thread runs the whole main loop (loads, MMAs, stage recycling); all warps share the epilogue.
-__global__ void __launch_bounds__(kGprThreads, 2) k_gpr_grad(const __grid_constant__ GprArgs A) {
+// Both operands by TMA: A = W rows, B = the species' M^T rows; one thread of warp 9 loads, one of warp 8 issues the MMAs;
+// warps 0-7 share the epilogue and request its first features beside the main loop.
+// Bound: reading p and writing dE/dp (0.84 GB, 126 us on the model above) behind a main loop of 8 k-blocks per tile, overlapped
+// only between the two CTAs of an SM: 256 us. It took 353 with a lane to a row (16-byte pieces of 32 rows per instruction) and
+// six 64-row loads per k-block issued by the MMAs' thread; 333 with eight lanes to a row, 272 with 128-byte rows and the
+// features requested early. Tiles of 128 features, three CTAs per SM: 391 us (the W tile is read twice as often).
+__global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_constant__ GprArgs A) {
+    constexpr int kKB = 32, kGprATile = 128 * 128;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem;                                          // [stages][8 KB]
-    unsigned char* sB = sA + kGprStages2 * kGprATile;                  // [stages][16 KB]
+    unsigned char* sB = sA + kGprStages2 * kGprATile;                  // [stages][8 KB]
     int* s_atom = reinterpret_cast<int*>(sB + kGprStages2 * kGprB2);  // [128]
-    int* s_off = s_atom + 128;
+    float* s_inv = reinterpret_cast<float*>(s_atom + 128);             // [128] 1 / |p|
+    float* s_c2 = s_inv + 128;                                         // [128] zeta E / |p|^2
+    int* s_off = reinterpret_cast<int*>(s_c2 + 128);
     int* s_per = s_off + kMaxSpecies + 1;                              // feature chunks per species
     uint64_t* bars = reinterpret_cast<uint64_t*>(s_per + kMaxSpecies + 1);
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * kGprStages2 + 1);
@@ -361,12 +410,12 @@ __global__ void __launch_bounds__(kGprThreads, 2) k_gpr_grad(const __grid_consta
     uint64_t* empty = bars;
     uint64_t* full = bars + kGprStages2;
     uint64_t* done = bars + 2 * kGprStages2;
-    const int n_fc = (int)((A.Fn + 255) / 256);
+    const int n_fc = (int)((A.Fn + kGprFT - 1) / kGprFT);
 
     for (int s = tid; s <= A.S; s += blockDim.x) s_off[s] = A.off[s];
     for (int s = tid; s < A.S; s += blockDim.x) s_per[s] = n_fc;
     if (warp == 0) {
-        tmem_alloc(s_tmem, 256);
+        tmem_alloc(s_tmem, kGprFT);
         tmem_relinquish();
     }
     if (tid == 0) {
@@ -378,7 +427,7 @@ __global__ void __launch_bounds__(kGprThreads, 2) k_gpr_grad(const __grid_consta
     tc_fence_after();
     const uint32_t taddr = *s_tmem;
     const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
-    int64_t g = 0;
+    int64_t g = 0, g_tma = 0;  // k-blocks of this CTA so far; last warp: loads issued
     uint32_t done_phase = 0;
     bool ok = true;
 
@@ -386,62 +435,76 @@ __global__ void __launch_bounds__(kGprThreads, 2) k_gpr_grad(const __grid_consta
         int s, row0, fc;
         if (!gpr_tile(s_off, A.S, s_per, t, s, row0, fc)) break;
         const int n_rows = min(128, s_off[s + 1] - row0);
-        const int f0 = fc * 256;
-        const int ncols = (int)(A.Fn - f0 < 256 ? A.Fn - f0 : 256);
-        const int nk = A.n_pad[s] / kGprKB;
-        const int nq = (ncols + 63) / 64;
-        if (tid < 128) s_atom[tid] = tid < n_rows ? A.perm[row0 + tid] : -1;
-        if (nk > 0) {
-            if (tid == 0) {
-                const CUtensorMap* tb = &A.tmMT[s];
-                auto load = [&](int kb, int stage) {
-                    const int k0 = kb * kGprKB;
-                    unsigned char* a = sA + stage * kGprATile;
-                    unsigned char* b = sB + stage * kGprB2;
-                    mbar_expect_tx(&full[stage], (uint32_t)(2 * 4096 + nq * 4096));
-                    for (int qq = 0; qq < 2; ++qq) tma_load_2d(a + qq * 4096, &A.tmW, k0, row0 + 64 * qq, &full[stage]);
-                    for (int qq = 0; qq < nq; ++qq) tma_load_2d(b + qq * 4096, tb, k0, f0 + 64 * qq, &full[stage]);
-                };
-                const uint32_t id = instr_desc(2u, 128u, (uint32_t)ncols);
-                int issued = 0;
-                for (int i = 0; i < kGprStages2 - 1 && i < nk; ++i, ++issued) load(i, (int)((g + i) % kGprStages2));
-                int kb = 0;
-                for (; kb < nk; ++kb) {
-                    const int64_t gi = g + kb;
-                    const int stage = (int)(gi % kGprStages2);
-                    if (!mbar_wait_bounded(&full[stage], (uint32_t)((gi / kGprStages2) & 1))) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t a0 = a_base + stage * kGprATile, b0 = b_base + stage * kGprB2;
+        const int f0 = fc * kGprFT;
+        const int ncols = (int)(A.Fn - f0 < kGprFT ? A.Fn - f0 : kGprFT);
+        const int nk = (A.n_pad[s] + kKB - 1) / kKB;
+        if (tid < 128) {
+            const int atom = tid < n_rows ? A.perm[row0 + tid] : -1;
+            s_atom[tid] = atom;
+            s_inv[tid] = atom >= 0 && nk > 0 ? A.inv[atom] : 0.0f;
+            s_c2[tid] = atom >= 0 && nk > 0 ? A.c2[atom] : 0.0f;
+        }
+        const int q = warp & 3, h = warp >> 2, row = 32 * q + lane, rr = lane >> 3, cl = 4 * (lane & 7);
+        const int c_end = min(ncols, kGprFT / 2 * (h + 1));
+        // the features of 32 columns of this warp's rows, eight lanes to a row
+        auto fetch = [&](int c, float4 (&pv)[8]) {
+            const int64_t f = f0 + c + cl;
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk)
-                        mma_tf32_ss(taddr, smem_desc_sw64(a0 + kk * 32, 512), smem_desc_sw64(b0 + kk * 32, 512), id,
-                                    (kb | kk) != 0);
-                    mma_commit(&empty[stage]);
-                    const int nxt = kb + kGprStages2 - 1;
-                    if (nxt < nk) {
-                        const int64_t prev = gi - 1;
-                        if (prev >= 0 &&
-                            !mbar_wait_bounded(&empty[prev % kGprStages2], (uint32_t)((prev / kGprStages2) & 1))) {
+            for (int u = 0; u < 8; ++u) {
+                const int atom = s_atom[32 * q + 4 * u + rr];
+                if (c + cl < c_end && f < A.F && atom >= 0) pv[u] = __ldcs(reinterpret_cast<const float4*>(A.p + (int64_t)atom * A.F + f));
+            }
+        };
+        float4 pn[8];
+        if (warp < kGprThreads / 32) {  // requested beside the main loop
+            asm volatile("bar.sync 1, %0;" ::"n"(kGprThreads) : "memory");  // s_atom
+            if (A.vec16) fetch(kGprFT / 2 * h, pn);
+        }
+        if (nk > 0) {
+            if (warp == kGprThreads / 32) {
+                if (lane == 0) {  // ---- MMAs
+                    const uint64_t da0 = smem_desc_sw128(a_base, 1024), db0 = smem_desc_sw128(b_base, 1024);
+                    const uint32_t id = instr_desc(2u, 128u, (uint32_t)ncols);
+                    GprRing<kGprStages2> use(g);
+                    for (int kb = 0; kb < nk; ++kb, use.next()) {
+                        if (!mbar_wait_spin(&full[use.stage], use.phase)) {
                             ok = false;
-                            ++kb;
                             break;
                         }
-                        load(nxt, (int)((g + nxt) % kGprStages2));
-                        ++issued;
+                        tc_fence_after();
+                        const uint64_t da = da0 + (uint32_t)(use.stage * (kGprATile >> 4)), db = db0 + (uint32_t)(use.stage * (kGprB2 >> 4));
+                        const int nkk = min(kKB, A.n_pad[s] - kb * kKB) / 8;  // columns of W past n_pad are not written
+#pragma unroll
+                        for (int kk = 0; kk < kKB / 8; ++kk)
+                            if (kk < nkk) mma_tf32_ss(taddr, da + 2 * kk, db + 2 * kk, id, (kb | kk) != 0);
+                        mma_commit(&empty[use.stage]);
+                    }
+                    mma_commit(done);
+                }
+                __syncwarp();
+            } else if (warp > kGprThreads / 32) {
+                if (lane == 0) {  // ---- loads
+                    GprRing<kGprStages2> ring(g);
+                    for (int kb = 0; kb < nk; ++kb, ring.next()) {
+                        if (ring.used && !mbar_wait_spin(&empty[ring.stage], ring.phase ^ 1u)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_expect_tx(&full[ring.stage], (uint32_t)(kGprATile + kGprB2));
+                        tma_load_2d(sA + ring.stage * kGprATile, &A.tmW, kb * kKB, row0, &full[ring.stage]);
+                        tma_load_2d(sB + ring.stage * kGprB2, &A.tmMT[s], kb * kKB, f0, &full[ring.stage]);
+                        ++g_tma;
                     }
                 }
-                mma_commit(done);
-                if (!ok) gpr_drain_tma(full, kGprStages2, g + kb, g + issued);
+                __syncwarp();
             }
-            if (warp == 0) __syncwarp();
             g += nk;
             const bool fin = mbar_wait_bounded(done, done_phase);
             done_phase ^= 1u;
             ok = __syncthreads_and(ok && fin) != 0;
             if (!ok) {
+                if (warp > kGprThreads / 32 && lane == 0)
+                    gpr_drain_tma(full, kGprStages2, g_tma > kGprStages2 ? g_tma - kGprStages2 : 0, g_tma);
                 gpr_fail(A, done, done_phase ^ 1u);
                 break;
             }
@@ -450,47 +513,61 @@ __global__ void __launch_bounds__(kGprThreads, 2) k_gpr_grad(const __grid_consta
             __syncthreads();
         }
         // epilogue: dE/dp = inv * G - c2 * p for this warp's rows and half of the columns
-        const int q = warp & 3, h = warp >> 2, row = 32 * q + lane;
-        const int atom = s_atom[row];
-        const float iv = atom >= 0 && nk > 0 ? A.inv[atom] : 0.0f;
-        const float cc = atom >= 0 && nk > 0 ? A.c2[atom] : 0.0f;
-        const int c_end = min(ncols, 128 * h + 128);
-        // the feature values of the next 16 columns are requested before this group's are used (latency overlap)
-        const float* pbase = atom >= 0 ? A.p + (int64_t)atom * A.F : A.p;
-        auto fetch = [&](int c, float4 (&pv)[4]) {
-            const int64_t f = f0 + c;
-            if (atom >= 0 && A.vec16 && f + 16 <= A.F) {
+        if (warp >= kGprThreads / 32) {
+        } else if (A.vec16) {
+            // 32 columns at a time through shared memory (the stages are free: every load has landed and every MMA is done),
+            // so that eight lanes read and write 128 contiguous bytes of a row
+            float* buf = reinterpret_cast<float*>(sA) + warp * 32 * 36;  // pitch 36: both directions conflict-free
+            for (int c = kGprFT / 2 * h; c < c_end; c += 32) {
+                const int64_t f = f0 + c + cl;
+                const bool in = c + cl < c_end && f < A.F;
+                float4 pv[8];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) pv[u] = __ldg(reinterpret_cast<const float4*>(pbase + f) + u);
-            }
-        };
-        float4 pn[4];
-        if (128 * h < c_end) fetch(128 * h, pn);
-        for (int c = 128 * h; c < c_end; c += 16) {
-            float4 pc[4] = {pn[0], pn[1], pn[2], pn[3]};
-            if (c + 16 < c_end) fetch(c + 16, pn);
-            float v[16];
-            if (nk > 0) {
-                tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
-            } else {
+                for (int u = 0; u < 8; ++u) pv[u] = pn[u];
+                if (c + 32 < c_end) fetch(c + 32, pn);
 #pragma unroll
-                for (int u = 0; u < 16; ++u) v[u] = 0.0f;
-            }
-            if (atom < 0) continue;
-            const int64_t f = f0 + c;
-            const float* prow = A.p + (int64_t)atom * A.F + f;
-            float* grow = A.grad + (int64_t)atom * A.F + f;
-            if (A.vec16 && f + 16 <= A.F) {
+                for (int w = 0; w < 32; w += 16) {
+                    if (c + w >= c_end) break;
+                    float v[16];
+                    if (nk > 0) {
+                        tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)(c + w), v);
+                    } else {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float4 o;
-                    o.x = fmaf(iv, v[4 * u], -cc * pc[u].x);
-                    o.y = fmaf(iv, v[4 * u + 1], -cc * pc[u].y);
-                    o.z = fmaf(iv, v[4 * u + 2], -cc * pc[u].z);
-                    o.w = fmaf(iv, v[4 * u + 3], -cc * pc[u].w);
-                    __stcs(reinterpret_cast<float4*>(grow) + u, o);
+                        for (int u = 0; u < 16; ++u) v[u] = 0.0f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 16; u += 4)
+                        *reinterpret_cast<float4*>(buf + lane * 36 + w + u) = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
                 }
-            } else {
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int r = 32 * q + 4 * u + rr, atom = s_atom[r];
+                    if (!in || atom < 0) continue;
+                    const float iv = s_inv[r], cc = s_c2[r];
+                    const float4 v = *reinterpret_cast<const float4*>(buf + (4 * u + rr) * 36 + cl);
+                    __stcs(reinterpret_cast<float4*>(A.grad + (int64_t)atom * A.F + f),
+                           make_float4(fmaf(iv, v.x, -cc * pv[u].x), fmaf(iv, v.y, -cc * pv[u].y),
+                                       fmaf(iv, v.z, -cc * pv[u].z), fmaf(iv, v.w, -cc * pv[u].w)));
+                }
+                __syncwarp();
+            }
+            fence_proxy_async_smem();  // the next tile's loads come by TMA
+        } else {
+            const int atom = s_atom[row];
+            const float iv = s_inv[row], cc = s_c2[row];
+            for (int c = kGprFT / 2 * h; c < c_end; c += 16) {
+                float v[16];
+                if (nk > 0) {
+                    tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) v[u] = 0.0f;
+                }
+                if (atom < 0) continue;
+                const int64_t f = f0 + c;
+                const float* prow = A.p + (int64_t)atom * A.F + f;
+                float* grow = A.grad + (int64_t)atom * A.F + f;
 #pragma unroll
                 for (int u = 0; u < 16; ++u)
                     if (f + u < A.F) grow[u] = fmaf(iv, v[u], -cc * prow[u]);
@@ -503,7 +580,7 @@ __global__ void __launch_bounds__(kGprThreads, 2) k_gpr_grad(const __grid_consta
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(taddr, 256);
+        tmem_dealloc(taddr, kGprFT);
     }
 }
 
@@ -599,12 +676,19 @@ __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict
     (void)passes_max;
 }
 
-static size_t gpr_smem1() {
-    return (size_t)kGprStages * (kGprATile + kGprB1) + sizeof(float) * (512 + 128 + 512) + sizeof(int) * 128 +
-           sizeof(int) * 2 * (kMaxSpecies + 1) + sizeof(uint64_t) * (2 * kGprStages + 1) + 16;
+static size_t gpr_smem1(int cols) {
+    const int stages = gpr_stages(cols);
+    return (size_t)stages * (128 + cols) * 4 * gpr_kb(cols) + sizeof(float) * (cols + 128 + 512) + sizeof(int) * 128 +
+           sizeof(int) * 2 * (kMaxSpecies + 1) + sizeof(uint64_t) * (3 * stages + 1) + 16;
+}
+using GprKernel = void (*)(GprArgs);
+static GprKernel gpr_kernel(bool vec16, int cols) {
+    if (cols == 128) return vec16 ? k_gpr_kernel<true, 128> : k_gpr_kernel<false, 128>;
+    if (cols == 256) return vec16 ? k_gpr_kernel<true, 256> : k_gpr_kernel<false, 256>;
+    return vec16 ? k_gpr_kernel<true, 512> : k_gpr_kernel<false, 512>;
 }
 static size_t gpr_smem2() {
-    return (size_t)kGprStages2 * (kGprATile + kGprB2) + sizeof(int) * 128 + sizeof(int) * 2 * (kMaxSpecies + 1) +
+    return (size_t)kGprStages2 * (128 * 128 + kGprB2) + sizeof(int) * 3 * 128 + sizeof(int) * 2 * (kMaxSpecies + 1) +
            sizeof(uint64_t) * (2 * kGprStages2 + 1) + 16;
 }
 
@@ -622,15 +706,15 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 // TMA map of a row-major FP32 matrix [rows][pitch] (cols used), boxes of 16 elements (64 bytes) x 64 rows written
 // with 64-byte swizzling (the operand layout of smem_desc_sw64); reads past the last row fill zeros
-static int tmap_2d(CUtensorMap* m, const float* base, uint64_t cols, uint64_t rows, uint64_t pitch) {
+static int tmap_2d(CUtensorMap* m, const float* base, uint64_t cols, uint64_t rows, uint64_t pitch, uint32_t box_cols, uint32_t box_rows) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
     if (!fn) return set_error(RASCAL_E_CUDA, "cuTensorMapEncodeTiled is not available from the CUDA driver library");
     cuuint64_t dims[2] = {cols, rows};
     cuuint64_t strides[1] = {pitch * sizeof(float)};
-    cuuint32_t box[2] = {16, 64};
+    cuuint32_t box[2] = {box_cols, box_rows};
     cuuint32_t es[2] = {1, 1};
     const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, es,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_error(RASCAL_E_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
     return RASCAL_OK;
@@ -688,7 +772,6 @@ extern "C" int rascal_gpr_create(rascal_ctx* ctx, int64_t n_sparse, int64_t n_fe
         r += m->n_pad[s];
         t += m->Fn * m->n_pad[s];
         m->n_pad_max = std::max(m->n_pad_max, m->n_pad[s]);
-        m->passes_max = std::max(m->passes_max, (m->n_pad[s] + 511) / 512);
     }
     m->rows = r;
     std::vector<float> hM((size_t)std::max<int64_t>(r, 1) * m->Fk, 0.0f), hMT((size_t)std::max<int64_t>(t, 1), 0.0f),
@@ -716,10 +799,10 @@ extern "C" int rascal_gpr_create(rascal_ctx* ctx, int64_t n_sparse, int64_t n_fe
     if (e == cudaSuccess) e = cudaMemcpy(m->d_M, hM.data(), sizeof(float) * hM.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->d_MT, hMT.data(), sizeof(float) * hMT.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->d_x, hx.data(), sizeof(float) * hx.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_gpr_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gpr_smem1());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_gpr_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gpr_smem1());
+    for (int cols = 128; cols <= 512; cols *= 2)
+        for (int v = 0; v < 2; ++v)
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(gpr_kernel(v, cols), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gpr_smem1(cols));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gpr_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gpr_smem2());
     if (e != cudaSuccess) {
         cudaFree(m->d_M);
@@ -729,10 +812,11 @@ extern "C" int rascal_gpr_create(rascal_ctx* ctx, int64_t n_sparse, int64_t n_fe
         return set_error(RASCAL_E_CUDA, "GPR model upload: %s", cudaGetErrorString(e));
     }
     int st = RASCAL_OK;
-    if (m->rows > 0) st = tmap_2d(&m->tmM, m->d_M, (uint64_t)m->Fk, (uint64_t)m->rows, (uint64_t)m->Fk);
+    if (m->rows > 0) st = tmap_2d(&m->tmM, m->d_M, (uint64_t)m->Fk, (uint64_t)m->rows, (uint64_t)m->Fk, 16, 256);
+    if (m->rows > 0 && !st) st = tmap_2d(&m->tmM32, m->d_M, (uint64_t)m->Fk, (uint64_t)m->rows, (uint64_t)m->Fk, 32, 128);
     for (int s = 0; s < S && !st; ++s)
         if (m->n_pad[s] > 0)
-            st = tmap_2d(&m->tmMT[s], m->d_MT + m->t_off[s], (uint64_t)m->n_pad[s], (uint64_t)m->Fn, (uint64_t)m->n_pad[s]);
+            st = tmap_2d(&m->tmMT[s], m->d_MT + m->t_off[s], (uint64_t)m->n_pad[s], (uint64_t)m->Fn, (uint64_t)m->n_pad[s], 32, kGprFT);
     if (st) {
         rascal_gpr_destroy(m);
         return st;
@@ -763,7 +847,12 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
     const int S = m->S;
     const int nb = (int)div_up(N, kSortBlock);
     const bool grad = d_grad != nullptr;
-    const int P = std::max(1, m->passes_max);
+    // Sparse points of a tile: as many as a species has, but fewer where that leaves SMs without a tile (8 960 centres of 4
+    // species are 72 tiles of 256 points or 144 of 128). The features are not split: a product's running sum stays one chain.
+    int cols = m->n_pad_max <= 128 ? 128 : (m->n_pad_max <= 256 ? 256 : 512);
+    auto tiles = [&](int w) { return ((int64_t)div_up(N, 128) + S - 1) * ((m->n_pad_max + w - 1) / w); };
+    while (cols > 128 && tiles(cols / 2) <= ctx->n_sm) cols /= 2;
+    const int P = std::max(1, (m->n_pad_max + cols - 1) / cols);  // passes
     void* base;
     st = arena_get(ctx->scratch, carve_bytes(sizeof(int) * N, sizeof(int) * nb * S, sizeof(int) * (S + 1),
                                              sizeof(int) * S, sizeof(float) * N, sizeof(float) * (size_t)P * N,
@@ -784,7 +873,7 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
     float* W = grad ? cv.take<float>((size_t)N * std::max(16, m->n_pad_max)) : nullptr;
 
     int hp[kMaxSpecies];
-    for (int s = 0; s < S; ++s) hp[s] = (m->n_pad[s] + 511) / 512;
+    for (int s = 0; s < S; ++s) hp[s] = (m->n_pad[s] + cols - 1) / cols;
     RASCAL_CUDA(cudaMemcpyAsync(npass, hp, sizeof(int) * S, cudaMemcpyHostToDevice, ctx->stream));
     k_gpr_count<<<nb, kSortBlock, 0, ctx->stream>>>(N, S, sys->d_species, ctx->d_lut, cnt);
     RASCAL_LAUNCH_CHECK("k_gpr_count");
@@ -822,13 +911,11 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
     A.grad = d_grad;
     A.flags = ctx->d_flags;
     A.tmM = m->tmM;
+    A.tmM32 = m->tmM32;
     for (int s = 0; s < S; ++s) A.tmMT[s] = m->tmMT[s];
-    if (grad && (st = tmap_2d(&A.tmW, W, (uint64_t)A.n_pad_max, (uint64_t)N, (uint64_t)A.n_pad_max))) return st;
+    if (grad && (st = tmap_2d(&A.tmW, W, (uint64_t)A.n_pad_max, (uint64_t)N, (uint64_t)A.n_pad_max, 32, 128))) return st;
     if (m->rows > 0) {
-        if (A.vec16)
-            k_gpr_kernel<true><<<ctx->n_sm, kGprThreads, gpr_smem1(), ctx->stream>>>(A);
-        else
-            k_gpr_kernel<false><<<ctx->n_sm, kGprThreads, gpr_smem1(), ctx->stream>>>(A);
+        gpr_kernel(A.vec16, cols)<<<ctx->n_sm, kGprThreads1, gpr_smem1(cols), ctx->stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_gpr_kernel");
     }
     k_gpr_finish<<<sys->n_structures, 256, 0, ctx->stream>>>(N, S, P, sys->d_struct_offsets, sys->d_species, ctx->d_lut,
@@ -837,7 +924,7 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
                                                              d_energy);
     RASCAL_LAUNCH_CHECK("k_gpr_finish");
     if (grad) {
-        k_gpr_grad<<<2 * ctx->n_sm, kGprThreads, gpr_smem2(), ctx->stream>>>(A);
+        k_gpr_grad<<<2 * ctx->n_sm, kGprThreads2, gpr_smem2(), ctx->stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_gpr_grad");
     }
     return RASCAL_OK;

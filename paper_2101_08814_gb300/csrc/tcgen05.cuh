@@ -75,6 +75,13 @@ __device__ inline bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint32_
     return false;
 }
 
+// the same for waits inside a pipeline, which are short: polls before it sleeps
+__device__ inline bool mbar_wait_spin(uint64_t* bar, uint32_t parity) {
+    for (int it = 0; it < 512; ++it)
+        if (mbar_test_wait(bar, parity)) return true;
+    return mbar_wait_bounded(bar, parity);
+}
+
 __device__ inline void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ inline void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // generic-proxy shared-memory writes -> visible to the tensor core (async proxy)
@@ -103,6 +110,20 @@ __device__ inline uint64_t smem_desc_sw64(uint32_t saddr, uint32_t sbo) {
 }
 __device__ inline uint32_t sw64_off(int row, int chunk) {
     return (uint32_t)((row >> 3) * 512 + (row & 7) * 64 + ((chunk ^ ((row >> 1) & 3)) << 4));
+}
+
+// the same with 128-byte rows: 8-row atoms of 1024 bytes, chunk c of row r at chunk c ^ (r & 7)
+__device__ inline uint64_t smem_desc_sw128(uint32_t saddr, uint32_t sbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;                     // swizzling mode: 128 bytes
+    return d;
+}
+__device__ inline uint32_t sw128_off(int row, int chunk) {
+    return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((chunk ^ (row & 7)) << 4));
 }
 
 // instruction descriptor: D FP32, A/B format (1 = BF16 for kind::f16, 2 = TF32 for kind::tf32), K-major A and B
@@ -203,6 +224,10 @@ __device__ inline void cp_async16_zfill(void* sdst, const void* gsrc, uint32_t s
 __device__ inline void cp_async4_zfill(void* sdst, const void* gsrc, uint32_t src_bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(src_bytes)
                  : "memory");
+}
+// one arrival on an mbarrier once this thread's cp.async copies so far have landed
+__device__ inline void cp_async_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>

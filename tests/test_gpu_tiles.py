@@ -10,6 +10,7 @@ from oracle import soap as osoap  # noqa: E402
 from oracle.neighbours import neighbour_list  # noqa: E402
 from synth import System, config_batch, mlp_initial_params, random_cell_atoms  # noqa: E402
 from tests.gpu_common import block_rel_err  # noqa: E402
+from tests.test_gpu_gpr import _emulated_energies, _grad_checks, _predict, _unit_tf32, tf32_trunc  # noqa: E402
 
 H = 64
 
@@ -230,3 +231,30 @@ def test_gradient_chunks(rg, n_max, l_max, S):
         e_size = torch.zeros(5, device="cuda", dtype=torch.float64).index_add(0, at, (pa * wa.abs()).sum(1))
         assert bool(((e - ref).abs() <= eps * e_size).all())
         assert bool(((fe - f).abs().amax(dim=1) <= eps * f_size).all()) and bool(((ve - v).abs().amax(dim=(1, 2)) <= eps * v_size).all())
+
+
+# Tiles of 128, 256 and 512 sparse points (one and several to a species, the wider ones where there are centres for every
+# SM), a species whose points are not a multiple of 32, features of less than a stage, of an odd number (4-byte copies) and of
+# half a stage past a whole one; gradient tiles of 256 features and what is left of them. Against the arithmetic on the inputs
+# as the tensor core sees them; the bounds are those of the model's other tests (1e-5 zeta sum |x|, 1e-4 of the terms).
+@pytest.mark.parametrize("N,F,points", [(140, 12, (3, 17)), (300, 301, (130, 40)), (260, 1040, (256, 48)), (19500, 36, (200, 16)),
+                                        (13000, 20, (600, 32)), (130, 272, (560, 0))])
+def test_gpr_tiles(rg, N, F, points):
+    rng = np.random.default_rng(47)
+    spe = rng.choice([1, 6], size=N).astype(np.int32)
+    s = System(rng.uniform(0, 20, size=(N, 3)), spe, np.eye(3)[None] * 20, np.ones((1, 3), np.int32), np.array([0, N], np.int32),
+               dict(r_cut=4.0, sigma=0.5, n_max=2, l_max=1, smooth_width=0.5, species=[1, 6]), "gpr-tiles")
+    p32 = np.abs(rng.normal(size=(N, F))).astype(np.float32)
+    M = np.abs(rng.normal(size=(sum(points), F)))
+    labels = np.repeat([1, 6], points).astype(np.int32)
+    x = rng.standard_normal(len(M)) / 30
+    Mt, zeta = _unit_tf32(M), 2
+    calc = rg.SoapCalculator(**s.hypers)
+    _, ea, g = _predict(rg, s, calc, p32, Mt, labels, x, zeta)
+    cs, ms = np.searchsorted([1, 6], spe), np.searchsorted([1, 6], labels)
+    E = _emulated_energies(p32, cs, Mt, ms, x, zeta, tf32_trunc)
+    assert np.max(np.abs(ea - E)) <= 1e-5 * zeta * np.sum(np.abs(x))
+    part = rng.choice(N, size=min(N, 600), replace=False)
+    r_emul, r_exact = _grad_checks(g[part], p32[part], cs[part], Mt, ms, x, zeta, Mt)
+    assert r_emul <= 1.0 and r_exact <= 1.0
+    assert np.all(g[~np.isin(cs, ms)] == 0.0)
