@@ -206,6 +206,7 @@ int64_t scan_tile_sums_len(int64_t n);
 int scan_exclusive_into(const int* in, int64_t* out, int64_t n, cudaStream_t stream, int64_t* sums);
 
 int validate_system(const rascal_ctx* ctx, const rascal_system* sys);
+int soap_supported(rascal_ctx* ctx);  // whether the fused FP32 PACKED power spectrum takes the context's hypers
 
 int radial_grid_fp64(rascal_ctx* ctx, int M, double* grid, double* ends, double* y, double* yend, double* dyend,
                      double* cp, double* y2);

@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
     int* s_start = s_list + chunk;                                    // [kMaxSpecies + 1]
     int* s_fmap = s_start + (kMaxSpecies + 1) + (kMaxLMax + 2);        // [F_pad]
     unsigned char* gram = smem_raw + A.gram_off;                      // CT or tiles
-    float* stage = s_G;                                               // reused once the pairs are done
+    // reused once the pairs are done (coefficients only: behind everything where a round's coefficients are more)
+    float* stage = GRAM == kGramNone ? reinterpret_cast<float*>(smem_raw + A.gram_off) : s_G;
 
     const int i = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -211,59 +212,39 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
             // comes first and only the round's pairs get rows (so too in the tensor-core forms, where the two
             // values warp 0 would hold through the phase cost more than the wait: 2.98 against 2.91 ms in BF16)
             const bool early = kCT && kRounds == 1;
-            int lab = -1;  // chunk <= 32: the neighbour's species label, held by lane p of warp 0
-            float vw = 0.0f;
+            int lab = -1;  // the neighbour's species label, held by lane p of warp 0 (a chunk is at most 32 pairs)
+            float vw = 0.0f;  // and its distance, where it would be read back long after (elsewhere it costs a spill)
             auto list_pairs = [&]() {  // warp 0
                 int a = -2;  // lanes without a pair match no species
-                if (chunk <= 32 && lane < nc) {
+                if (lane < nc) {
                     a = (lab >= 0 && lab < 256) ? A.lut[lab] : -1;
                     if (a < 0) atomicOr(A.flags, kFlagSpecies);
-                    if (!(vw > 1e-6f)) a = -1;  // coincident atoms are flagged by the neighbour search
+                    if (!((kCT ? vw : s_vec[lane].w) > 1e-6f)) a = -1;  // coincident atoms are flagged by the neighbour search
                 }
                 int base = 0;
                 #pragma unroll 1
                 for (int ga = 0; ga < na; ++ga) {
                     if (lane == 0) s_start[ga] = base;
-                    #pragma unroll 1
-                    for (int p0 = 0; p0 < nc; p0 += 32) {
-                        const int p = p0 + lane;
-                        const bool mine = chunk <= 32 ? (a == a0 + ga) : (p < nc && s_spc[p] == a0 + ga);
-                        const unsigned m = __ballot_sync(0xffffffffu, mine);
-                        if (mine) s_list[base + __popc(m & ((1u << lane) - 1u))] = p;
-                        base += __popc(m);
-                    }
+                    const bool mine = a == a0 + ga;
+                    const unsigned m = __ballot_sync(0xffffffffu, mine);
+                    if (mine) s_list[base + __popc(m & ((1u << lane) - 1u))] = lane;
+                    base += __popc(m);
                 }
                 if (lane == 0) s_start[na] = base;
             };
-            if (chunk <= 32) {
-                if (warp == 0) {
-                    if (lane < nc) {
-                        const float4 v = seg_rij[pos + lane];
-                        const int j = seg_j[pos + lane];
-                        s_vec[lane] = v;
-                        s_fc[lane] = cutoff_fp32(v.w, A.r_cut, A.width);
-                        vw = v.w;
-                        lab = A.species[j];
-                    }
-                    if (!early) list_pairs();
+            if (warp == 0) {
+                if (lane < nc) {
+                    const float4 v = seg_rij[pos + lane];
+                    const int j = seg_j[pos + lane];
+                    s_vec[lane] = v;
+                    s_fc[lane] = cutoff_fp32(v.w, A.r_cut, A.width);
+                    if (kCT) vw = v.w;
+                    lab = A.species[j];
                 }
-            } else {
-            #pragma unroll 1
-            for (int t = tid; t < nc; t += blockDim.x) {
-                const float4 v = seg_rij[pos + t];
-                const int j = seg_j[pos + t];
-                const int lb = A.species[j];
-                int a = (lb >= 0 && lb < 256) ? A.lut[lb] : -1;
-                if (a < 0) atomicOr(A.flags, kFlagSpecies);
-                if (!(v.w > 1e-6f)) a = -1;  // coincident atoms are flagged by the neighbour search
-                s_vec[t] = v;
-                s_spc[t] = a;
-                s_fc[t] = cutoff_fp32(v.w, A.r_cut, A.width);
-            }
-            if (!early) {
-                __syncthreads();
-                if (warp == 0) list_pairs();
-            }
+                if (!early) {
+                    __syncwarp();
+                    list_pairs();
+                }
             }
             __syncthreads();
             const int n_rows = early ? nc : s_start[na];
@@ -358,6 +339,8 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
             // CT, and the barrier that hands CT over comes before anything reuses the pair buffers
             if (!kCT || pos + chunk < seg_len || round + 1 < kRounds) __syncthreads();
         }
+        float* cdst = A.coeffs + ((int64_t)i * kS + a0) * kNmax * kNlm;  // the round's coefficients
+        float* cst = stage + stage_shift(cdst);
         float acc[4][4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -378,12 +361,12 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                     }
                 }
             }
-            if (RTC) {  // c[q][lm] staged in the (free) pair rows; the operand rounds read it from there
+            if (RTC || GRAM == kGramNone) {  // c[q][lm] staged in the (free) pair rows, whence it leaves by one bulk copy
                 const int s_end = 2 * my_l + 1 - 4 * my_mt;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     if (4 * my_nt + u >= kNmax) continue;
-                    float* crow = cst_r + (a * kNmax + 4 * my_nt + u) * kNlm + my_l * my_l + 4 * my_mt;
+                    float* crow = cst + (g * kNmax + 4 * my_nt + u) * kNlm + my_l * my_l + 4 * my_mt;
                     if (s_end >= 4 && (reinterpret_cast<uintptr_t>(crow) & 15) == 0) {
                         *reinterpret_cast<float4*>(crow) = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
                     } else {
@@ -392,7 +375,6 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                             if (v < s_end) crow[v] = acc[u][v];
                     }
                 }
-                continue;
             }
             if (kCT) {  // tile -> CT[l^2 + s][a n_max + n]; c reaches HBM from CT afterwards
                 float* ct = reinterpret_cast<float*>(gram) + (my_l * my_l + 4 * my_mt) * kQp + a * kNmax + 4 * my_nt;
@@ -410,26 +392,41 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                             if (u < u_end) row[u] = acc[u][v];
                     }
                 }
-                continue;
             }
-            float* out = A.coeffs + ((int64_t)i * kS + a) * kNmax * kNlm + my_l * my_l;
+            if (TC) {
+                float* out = A.coeffs + ((int64_t)i * kS + a) * kNmax * kNlm + my_l * my_l;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int n = 4 * my_nt + u;
-                if (n >= kNmax) continue;
-                const int q = a * kNmax + n;
+                for (int u = 0; u < 4; ++u) {
+                    const int n = 4 * my_nt + u;
+                    if (n >= kNmax) continue;
+                    const int q = a * kNmax + n;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int s = 4 * my_mt + v;
-                    if (s > 2 * my_l) continue;
-                    const float cv = acc[u][v];
-                    out[n * kNlm + s] = cv;
-                    if (TC) put_operand<GRAM>(gram, A, my_l, q, s, cv);
+                    for (int v = 0; v < 4; ++v) {
+                        const int s = 4 * my_mt + v;
+                        if (s > 2 * my_l) continue;
+                        const float cv = acc[u][v];
+                        out[n * kNlm + s] = cv;
+                        put_operand<GRAM>(gram, A, my_l, q, s, cv);
+                    }
                 }
             }
         }
+        // coefficients only: 16 scattered 4-byte stores per thread were 210 of 808 us on 8 192 centres (n_max 16, l_max 12, 8
+        // species: 0.71 GB of coefficients); staged like this the kernel takes 670
+        if (GRAM == kGramNone) {
+            fence_proxy_async_smem();
+            __syncthreads();
+            store_staged(cdst, cst, na * kNmax * kNlm);
+            if (round + 1 < kRounds) {  // the next round's rows take its place
+                if (tid == 0) bulk_wait_read<0>();
+                __syncthreads();
+            }
+        }
     }
-    if (GRAM == kGramNone) return;
+    if (GRAM == kGramNone) {
+        if (tid == 0) bulk_wait_all();
+        return;
+    }
     if (RTC) {
         // ---------------------------------------------------------------- tensor-core Gram in rounds of one l
         fence_proxy_async_smem();
@@ -1027,6 +1024,11 @@ static int exp_shape_of(const rascal_ctx* ctx, const ExpArgs& A, bool with_qp) {
 
 template <int GRAM, int SHAPE = 0>
 static int launch_expansion(rascal_ctx* ctx, const ExpArgs& A, int n_atoms, int threads, size_t smem) {
+    // Warps beyond the ones that hold coefficient tiles share the harmonics, the radial rows and the Gram tiles. A basis of one
+    // or two tile warps takes four: 4 096 centres of n_max 8, l_max 6, 2 species 34 -> 27 us (six warps 28, eight 30), and
+    // eight where no SM has more than two centres: 64 centres of 1 species 29 -> 10 us (four warps 13).
+    if (GRAM == kGramNone || GRAM == kGramSimt || GRAM == kGramSel)
+        threads = std::max(threads, n_atoms <= 2 * ctx->n_sm ? 256 : 128);
     k_expansion<GRAM, SHAPE><<<n_atoms, threads, smem, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_expansion");
     return RASCAL_OK;
@@ -1042,6 +1044,13 @@ static int launch_shaped(rascal_ctx* ctx, const ExpArgs& A, int n_atoms, int thr
         case 4: return launch_expansion<GRAM, 4>(ctx, A, n_atoms, threads, smem);
         default: return launch_expansion<GRAM>(ctx, A, n_atoms, threads, smem);
     }
+}
+
+int soap_supported(rascal_ctx* ctx) {
+    ExpArgs A = make_args(ctx, nullptr, nullptr, nullptr, nullptr, nullptr);
+    size_t smem;
+    int threads;
+    return make_gram(ctx, kGramSimt, RASCAL_LAYOUT_PACKED, nullptr, A, &smem, &threads);
 }
 
 int power_spectrum_tc(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps) {
@@ -1077,7 +1086,17 @@ extern "C" int rascal_spherical_expansion(rascal_ctx* ctx, const rascal_system* 
     ExpArgs A = make_args(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs);
     const float* pre_D;
     if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, false, &A.pre_G, &pre_D))) return st;
-    return launch_shaped<kGramNone>(ctx, A, sys->n_atoms, ctx->plan.threads, ctx->plan.smem);
+    // a round's coefficients, staged over the pair rows or behind everything (where a chunk has few values per pair for the
+    // species of a round)
+    const ExpPlan& P = ctx->plan;
+    const size_t rows = sizeof(float) * P.chunk * (P.F_pad + P.Ly), need = sizeof(float) * ((size_t)P.S_c * ctx->n_max * ctx->n_lm + 3);
+    size_t smem = P.smem;
+    A.gram_off = (int)(sizeof(float4) * P.chunk);
+    if (need > rows) {
+        A.gram_off = (int)align_up(smem, 16);
+        smem = A.gram_off + need;
+    }
+    return launch_shaped<kGramNone>(ctx, A, sys->n_atoms, P.threads, smem);
 }
 
 // PACKED feature index -> (l | q1 << 8 | q2 << 16); out-of-range indices flag an error and decode to l = 255 (zero)

@@ -258,3 +258,27 @@ def test_gpr_tiles(rg, N, F, points):
     r_emul, r_exact = _grad_checks(g[part], p32[part], cs[part], Mt, ms, x, zeta, Mt)
     assert r_emul <= 1.0 and r_exact <= 1.0
     assert np.all(g[~np.isin(cs, ms)] == 0.0)
+
+
+# Coefficients alone equal those of the fused call bit for bit: one and several species rounds, coefficients of a round that fit
+# the pair rows and that do not (16 species), targets at every alignment, four warps and eight (at most two centres per SM), no
+# neighbours, one chunk and several.
+@pytest.mark.parametrize("n_max,l_max,S,n,copies", [(1, 0, 1, 40, 1), (8, 6, 1, 64, 1), (8, 6, 2, 50, 8), (5, 3, 3, 50, 8),
+                                                    (4, 6, 16, 60, 1), (16, 12, 8, 30, 1), (10, 8, 3, 90, 1)])
+def test_coefficients_alone(rg, n_max, l_max, S, n, copies):
+    import torch
+
+    calc = rg.SoapCalculator(5.0, 0.5, n_max, l_max, list(range(1, S + 1)), include_center=True, spline_intervals=64)
+    rng = np.random.default_rng(53)
+    L = (n / 0.08) ** (1 / 3)
+    pos = np.concatenate([np.concatenate([random_cell_atoms(n, np.eye(3) * L, 1.0, rng), [[0.0, 0.0, 60.0]]])] * copies)
+    s = System(pos, rng.integers(1, S + 1, len(pos)).astype(np.int32), np.tile(np.diag([L, L, 200.0])[None], (copies, 1, 1)),
+               np.tile([[1, 1, 0]], (copies, 1)).astype(np.int32), np.arange(0, len(pos) + 1, n + 1).astype(np.int32), {})
+    ds = rg.DeviceSystem.from_numpy(s)
+    pairs = calc.neighbours(ds)
+    ref, _ = calc.soap(ds, pairs)
+    for shift in range(4):
+        out = torch.full((ref.numel() + 8,), 7.0, device="cuda")
+        calc.spherical_expansion(ds, pairs, out=out[shift:])
+        assert torch.equal(out[shift:shift + ref.numel()].view_as(ref), ref)
+        assert bool((out[:shift] == 7.0).all()) and bool((out[shift + ref.numel():] == 7.0).all())
