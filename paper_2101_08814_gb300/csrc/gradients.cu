@@ -135,12 +135,19 @@ __host__ __device__ constexpr int grad_h_pitch(int l_max, int n_max) {
 }
 __host__ __device__ constexpr int grad_g_pitch(int F_pad) { return 2 * F_pad + 2; }
 
-// Dense symmetric adjoint weights: Ws[a][l][k][q] = k_l (W_l + W_l^T)[k][q] from the packed upper-triangular
-// weight rows (entry (q1 <= q2) at q1 (2Q - q1 - 1) / 2 + q2), zero in the padding columns q >= Q.
-__global__ void k_wsym(int S, int L1, int Q, int Qw, int ps_norm, const float* __restrict__ w, int64_t Fp,
-                       float* __restrict__ ws) {
-    const int64_t total = (int64_t)S * L1 * Q * Qw;
+// What a call needs before the gradient kernel, in one launch instead of four: dense symmetric adjoint weights (linear model)
+// Ws[a][l][k][q] = k_l (W_l + W_l^T)[k][q] from the packed upper-triangular weight rows (entry (q1 <= q2) at
+// q1 (2Q - q1 - 1) / 2 + q2), zero in the padding columns q >= Q, and zeros in the sums that the gradient kernel adds to.
+__global__ void k_prepare(int S, int L1, int Q, int Qw, int ps_norm, const float* __restrict__ w, int64_t Fp,
+                          float* __restrict__ ws, int64_t n3, float* __restrict__ forces, int n_s, double* __restrict__ virial,
+                          double* __restrict__ energy) {
+    const int64_t total = ws ? (int64_t)S * L1 * Q * Qw : 0;
     const int Qpk = Q * (Q + 1) / 2;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n3; e += (int64_t)gridDim.x * blockDim.x) forces[e] = 0.0f;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 9 * (int64_t)n_s; e += (int64_t)gridDim.x * blockDim.x) {
+        virial[e] = 0.0;
+        if (energy && e < n_s) energy[e] = 0.0;
+    }
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int q = (int)(e % Qw);
         const int64_t r = e / Qw;
@@ -968,10 +975,12 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     if (!d_forces || !d_virial) return set_error(RASCAL_E_ARG, "NULL forces or virial");
     if ((d_grad_ps == nullptr) == (d_weights == nullptr))
         return set_error(RASCAL_E_ARG, "exactly one of grad_ps and weights must be given");
-    RASCAL_CUDA(cudaMemsetAsync(d_forces, 0, sizeof(double) * 3 * sys->n_atoms, ctx->stream));
-    RASCAL_CUDA(cudaMemsetAsync(d_virial, 0, sizeof(double) * 9 * sys->n_structures, ctx->stream));
-    if (d_energy) RASCAL_CUDA(cudaMemsetAsync(d_energy, 0, sizeof(double) * sys->n_structures, ctx->stream));
-    if (sys->n_atoms == 0) return RASCAL_OK;
+    if (sys->n_atoms == 0) {
+        RASCAL_CUDA(cudaMemsetAsync(d_virial, 0, sizeof(double) * 9 * sys->n_structures, ctx->stream));
+        if (d_energy) RASCAL_CUDA(cudaMemsetAsync(d_energy, 0, sizeof(double) * sys->n_structures, ctx->stream));
+        return RASCAL_OK;
+    }
+    if (!d_offsets || !d_nbr_j || !d_rij || !d_coeffs) return set_error(RASCAL_E_ARG, "NULL device pointer");
     const int L1 = ctx->l_max + 1;
     const int Qw = (ctx->Q + 3) / 4 * 4;
     const size_t n_ws = d_weights ? (size_t)ctx->n_species * L1 * ctx->Q * Qw : 0;
@@ -982,8 +991,6 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     Carver wcv(wbase);
     float* f32 = wcv.take<float>(3 * (size_t)sys->n_atoms);
     float* ws = wcv.take<float>(n_ws);
-    RASCAL_CUDA(cudaMemsetAsync(f32, 0, sizeof(float) * 3 * sys->n_atoms, ctx->stream));
-    if (!d_offsets || !d_nbr_j || !d_rij || !d_coeffs) return set_error(RASCAL_E_ARG, "NULL device pointer");
     const ExpPlan& P = ctx->plan;
     GradArgs A = {};
     A.offsets = d_offsets;
@@ -1019,16 +1026,10 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     A.r_cut = (float)ctx->r_cut;
     A.width = (float)ctx->smooth_width;
     for (int l = 0; l < kMaxLMax + 2; ++l) A.lp[l] = P.lp[l];
-    A.wsym = nullptr;
-    if (d_weights) {  // dense symmetric adjoint weights per species and l, for the tiled adjoint
-        A.Qw = Qw;
-        A.Lp_adj = P.Lp;
-        const int blocks = (int)std::min<size_t>((n_ws + 255) / 256, 4096);
-        k_wsym<<<blocks, 256, 0, ctx->stream>>>(ctx->n_species, L1, ctx->Q, A.Qw, ctx->ps_norm, d_weights, A.Fp, ws);
-        RASCAL_LAUNCH_CHECK("k_wsym");
-        A.wsym = ws;
-        A.n_adj_tasks = (ctx->Q + 3) / 4 * (P.Lp / 4);
-    }
+    A.wsym = d_weights ? ws : nullptr;
+    A.Qw = Qw;
+    A.Lp_adj = P.Lp;
+    A.n_adj_tasks = (ctx->Q + 3) / 4 * (P.Lp / 4);
     size_t smem = 0;
     // a per-centre dE/dp: all its l blocks staged at once where two CTAs per SM still fit, else as many as fit
     A.w_lg = d_weights ? 0 : L1;
@@ -1045,7 +1046,6 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
         A.chunk = 32;
         A.w_off = (int)(grad_c_off(ctx) + grad_c_bytes(ctx, true));
         A.aux_off = 0;
-        if (A.w_lg) A.Lp_adj = P.Lp;
     } else {
         // the largest chunk (<= 32: one warp stages a chunk, a pair per lane) that keeps five CTAs per SM (48 registers)
         const bool tiled = A.wsym != nullptr;
@@ -1064,6 +1064,11 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
         if (smem > 220 * 1024) return set_error(RASCAL_E_UNSUPPORTED, "hypers too large for the gradient kernel");
     }
     if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, true, &A.pre_G, &A.pre_D))) return st;
+    const int64_t n3 = 3 * (int64_t)sys->n_atoms, n_prep = std::max({n3, (int64_t)n_ws, 9 * (int64_t)sys->n_structures});
+    k_prepare<<<(unsigned)std::min<int64_t>((n_prep + 255) / 256, 4096), 256, 0, ctx->stream>>>(
+        ctx->n_species, L1, ctx->Q, Qw, ctx->ps_norm, d_weights, A.Fp, d_weights ? ws : nullptr, n3, f32, sys->n_structures,
+        d_virial, d_energy);
+    RASCAL_LAUNCH_CHECK("k_prepare");
     // a compiled instance for the hyper shape when the plan's sizes match it (kExpShapes), else the generic kernel
     int shape = 0;
     for (int k = 1; k < kNumExpShapes && !shape; ++k) {
@@ -1078,7 +1083,6 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     else
         k_gradients_wide<<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_gradients");
-    const int64_t n3 = 3 * (int64_t)sys->n_atoms;
     k_forces_f64<<<(unsigned)std::min<int64_t>((n3 + 255) / 256, 8192), 256, 0, ctx->stream>>>(n3, f32, d_forces);
     RASCAL_LAUNCH_CHECK("k_forces_f64");
     return RASCAL_OK;
@@ -1093,10 +1097,10 @@ extern "C" int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const
 extern "C" int rascal_linear_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets,
                                        const int* d_nbr_j, const float* d_rij, const float* d_coeffs, const float* d_weights,
                                        double* d_energy, double* d_forces, double* d_virial) {
-    if (!d_energy) {
-        clear_error();
-        return set_error(RASCAL_E_ARG, "NULL energy");
-    }
+    clear_error();
+    if (!ctx) return set_error(RASCAL_E_ARG, "NULL context");
+    if (!d_energy) return set_error(RASCAL_E_ARG, "NULL energy");
+    if (int st = soap_supported(ctx)) return st;  // the same bases with forces as without (which take a power spectrum)
     return gradients(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs, nullptr, d_weights, d_energy, d_forces, d_virial);
 }
 
