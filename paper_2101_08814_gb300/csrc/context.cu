@@ -462,6 +462,7 @@ extern "C" void rascal_destroy(rascal_ctx* ctx) {
     cudaFree(ctx->mlp_w3t);
     cudaFreeHost(ctx->h_flags);
     cudaFreeHost(ctx->h_pinned);
+    if (ctx->counted) cudaEventDestroy(ctx->counted);
     cudaFree(ctx->scratch.ptr);
     cudaFree(ctx->scratch_w.ptr);
     cudaFree(ctx->d_dvr);
@@ -533,6 +534,7 @@ static int create_impl(const rascal_hypers* h, void* stream, rascal_ctx** out) {
     RASCAL_CUDA(cudaMalloc(&ctx->d_flags, sizeof(unsigned)));
     RASCAL_CUDA(cudaMallocHost(&ctx->h_flags, sizeof(unsigned)));
     RASCAL_CUDA(cudaMallocHost(&ctx->h_pinned, sizeof(int64_t) * 8));
+    RASCAL_CUDA(cudaEventCreateWithFlags(&ctx->counted, cudaEventDisableTiming));
     RASCAL_CUDA(cudaMemsetAsync(ctx->d_flags, 0, sizeof(unsigned), ctx->stream));
     int lut[256];
     for (int i = 0; i < 256; ++i) lut[i] = -1;

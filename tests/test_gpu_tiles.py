@@ -282,3 +282,41 @@ def test_coefficients_alone(rg, n_max, l_max, S, n, copies):
         calc.spherical_expansion(ds, pairs, out=out[shift:])
         assert torch.equal(out[shift:shift + ref.numel()].view_as(ref), ref)
         assert bool((out[:shift] == 7.0).all()) and bool((out[shift + ref.numel():] == 7.0).all())
+
+
+# The fill pass is queued before the host knows the counts: where they do not fit it writes nothing (too small a capacity, a
+# flagged geometry), and where a centre has more pairs than a warp sorts in shared memory (150) it runs once they are known.
+@pytest.mark.parametrize("entry,n", [("rascal_neighbours", 60), ("rascal_neighbours_noalloc", 60), ("rascal_neighbours", 151)])
+def test_neighbour_fill_waits_for_the_counts(rg, entry, n):
+    import ctypes as C
+
+    import torch
+
+    s = _cell(n, np.eye(3) * (11.0 if n == 60 else 2.2), 5.0 if n == 60 else 3.9, (1, 1, 1) if n == 60 else (0, 0, 0),
+              **({} if n == 60 else dict(d_min=0.3)))
+    ref = neighbour_list(s, s.hypers["r_cut"])
+    P = len(ref["nbr_j"])
+    calc = rg.SoapCalculator(**s.hypers)
+
+    def call(system, capacity):
+        ds = rg.DeviceSystem.from_numpy(system)
+        off = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+        j = torch.full((P,), -5, dtype=torch.int32, device="cuda")
+        sh = torch.full((P, 3), -5, dtype=torch.int32, device="cuda")
+        rij = torch.full((P, 4), -5.0, device="cuda")
+        sys_c, count = ds.c_struct(), C.c_int64(0)
+        st = getattr(rg._lib.lib(), entry)(calc._ctx, C.byref(sys_c), capacity, *(C.c_void_p(t.data_ptr()) for t in (off, j, sh, rij)),
+                                           C.byref(count))
+        torch.cuda.synchronize()
+        return st, count.value, j.cpu().numpy(), sh.cpu().numpy(), rij.cpu().numpy()
+
+    calc._bind_stream()
+    st, count, j, sh, rij = call(s, P - 1)
+    assert st == rg._lib.RASCAL_E_CAPACITY and count == P and np.all(j == -5) and np.all(sh == -5) and np.all(rij == -5.0)
+    same = s.positions.copy()
+    same[1] = same[0]
+    st, _, j, sh, rij = call(System(same, s.species, s.cells, s.pbc, s.struct_offsets, s.hypers), P)
+    assert st == rg._lib.RASCAL_E_GEOMETRY and np.all(j == -5) and np.all(sh == -5) and np.all(rij == -5.0)
+    st, count, j, sh, rij = call(s, P)
+    assert st == 0 and count == P and np.array_equal(j, ref["nbr_j"]) and np.array_equal(sh, ref["shifts"])
+    assert np.allclose(rij[:, :3], ref["rij"], rtol=0, atol=2e-6)
