@@ -320,3 +320,24 @@ def test_neighbour_fill_waits_for_the_counts(rg, entry, n):
     st, count, j, sh, rij = call(s, P)
     assert st == 0 and count == P and np.array_equal(j, ref["nbr_j"]) and np.array_equal(sh, ref["shifts"])
     assert np.allclose(rij[:, :3], ref["rij"], rtol=0, atol=2e-6)
+
+
+# Outputs of one 16-column tile, of half a 32-column slab, not a multiple of 4 (scalar stores), the most TMEM holds; batches
+# of one, one short of and one past a tile, several tiles; with and without derivatives; nothing written past the last row.
+# Bounds of the other inference test: 2e-2 (values) and 3e-2 (derivatives) of the largest, from the 16-bit operands.
+@pytest.mark.parametrize("n_max,l_max", [(1, 0), (5, 2), (4, 3), (7, 6), (16, 12), (16, 15)])
+def test_inference_tiles(rg, n_max, l_max):
+    calc = rg.SoapCalculator(5.0, 0.5, n_max, l_max, [1], spline_intervals=64)
+    F = n_max * (l_max + 1)
+    p = mlp_initial_params(H, F)
+    calc.mlp_set_params(p, np.ones(F, np.float32))
+    rng = np.random.default_rng(59)
+    r = rng.uniform(0.2, 5.0, 700).astype(np.float32)
+    y, dy, _ = omlp.forward(_network(p, F), r.astype(np.float64) / 5.0, tangent=True)
+    dy = dy / 5.0
+    whole, dwhole = (t.cpu().numpy() for t in calc.mlp_eval(r, derivative=True))
+    assert np.max(np.abs(whole - y)) <= 2e-2 * np.max(np.abs(y)) and np.max(np.abs(dwhole - dy)) <= 3e-2 * np.max(np.abs(dy))
+    for n in (1, 127, 129, 700):
+        v, d = (t.cpu().numpy() for t in calc.mlp_eval(r[:n], derivative=True))
+        assert np.array_equal(v, whole[:n]) and np.array_equal(d, dwhole[:n])
+        assert np.array_equal(calc.mlp_eval(r[:n]).cpu().numpy(), whole[:n])
