@@ -1105,17 +1105,8 @@ int power_spectrum_tc(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs,
 
 using namespace rascal;
 
-extern "C" int rascal_spherical_expansion(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets,
-                                          const int* d_nbr_j, const float* d_rij, float* d_coeffs) {
-    clear_error();
-    if (!ctx) return set_error(RASCAL_E_ARG, "NULL context");
-    int st = validate_system(ctx, sys);
-    if (st) return st;
-    if (sys->n_atoms == 0) return RASCAL_OK;
-    if (!d_offsets || !d_nbr_j || !d_rij || !d_coeffs) return set_error(RASCAL_E_ARG, "NULL device pointer");
-    ExpArgs A = make_args(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs);
-    const float* pre_D;
-    if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, false, &A.pre_G, &pre_D))) return st;
+// c alone
+static int coefficients(rascal_ctx* ctx, const rascal_system* sys, ExpArgs A) {
     // a round's coefficients, staged over the pair rows or behind everything (where a chunk has few values per pair for the
     // species of a round)
     const ExpPlan& P = ctx->plan;
@@ -1127,6 +1118,20 @@ extern "C" int rascal_spherical_expansion(rascal_ctx* ctx, const rascal_system* 
         smem = A.gram_off + need;
     }
     return launch_shaped<kGramNone>(ctx, A, sys->n_atoms, P.threads, smem);
+}
+
+extern "C" int rascal_spherical_expansion(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets,
+                                          const int* d_nbr_j, const float* d_rij, float* d_coeffs) {
+    clear_error();
+    if (!ctx) return set_error(RASCAL_E_ARG, "NULL context");
+    int st = validate_system(ctx, sys);
+    if (st) return st;
+    if (sys->n_atoms == 0) return RASCAL_OK;
+    if (!d_offsets || !d_nbr_j || !d_rij || !d_coeffs) return set_error(RASCAL_E_ARG, "NULL device pointer");
+    ExpArgs A = make_args(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs);
+    const float* pre_D;
+    if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, false, &A.pre_G, &pre_D))) return st;
+    return coefficients(ctx, sys, A);
 }
 
 // PACKED feature index -> (l | q1 << 8 | q2 << 16); out-of-range indices flag an error and decode to l = 255 (zero)
@@ -1188,19 +1193,29 @@ extern "C" int rascal_soap(rascal_ctx* ctx, const rascal_system* sys, const int6
     ExpArgs A = make_args(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs);
     const float* pre_D;
     if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, false, &A.pre_G, &pre_D))) return st;
-    if (precision == RASCAL_PS_TF32X3) {  // TF32x3: the tensor-core Gram in rounds of one l where the hypers fit it
-        ExpArgs R = A;
-        size_t smem_r;
-        int threads_r;
-        st = make_gram(ctx, kGramRTf32, layout, d_ps, R, &smem_r, &threads_r);
-        if (st == RASCAL_OK) return launch_shaped<kGramRTf32>(ctx, R, sys->n_atoms, threads_r, smem_r);
+    const int mode = precision == RASCAL_PS_FP32 ? kGramSimt : (precision == RASCAL_PS_BF16 ? kGramBf16 : kGramTf32x3);
+    const ExpArgs plain = A;
+    ExpArgs R = A;
+    size_t smem, smem_r;
+    int threads, threads_r;
+    // TF32x3: the tensor-core Gram in rounds of one l where the hypers fit it
+    const int st_r = precision == RASCAL_PS_TF32X3 ? make_gram(ctx, kGramRTf32, layout, d_ps, R, &smem_r, &threads_r)
+                                                  : RASCAL_E_UNSUPPORTED;
+    if (st_r != RASCAL_OK && st_r != RASCAL_E_UNSUPPORTED) return st_r;
+    clear_error();
+    if (st_r && (st = make_gram(ctx, mode, layout, d_ps, A, &smem, &threads))) return st;
+    // The tensor-core precisions as two launches, coefficients and the spectrum kernel of stored coefficients: 13 440 centres of
+    // 25 pairs (12, 9, 4) BF16 564 -> 357 us and TF32x3 698 -> 417, of 2 species (8, 6) 301 -> 119 and 414 -> 125, of 30 pairs (9,
+    // 7, 3) 528 -> 239 and 551 -> 256, 200 centres 24 -> 22 and 27 -> 23; TF32x3 errors 4.8e-7 -> 1.2e-7. The one-launch forms
+    // wait for a chain of barriers and MMAs per l; they serve what the spectrum kernel does not take, and the test hook
+    // that makes their waits run out.
+    if (mode != kGramSimt && !ctx->stall_polls) {
+        if ((st = coefficients(ctx, sys, plain))) return st;
+        st = power_spectrum_warp(ctx, sys->n_atoms, d_coeffs, precision, layout, d_ps);
         if (st != RASCAL_E_UNSUPPORTED) return st;
         clear_error();
     }
-    const int mode = precision == RASCAL_PS_FP32 ? kGramSimt : (precision == RASCAL_PS_BF16 ? kGramBf16 : kGramTf32x3);
-    size_t smem;
-    int threads;
-    if ((st = make_gram(ctx, mode, layout, d_ps, A, &smem, &threads))) return st;
+    if (!st_r) return launch_shaped<kGramRTf32>(ctx, R, sys->n_atoms, threads_r, smem_r);
     if (mode == kGramSimt) return launch_shaped<kGramSimt>(ctx, A, sys->n_atoms, threads, smem);
     if (mode == kGramBf16) return launch_shaped<kGramBf16>(ctx, A, sys->n_atoms, threads, smem);
     return launch_expansion<kGramTf32x3>(ctx, A, sys->n_atoms, threads, smem);

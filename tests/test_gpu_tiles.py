@@ -341,3 +341,30 @@ def test_inference_tiles(rg, n_max, l_max):
         v, d = (t.cpu().numpy() for t in calc.mlp_eval(r[:n], derivative=True))
         assert np.array_equal(v, whole[:n]) and np.array_equal(d, dwhole[:n])
         assert np.array_equal(calc.mlp_eval(r[:n]).cpu().numpy(), whole[:n])
+
+
+# The fused call in the tensor-core precisions is the coefficients followed by the spectrum of stored coefficients, whatever
+# the layout and the alignment of its outputs: Q = 1, 21, 24, 48, one species round and several, no atoms' worth of pairs.
+@pytest.mark.parametrize("n_max,l_max,S,n", [(1, 0, 1, 9), (7, 5, 3, 70), (8, 6, 3, 70), (12, 9, 4, 70), (16, 7, 5, 40)])
+@pytest.mark.parametrize("precision", ["bf16", "tf32x3"])
+def test_fused_tensor_core_precisions(rg, n_max, l_max, S, n, precision):
+    import torch
+
+    calc = rg.SoapCalculator(4.5, 0.5, n_max, l_max, list(range(1, S + 1)), include_center=n_max > 1, spline_intervals=64)
+    rng = np.random.default_rng(67)
+    L = (n / 0.08) ** (1 / 3)
+    s = System(np.concatenate([random_cell_atoms(n, np.eye(3) * L, 1.0, rng), [[0.0, 0.0, 60.0]]]),
+               rng.integers(1, S + 1, n + 1).astype(np.int32), np.diag([L, L, 200.0])[None], np.array([[1, 1, 0]], np.int32),
+               np.array([0, n + 1], np.int32), {})
+    ds = rg.DeviceSystem.from_numpy(s)
+    pairs = calc.neighbours(ds)
+    c_ref = calc.spherical_expansion(ds, pairs)
+    for layout in ("packed", "full"):
+        p_ref = calc.power_spectrum(c_ref, precision=precision, layout=layout)
+        for shift in range(0, 4, 1 + 2 * (layout == "full")):
+            c = torch.full((c_ref.numel() + 8,), 7.0, device="cuda")
+            p = torch.full((p_ref.numel() + 8,), 7.0, device="cuda")
+            calc.soap(ds, pairs, layout=layout, precision=precision, coeffs=c[shift:], ps=p[3 - shift:])
+            assert torch.equal(c[shift:shift + c_ref.numel()].view_as(c_ref), c_ref)
+            assert torch.equal(p[3 - shift:3 - shift + p_ref.numel()].view_as(p_ref), p_ref)
+            assert bool((c[:shift] == 7.0).all()) and bool((p[3 - shift + p_ref.numel():] == 7.0).all())
