@@ -125,8 +125,8 @@ static void lsoap_pairs(int l_max, int lam, std::vector<int2>& p) {
 constexpr int kLsoapThreads = 128, kLsoapCtas = 4;
 constexpr int kLsoapGroups = 36;  // row groups per chunk: X takes 11.5 KB (PX = 20) or 20.7 KB (PX = 36) per buffer
 
-template <bool VEC, int PX>
-__global__ void __launch_bounds__(kLsoapThreads, kLsoapCtas) k_lambda_soap(const float* __restrict__ c, int Q, int l_max, int lam,
+template <bool VEC, int PX, int G>
+__global__ void __launch_bounds__(kLsoapThreads, G == 1 ? 6 : kLsoapCtas) k_lambda_soap(const float* __restrict__ c, int Q, int l_max, int lam,
                                                                            int chunk, unsigned qt_inv, int n_pairs,
                                                                            const int4* __restrict__ hdr,
                                                                            const float4* __restrict__ R,
@@ -192,16 +192,16 @@ __global__ void __launch_bounds__(kLsoapThreads, kLsoapCtas) k_lambda_soap(const
             }
             __syncthreads();
             if (!t_on) continue;
-            const int half = (ng + 1) >> 1;  // a thread's two row groups: r and r + half, if there is one
+            const int half = G == 2 ? (ng + 1) >> 1 : ng;  // a thread's row groups: r and, with G = 2, r + half, if there is one
 #pragma unroll 1
             for (int r = t_r; r < half; r += r_step) {
-                uint64_t acc[8][4];
-                const bool two = r + half < ng;
+                uint64_t acc[4 * G][4];
+                const bool two = G == 2 && r + half < ng;
                 const float* x0 = X + r * 4 * PX;
                 const float* x1 = two ? x0 + half * 4 * PX : x0;
                 const float *b0 = Bt, *b1 = Bt + pitch, *b2 = b1 + pitch, *b3 = b2 + pitch;
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
+                for (int u = 0; u < 4 * G; ++u)
 #pragma unroll
                     for (int v = 0; v < 4; ++v) acc[u][v] = 0ull;
 #pragma unroll 1
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kLsoapThreads, kLsoapCtas) k_lambda_soap(const
                     b[2] = *reinterpret_cast<const ulonglong2*>(b2);
                     b[3] = *reinterpret_cast<const ulonglong2*>(b3);
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
+                    for (int u = 0; u < 4 * G; ++u) {
                         const ulonglong2 x = *reinterpret_cast<const ulonglong2*>((u < 4 ? x0 : x1) + (u & 3) * PX);
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kLsoapThreads, kLsoapCtas) k_lambda_soap(const
                     x1 += 4;
                 }
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
+                for (int k = 0; k < G; ++k) {
                     if (k == 1 && !two) break;
                     const int tau = g0 + r + k * half, mu = div_qt(tau), g = tau - mu * QT;
                     float* o = op + (mu * Q + (VEC ? 4 * g : g)) * Q;
@@ -260,10 +260,23 @@ __global__ void __launch_bounds__(kLsoapThreads, kLsoapCtas) k_lambda_soap(const
 // row pitch of X: 20 holds the widest pair up to l_max 9 (2 l_max + 1 <= 20), 36 every other; an odd number of 16-byte words
 static int lsoap_px(int l_max) { return l_max <= 9 ? 20 : 36; }
 
-static auto lsoap_kernel(int Q, int l_max) {
+// Row groups of a thread's tiles: one where a chunk's 4 x 4 tiles do not exceed the threads (small bases, small ranks), else two;
+// with one, six CTAs per SM (78 registers). Two groups (and 2 x 4 tiles) -> one: 4 000 centres, Q = 15, l_max 9, lambda 0 106
+// (100) -> 72 us; 9 000 centres, Q = 21, l_max 3, lambda 1 90 (167) -> 72 us; 5 000 centres, Q = 12, l_max 4, lambda 0 53 (45) ->
+// 37 us. Past the line two groups win: 3 000 centres, Q = 30, l_max 5, lambda 1 62 against 70 us.
+static bool lsoap_small(int Q, int lam) {
+    const int QT = (Q + 3) / 4;
+    return std::min((2 * lam + 1) * QT, kLsoapGroups) * QT <= kLsoapThreads;
+}
+
+template <int G>
+static auto lsoap_kernel_of(int Q, int l_max) {
     const bool vec = Q % 4 == 0;
-    return lsoap_px(l_max) == 20 ? (vec ? k_lambda_soap<true, 20> : k_lambda_soap<false, 20>)
-                                 : (vec ? k_lambda_soap<true, 36> : k_lambda_soap<false, 36>);
+    return lsoap_px(l_max) == 20 ? (vec ? k_lambda_soap<true, 20, G> : k_lambda_soap<false, 20, G>)
+                                 : (vec ? k_lambda_soap<true, 36, G> : k_lambda_soap<false, 36, G>);
+}
+static auto lsoap_kernel(int Q, int l_max, int lam) {
+    return lsoap_small(Q, lam) ? lsoap_kernel_of<1>(Q, l_max) : lsoap_kernel_of<2>(Q, l_max);
 }
 
 int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const float4** R) {
@@ -302,7 +315,7 @@ int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const 
         LsoapTable* t = new LsoapTable();
         t->lambda = lam;
         t->n_pairs = (int)P.size();
-        cudaError_t e = cudaFuncSetAttribute(lsoap_kernel(ctx->Q, ctx->l_max), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(lsoap_kernel(ctx->Q, ctx->l_max, lam), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              227 * 1024);
         if (e == cudaSuccess) e = cudaMalloc(&t->d_hdr, sizeof(int4) * std::max<size_t>(1, h.size()));
         if (e == cudaSuccess) e = cudaMalloc(&t->d_R, sizeof(float4) * std::max<size_t>(1, all.size()));
@@ -385,7 +398,7 @@ extern "C" int rascal_lambda_soap(rascal_ctx* ctx, int64_t n_centres, const floa
     int chunk = std::min((2 * lambda + 1) * QT, kLsoapGroups);
     while (chunk > 6 && sizeof(float) * (c_floats + (size_t)2 * 4 * chunk * px) > 227 * 1024) --chunk;
     const size_t smem = sizeof(float) * (c_floats + (size_t)2 * 4 * chunk * px);
-    lsoap_kernel(ctx->Q, ctx->l_max)<<<(unsigned)n_centres, kLsoapThreads, smem, ctx->stream>>>(
+    lsoap_kernel(ctx->Q, ctx->l_max, lambda)<<<(unsigned)n_centres, kLsoapThreads, smem, ctx->stream>>>(
         d_coeffs, ctx->Q, ctx->l_max, lambda, chunk, (unsigned)((0x100000000ull + QT - 1) / QT), np, hdr, R, d_out);
     RASCAL_LAUNCH_CHECK("k_lambda_soap");
     return RASCAL_OK;
