@@ -390,9 +390,9 @@ __device__ __forceinline__ void warp_energy(float dot, float* s_e) {
     for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = dot;
 }
-__device__ __forceinline__ void add_energy(const float* s_e, double* energy) {
+__device__ __forceinline__ void add_energy(const float* s_e, int nwarps, double* energy) {
     double e = 0.0;
-    for (int w = 0; w < kGradThreads / 32; ++w) e += (double)s_e[w];
+    for (int w = 0; w < nwarps; ++w) e += (double)s_e[w];
     atomicAdd(energy, 0.5 * e);
 }
 
@@ -410,11 +410,12 @@ __device__ __forceinline__ void add_energy(const float* s_e, double* energy) {
 // 1 390 us on 32 768 centres with 90 pairs (n_max 10, l_max 8, 3 species), the contraction takes 500, the radial values 420
 // (4.2 GB from L2) and the adjoint 180. With a warp per pair, lanes over lm and Y in shared memory (two loads per two
 // products) the kernel took 2 328 us; with a warp per m, up in l, radial values loaded for every m, 1 422; with half of n_max
-// 10 per task 1 526; with three CTAs per SM 1 510. 4 096 centres with 34 pairs (8, 6, 2): 81 -> 63 us.
-template <int SHAPE, int W>
-__global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradients(const GradArgs A) {
+// 10 per task 1 526; with three CTAs per SM 1 510. 4 096 centres with 34 pairs (8, 6, 2): 81 -> 63 us, with CTAs of 128
+// threads (below) 45.
+template <int SHAPE, int W, int T>
+__global__ void __launch_bounds__(T, (W == kLinear ? 4 : 3) * 256 / T) k_gradients(const GradArgs A) {
     const GradShape<SHAPE> K(A);
-    constexpr int chunk = 32, nwarps = kGradThreads / 32;
+    constexpr int chunk = 32, nwarps = T / 32;
     const int L1 = K.Lmax + 1, n2 = (K.Nmax + 1) & ~1;             // n in pairs
     const int Hl = 2 * n2, Hs = grad_h_pitch(K.Lmax, K.Nmax);      // floats of an (l, m) and of a species in H
     const int NP = n2 / 2;                                         // pairs of n
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     const int lab_i = A.species[i];
     const int a_i = (lab_i >= 0 && lab_i < 256) ? A.lut[lab_i] : -1;
     // what the adjoint leaves out (m = 0 has no partner, an odd n_max a last n) reads as zero; its first barrier follows
-    for (int e = tid; e < A.S * Hs / 4; e += kGradThreads) reinterpret_cast<float4*>(s_H)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int e = tid; e < A.S * Hs / 4; e += T) reinterpret_cast<float4*>(s_H)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     float* s_W = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sm) + A.w_off);
     const float dot = adjoint<SHAPE, W>(A, K, i, a_i, s_C, s_W, [&](int q, int l, int s, float v) {
         const int a = q / K.Nmax, n = q - a * K.Nmax, m = s - l;
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
             gd[K.Fpad + f] = dg;
         };
         if (pos == 0 && K.Npad != K.Nmax)  // the padding slots are read as zero and written only here
-            for (int e = tid; e < chunk * L1 * (K.Npad - K.Nmax); e += kGradThreads) {
+            for (int e = tid; e < chunk * L1 * (K.Npad - K.Nmax); e += T) {
                 const int q = K.Npad - K.Nmax, n = e % q, l = e / q % L1;
                 put(s_G + e / q / L1 * Gp, l * K.Npad + K.Nmax + n, 0.0f, 0.0f);
             }
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(kGradThreads, W == kLinear ? 4 : 3) k_gradient
     if (last && seg_len > 0) finish((seg_len - 1) / chunk * chunk, b ^ 1);
     // F_i and the virial from the last warp's lanes
     if (!last) return;
-    if (W == kLinear && A.energy && lane == 0) add_energy(s_e, &A.energy[s_sid]);
+    if (W == kLinear && A.energy && lane == 0) add_energy(s_e, nwarps, &A.energy[s_sid]);
     float t = 0.0f;  // of component `lane`
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
@@ -885,7 +886,7 @@ static __global__ void __launch_bounds__(kGradThreads, 5) k_gradients_wide(const
             atomicAdd(&A.virial[9 * (int64_t)s_sid + (tid - 3)], s);
         }
     } else if (tid == 32 && A.energy) {
-        add_energy(s_e, &A.energy[s_sid]);
+        add_energy(s_e, nwarps, &A.energy[s_sid]);
     }
 }
 
@@ -914,33 +915,37 @@ static size_t grad_smem(const rascal_ctx* ctx, int chunk, bool tiled) {
 
 // bytes of k_gradients' shared memory before the area that the coefficients (with the dense weight block of a per-centre
 // dE/dp behind them) and then the radial values use, and in all
-static size_t grad_c_off(const rascal_ctx* ctx) {
-    return sizeof(float) * ctx->n_species * grad_h_pitch(ctx->l_max, ctx->n_max) + 32 * (2 * 16 + kGradThreads / 32 * 16 + 2 * 16);
+static size_t grad_c_off(const rascal_ctx* ctx, int threads) {
+    return sizeof(float) * ctx->n_species * grad_h_pitch(ctx->l_max, ctx->n_max) + 32 * (2 * 16 + threads / 32 * 16 + 2 * 16);
 }
 static size_t grad_c_bytes(const rascal_ctx* ctx, bool tiled) {
     return align_up(sizeof(float) * ctx->Q * (tiled ? ctx->plan.Lp : ctx->n_lm), 16);
 }
 static size_t grad_w_bytes(const rascal_ctx* ctx, int w_lg) { return sizeof(float) * w_lg * ((ctx->Q * (ctx->Q + 1) / 2) | 1); }
-static size_t grad_chain_smem(const rascal_ctx* ctx, bool tiled, int w_lg) {
+static size_t grad_chain_smem(const rascal_ctx* ctx, int threads, bool tiled, int w_lg) {
     const size_t c = grad_c_bytes(ctx, tiled) + grad_w_bytes(ctx, w_lg);
-    return grad_c_off(ctx) + std::max(c, sizeof(float) * 32 * grad_g_pitch(ctx->plan.F_pad));
+    return grad_c_off(ctx, threads) + std::max(c, sizeof(float) * 32 * grad_g_pitch(ctx->plan.F_pad));
 }
 
 using GradKernel = void (*)(GradArgs);
-static const GradKernel kGradLinear[] = {k_gradients<0, kLinear>, k_gradients<1, kLinear>, k_gradients<2, kLinear>,
-                                         k_gradients<3, kLinear>, k_gradients<4, kLinear>};
-static const GradKernel kGradPerCentre[] = {k_gradients<0, kPerCentre>, k_gradients<1, kPerCentre>, k_gradients<2, kPerCentre>,
-                                            k_gradients<3, kPerCentre>, k_gradients<4, kPerCentre>};
+// by threads (256, 128), kind of weights and shape; no shape that is not listed for 128 threads is small enough for them
+static const GradKernel kGradKernels[2][2][5] = {
+    {{k_gradients<0, kLinear, 256>, k_gradients<1, kLinear, 256>, k_gradients<2, kLinear, 256>, k_gradients<3, kLinear, 256>,
+      k_gradients<4, kLinear, 256>},
+     {k_gradients<0, kPerCentre, 256>, k_gradients<1, kPerCentre, 256>, k_gradients<2, kPerCentre, 256>,
+      k_gradients<3, kPerCentre, 256>, k_gradients<4, kPerCentre, 256>}},
+    {{k_gradients<0, kLinear, 128>, nullptr, nullptr, k_gradients<3, kLinear, 128>, nullptr},
+     {k_gradients<0, kPerCentre, 128>, nullptr, nullptr, k_gradients<3, kPerCentre, 128>, nullptr}}};
 static_assert(kNumExpShapes == 5, "an instance per shape");
 
 int gradients_setup(rascal_ctx* ctx) {
     RASCAL_CUDA(upload_ylm_constants(ctx->stream));
     RASCAL_CUDA(upload_ylm_down(ctx->stream));
     RASCAL_CUDA(cudaFuncSetAttribute(k_gradients_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    for (int k = 0; k < kNumExpShapes; ++k) {
-        RASCAL_CUDA(cudaFuncSetAttribute(kGradLinear[k], cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-        RASCAL_CUDA(cudaFuncSetAttribute(kGradPerCentre[k], cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    }
+    for (int t = 0; t < 2; ++t)
+        for (int w = 0; w < 2; ++w)
+            for (GradKernel k : kGradKernels[t][w])
+                if (k) RASCAL_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     return RASCAL_OK;
 }
 
@@ -1030,21 +1035,26 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     A.Qw = Qw;
     A.Lp_adj = P.Lp;
     A.n_adj_tasks = (ctx->Q + 3) / 4 * (P.Lp / 4);
-    size_t smem = 0;
+    // Small bases take CTAs of 128 threads, of which eight (six with dE/dp) fit an SM: their few l leave half of eight warps
+    // without a task, and more CTAs hide each other's barriers: 16 000 centres of 31 pairs (8, 6, 2) 205 -> 155 us, of 25 pairs (7, 5,
+    // 2) 293 -> 228, of 29 pairs (5, 3, 1) 227 -> 152; with dE/dp 25 262 centres (5, 4, 2) 519 -> 350.
+    const int per_sm = d_weights ? 8 : 6;
+    const bool small = grad_chain_smem(ctx, 128, true, d_weights ? 0 : L1) <= 226 * 1024 / per_sm - 2 * 1024;
+    const int threads = small ? 128 : 256;
     // a per-centre dE/dp: all its l blocks staged at once where two CTAs per SM still fit, else as many as fit
     A.w_lg = d_weights ? 0 : L1;
-    while (A.w_lg > 1 && grad_chain_smem(ctx, true, A.w_lg) > 112 * 1024) --A.w_lg;
-    if (A.w_lg && grad_chain_smem(ctx, true, A.w_lg) > 220 * 1024) A.w_lg = 0;
-    smem = grad_chain_smem(ctx, A.wsym || A.w_lg, A.w_lg);
+    while (A.w_lg > 1 && grad_chain_smem(ctx, threads, true, A.w_lg) > 112 * 1024) --A.w_lg;
+    if (A.w_lg && grad_chain_smem(ctx, threads, true, A.w_lg) > 220 * 1024) A.w_lg = 0;
+    size_t smem = grad_chain_smem(ctx, threads, A.wsym || A.w_lg, A.w_lg);
     const bool chains = smem <= 220 * 1024;  // all but the widest bases (about n_species n_max (l_max + 1)^2 > 24 500)
     {  // rows of a warp: the fewest rounds x (loads of a step)
-        const int w = kGradThreads / 32;
+        const int w = threads / 32;
         auto cost = [&](int r) { return (ctx->Q + r * w - 1) / (r * w) * (r + 4); };
         A.w_rows = cost(6) < cost(4) ? 6 : 4;
     }
     if (chains) {
         A.chunk = 32;
-        A.w_off = (int)(grad_c_off(ctx) + grad_c_bytes(ctx, true));
+        A.w_off = (int)(grad_c_off(ctx, threads) + grad_c_bytes(ctx, true));
         A.aux_off = 0;
     } else {
         // the largest chunk (<= 32: one warp stages a chunk, a pair per lane) that keeps five CTAs per SM (48 registers)
@@ -1078,10 +1088,13 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
             ctx->n_lm == (c.l_max + 1) * (c.l_max + 1) && ctx->F == (c.l_max + 1) * c.n_max && (!A.wsym || A.Qw == (ctx->Q + 3) / 4 * 4))
             shape = k;
     }
-    if (chains)
-        (d_weights ? kGradLinear : kGradPerCentre)[shape]<<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A);
-    else
+    if (chains) {
+        GradKernel kernel = kGradKernels[small][d_weights ? 0 : 1][shape];
+        if (!kernel) kernel = kGradKernels[small][d_weights ? 0 : 1][0];
+        kernel<<<sys->n_atoms, threads, smem, ctx->stream>>>(A);
+    } else {
         k_gradients_wide<<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A);
+    }
     RASCAL_LAUNCH_CHECK("k_gradients");
     k_forces_f64<<<(unsigned)std::min<int64_t>((n3 + 255) / 256, 8192), 256, 0, ctx->stream>>>(n3, f32, d_forces);
     RASCAL_LAUNCH_CHECK("k_forces_f64");
