@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
 // Bound: reading p and writing dE/dp (0.84 GB, 126 us on the model above) behind a main loop of 8 k-blocks per tile, overlapped
 // only between the two CTAs of an SM: 256 us. It took 353 with a lane to a row (16-byte pieces of 32 rows per instruction) and
 // six 64-row loads per k-block issued by the MMAs' thread; 333 with eight lanes to a row, 272 with 128-byte rows and the
-// features requested early. Tiles of 128 features, three CTAs per SM: 391 us (the W tile is read twice as often).
+// features requested early. Rows that are not 16-byte aligned (25 262 centres, 275 features): 189 -> 94 us with 32 lanes to a
+// row. Tiles of 128 features, three CTAs per SM: 391 us (the W tile is read twice as often).
 __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_constant__ GprArgs A) {
     constexpr int kKB = 32, kGprATile = 128 * 128;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -444,7 +445,7 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
             s_inv[tid] = atom >= 0 && nk > 0 ? A.inv[atom] : 0.0f;
             s_c2[tid] = atom >= 0 && nk > 0 ? A.c2[atom] : 0.0f;
         }
-        const int q = warp & 3, h = warp >> 2, row = 32 * q + lane, rr = lane >> 3, cl = 4 * (lane & 7);
+        const int q = warp & 3, h = warp >> 2, rr = lane >> 3, cl = 4 * (lane & 7);
         const int c_end = min(ncols, kGprFT / 2 * (h + 1));
         // the features of 32 columns of this warp's rows, eight lanes to a row
         auto fetch = [&](int c, float4 (&pv)[8]) {
@@ -513,10 +514,9 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
             __syncthreads();
         }
         // epilogue: dE/dp = inv * G - c2 * p for this warp's rows and half of the columns
-        if (warp >= kGprThreads / 32) {
-        } else if (A.vec16) {
+        if (warp < kGprThreads / 32) {
             // 32 columns at a time through shared memory (the stages are free: every load has landed and every MMA is done),
-            // so that eight lanes read and write 128 contiguous bytes of a row
+            // so that eight lanes read and write 128 contiguous bytes of a row, or 32 lanes where rows are not 16-byte aligned
             float* buf = reinterpret_cast<float*>(sA) + warp * 32 * 36;  // pitch 36: both directions conflict-free
             for (int c = kGprFT / 2 * h; c < c_end; c += 32) {
                 const int64_t f = f0 + c + cl;
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
                 float4 pv[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) pv[u] = pn[u];
-                if (c + 32 < c_end) fetch(c + 32, pn);
+                if (A.vec16 && c + 32 < c_end) fetch(c + 32, pn);
 #pragma unroll
                 for (int w = 0; w < 32; w += 16) {
                     if (c + w >= c_end) break;
@@ -540,38 +540,29 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
                         *reinterpret_cast<float4*>(buf + lane * 36 + w + u) = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
                 }
                 __syncwarp();
+                if (A.vec16) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int r = 32 * q + 4 * u + rr, atom = s_atom[r];
-                    if (!in || atom < 0) continue;
-                    const float iv = s_inv[r], cc = s_c2[r];
-                    const float4 v = *reinterpret_cast<const float4*>(buf + (4 * u + rr) * 36 + cl);
-                    __stcs(reinterpret_cast<float4*>(A.grad + (int64_t)atom * A.F + f),
-                           make_float4(fmaf(iv, v.x, -cc * pv[u].x), fmaf(iv, v.y, -cc * pv[u].y),
-                                       fmaf(iv, v.z, -cc * pv[u].z), fmaf(iv, v.w, -cc * pv[u].w)));
+                    for (int u = 0; u < 8; ++u) {
+                        const int r = 32 * q + 4 * u + rr, atom = s_atom[r];
+                        if (!in || atom < 0) continue;
+                        const float iv = s_inv[r], cc = s_c2[r];
+                        const float4 v = *reinterpret_cast<const float4*>(buf + (4 * u + rr) * 36 + cl);
+                        __stcs(reinterpret_cast<float4*>(A.grad + (int64_t)atom * A.F + f),
+                               make_float4(fmaf(iv, v.x, -cc * pv[u].x), fmaf(iv, v.y, -cc * pv[u].y),
+                                           fmaf(iv, v.z, -cc * pv[u].z), fmaf(iv, v.w, -cc * pv[u].w)));
+                    }
+                } else if (c + lane < c_end && f0 + c + lane < A.F) {
+#pragma unroll 8
+                    for (int u = 0; u < 32; ++u) {
+                        const int r = 32 * q + u, atom = s_atom[r];
+                        if (atom < 0) continue;
+                        const int64_t o = (int64_t)atom * A.F + f0 + c + lane;
+                        A.grad[o] = fmaf(s_inv[r], buf[u * 36 + lane], -s_c2[r] * __ldg(A.p + o));
+                    }
                 }
                 __syncwarp();
             }
             fence_proxy_async_smem();  // the next tile's loads come by TMA
-        } else {
-            const int atom = s_atom[row];
-            const float iv = s_inv[row], cc = s_c2[row];
-            for (int c = kGprFT / 2 * h; c < c_end; c += 16) {
-                float v[16];
-                if (nk > 0) {
-                    tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
-                } else {
-#pragma unroll
-                    for (int u = 0; u < 16; ++u) v[u] = 0.0f;
-                }
-                if (atom < 0) continue;
-                const int64_t f = f0 + c;
-                const float* prow = A.p + (int64_t)atom * A.F + f;
-                float* grow = A.grad + (int64_t)atom * A.F + f;
-#pragma unroll
-                for (int u = 0; u < 16; ++u)
-                    if (f + u < A.F) grow[u] = fmaf(iv, v[u], -cc * prow[u]);
-            }
         }
         tc_fence_before();
         __syncthreads();
@@ -645,7 +636,8 @@ __global__ void k_gpr_scatter(int N, int S, const int* __restrict__ species, con
     }
 }
 
-// per structure: E_i over the passes, zeta E_i / |p_i|^2, and the FP64 structure sum
+// per structure: E_i over the passes, zeta E_i / |p_i|^2, and the FP64 structure sum; gridDim.y CTAs share a structure (one CTA
+// took 96 us on a single structure of 25 262 atoms)
 __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict__ struct_off,
                              const int* __restrict__ species, const int* __restrict__ lut, const int* __restrict__ npass,
                              const float* __restrict__ e_part, const float* __restrict__ inv, int zeta, int normalize,
@@ -654,7 +646,7 @@ __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict
     const int st = blockIdx.x;
     const int i0 = struct_off[st], i1 = struct_off[st + 1];
     double acc = 0.0;
-    for (int i = i0 + (int)threadIdx.x; i < i1; i += blockDim.x) {
+    for (int i = i0 + (int)(blockIdx.y * blockDim.x + threadIdx.x); i < i1; i += gridDim.y * blockDim.x) {
         const int lab = species[i];
         const int a = (lab >= 0 && lab < 256) ? lut[lab] : -1;
         const int np = a >= 0 ? npass[a] : 0;
@@ -670,7 +662,12 @@ __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict
     if (threadIdx.x < 32) {
         double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0 && energy) energy[st] = v;
+        if (threadIdx.x == 0 && energy) {
+            if (gridDim.y == 1)
+                energy[st] = v;
+            else
+                atomicAdd(&energy[st], v);  // cleared before
+        }
     }
     (void)S;
     (void)passes_max;
@@ -918,7 +915,8 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
         gpr_kernel(A.vec16, cols)<<<ctx->n_sm, kGprThreads1, gpr_smem1(cols), ctx->stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_gpr_kernel");
     }
-    k_gpr_finish<<<sys->n_structures, 256, 0, ctx->stream>>>(N, S, P, sys->d_struct_offsets, sys->d_species, ctx->d_lut,
+    const dim3 finish((unsigned)sys->n_structures, (unsigned)std::max(1, std::min(64, N / sys->n_structures / 512)));
+    k_gpr_finish<<<finish, 256, 0, ctx->stream>>>(N, S, P, sys->d_struct_offsets, sys->d_species, ctx->d_lut,
                                                              npass, e_part, inv, m->zeta, m->normalize, atomic,
                                                              grad ? c2 : nullptr,
                                                              d_energy);
