@@ -54,8 +54,8 @@ extern "C" {
 
 /* power-spectrum arithmetic */
 #define RASCAL_PS_FP32 0   /* FP32 inputs and accumulation (CUDA cores) */
-#define RASCAL_PS_BF16 1   /* BF16 inputs, FP32 accumulation (tcgen05 tensor cores) */
-#define RASCAL_PS_TF32X3 2 /* FP32 inputs split into TF32 hi + lo, three tcgen05 MMAs, FP32 accumulation:
+#define RASCAL_PS_BF16 1   /* BF16 inputs, FP32 accumulation (tensor cores) */
+#define RASCAL_PS_TF32X3 2 /* FP32 inputs split into TF32 hi + lo, three tensor-core MMAs, FP32 accumulation:
                               about 2^-21 relative per product, FP32-grade results on tensor cores */
 
 /* radial basis */
@@ -133,7 +133,8 @@ int rascal_info(const rascal_ctx* ctx, rascal_info_t* out);
  * label, degenerate geometry, ...) into a status. */
 int rascal_sync(rascal_ctx* ctx);
 
-/* Test hook for the failure path of the fused tensor-core Gram (no counterpart in the paper). With polls > 0, the
+/* Test hook for the failure path of the tcgen05 forms of the Gram (no counterpart in the paper). With polls > 0,
+ * rascal_soap (precision BF16 or TF32X3) and the tensor-core precisions of rascal_power_spectrum run those forms, and the
  * first MMA-completion wait of every CTA of rascal_soap (precision BF16 or TF32X3) and of the tensor-core forms of
  * rascal_power_spectrum is made on an mbarrier that nothing arrives at, and gives up after `polls` polls (about
  * 20 ns apart). The kernel then raises the timeout flag, skips the remaining epilogues, waits (with the built-in
@@ -213,9 +214,10 @@ int rascal_debug_pair_gradients(rascal_ctx* ctx, int64_t n_pairs, const float* d
 int rascal_power_spectrum(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout,
                           float* d_ps);
 
-/* Expansion and power spectrum in one kernel: each centre's c is written to d_coeffs and kept in shared memory,
- * where its Gram is formed (precision as in rascal_power_spectrum; RASCAL_PS_FP32 uses the CUDA cores, the
- * others tcgen05), so c is never read back from global memory. */
+/* Expansion and power spectrum in one call, precision as in rascal_power_spectrum. RASCAL_PS_FP32 is one kernel on the
+ * CUDA cores: each centre's c is written to d_coeffs and kept in shared memory, where its Gram is formed, so that it is
+ * never read back from global memory. The tensor-core precisions run the coefficients and then the kernel of
+ * rascal_power_spectrum on them, which is faster than their one-kernel forms. */
 int rascal_soap(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets, const int* d_nbr_j,
                 const float* d_rij, int precision, int layout, float* d_coeffs, float* d_ps);
 

@@ -196,7 +196,7 @@ class SoapCalculator:
         return p
 
     def soap(self, system: DeviceSystem, pairs: PairList, layout="packed", precision="fp32", coeffs=None, ps=None):
-        """Expansion and power spectrum in one fused kernel launch."""
+        """Expansion and power spectrum in one call (FP32: one fused kernel; BF16, TF32x3: two)."""
         import torch
 
         self._bind_stream()

@@ -16,7 +16,8 @@
 // memory and, when the power spectrum is fused, also into shared memory, where the Gram runs without c ever being
 // read back from HBM:
 //   kGramSimt    FP32 register-tiled Gram on the CUDA cores from CT[lm][q] (ps_fp32.cuh);
-//   kGramBf16    tcgen05 MMA, BF16 operands, FP32 accumulators in TMEM (tcgen05.cuh);
+//   kGramBf16    tcgen05 MMA, BF16 operands, FP32 accumulators in TMEM (tcgen05.cuh); this form and the next serve what the
+//                spectrum kernel of stored coefficients, which is faster, does not take, and the wait-timeout hook;
 //   kGramTf32x3  tcgen05 MMA, TF32 hi/lo split, three MMAs per K step (FP32-grade).
 // The Gram output is staged per group of l values in the (then free) pair-staging buffers and written to global
 // memory by bulk copies.
@@ -822,16 +823,12 @@ int expansion_setup(rascal_ctx* ctx) {
     RASCAL_CUDA(cudaMemcpyAsync(ctx->d_fmap, fmap.data(), sizeof(int) * fmap.size(), cudaMemcpyHostToDevice, ctx->stream));
     RASCAL_CUDA(upload_ylm_constants(ctx->stream));
     int st;
-    if ((st = set_attr<kGramNone>()) || (st = set_attr<kGramSimt>()) || (st = set_attr<kGramSel>()) ||
-        (st = set_attr<kGramBf16>()) ||
-        (st = set_attr<kGramTf32x3>()) || (st = set_attr<kGramRTf32>()) || (st = set_attr<kGramRBf16>()) ||
+    if ((st = set_attr<kGramNone>()) || (st = set_attr<kGramNone, 1>()) || (st = set_attr<kGramNone, 2>()) ||
+        (st = set_attr<kGramNone, 3>()) || (st = set_attr<kGramNone, 4>()) || (st = set_attr<kGramSimt>()) ||
         (st = set_attr<kGramSimt, 1>()) || (st = set_attr<kGramSimt, 2>()) || (st = set_attr<kGramSimt, 3>()) ||
-        (st = set_attr<kGramNone, 1>()) || (st = set_attr<kGramNone, 2>()) || (st = set_attr<kGramNone, 3>()) ||
-        (st = set_attr<kGramBf16, 1>()) || (st = set_attr<kGramBf16, 2>()) || (st = set_attr<kGramBf16, 3>()) ||
-        (st = set_attr<kGramRTf32, 1>()) || (st = set_attr<kGramRTf32, 2>()) || (st = set_attr<kGramRTf32, 3>()) ||
-        (st = set_attr<kGramSel, 1>()) || (st = set_attr<kGramSel, 2>()) || (st = set_attr<kGramSel, 3>()) ||
-        (st = set_attr<kGramSimt, 4>()) || (st = set_attr<kGramNone, 4>()) || (st = set_attr<kGramBf16, 4>()) ||
-        (st = set_attr<kGramRTf32, 4>()) || (st = set_attr<kGramSel, 4>()))
+        (st = set_attr<kGramSimt, 4>()) || (st = set_attr<kGramSel>()) || (st = set_attr<kGramSel, 1>()) ||
+        (st = set_attr<kGramSel, 2>()) || (st = set_attr<kGramSel, 3>()) || (st = set_attr<kGramSel, 4>()) ||
+        (st = set_attr<kGramBf16>()) || (st = set_attr<kGramTf32x3>()) || (st = set_attr<kGramRTf32>()))
         return st;
     RASCAL_CUDA(cudaStreamSynchronize(ctx->stream));
     return RASCAL_OK;
@@ -1215,8 +1212,8 @@ extern "C" int rascal_soap(rascal_ctx* ctx, const rascal_system* sys, const int6
         if (st != RASCAL_E_UNSUPPORTED) return st;
         clear_error();
     }
-    if (!st_r) return launch_shaped<kGramRTf32>(ctx, R, sys->n_atoms, threads_r, smem_r);
+    if (!st_r) return launch_expansion<kGramRTf32>(ctx, R, sys->n_atoms, threads_r, smem_r);
     if (mode == kGramSimt) return launch_shaped<kGramSimt>(ctx, A, sys->n_atoms, threads, smem);
-    if (mode == kGramBf16) return launch_shaped<kGramBf16>(ctx, A, sys->n_atoms, threads, smem);
+    if (mode == kGramBf16) return launch_expansion<kGramBf16>(ctx, A, sys->n_atoms, threads, smem);
     return launch_expansion<kGramTf32x3>(ctx, A, sys->n_atoms, threads, smem);
 }
