@@ -973,7 +973,9 @@ extern "C" int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* s
     int64_t P;
     int maxc;
     bool filled;
-    if ((st = nbr_search<kNoallocCap>(ctx, sys, nbr_carve(base, N, n_s), capacity, d_offsets, d_nbr_j, d_shift, d_rij, A, &grid,
+    // the fill is launched only once the call is known to succeed: its scratch is shared by all contexts of the device, and a
+    // refused call leaves nothing queued that reads it
+    if ((st = nbr_search<kNoallocCap>(ctx, sys, nbr_carve(base, N, n_s), capacity, d_offsets, nullptr, nullptr, nullptr, A, &grid,
                                       &P, &maxc, &filled)))
         return st;
     *n_pairs = P;
@@ -984,5 +986,10 @@ extern "C" int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* s
     if (P > capacity) return set_error(RASCAL_E_CAPACITY, "pair capacity %lld < required %lld", (long long)capacity, (long long)P);
     if (P == 0) return RASCAL_OK;
     if (!d_nbr_j || !d_shift || !d_rij) return set_error(RASCAL_E_ARG, "NULL pair output arrays");
-    return RASCAL_OK;  // filled: every other case has returned
+    A.out_j = d_nbr_j;
+    A.out_shift = d_shift;
+    A.out_rij = reinterpret_cast<float4*>(d_rij);
+    k_pairs<true, kNoallocCap><<<grid, kPairWarps * 32, 0, ctx->stream>>>(A);
+    RASCAL_LAUNCH_CHECK("k_pairs<fill>");
+    return RASCAL_OK;
 }
