@@ -147,6 +147,7 @@ struct rascal_ctx {
     rascal::Arena scratch_sel;  // decoded feature selection of rascal_soap_selected
     int64_t* h_pinned;      // pinned host words for small read-backs
     cudaEvent_t counted;    // recorded once a neighbour search has written them
+    int searches;           // neighbour searches so far: a queued fill pass runs for its own search only
 
     rascal::ExpPlan plan;
     int* d_tasks;   // [T_s] packed (l, n-tile, m-tile) of the accumulation tasks

@@ -352,8 +352,8 @@ struct PairArgs {
     const int4* atom_wrap;
     const float4* atom_lo;
     const int4* items;
-    int* words;              // [0] number of work items, [1] largest count of a centre, [3] whether the fill may run
-    bool ask;                // fill: launched before the host has seen the counts, runs only where words[3] says so
+    int* words;              // [0] number of work items, [1] largest count of a centre, [3] the search whose fill may run
+    int search;              // fill launched before the host has seen the counts: runs only where words[3] names it; else 0
     double rc2;
     int* counts;             // count: pairs per centre
     const int64_t* offsets;  // fill
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) :
     __shared__ float4 s_vec[FILL ? kPairWarps * CAP : 1];
     __shared__ unsigned short s_rec[FILL ? kPairWarps * kPairRec : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (FILL && A.ask && !A.words[3]) return;
+    if (FILL && A.search && A.words[3] != A.search) return;
     const int n_work = min(A.words[0], A.n_atoms);
     unsigned local_flags = 0;
     int local_max = 0;
@@ -693,16 +693,16 @@ __global__ void __launch_bounds__(kPairWarps * 32, CAP <= 128 ? (FILL ? 6 : 8) :
 // and the error flags to the host's pinned words. Three launches (scan.cu) and k_report serve larger systems.
 constexpr int kOffsetsThreads = 1024;
 constexpr int kOffsetsMax = 131072;
-// h_words: pairs, largest count of a centre. words[3]: whether a fill pass with these limits fits the search.
+// h_words: pairs, largest count of a centre. words[3]: the search's number if a fill pass with these limits fits it.
 struct Report {
     int* words;
     const unsigned* flags;
     int64_t* h_words;
     unsigned* h_flags;
     int64_t capacity;
-    int largest;
+    int largest, search;
     __device__ void operator()(int64_t total) const {
-        words[3] = *flags == 0 && total <= capacity && words[1] <= largest;
+        words[3] = *flags == 0 && total <= capacity && words[1] <= largest ? search : 0;
         h_words[0] = total;
         h_words[1] = words[1];
         *h_flags = *flags;
@@ -820,7 +820,8 @@ static int nbr_search(rascal_ctx* ctx, const rascal_system* sys, const NbrScratc
     A.out_j = d_nbr_j;
     A.out_shift = d_shift;
     A.out_rij = reinterpret_cast<float4*>(d_rij);
-    const Report report = {W.words, ctx->d_flags, ctx->h_pinned, ctx->h_flags, capacity, CAP};
+    ctx->searches = ctx->searches % 0x7fffffff + 1;
+    const Report report = {W.words, ctx->d_flags, ctx->h_pinned, ctx->h_flags, capacity, CAP, ctx->searches};
     *grid = (unsigned)std::min<int64_t>(N, 8LL * ctx->n_sm);
     k_pairs<false, CAP><<<*grid, kPairWarps * 32, 0, stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_pairs<count>");
@@ -836,10 +837,10 @@ static int nbr_search(rascal_ctx* ctx, const rascal_system* sys, const NbrScratc
     RASCAL_CUDA(cudaEventRecord(ctx->counted, stream));
     const bool outputs = d_nbr_j && d_shift && d_rij;
     if (outputs) {
-        A.ask = true;
+        A.search = ctx->searches;
         k_pairs<true, CAP><<<*grid, kPairWarps * 32, 0, stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_pairs<fill>");
-        A.ask = false;
+        A.search = 0;
     }
     RASCAL_CUDA(cudaEventSynchronize(ctx->counted));
     const int st = flags_status(ctx, *ctx->h_flags);
