@@ -223,9 +223,7 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
                     lim[j] = atom >= 0 ? A.F : 0;
                 }
                 for (int kb = 0; kb < nk; ++kb, ring.next()) {
-                    bool free = true;
-                    if (ring.used && lane == 0) free = mbar_wait_spin(&empty[ring.stage], ring.phase ^ 1u);
-                    if (!__shfl_sync(0xffffffffu, free, 0)) {
+                    if (!mbar_wait_warp(ring.used, &empty[ring.stage], ring.phase ^ 1u)) {
                         ok = false;
                         break;
                     }
@@ -253,9 +251,7 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
             } else {
                 float nrm[kRows] = {};
                 for (int kb = 0; kb < nk; ++kb, ring.next()) {
-                    bool here = true;
-                    if (lane == 0) here = mbar_wait_spin(&landed[ring.stage], ring.phase);
-                    if (!__shfl_sync(0xffffffffu, here, 0)) {
+                    if (!mbar_wait_warp(true, &landed[ring.stage], ring.phase)) {
                         ok = false;
                         break;
                     }

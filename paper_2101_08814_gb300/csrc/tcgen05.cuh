@@ -82,6 +82,17 @@ __device__ inline bool mbar_wait_spin(uint64_t* bar, uint32_t parity) {
     return mbar_wait_bounded(bar, parity);
 }
 
+// One lane waits for its whole warp (32 polling lanes take issue slots from the working warps); every lane gets the outcome.
+// The shuffle passes it on but orders no memory: the __syncwarp does, so that what the wait acquired holds for all lanes
+// before they read or refill what the barrier guards. All lanes call it; wait is false where there is nothing to wait for.
+__device__ inline bool mbar_wait_warp(bool wait, uint64_t* bar, uint32_t parity) {
+    bool ok = true;
+    if (wait && (threadIdx.x & 31) == 0) ok = mbar_wait_spin(bar, parity);
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();
+    return ok;
+}
+
 __device__ inline void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ inline void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // generic-proxy shared-memory writes -> visible to the tensor core (async proxy)
