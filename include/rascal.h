@@ -126,6 +126,9 @@ long long rascal_launch_count(void);
  * coefficients. `cuda_stream` is a cudaStream_t (NULL = legacy default stream). Synchronises the stream. */
 int rascal_create(const rascal_hypers* hypers, void* cuda_stream, rascal_ctx** out);
 void rascal_destroy(rascal_ctx* ctx);
+/* Later calls enqueue their work on `cuda_stream`. A neighbour search returns while it still writes its pair arrays: the new
+ * stream waits for that on the device (not where it is being captured). All calls of a context share its scratch: other work
+ * that is still running on the earlier stream is ordered by the caller. */
 int rascal_set_stream(rascal_ctx* ctx, void* cuda_stream);
 int rascal_info(const rascal_ctx* ctx, rascal_info_t* out);
 

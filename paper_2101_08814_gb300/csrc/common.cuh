@@ -148,6 +148,8 @@ struct rascal_ctx {
     int64_t* h_pinned;      // pinned host words for small read-backs
     cudaEvent_t counted;    // recorded once a neighbour search has written them
     int searches;           // neighbour searches so far: a queued fill pass runs for its own search only
+    cudaEvent_t searched;   // recorded behind the fill pass that a search leaves running: another stream waits for it
+    bool fill_queued;       // whether it has been recorded
 
     rascal::ExpPlan plan;
     int* d_tasks;   // [T_s] packed (l, n-tile, m-tile) of the accumulation tasks

@@ -463,6 +463,7 @@ extern "C" void rascal_destroy(rascal_ctx* ctx) {
     cudaFreeHost(ctx->h_flags);
     cudaFreeHost(ctx->h_pinned);
     if (ctx->counted) cudaEventDestroy(ctx->counted);
+    if (ctx->searched) cudaEventDestroy(ctx->searched);
     cudaFree(ctx->scratch.ptr);
     cudaFree(ctx->scratch_w.ptr);
     cudaFree(ctx->d_dvr);
@@ -535,6 +536,7 @@ static int create_impl(const rascal_hypers* h, void* stream, rascal_ctx** out) {
     RASCAL_CUDA(cudaMallocHost(&ctx->h_flags, sizeof(unsigned)));
     RASCAL_CUDA(cudaMallocHost(&ctx->h_pinned, sizeof(int64_t) * 8));
     RASCAL_CUDA(cudaEventCreateWithFlags(&ctx->counted, cudaEventDisableTiming));
+    RASCAL_CUDA(cudaEventCreateWithFlags(&ctx->searched, cudaEventDisableTiming));
     RASCAL_CUDA(cudaMemsetAsync(ctx->d_flags, 0, sizeof(unsigned), ctx->stream));
     int lut[256];
     for (int i = 0; i < 256; ++i) lut[i] = -1;
@@ -588,7 +590,17 @@ extern "C" int rascal_set_radial(rascal_ctx* ctx, int radial) {
 
 extern "C" int rascal_set_stream(rascal_ctx* ctx, void* stream) {
     if (!ctx) return set_error(RASCAL_E_ARG, "NULL context");
-    ctx->stream = static_cast<cudaStream_t>(stream);
+    const cudaStream_t next = static_cast<cudaStream_t>(stream);
+    if (next != ctx->stream && ctx->fill_queued) {
+        // A search returns while its fill pass still reads the scratch that the next call writes. The event stands for it (the
+        // earlier stream may be gone by now). A stream under capture takes no event from outside the capture.
+        cudaStreamCaptureStatus capture;
+        if (cudaStreamIsCapturing(next, &capture) != cudaSuccess)
+            cudaGetLastError();
+        else if (capture == cudaStreamCaptureStatusNone)
+            RASCAL_CUDA(cudaStreamWaitEvent(next, ctx->searched, 0));
+    }
+    ctx->stream = next;
     return RASCAL_OK;
 }
 

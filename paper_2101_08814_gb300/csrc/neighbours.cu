@@ -773,6 +773,13 @@ static NbrScratch nbr_carve(void* base, int N, int n_s) {
     return W;
 }
 
+// The fill pass outlives the call: rascal_set_stream makes another stream wait for it.
+static int fill_queued(rascal_ctx* ctx) {
+    RASCAL_CUDA(cudaEventRecord(ctx->searched, ctx->stream));
+    ctx->fill_queued = true;
+    return RASCAL_OK;
+}
+
 // Everything up to the pair count: *total pairs and *largest count of a centre, after one synchronisation. With output arrays
 // (A.out_j) the fill pass is launched before that synchronisation, which then waits for the counts alone; it writes nothing
 // unless the counts fit capacity and CAP and no flag is raised (*filled). Waiting for the counts first left the GPU idle for a
@@ -841,6 +848,7 @@ static int nbr_search(rascal_ctx* ctx, const rascal_system* sys, const NbrScratc
         k_pairs<true, CAP><<<*grid, kPairWarps * 32, 0, stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_pairs<fill>");
         A.search = 0;
+        if (const int st = fill_queued(ctx)) return st;
     }
     RASCAL_CUDA(cudaEventSynchronize(ctx->counted));
     const int st = flags_status(ctx, *ctx->h_flags);
@@ -891,7 +899,7 @@ extern "C" int rascal_neighbours(rascal_ctx* ctx, const rascal_system* sys, int6
     }
     k_pairs<true><<<grid, kPairWarps * 32, 0, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_pairs<fill>");
-    return RASCAL_OK;
+    return fill_queued(ctx);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -992,5 +1000,5 @@ extern "C" int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* s
     A.out_rij = reinterpret_cast<float4*>(d_rij);
     k_pairs<true, kNoallocCap><<<grid, kPairWarps * 32, 0, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_pairs<fill>");
-    return RASCAL_OK;
+    return fill_queued(ctx);
 }
