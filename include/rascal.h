@@ -136,13 +136,14 @@ int rascal_info(const rascal_ctx* ctx, rascal_info_t* out);
  * label, degenerate geometry, ...) into a status. */
 int rascal_sync(rascal_ctx* ctx);
 
-/* Test hook for the failure path of the tcgen05 forms of the Gram (no counterpart in the paper). With polls > 0,
+/* Test hook for the failure path of the tcgen05 kernels (no counterpart in the paper). With polls > 0,
  * rascal_soap (precision BF16 or TF32X3) and the tensor-core precisions of rascal_power_spectrum run those forms, and the
  * first MMA-completion wait of every CTA of rascal_soap (precision BF16 or TF32X3) and of the tensor-core forms of
  * rascal_power_spectrum is made on an mbarrier that nothing arrives at, and gives up after `polls` polls (about
  * 20 ns apart). The kernel then raises the timeout flag, skips the remaining epilogues, waits (with the built-in
  * bound of 2^22 polls) for every MMA it issued and frees its tensor memory; the next synchronising call returns
- * RASCAL_E_TIMEOUT. The outputs of that call are incomplete. polls = 0 switches the hook off; the context stays
+ * RASCAL_E_TIMEOUT. The outputs of that call are incomplete. The MLP inference (rascal_mlp_eval, radial mode MLP) has the
+ * same hook in the kernel that it always runs. polls = 0 switches the hook off; the context stays
  * usable throughout. Returns RASCAL_E_ARG for a NULL context. */
 int rascal_debug_wait_timeout(rascal_ctx* ctx, unsigned polls);
 

@@ -138,7 +138,7 @@ struct rascal_ctx {
     int* d_lut;         // [256] label -> species index or -1
 
     unsigned* d_flags;  // device error flags (see kFlag*)
-    unsigned stall_polls;  // test hook: > 0 makes the fused tensor-core Gram's first completion wait run out
+    unsigned stall_polls;  // test hook: > 0 makes the first completion wait of the tcgen05 kernels run out
     unsigned* h_flags;  // pinned host mirror
 
     rascal::Arena scratch;  // grown on demand, reused across calls

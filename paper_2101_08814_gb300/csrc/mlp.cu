@@ -417,6 +417,7 @@ struct MlpInferArgs {
     int F_pad;              // F rounded up to 16
     float inv_rscale;       // 1 / r_cut
     unsigned* flags;
+    uint32_t stall_polls;   // test hook: > 0 makes the first completion wait run out
 };
 
 constexpr int kMlpH = 64;
@@ -447,7 +448,7 @@ __device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
 // and sleeping waits the kernel took 341 us there, now 164; outputs bit-identical.
 __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_infer(const MlpInferArgs A) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t s_bar;
+    __shared__ uint64_t s_bar, s_dead;
     __shared__ uint32_t s_tmem;
     const int H = kMlpH, F = A.L.F;
     unsigned char* w2 = smem;                              // 64 x 64 bf16 = 8 KB
@@ -481,6 +482,7 @@ __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_infer(const MlpInferArgs
     }
     if (tid == 0) {
         mbar_init(&s_bar, 1);
+        mbar_init(&s_dead, 1);
         fence_mbar_init();
     }
     tc_fence_before();
@@ -527,10 +529,11 @@ __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_infer(const MlpInferArgs
             }
             mma_commit(&s_bar);
         }
-        bool done = mbar_wait_spin(&s_bar, phase);
+        // the test hook makes this wait, a CTA's first, on a barrier that nothing arrives at
+        bool done = A.stall_polls ? mbar_wait_bounded(&s_dead, 0u, A.stall_polls) : mbar_wait_spin(&s_bar, phase);
         ok = __syncthreads_and(done) != 0;
-        phase ^= 1u;
         if (!ok) break;
+        phase ^= 1u;
         tc_fence_after();
 #pragma unroll 1
         for (int c0 = H / 2 * half; c0 < H / 2 * (half + 1); c0 += 16) {
@@ -565,8 +568,8 @@ __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_infer(const MlpInferArgs
         }
         done = mbar_wait_spin(&s_bar, phase);
         ok = __syncthreads_and(done) != 0;
-        phase ^= 1u;
         if (!ok) break;
+        phase ^= 1u;
         tc_fence_after();
         const int64_t row0 = tile * kMlpTile + 32 * (warp & 3);  // this warp's 32 rows (pairs)
         // 32 columns at a time through the slab, values then derivatives: eight lanes store 128 bytes of a row
@@ -612,7 +615,7 @@ __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_infer(const MlpInferArgs
         __syncthreads();
     }
     if (!ok && tid == 0) atomicOr(A.flags, kFlagTimeout);
-    if (!ok) mbar_wait_bounded(&s_bar, phase);
+    if (!ok) mbar_wait_bounded(&s_bar, phase);  // the MMAs of the wait that ran out, before their TMEM is freed
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -678,6 +681,7 @@ int mlp_infer(rascal_ctx* ctx, int64_t n, const float4* rij, const float* r, flo
     A.F_pad = F_pad;
     A.inv_rscale = (float)(1.0 / ctx->r_cut);
     A.flags = ctx->d_flags;
+    A.stall_polls = ctx->stall_polls;
     const size_t smem = 8192 + (size_t)F_pad * 128 + (dout ? 4 : 2) * 16384 +
                         sizeof(float) * ((3 * kMlpH + 2 * ctx->F + 3) / 4 * 4 + kMlpThreads / 32 * 32 * 36) + 64;
     const int64_t tiles = (n + kMlpTile - 1) / kMlpTile;

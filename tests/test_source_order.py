@@ -30,3 +30,11 @@ def test_a_wait_by_one_lane_orders_memory_for_its_warp():
             found += 1
             assert nxt and nxt[0].strip() == "__syncwarp();", (name, nxt)
     assert found >= 1
+
+
+def test_a_wait_that_ran_out_is_repeated_on_its_own_phase():
+    # after a timeout the inference kernel waits once more for the MMAs it issued; on the next phase's parity that wait would
+    # return at once and tensor memory be freed under them
+    code = _code("mlp.cu")
+    waits = re.findall(r"ok = __syncthreads_and\(done\) != 0;\s*(.*?)\n\s*(.*?)\n", code)
+    assert waits == [("if (!ok) break;", "phase ^= 1u;")] * 2, waits
