@@ -142,8 +142,8 @@ int rascal_sync(rascal_ctx* ctx);
  * rascal_power_spectrum is made on an mbarrier that nothing arrives at, and gives up after `polls` polls (about
  * 20 ns apart). The kernel then raises the timeout flag, skips the remaining epilogues, waits (with the built-in
  * bound of 2^22 polls) for every MMA it issued and frees its tensor memory; the next synchronising call returns
- * RASCAL_E_TIMEOUT. The outputs of that call are incomplete. The MLP inference (rascal_mlp_eval, radial mode MLP) has the
- * same hook in the kernel that it always runs. polls = 0 switches the hook off; the context stays
+ * RASCAL_E_TIMEOUT. The outputs of that call are incomplete. The MLP inference (rascal_mlp_eval, radial mode MLP) and
+ * rascal_gpr_predict have the same hook in the kernels that they always run. polls = 0 switches the hook off; the context stays
  * usable throughout. Returns RASCAL_E_ARG for a NULL context. */
 int rascal_debug_wait_timeout(rascal_ctx* ctx, unsigned polls);
 

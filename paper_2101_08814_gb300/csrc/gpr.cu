@@ -78,6 +78,7 @@ struct GprArgs {
     const float* c2;      // [N] zeta E_i / |p_i|^2
     float* grad;          // [N][F]
     unsigned* flags;
+    uint32_t stall_polls; // test hook: > 0 makes the MMAs' first wait run out
     CUtensorMap tmM, tmM32;            // M^ rows [rows][Fk], boxes of 256 rows x 16 or 128 rows x 32 columns
     CUtensorMap tmW;                   // W [N sorted][n_pad_max]
     CUtensorMap tmMT[kMaxSpecies];     // per species M^T [Fn][n_pad]
@@ -161,13 +162,14 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
     int* s_atom = reinterpret_cast<int*>(s_E + 512);                 // [128]
     int* s_off = s_atom + 128;                                       // [S + 1]
     int* s_per = s_off + kMaxSpecies + 1;                            // [S] passes per species
-    uint64_t* bars = reinterpret_cast<uint64_t*>(s_per + kMaxSpecies + 1);  // [stages] empty, full, landed; done
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 3 * kGprStages + 1);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(s_per + kMaxSpecies + 1);  // [stages] empty, full, landed; done, dead
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 3 * kGprStages + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint64_t* empty = bars;
     uint64_t* full = bars + kGprStages;
     uint64_t* landed = bars + 2 * kGprStages;
     uint64_t* done = bars + 3 * kGprStages;
+    uint64_t* dead = done + 1;  // nothing arrives at it (test hook)
 
     for (int s = tid; s <= A.S; s += blockDim.x) s_off[s] = A.off[s];
     for (int s = tid; s < A.S; s += blockDim.x) s_per[s] = (A.n_pad[s] + COLS - 1) / COLS;
@@ -182,6 +184,7 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
             mbar_init(&landed[i], kGprProducers);
         }
         mbar_init(done, 1);
+        mbar_init(dead, 1);
         fence_mbar_init();
     }
     tc_fence_before();
@@ -285,7 +288,8 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
                 auto desc = [&](uint32_t at) { return kKB == 16 ? smem_desc_sw64(at, 512) : smem_desc_sw128(at, 1024); };
                 const uint64_t da0 = desc(a_base), db0 = desc(b_base);  // the address is the descriptor's low field, in 16 bytes
                 GprRing<kGprStages> use(g);
-                for (int kb = 0; kb < nk; ++kb, use.next()) {
+                if (A.stall_polls) ok = mbar_wait_bounded(dead, 0u, A.stall_polls);
+                for (int kb = ok ? 0 : nk; kb < nk; ++kb, use.next()) {
                     if (!mbar_wait_spin(&full[use.stage], use.phase)) {
                         ok = false;
                         break;
@@ -402,11 +406,12 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
     int* s_off = reinterpret_cast<int*>(s_c2 + 128);
     int* s_per = s_off + kMaxSpecies + 1;                              // feature chunks per species
     uint64_t* bars = reinterpret_cast<uint64_t*>(s_per + kMaxSpecies + 1);
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * kGprStages2 + 1);
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * kGprStages2 + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint64_t* empty = bars;
     uint64_t* full = bars + kGprStages2;
     uint64_t* done = bars + 2 * kGprStages2;
+    uint64_t* dead = done + 1;  // nothing arrives at it (test hook)
     const int n_fc = (int)((A.Fn + kGprFT - 1) / kGprFT);
 
     for (int s = tid; s <= A.S; s += blockDim.x) s_off[s] = A.off[s];
@@ -416,7 +421,7 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
         tmem_relinquish();
     }
     if (tid == 0) {
-        for (int i = 0; i <= 2 * kGprStages2; ++i) mbar_init(&bars[i], 1);
+        for (int i = 0; i < 2 * kGprStages2 + 2; ++i) mbar_init(&bars[i], 1);
         fence_mbar_init();
     }
     tc_fence_before();
@@ -463,7 +468,8 @@ __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_const
                     const uint64_t da0 = smem_desc_sw128(a_base, 1024), db0 = smem_desc_sw128(b_base, 1024);
                     const uint32_t id = instr_desc(2u, 128u, (uint32_t)ncols);
                     GprRing<kGprStages2> use(g);
-                    for (int kb = 0; kb < nk; ++kb, use.next()) {
+                    if (A.stall_polls) ok = mbar_wait_bounded(dead, 0u, A.stall_polls);
+                    for (int kb = ok ? 0 : nk; kb < nk; ++kb, use.next()) {
                         if (!mbar_wait_spin(&full[use.stage], use.phase)) {
                             ok = false;
                             break;
@@ -672,7 +678,7 @@ __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict
 static size_t gpr_smem1(int cols) {
     const int stages = gpr_stages(cols);
     return (size_t)stages * (128 + cols) * 4 * gpr_kb(cols) + sizeof(float) * (cols + 128 + 512) + sizeof(int) * 128 +
-           sizeof(int) * 2 * (kMaxSpecies + 1) + sizeof(uint64_t) * (3 * stages + 1) + 16;
+           sizeof(int) * 2 * (kMaxSpecies + 1) + sizeof(uint64_t) * (3 * stages + 2) + 16;
 }
 using GprKernel = void (*)(GprArgs);
 static GprKernel gpr_kernel(bool vec16, int cols) {
@@ -682,7 +688,7 @@ static GprKernel gpr_kernel(bool vec16, int cols) {
 }
 static size_t gpr_smem2() {
     return (size_t)kGprStages2 * (128 * 128 + kGprB2) + sizeof(int) * 3 * 128 + sizeof(int) * 2 * (kMaxSpecies + 1) +
-           sizeof(uint64_t) * (2 * kGprStages2 + 1) + 16;
+           sizeof(uint64_t) * (2 * kGprStages2 + 2) + 16;
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -903,6 +909,7 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
     A.c2 = c2;
     A.grad = d_grad;
     A.flags = ctx->d_flags;
+    A.stall_polls = ctx->stall_polls;
     A.tmM = m->tmM;
     A.tmM32 = m->tmM32;
     for (int s = 0; s < S; ++s) A.tmMT[s] = m->tmMT[s];
