@@ -229,6 +229,7 @@ int power_spectrum_tc(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs,
 // FP32, BF16 or TF32x3 power spectrum of given coefficients by the kernel of power_spectrum.cu; RASCAL_E_UNSUPPORTED
 // (without a message) where a centre does not fit its shared memory
 int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps);
+bool power_spectrum_fits(const rascal_ctx* ctx, int precision, int layout);  // whether that kernel takes the context's hypers
 int gradients_setup(rascal_ctx* ctx);
 // caches the device address of the no-allocation neighbour scratch for ctx->device (neighbours.cu)
 int nbr_static_prepare(rascal_ctx* ctx);

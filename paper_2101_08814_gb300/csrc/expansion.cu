@@ -1206,11 +1206,9 @@ extern "C" int rascal_soap(rascal_ctx* ctx, const rascal_system* sys, const int6
     // 7, 3) 528 -> 239 and 551 -> 256, 200 centres 24 -> 22 and 27 -> 23; TF32x3 errors 4.8e-7 -> 1.2e-7. The one-launch forms
     // wait for a chain of barriers and MMAs per l; they serve what the spectrum kernel does not take, and the test hook
     // that makes their waits run out.
-    if (mode != kGramSimt && !ctx->stall_polls) {
+    if (mode != kGramSimt && !ctx->stall_polls && power_spectrum_fits(ctx, precision, layout)) {
         if ((st = coefficients(ctx, sys, plain))) return st;
-        st = power_spectrum_warp(ctx, sys->n_atoms, d_coeffs, precision, layout, d_ps);
-        if (st != RASCAL_E_UNSUPPORTED) return st;
-        clear_error();
+        return power_spectrum_warp(ctx, sys->n_atoms, d_coeffs, precision, layout, d_ps);
     }
     if (!st_r) return launch_expansion<kGramRTf32>(ctx, R, sys->n_atoms, threads_r, smem_r);
     if (mode == kGramSimt) return launch_shaped<kGramSimt>(ctx, A, sys->n_atoms, threads, smem);

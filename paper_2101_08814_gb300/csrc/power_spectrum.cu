@@ -400,12 +400,10 @@ int power_spectrum_setup(rascal_ctx* ctx) {
     return RASCAL_OK;
 }
 
-int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps) {
+// Sizes of a launch of k_power_spectrum, without its pointers; false where a centre does not fit its shared memory
+static bool ps_plan(const rascal_ctx* ctx, int precision, int layout, PsArgs& A, size_t* smem) {
     const int Q = ctx->Q, L1 = ctx->l_max + 1;
     const bool full = layout == RASCAL_LAYOUT_FULL;
-    PsArgs A;
-    A.c = d_coeffs;
-    A.ps = d_ps;
     A.Q = Q;
     A.l_max = ctx->l_max;
     A.per_l = full ? Q * Q : Q * (Q + 1) / 2;
@@ -420,9 +418,24 @@ int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeff
     A.n_half = std::max(1, std::min(L1, (kPsStage / 2 - 3) / A.per_l));
     A.half = (A.n_half * A.per_l + 3 + 3) / 4 * 4;
     const int rows = std::max((Q + 15) / 16 * 16, (Q + 7) / 8 * 8);
-    A.copy16 = A.pitch == ctx->n_lm && Q * ctx->n_lm % 4 == 0 && (reinterpret_cast<uintptr_t>(d_coeffs) & 15) == 0;
-    const size_t smem = sizeof(float) * ((size_t)2 * A.half + (size_t)rows * A.pitch + 32);
-    if (smem > 220 * 1024) return RASCAL_E_UNSUPPORTED;
+    *smem = sizeof(float) * ((size_t)2 * A.half + (size_t)rows * A.pitch + 32);
+    return *smem <= 220 * 1024;
+}
+
+bool power_spectrum_fits(const rascal_ctx* ctx, int precision, int layout) {
+    PsArgs A;
+    size_t smem;
+    return ps_plan(ctx, precision, layout, A, &smem);
+}
+
+int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps) {
+    const bool full = layout == RASCAL_LAYOUT_FULL;
+    PsArgs A;
+    size_t smem;
+    if (!ps_plan(ctx, precision, layout, A, &smem)) return RASCAL_E_UNSUPPORTED;
+    A.c = d_coeffs;
+    A.ps = d_ps;
+    A.copy16 = A.pitch == ctx->n_lm && A.Q * ctx->n_lm % 4 == 0 && (reinterpret_cast<uintptr_t>(d_coeffs) & 15) == 0;
     auto kernel = precision == RASCAL_PS_BF16 ? (full ? k_power_spectrum<RASCAL_PS_BF16, true> : k_power_spectrum<RASCAL_PS_BF16, false>)
                   : precision == RASCAL_PS_TF32X3
                       ? (full ? k_power_spectrum<RASCAL_PS_TF32X3, true> : k_power_spectrum<RASCAL_PS_TF32X3, false>)

@@ -9,7 +9,9 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-from synth import System, mlp_initial_params  # noqa: E402
+from oracle import soap as osoap  # noqa: E402
+from synth import System, mlp_initial_params, random_cell_atoms  # noqa: E402
+from tests.gpu_common import block_rel_err, ps_blocks  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -68,5 +70,43 @@ def test_gpr(rg, N, F, points):
     before = run()
     _times_out(rg, calc, run)
     for a, b in zip(run(), before):
+        assert np.array_equal(a, b)
+    calc.sync()
+
+
+# The tcgen05 form of the BF16 Gram serves bases whose FULL l blocks do not fit the spectrum kernel beside the coefficients
+# (Q = 128, l_max 14). One launch that computes c and p, against the oracle: c 1e-5 per block, p the bars of the other BF16
+# tests; and the same kernel, with the same bits, after its wait has run out.
+@pytest.mark.parametrize("n_max,S,l_max", [(16, 8, 14), (12, 10, 14), (16, 8, 13)])
+def test_bf16_gram_of_wide_bases(rg, n_max, S, l_max):
+    rng = np.random.default_rng(7)
+    species, n = list(range(1, S + 1)), 41
+    s = System(np.concatenate([random_cell_atoms(n - 1, np.eye(3) * 8.0, 1.2, rng), [[4.0, 4.0, 60.0]]]),
+               rng.integers(1, S + 1, n).astype(np.int32), np.diag([8.0, 8.0, 200.0])[None], np.array([[1, 1, 0]], np.int32),
+               np.array([0, n], np.int32), dict(r_cut=4.5, sigma=0.5, n_max=n_max, l_max=l_max, smooth_width=0.5, species=species))
+    calc = rg.SoapCalculator(**s.hypers)
+    ds = rg.DeviceSystem.from_numpy(s)
+    pairs = calc.neighbours(ds)
+
+    def run():
+        return [t.cpu().numpy() for t in calc.soap(ds, pairs, layout="full", precision="bf16")]
+
+    launches = rg.launch_count()
+    c, p = run()
+    assert rg.launch_count() == launches + 1
+    p_separate = calc.power_spectrum(calc.spherical_expansion(ds, pairs), layout="full", precision="bf16").cpu().numpy()
+    h = osoap.Hypers(**s.hypers)
+    sel = [0, 7, 23, n - 1]
+    c_ref = osoap.spherical_expansion(s, h, centres=sel)
+    ref = osoap.power_spectrum(c_ref, h, "full").reshape(len(sel), l_max + 1, -1)
+    assert block_rel_err(c[sel], c_ref, 2) <= 1e-5
+    for got in (p, p_separate):
+        assert np.all(np.isfinite(got)) and np.all(got[-1] == 0.0)
+        blocks = ps_blocks(got[sel], l_max)
+        assert block_rel_err(blocks, ref, 2) <= 2.0 ** -7
+        fro = np.sqrt(np.sum((blocks - ref) ** 2, axis=-1) / np.maximum(np.sum(ref ** 2, axis=-1), 1e-300))
+        assert np.max(fro) <= 5e-3
+    _times_out(rg, calc, run)
+    for a, b in zip(run(), (c, p)):
         assert np.array_equal(a, b)
     calc.sync()
