@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(T, (W == kLinear ? 4 : 3) * 256 / T) k_gradien
     float* s_C = reinterpret_cast<float*>(s_j + 2 * chunk);
     float* s_G = s_C;                                              // [chunk][Gp]: f I, then (f I)'
     __shared__ float s_e[nwarps];
-    __shared__ float s_acc[12][32];  // per lane of the last warp: sums of F_i and of the virial
+    __shared__ float s_acc[12][33];  // per lane of the last warp: sums of F_i and of the virial (odd pitch: read down a lane)
     __shared__ int s_sid;
 
     const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -635,18 +635,27 @@ __global__ void __launch_bounds__(T, (W == kLinear ? 4 : 3) * 256 / T) k_gradien
     // F_i and the virial from the last warp's lanes
     if (!last) return;
     if (W == kLinear && A.energy && lane == 0) add_energy(s_e, nwarps, &A.energy[s_sid]);
-    float t = 0.0f;  // of component `lane`
+    // Across the lanes beyond FP32, as the wide form adds its warps' sums in FP64: lane k + 12 h adds half h of component k's
+    // lanes with the roundings' errors kept beside the sum (left out where the sum is not finite). Sixteen FP64 additions instead
+    // took 1 to 2 % of the kernel (FP64 issues at a sixty-fourth of the FP32 rate).
+    __syncwarp();
+    double t = 0.0;
+    if (lane < 24) {
+        const float* v = s_acc[lane % 12] + lane / 12 * 16;
+        float s = v[0], c = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        float v = s_acc[k][lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == k) t = v;
+        for (int e = 1; e < 16; ++e) {
+            const float a = v[e], n = s + a, b = n - s;
+            c += (s - (n - b)) + (a - b);
+            s = n;
+        }
+        t = (double)s + (double)(c == c ? c : 0.0f);
     }
+    t += __shfl_down_sync(0xffffffffu, t, 12);
     if (lane < 3) {
-        if (t != 0.0f) atomicAdd(&A.forces[3 * (int64_t)i + lane], t);
+        if (t != 0.0) atomicAdd(&A.forces[3 * (int64_t)i + lane], (float)t);
     } else if (lane < 12) {
-        atomicAdd(&A.virial[9 * (int64_t)s_sid + (lane - 3)], (double)t);
+        atomicAdd(&A.virial[9 * (int64_t)s_sid + (lane - 3)], t);
     }
 }
 
