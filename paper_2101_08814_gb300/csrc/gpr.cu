@@ -639,11 +639,11 @@ __global__ void k_gpr_scatter(int N, int S, const int* __restrict__ species, con
 }
 
 // per structure: E_i over the passes, zeta E_i / |p_i|^2, and the FP64 structure sum; gridDim.y CTAs share a structure (one CTA
-// took 96 us on a single structure of 25 262 atoms)
+// took 96 us on a single structure of 25 262 atoms), whose sums k_gpr_sum adds in order: the same bits in every run
 __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict__ struct_off,
                              const int* __restrict__ species, const int* __restrict__ lut, const int* __restrict__ npass,
                              const float* __restrict__ e_part, const float* __restrict__ inv, int zeta, int normalize,
-                             float* atomic, float* c2, double* energy) {
+                             float* atomic, float* c2, double* energy, double* part) {
     __shared__ double red[32];
     const int st = blockIdx.x;
     const int i0 = struct_off[st], i1 = struct_off[st + 1];
@@ -668,11 +668,19 @@ __global__ void k_gpr_finish(int N, int S, int passes_max, const int* __restrict
             if (gridDim.y == 1)
                 energy[st] = v;
             else
-                atomicAdd(&energy[st], v);  // cleared before
+                part[(int64_t)st * gridDim.y + blockIdx.y] = v;
         }
     }
     (void)S;
     (void)passes_max;
+}
+
+__global__ void k_gpr_sum(int n_s, int n, const double* __restrict__ part, double* __restrict__ energy) {
+    const int st = blockIdx.x * blockDim.x + threadIdx.x;
+    if (st >= n_s) return;
+    double v = 0.0;
+    for (int k = 0; k < n; ++k) v += part[(int64_t)st * n + k];
+    energy[st] = v;
 }
 
 static size_t gpr_smem1(int cols) {
@@ -852,11 +860,14 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
     auto tiles = [&](int w) { return ((int64_t)div_up(N, 128) + S - 1) * ((m->n_pad_max + w - 1) / w); };
     while (cols > 128 && tiles(cols / 2) <= ctx->n_sm) cols /= 2;
     const int P = std::max(1, (m->n_pad_max + cols - 1) / cols);  // passes
+    const dim3 finish((unsigned)sys->n_structures, (unsigned)std::max(1, std::min(64, N / sys->n_structures / 512)));
+    const bool shared = d_energy && finish.y > 1;  // several CTAs to a structure
     void* base;
     st = arena_get(ctx->scratch, carve_bytes(sizeof(int) * N, sizeof(int) * nb * S, sizeof(int) * (S + 1),
                                              sizeof(int) * S, sizeof(float) * N, sizeof(float) * (size_t)P * N,
                                              sizeof(float) * N, sizeof(float) * N,
-                                             grad ? sizeof(float) * (size_t)N * std::max(16, m->n_pad_max) : 16),
+                                             grad ? sizeof(float) * (size_t)N * std::max(16, m->n_pad_max) : 16,
+                                             shared ? sizeof(double) * finish.x * finish.y : 16),
                    &base);
     if (st) return st;
     Carver cv(base);
@@ -870,6 +881,7 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
     if (d_atomic) cv.take<float>(N);
     float* c2 = cv.take<float>(N);
     float* W = grad ? cv.take<float>((size_t)N * std::max(16, m->n_pad_max)) : nullptr;
+    double* part = shared ? cv.take<double>((size_t)finish.x * finish.y) : nullptr;
 
     int hp[kMaxSpecies];
     for (int s = 0; s < S; ++s) hp[s] = (m->n_pad[s] + cols - 1) / cols;
@@ -918,12 +930,13 @@ extern "C" int rascal_gpr_predict(rascal_ctx* ctx, const rascal_gpr* m, const ra
         gpr_kernel(A.vec16, cols)<<<ctx->n_sm, kGprThreads1, gpr_smem1(cols), ctx->stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_gpr_kernel");
     }
-    const dim3 finish((unsigned)sys->n_structures, (unsigned)std::max(1, std::min(64, N / sys->n_structures / 512)));
-    k_gpr_finish<<<finish, 256, 0, ctx->stream>>>(N, S, P, sys->d_struct_offsets, sys->d_species, ctx->d_lut,
-                                                             npass, e_part, inv, m->zeta, m->normalize, atomic,
-                                                             grad ? c2 : nullptr,
-                                                             d_energy);
+    k_gpr_finish<<<finish, 256, 0, ctx->stream>>>(N, S, P, sys->d_struct_offsets, sys->d_species, ctx->d_lut, npass, e_part, inv,
+                                                  m->zeta, m->normalize, atomic, grad ? c2 : nullptr, d_energy, part);
     RASCAL_LAUNCH_CHECK("k_gpr_finish");
+    if (shared) {
+        k_gpr_sum<<<(unsigned)div_up(sys->n_structures, 256), 256, 0, ctx->stream>>>(sys->n_structures, (int)finish.y, part, d_energy);
+        RASCAL_LAUNCH_CHECK("k_gpr_sum");
+    }
     if (grad) {
         k_gpr_grad<<<2 * ctx->n_sm, kGprThreads2, gpr_smem2(), ctx->stream>>>(A);
         RASCAL_LAUNCH_CHECK("k_gpr_grad");

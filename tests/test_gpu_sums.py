@@ -50,3 +50,28 @@ def test_centre_sums_are_wider_than_fp32(rg, n_max, l_max, S, linear, P):
     eps = 15 ** 2 * 2.0 ** -48
     assert np.all(np.abs(v - vs.sum(0)) <= eps * np.abs(vs).sum(0))
     assert np.all(np.abs(f - fs.sum(0)) <= 2.0 ** -24 * np.abs(fs.sum(0)) + 2 * eps * np.abs(fs).sum(0))
+
+
+# The structure energies are the same bits in every call, one CTA to a structure and several (one structure of 25 000 atoms; a
+# large and two small ones), and the FP64 sums of the atoms' energies. Those spread over 24 decades, so that FP64 sums round.
+@pytest.mark.parametrize("sizes", [(25000,), (700, 650), (6000, 3, 300)])
+def test_gpr_energies_repeat(rg, sizes):
+    import torch
+
+    N, F = sum(sizes), 20
+    rng = np.random.default_rng(73)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    n = len(sizes)
+    s = System(rng.uniform(0, 20, (N, 3)), rng.choice([1, 6], N).astype(np.int32), np.tile(np.eye(3) * 20, (n, 1, 1)),
+               np.ones((n, 3), np.int32), off, {})
+    calc = rg.SoapCalculator(4.0, 0.5, 2, 1, [1, 6], spline_intervals=64)
+    model = rg.GprModel(calc, rng.random((60, F)), np.repeat([1, 6], 30), rng.standard_normal(60), normalize=False)
+    ds = rg.DeviceSystem.from_numpy(s)
+    p = torch.tensor(rng.random((N, F)) * 10.0 ** rng.uniform(-6, 6, (N, 1)), dtype=torch.float32, device="cuda")
+    e, ea, _ = model.predict(ds, p)
+    for _ in range(40):
+        assert torch.equal(model.predict(ds, p)[0], e)
+    ea = ea.double().cpu().numpy()
+    for k in range(n):
+        atoms = ea[off[k]:off[k + 1]]
+        assert abs(e[k].item() - atoms.sum()) <= len(atoms) * 2.0 ** -53 * np.abs(atoms).sum()
