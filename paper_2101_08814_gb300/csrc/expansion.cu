@@ -121,11 +121,14 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
     const int kSc = SHAPE ? exp_sc(C.n_max, C.l_max, C.S) : A.S_c;
     const int kRounds = SHAPE ? (C.S + exp_sc(C.n_max, C.l_max, C.S) - 1) / exp_sc(C.n_max, C.l_max, C.S) : A.rounds;
     const int kChunk = SHAPE ? exp_chunk(C.n_max, C.l_max) : A.chunk;
-    // Coefficients only, n_max not a multiple of 4, known at compile time: radial rows two at a time with the lanes over the
-    // table's own columns instead of the padded slots and their map (16 000 centres with 86 pairs, 10, 8, 3: 472 -> 409 us). With
-    // n_max a multiple of 4 there is no map and nothing to gain but spills (12, 9, 4: 191 -> 252 us; 16, 12, 8: 311 -> 492 us), and
-    // the runtime-shaped kernel spills as well (9, 7, 3: 383 -> 467 us).
-    constexpr bool kTwoRows = GRAM == kGramNone && SHAPE != 0 && C.n_max % 4 != 0;
+    // Coefficients only, padded slots other than the table's columns or not known to be the same: the lanes go over the table's own
+    // columns with a running slot, without the map and the padding's loads, runtime shapes two rows at a time (one after the
+    // other's columns: more in flight spill). Over the map -> so: 16 000 centres with 86 pairs (10, 8, 3) 471 -> 397 us, two rows
+    // 449; runtime shapes of 9 000 to 16 000 centres (9, 7, 3) 226 -> 215, (5, 4, 2) 92 -> 82, (6, 4, 3) 103 -> 86, (11, 8, 4)
+    // 150 -> 146, (13, 9, 3) 166 -> 166, (8, 5, 3) 109 -> 102, (16, 8, 4) 173 -> 165; one row (7, 5, 2) 98 -> 112, two 94. Where the
+    // slots are the columns (n_max a multiple of 4, compiled) there is nothing to gain but spills: (12, 9, 4) two rows 191 -> 252 us.
+    constexpr bool kOwnColumns = GRAM == kGramNone && !kFmapId;
+    constexpr int kRowsAtOnce = SHAPE ? 1 : 2, kColumnUnroll = SHAPE ? 4 : 1;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ uint64_t s_bar[4];  // two MMA slots, a drain barrier and one that nothing arrives at (test hook)
     __shared__ uint32_t s_tmem;
@@ -146,6 +149,9 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
 
     const int i = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    // n and padded slot of this lane's first table column, and the steps of 32 columns (divided once)
+    const int pad = kNpad - kNmax, col_n = lane % kNmax, col_slot = lane + lane / kNmax * pad;
+    const int step_n = 32 % kNmax, step_slot = 32 + 32 / kNmax * pad;
     if (!kFmapId) {
         #pragma unroll 1
         for (int t = tid; t < kFpad; t += blockDim.x) s_fmap[t] = A.fmap[t];
@@ -299,15 +305,14 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
             }
             // radial values G = f_cut I^o_nl: one warp per row, lanes over padded (l, n); the warps without a Y chain
             // take the first rows
-            if (kTwoRows && !A.pre_G) {
-                const int pad = kNpad - kNmax;
+            if (kOwnColumns && !A.pre_G) {
                 #pragma unroll 1
                 for (int e = tid; e < n_rows * L1; e += blockDim.x)
                     #pragma unroll 1
                     for (int c = kNmax; c < kNpad; ++c) s_G[e / L1 * kFpad + e % L1 * kNpad + c] = 0.0f;
                 #pragma unroll 1
-                for (int q = 2 * (nwarps - 1 - warp); q < n_rows; q += 2 * nwarps) {
-                    const bool two = q + 1 < n_rows;
+                for (int q = kRowsAtOnce * (nwarps - 1 - warp); q < n_rows; q += kRowsAtOnce * nwarps) {
+                    const bool two = kRowsAtOnce == 2 && q + 1 < n_rows;
                     const int p0 = s_list[q], p1 = s_list[two ? q + 1 : q];
                     const float f0 = s_fc[p0], f1 = s_fc[p1];
                     const float x0 = s_vec[p0].w * A.inv_delta, x1 = s_vec[p1].w * A.inv_delta;
@@ -315,12 +320,18 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                     const float u0 = x0 - (float)k0, u1 = x1 - (float)k1;
                     const float4 *t0 = A.table + k0 * kF, *t1 = A.table + k1 * kF;
                     float* g0 = s_G + q * kFpad;
-                    #pragma unroll 4
+                    int n = col_n, slot = col_slot;  // of column c = l n_max + n: slot l n_pad + n
+                    #pragma unroll (kColumnUnroll)
                     for (int c = lane; c < kF; c += 32) {
-                        const float4 a = __ldg(t0 + c), b = __ldg(t1 + c);
-                        float* o = g0 + c + c / kNmax * pad;
-                        o[0] = f0 * fmaf(u0, fmaf(u0, fmaf(u0, a.w, a.z), a.y), a.x);
-                        if (two) o[kFpad] = f1 * fmaf(u1, fmaf(u1, fmaf(u1, b.w, b.z), b.y), b.x);
+                        const float4 a = __ldg(t0 + c), b = kRowsAtOnce == 2 ? __ldg(t1 + c) : a;
+                        g0[slot] = f0 * fmaf(u0, fmaf(u0, fmaf(u0, a.w, a.z), a.y), a.x);
+                        if (two) g0[slot + kFpad] = f1 * fmaf(u1, fmaf(u1, fmaf(u1, b.w, b.z), b.y), b.x);
+                        n += step_n;
+                        slot += step_slot;
+                        if (n >= kNmax) {
+                            n -= kNmax;
+                            slot += pad;
+                        }
                     }
                 }
             } else
