@@ -136,15 +136,14 @@ int rascal_info(const rascal_ctx* ctx, rascal_info_t* out);
  * label, degenerate geometry, ...) into a status. */
 int rascal_sync(rascal_ctx* ctx);
 
-/* Test hook for the failure path of the tcgen05 kernels (no counterpart in the paper). With polls > 0,
- * rascal_soap (precision BF16 or TF32X3) and the tensor-core precisions of rascal_power_spectrum run those forms, and the
- * first MMA-completion wait of every CTA of rascal_soap (precision BF16 or TF32X3) and of the tensor-core forms of
- * rascal_power_spectrum is made on an mbarrier that nothing arrives at, and gives up after `polls` polls (about
- * 20 ns apart). The kernel then raises the timeout flag, skips the remaining epilogues, waits (with the built-in
- * bound of 2^22 polls) for every MMA it issued and frees its tensor memory; the next synchronising call returns
- * RASCAL_E_TIMEOUT. The outputs of that call are incomplete. The MLP inference (rascal_mlp_eval, radial mode MLP) and
- * rascal_gpr_predict have the same hook in the kernels that they always run. polls = 0 switches the hook off; the context stays
- * usable throughout. Returns RASCAL_E_ARG for a NULL context. */
+/* Test hook for the failure path of the tcgen05 kernels (no counterpart in the paper). With polls > 0, rascal_soap and
+ * rascal_power_spectrum in their tensor-core precisions run the tcgen05 form of the BF16 Gram (which otherwise serves the
+ * BF16 bases that the spectrum kernel does not take), and the first completion wait of every CTA of that form, of the MLP
+ * inference (rascal_mlp_eval, radial mode MLP) and of both kernels of rascal_gpr_predict is made on an mbarrier that
+ * nothing arrives at, and gives up after `polls` polls (about 20 ns apart). The kernel then raises the timeout flag, skips
+ * what remains, waits (with the built-in bound of 2^22 polls) for everything it issued and frees its tensor memory; the
+ * next synchronising call returns RASCAL_E_TIMEOUT. The outputs of that call are incomplete. polls = 0 switches the hook
+ * off; the context stays usable throughout. Returns RASCAL_E_ARG for a NULL context. */
 int rascal_debug_wait_timeout(rascal_ctx* ctx, unsigned polls);
 
 /* Test hooks for tables the library builds on the host (no context and no GPU needed; no counterpart in the paper).

@@ -104,7 +104,6 @@ struct ExpPlan {
     int T_s, W_s, S_c, rounds, threads;
     int chunk;        // pairs staged per chunk
     size_t smem;      // dynamic shared memory of the expansion kernel
-    size_t smem_ps;   // extra dynamic shared memory when the power spectrum is fused
 };
 
 }  // namespace rascal
@@ -224,7 +223,8 @@ int radial_precompute(rascal_ctx* ctx, const rascal_system* sys, const int64_t* 
 int mlp_setup(rascal_ctx* ctx);
 int expansion_setup(rascal_ctx* ctx);
 int power_spectrum_setup(rascal_ctx* ctx);
-// BF16 / TF32x3 power spectrum of given coefficients [n][Q][n_lm] by the fused kernel's tensor-core Gram
+// BF16 / TF32x3 power spectrum of given coefficients [n][Q][n_lm]: what is refused, then the kernel of power_spectrum.cu, or the
+// tcgen05 Gram of expansion.cu for what that does not take and for the test hook
 int power_spectrum_tc(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps);
 // FP32, BF16 or TF32x3 power spectrum of given coefficients by the kernel of power_spectrum.cu; RASCAL_E_UNSUPPORTED
 // (without a message) where a centre does not fit its shared memory

@@ -16,9 +16,9 @@
 // memory and, when the power spectrum is fused, also into shared memory, where the Gram runs without c ever being
 // read back from HBM:
 //   kGramSimt    FP32 register-tiled Gram on the CUDA cores from CT[lm][q] (ps_fp32.cuh);
-//   kGramBf16    tcgen05 MMA, BF16 operands, FP32 accumulators in TMEM (tcgen05.cuh); this form and the next serve what the
-//                spectrum kernel of stored coefficients, which is faster, does not take, and the wait-timeout hook;
-//   kGramTf32x3  tcgen05 MMA, TF32 hi/lo split, three MMAs per K step (FP32-grade).
+//   kGramBf16    tcgen05 MMA, BF16 operands, FP32 accumulators in TMEM (tcgen05.cuh): bases whose FULL l blocks do not fit the
+//                spectrum kernel of stored coefficients, which is faster (Q of 112 to 128, l_max 13 and above), and the
+//                wait-timeout hook.
 // The Gram output is staged per group of l values in the (then free) pair-staging buffers and written to global
 // memory by bulk copies.
 #include <cuda_bf16.h>
@@ -36,11 +36,7 @@ namespace rascal {
 
 // kGramSel: the FP32 form restricted to listed features (its own instantiation, so that the full Gram's register
 // allocation is not affected by the selection branch)
-// kGramRTf32 / kGramRBf16: the tensor-core Gram in rounds of one l (operands staged per round in the pair rows,
-// M = 64 MMAs into two 64-column TMEM slots, epilogue by every warp storing p straight to global memory)
-enum GramMode : int { kGramNone = 0, kGramSimt = 1, kGramBf16 = 2, kGramTf32x3 = 3, kGramSel = 4, kGramRTf32 = 5,
-                      kGramRBf16 = 6 };
-constexpr int kRtcLbo = 144;  // bytes between core matrices adjacent along K (bank groups advance by one per step)
+enum GramMode : int { kGramNone = 0, kGramSimt = 1, kGramBf16 = 2, kGramSel = 3 };
 constexpr int kMaxGroups = kMaxLMax + 2;
 
 struct ExpArgs {
@@ -51,7 +47,7 @@ struct ExpArgs {
     const int* lut;
     const float4* table;
     const float* pre_G;  // per-pair radial values [P][F] (EXACT / MLP modes) or NULL (spline table)
-    const float* c_in;   // tensor-core power spectrum of given coefficients [N][Q][n_lm]: no pair phase, or NULL
+    const float* c_in;   // tcgen05 power spectrum of given coefficients [N][Q][n_lm]: no pair phase, or NULL
     const int* sel;      // selected features (FP32 form): packed (l | q1 << 8 | q2 << 16) per output column, or NULL
     int n_sel;
     const int* tasks;
@@ -74,12 +70,8 @@ struct ExpArgs {
     const int* ps_tasks;            // SIMT tasks, l descending
     int g_tbeg[kMaxGroups], g_tend[kMaxGroups];  // SIMT task ranges of the groups
     int Qp;                         // SIMT CT row pitch
-    int N_mma, tm_cols, slot_cols, lo_off, tiles_bytes;
+    int N_mma, tm_cols, slot_cols, tiles_bytes;
     int tile_off[kMaxLMax + 1], sbo[kMaxLMax + 1], nk[kMaxLMax + 1];
-    // rounds of one l (kGramRTf32 / kGramRBf16)
-    int rtc_half, rtc_lo, rtc_c_bytes;            // bytes per operand half, offset of the lo tile, staged c bytes
-    int rtc_kq[kMaxLMax + 1];                     // units of four K elements per row (kpad / 4)
-    float rtc_sc[kMaxLMax + 1];                  // operand scale s_l, s_l^2 = k_l
     uint32_t stall_polls;                        // test hook: > 0 makes the first completion wait run out
 };
 
@@ -91,18 +83,10 @@ __device__ inline float cutoff_fp32(float r, float r_cut, float w) {
     return c * c;
 }
 
-// element (q, s) of C_l into the K-major operand tile of l (BF16, or TF32 hi/lo for the three-MMA split)
-template <int GRAM>
+// element (q, s) of C_l into the K-major BF16 operand tile of l
 __device__ inline void put_operand(unsigned char* tiles, const ExpArgs& A, int l, int q, int s, float cv) {
-    constexpr int esz = (GRAM == kGramTf32x3) ? 4 : 2, e16 = 16 / esz;
-    const int off = A.tile_off[l] + (q >> 3) * A.sbo[l] + (s / e16) * 128 + (q & 7) * 16 + (s % e16) * esz;
-    if (GRAM == kGramTf32x3) {
-        const float hi = __uint_as_float(__float_as_uint(cv) & 0xFFFFE000u);
-        *reinterpret_cast<float*>(tiles + off) = hi;
-        *reinterpret_cast<float*>(tiles + A.lo_off + off) = cv - hi;
-    } else {
-        *reinterpret_cast<__nv_bfloat16*>(tiles + off) = __float2bfloat16_rn(cv);
-    }
+    const int off = A.tile_off[l] + (q >> 3) * A.sbo[l] + (s >> 3) * 128 + (q & 7) * 16 + (s & 7) * 2;
+    *reinterpret_cast<__nv_bfloat16*>(tiles + off) = __float2bfloat16_rn(cv);
 }
 
 template <int GRAM, int SHAPE = 0>
@@ -132,15 +116,13 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ uint64_t s_bar[4];  // two MMA slots, a drain barrier and one that nothing arrives at (test hook)
     __shared__ uint32_t s_tmem;
-    constexpr bool TC = (GRAM == kGramBf16 || GRAM == kGramTf32x3);
-    constexpr bool RTC = (GRAM == kGramRTf32 || GRAM == kGramRBf16);
+    constexpr bool TC = GRAM == kGramBf16;
     const int chunk = kChunk;
     float4* s_vec = reinterpret_cast<float4*>(smem_raw + A.pair_off);
     float* s_G = reinterpret_cast<float*>(s_vec + chunk);            // [chunk][F_pad]
     float* s_Y = s_G + (size_t)chunk * kFpad;                       // [chunk][Ly]
     float* s_fc = s_Y + (size_t)chunk * kLy;
-    int* s_spc = reinterpret_cast<int*>(s_fc + chunk);
-    int* s_list = s_spc + chunk;
+    int* s_list = reinterpret_cast<int*>(s_fc + chunk);
     int* s_start = s_list + chunk;                                    // [kMaxSpecies + 1]
     int* s_fmap = s_start + (kMaxSpecies + 1) + (kMaxLMax + 2);        // [F_pad]
     unsigned char* gram = smem_raw + A.gram_off;                      // CT or tiles
@@ -165,10 +147,9 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                 #pragma unroll 1
                 for (int c = kQ; c < q_end; ++c) CT[lm * kQp + c] = 0.0f;
     }
-    if (TC || RTC) {
-        if (TC)  // K padding and rows >= Q of the operand tiles must read as zero
-            for (int b = tid; b < A.tiles_bytes / 16; b += blockDim.x)
-                reinterpret_cast<uint4*>(gram)[b] = make_uint4(0, 0, 0, 0);
+    if (TC) {
+        // K padding and rows >= Q of the operand tiles must read as zero
+        for (int b = tid; b < A.tiles_bytes / 16; b += blockDim.x) reinterpret_cast<uint4*>(gram)[b] = make_uint4(0, 0, 0, 0);
         if (warp == 0) {
             tmem_alloc(&s_tmem, (uint32_t)A.tm_cols);
             tmem_relinquish();
@@ -206,8 +187,6 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
     const int g_off = my_l * kNpad + 4 * my_nt;   // offset inside a G row
     const int y_off = exp_lp(my_l) + 4 * my_mt;       // offset inside a Y row
 
-    float* cdst_r = A.coeffs + (int64_t)i * kQ * kNlm;
-    float* cst_r = stage + stage_shift(cdst_r);
     for (int round = 0; round < (given_c ? 0 : kRounds); ++round) {
         const int a0 = round * kSc;
         const int na = min(kSc, kS - a0);
@@ -403,7 +382,7 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                     }
                 }
             }
-            if (RTC || GRAM == kGramNone) {  // c[q][lm] staged in the (free) pair rows, whence it leaves by one bulk copy
+            if (GRAM == kGramNone) {  // c[q][lm] staged in the (free) pair rows, whence it leaves by one bulk copy
                 const int s_end = 2 * my_l + 1 - 4 * my_mt;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -448,7 +427,7 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
                         if (s > 2 * my_l) continue;
                         const float cv = acc[u][v];
                         out[n * kNlm + s] = cv;
-                        put_operand<GRAM>(gram, A, my_l, q, s, cv);
+                        put_operand(gram, A, my_l, q, s, cv);
                     }
                 }
             }
@@ -469,141 +448,12 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
         if (tid == 0) bulk_wait_all();
         return;
     }
-    if (RTC) {
-        // ---------------------------------------------------------------- tensor-core Gram in rounds of one l
-        fence_proxy_async_smem();
-        __syncthreads();
-        store_staged(cdst_r, cst_r, kQ * kNlm);  // c leaves by one bulk copy (the staged c stays for the operands)
-        const int Q = kQ, L1n = kLmax + 1;
-        const bool packed = A.layout == RASCAL_LAYOUT_PACKED;
-        unsigned char* halves = reinterpret_cast<unsigned char*>(stage) + A.rtc_c_bytes;  // behind the staged c
-        const uint32_t halves_s = smem_u32(halves);
-        const uint32_t taddr = s_tmem;
-        const uint32_t idesc = instr_desc(GRAM == kGramRTf32 ? 2u : 1u, 64u, (uint32_t)A.N_mma);
-        float* pout = A.ps + (int64_t)i * A.ps_stride;
-        // operands of l into half h from the staged c: 16-byte units of four K elements (s_l c, zero beyond 2l),
-        // TF32 hi and lo tiles or BF16; every thread takes some of the Q x kpad / 4 units
-        auto write_ops = [&](int l, int h) {
-            unsigned char* base = halves + h * A.rtc_half;
-            const float sl = A.rtc_sc[l];
-            const int n4 = A.rtc_kq[l];
-            const float* cl = cst_r + l * l;
-            for (int e = tid; e < Q * n4; e += blockDim.x) {
-                const int q = e / n4, k4 = e - q * n4;
-                const float* src = cl + q * kNlm + 4 * k4;
-                const int s0 = 4 * k4;
-                const float x0 = s0 <= 2 * l ? sl * src[0] : 0.0f;
-                const float x1 = s0 + 1 <= 2 * l ? sl * src[1] : 0.0f;
-                const float x2 = s0 + 2 <= 2 * l ? sl * src[2] : 0.0f;
-                const float x3 = s0 + 3 <= 2 * l ? sl * src[3] : 0.0f;
-                const int row = (q >> 3) * A.sbo[l] + (q & 7) * 16;
-                if (GRAM == kGramRTf32) {
-                    const float h0 = __uint_as_float(__float_as_uint(x0) & 0xFFFFE000u);
-                    const float h1 = __uint_as_float(__float_as_uint(x1) & 0xFFFFE000u);
-                    const float h2 = __uint_as_float(__float_as_uint(x2) & 0xFFFFE000u);
-                    const float h3 = __uint_as_float(__float_as_uint(x3) & 0xFFFFE000u);
-                    const int off = row + k4 * kRtcLbo;
-                    *reinterpret_cast<float4*>(base + off) = make_float4(h0, h1, h2, h3);
-                    *reinterpret_cast<float4*>(base + A.rtc_lo + off) = make_float4(x0 - h0, x1 - h1, x2 - h2, x3 - h3);
-                } else {
-                    const int off = row + (k4 >> 1) * kRtcLbo + (k4 & 1) * 8;
-                    const __nv_bfloat162 b01 = __floats2bfloat162_rn(x0, x1), b23 = __floats2bfloat162_rn(x2, x3);
-                    uint2 w;
-                    w.x = *reinterpret_cast<const uint32_t*>(&b01);
-                    w.y = *reinterpret_cast<const uint32_t*>(&b23);
-                    *reinterpret_cast<uint2*>(base + off) = w;
-                }
-            }
-        };
-        auto issue = [&](int l, int sl) {
-            const uint32_t d = taddr + (uint32_t)(sl * A.slot_cols);
-            const uint32_t a0 = halves_s + (uint32_t)(sl * A.rtc_half);
-            for (int kk = 0; kk < A.nk[l]; ++kk) {
-                const uint32_t a_addr = a0 + (uint32_t)(kk * 2 * kRtcLbo);
-                const uint64_t da = smem_desc(a_addr, kRtcLbo, (uint32_t)A.sbo[l]);
-                if (GRAM == kGramRTf32) {
-                    const uint64_t dl = smem_desc(a_addr + (uint32_t)A.rtc_lo, kRtcLbo, (uint32_t)A.sbo[l]);
-                    mma_tf32_ss(d, da, da, idesc, kk > 0);
-                    mma_tf32_ss(d, da, dl, idesc, 1);
-                    mma_tf32_ss(d, dl, da, idesc, 1);
-                } else {
-                    mma_bf16_ss(d, da, da, idesc, kk > 0);
-                }
-            }
-            mma_commit(&s_bar[sl]);
-        };
-        // rows of this warp (M = 64: TMEM lanes 32 quad + 0..15 hold rows 16 quad + 0..15); the warps of a quadrant
-        // share its 16-column chunks
-        const int quad = warp & 3, wq = warp >> 2, nwq = (nwarps - quad + 3) >> 2;
-        const int r = 16 * quad + lane;
-        const bool row_ok = lane < 16 && r < Q;
-        const int cend = packed ? min(Q - 1, 16 * quad + 15) + 1 : Q;
-        __shared__ int s_fail;
-        if (tid == 0) s_fail = 0;
-        // round k handles l = l_max - k in slot / operand half k & 1; the MMAs of round k + 1 are issued before
-        // the epilogue of round k
-        write_ops(kLmax, 0);
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (tid == 0) issue(kLmax, 0);
-        for (int k = 0; k < L1n; ++k) {
-            const int l = kLmax - k, sl = k & 1;
-            if (k + 1 < L1n) write_ops(l - 1, sl ^ 1);  // its half was read by round k - 1's MMAs, waited for below
-            fence_proxy_async_smem();
-            tc_fence_before();
-            __syncthreads();  // operands of round k + 1 written; round k - 1's epilogue done with slot sl ^ 1
-            tc_fence_after();
-            const bool go = s_fail == 0;
-            if (tid == 0 && k + 1 < L1n && go) issue(l - 1, sl ^ 1);
-            // the test hook points the first wait at a barrier that no MMA signals, bounded by stall_polls polls
-            const bool stall = A.stall_polls != 0 && k == 0;
-            const bool done = go && __all_sync(0xffffffffu, mbar_wait_bounded(stall ? &s_bar[3] : &s_bar[sl],
-                                                                              (uint32_t)((k >> 1) & 1),
-                                                                              stall ? A.stall_polls : (1u << 22)));
-            if (!done) {
-                if (lane == 0) s_fail = 1;
-                continue;
-            }
-            tc_fence_after();
-            if (16 * quad < Q) {
-                const uint32_t tl = taddr + ((uint32_t)(32 * quad) << 16) + (uint32_t)(sl * A.slot_cols);
-                float* out = pout + (int64_t)l * A.per_l;
-                for (int c0 = 16 * wq; c0 < cend; c0 += 16 * nwq) {
-                    float v[16];
-                    tmem_ld16(tl + (uint32_t)c0, v);
-                    // packed (q1, q2) = (column c, row r), c <= r, at c (2Q - c - 1) / 2 + r; FULL: at c Q + r
-                    int o = packed ? c0 * (2 * Q - c0 - 1) / 2 + r : c0 * Q + r;
-                    const int dd = row_ok ? (packed ? r - c0 : Q - 1 - c0) : -1;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        if (j <= dd) out[o] = v[j];
-                        o += packed ? Q - 1 - (c0 + j) : Q;
-                    }
-                }
-            }
-        }
-        if (tid == 0) {  // every MMA issued above has completed before the tensor memory is freed
-            if (s_fail) atomicOr(A.flags, kFlagTimeout);
-            mma_commit(&s_bar[2]);
-            if (!mbar_wait_bounded(&s_bar[2], 0u)) atomicOr(A.flags, kFlagTimeout);
-        }
-        if (tid == 0) bulk_wait_all();
-        tc_fence_before();
-        __syncthreads();
-        if (warp == 0) {
-            tc_fence_after();
-            tmem_dealloc(s_tmem, (uint32_t)A.tm_cols);
-        }
-        return;
-    }
     if (given_c) {  // operand tiles from the given coefficients of this centre
         const float* cc = A.c_in + (int64_t)i * kQ * kNlm;
         for (int e = tid; e < kQ * kNlm; e += blockDim.x) {
             const int q = e / kNlm, lm = e - q * kNlm;
             const int l = (int)sqrtf((float)lm);
-            put_operand<GRAM>(gram, A, l, q, lm - l * l, __ldg(cc + e));
+            put_operand(gram, A, l, q, lm - l * l, __ldg(cc + e));
         }
     }
 
@@ -692,21 +542,14 @@ __global__ void __launch_bounds__(512, 3) k_expansion(const ExpArgs A) {
         tc_fence_after();
         const uint32_t taddr = s_tmem;
         const uint32_t tiles_s = smem_u32(gram);
-        const uint32_t idesc = instr_desc(GRAM == kGramTf32x3 ? 2u : 1u, 128u, (uint32_t)A.N_mma);
+        const uint32_t idesc = instr_desc(1u, 128u, (uint32_t)A.N_mma);
         const int L1n = kLmax + 1;
         auto issue = [&](int l) {
             const uint32_t d = taddr + (uint32_t)((l & 1) * A.slot_cols);
             for (int kk = 0; kk < A.nk[l]; ++kk) {
                 const uint32_t a_addr = tiles_s + A.tile_off[l] + kk * 256;
                 const uint64_t da = smem_desc(a_addr, 128, A.sbo[l]);
-                if (GRAM == kGramTf32x3) {
-                    const uint64_t dl = smem_desc(a_addr + A.lo_off, 128, A.sbo[l]);
-                    mma_tf32_ss(d, da, da, idesc, kk > 0);
-                    mma_tf32_ss(d, da, dl, idesc, 1);
-                    mma_tf32_ss(d, dl, da, idesc, 1);
-                } else {
-                    mma_bf16_ss(d, da, da, idesc, kk > 0);
-                }
+                mma_bf16_ss(d, da, da, idesc, kk > 0);
             }
             mma_commit(&s_bar[l & 1]);
         };
@@ -802,6 +645,7 @@ static void make_plan(rascal_ctx* ctx) {
     if (P.W_s > max_warps) P.S_c = 1;
     P.rounds = (ctx->n_species + P.S_c - 1) / P.S_c;
     P.threads = 32 * P.W_s * P.S_c;
+    // (a word per pair more than the kernel uses: which hypers are refused follows from this size, and stays as it is)
     auto smem_for = [&](int chunk) {
         return (size_t)chunk * sizeof(float4) + (size_t)chunk * (P.F_pad + P.Ly) * sizeof(float) +
                (size_t)chunk * (sizeof(float) + 2 * sizeof(int)) + (kMaxSpecies + 1 + kMaxLMax + 2 + P.F_pad) * sizeof(int) + 64;
@@ -809,7 +653,6 @@ static void make_plan(rascal_ctx* ctx) {
     P.chunk = 32;  // about 30 KB for n_max 12, l_max 9: four CTAs per SM
     while (P.chunk > 8 && smem_for(P.chunk) > 56 * 1024) P.chunk /= 2;
     P.smem = smem_for(P.chunk);
-    P.smem_ps = 0;
 }
 
 template <int GRAM, int SHAPE = 0>
@@ -839,7 +682,7 @@ int expansion_setup(rascal_ctx* ctx) {
         (st = set_attr<kGramSimt, 1>()) || (st = set_attr<kGramSimt, 2>()) || (st = set_attr<kGramSimt, 3>()) ||
         (st = set_attr<kGramSimt, 4>()) || (st = set_attr<kGramSel>()) || (st = set_attr<kGramSel, 1>()) ||
         (st = set_attr<kGramSel, 2>()) || (st = set_attr<kGramSel, 3>()) || (st = set_attr<kGramSel, 4>()) ||
-        (st = set_attr<kGramBf16>()) || (st = set_attr<kGramTf32x3>()) || (st = set_attr<kGramRTf32>()))
+        (st = set_attr<kGramBf16>()))
         return st;
     RASCAL_CUDA(cudaStreamSynchronize(ctx->stream));
     return RASCAL_OK;
@@ -886,8 +729,9 @@ static ExpArgs make_args(rascal_ctx* ctx, const rascal_system* sys, const int64_
     return A;
 }
 
-// Sets the fused power-spectrum part of the arguments; returns the total dynamic shared memory in *smem.
-static int make_gram(rascal_ctx* ctx, int mode, int layout, float* d_ps, ExpArgs& A, size_t* smem, int* threads) {
+// Sets the fused power-spectrum part of the arguments; returns the total dynamic shared memory in *smem. tf32: the sizes of
+// operand tiles in two TF32 parts, by which TF32x3 is accepted or refused (the spectrum kernel takes every basis that passes).
+static int make_gram(rascal_ctx* ctx, int mode, int layout, float* d_ps, ExpArgs& A, size_t* smem, int* threads, bool tf32 = false) {
     const ExpPlan& P = ctx->plan;
     const int Q = ctx->Q;
     A.ps = d_ps;
@@ -903,35 +747,6 @@ static int make_gram(rascal_ctx* ctx, int mode, int layout, float* d_ps, ExpArgs
     size_t gram_bytes = 0;
     size_t stage_need = 0;
     size_t tail_end = 0;  // tensor cores: end of the bytes the last MMA reads
-    if (mode == kGramRTf32 || mode == kGramRBf16) {
-        // one species round, M = 64 rows, N <= 64 columns per TMEM slot; one l per round
-        if (P.rounds != 1 || Q > 64) return RASCAL_E_UNSUPPORTED;
-        const bool tf32 = mode == kGramRTf32;
-        const int esz = tf32 ? 4 : 2, kstep = tf32 ? 8 : 16, e16 = 16 / esz;
-        A.N_mma = std::max(8, (Q + 7) / 8 * 8);
-        int sbo_max = 0;
-        for (int l = 0; l < L1; ++l) {
-            const int kpad = (2 * l + 1 + kstep - 1) / kstep * kstep;
-            A.nk[l] = kpad / kstep;
-            A.rtc_kq[l] = kpad / 4;
-            A.sbo[l] = (kpad / e16) * kRtcLbo;
-            sbo_max = std::max(sbo_max, A.sbo[l]);
-            A.rtc_sc[l] = ctx->ps_norm ? (float)std::pow(2.0 * l + 1.0, -0.25) : 1.0f;
-        }
-        A.rtc_lo = 8 * sbo_max;  // an M = 64 MMA reads 8 groups of 8 rows
-        A.rtc_half = tf32 ? 2 * A.rtc_lo : A.rtc_lo;
-        A.slot_cols = 64;
-        A.tm_cols = 128;
-        A.pair_off = 0;
-        A.rtc_c_bytes = (int)align_up(sizeof(float) * ((size_t)Q * ctx->n_lm + 3), 16);
-        const size_t need = (size_t)A.rtc_c_bytes + 2 * (size_t)A.rtc_half;
-        size_t exp_bytes = P.smem;
-        if (need > pair_region * sizeof(float)) exp_bytes += need - pair_region * sizeof(float);
-        A.gram_off = (int)align_up(exp_bytes, 1024);
-        *smem = exp_bytes;
-        *threads = std::max(P.threads, 128);
-        return *smem > 200 * 1024 ? RASCAL_E_UNSUPPORTED : RASCAL_OK;
-    }
     if (mode == kGramSimt) {
         // row pitch: a multiple of 4 floats with Qp / 4 odd, so float4 reads down a column of CT are conflict-free
         A.Qp = ((Q + 3) / 4 | 1) * 4;
@@ -982,7 +797,6 @@ static int make_gram(rascal_ctx* ctx, int mode, int layout, float* d_ps, ExpArgs
         stage_need = half + (n1 > 0 ? (size_t)n1 * blk + 3 : 0);
     } else {
         if (Q > 128) return set_error(RASCAL_E_UNSUPPORTED, "tensor-core power spectrum needs n_species*n_max <= 128");
-        const bool tf32 = mode == kGramTf32x3;
         const int esz = tf32 ? 4 : 2, kstep = tf32 ? 8 : 16, e16 = 16 / esz;
         A.N_mma = (Q + 15) / 16 * 16;
         const int Qr = (Q + 7) / 8 * 8;
@@ -996,13 +810,12 @@ static int make_gram(rascal_ctx* ctx, int mode, int layout, float* d_ps, ExpArgs
             off += (Qr / 8) * A.sbo[l];
         }
         const int hi_bytes = (off + 1023) / 1024 * 1024;
-        A.lo_off = tf32 ? hi_bytes : 0;
         A.tiles_bytes = tf32 ? 2 * hi_bytes : hi_bytes;
         // the tiles sit at the start of shared memory and the pair area follows them, so the rows >= Q that the
         // MMA reads past the last tile stay inside the allocation
         A.gram_off = 0;
         A.pair_off = A.tiles_bytes;
-        tail_end = (size_t)A.lo_off + read_end;
+        tail_end = (size_t)(tf32 ? hi_bytes : 0) + read_end;
         A.slot_cols = A.N_mma <= 64 ? 64 : 128;
         A.tm_cols = 2 * A.slot_cols;
         size_t half = std::max((pair_region / 2) / 4 * 4, ((size_t)A.per_l + 3 + 3) / 4 * 4);
@@ -1095,18 +908,15 @@ int power_spectrum_tc(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs,
     ExpArgs A = make_args(ctx, nullptr, nullptr, nullptr, nullptr, nullptr);
     A.N = (int)n_centres;
     A.c_in = d_coeffs;
-    const int mode = precision == RASCAL_PS_TF32X3 ? kGramTf32x3 : kGramBf16;
     size_t smem;
     int threads;
-    int st = make_gram(ctx, mode, layout, d_ps, A, &smem, &threads);  // also decides what is refused
+    int st = make_gram(ctx, kGramBf16, layout, d_ps, A, &smem, &threads, precision == RASCAL_PS_TF32X3);  // decides what is refused
     if (st) return st;
-    // the waits that the test hook makes run out are this kernel's; without it the kernel of power_spectrum.cu runs
-    if (!ctx->stall_polls) {
-        st = power_spectrum_warp(ctx, n_centres, d_coeffs, precision, layout, d_ps);
-        if (st != RASCAL_E_UNSUPPORTED) return st;
-    }
-    return mode == kGramTf32x3 ? launch_expansion<kGramTf32x3>(ctx, A, (int)n_centres, threads, smem)
-                               : launch_expansion<kGramBf16>(ctx, A, (int)n_centres, threads, smem);
+    // the waits that the test hook makes run out are the tcgen05 kernel's; without it the kernel of power_spectrum.cu runs
+    if (!ctx->stall_polls && power_spectrum_fits(ctx, precision, layout))
+        return power_spectrum_warp(ctx, n_centres, d_coeffs, precision, layout, d_ps);
+    if ((st = make_gram(ctx, kGramBf16, layout, d_ps, A, &smem, &threads))) return st;
+    return launch_expansion<kGramBf16>(ctx, A, (int)n_centres, threads, smem);
 }
 
 }  // namespace rascal
@@ -1201,28 +1011,22 @@ extern "C" int rascal_soap(rascal_ctx* ctx, const rascal_system* sys, const int6
     ExpArgs A = make_args(ctx, sys, d_offsets, d_nbr_j, d_rij, d_coeffs);
     const float* pre_D;
     if ((st = radial_precompute(ctx, sys, d_offsets, d_rij, false, &A.pre_G, &pre_D))) return st;
-    const int mode = precision == RASCAL_PS_FP32 ? kGramSimt : (precision == RASCAL_PS_BF16 ? kGramBf16 : kGramTf32x3);
+    const bool fp32 = precision == RASCAL_PS_FP32;
     const ExpArgs plain = A;
-    ExpArgs R = A;
-    size_t smem, smem_r;
-    int threads, threads_r;
-    // TF32x3: the tensor-core Gram in rounds of one l where the hypers fit it
-    const int st_r = precision == RASCAL_PS_TF32X3 ? make_gram(ctx, kGramRTf32, layout, d_ps, R, &smem_r, &threads_r)
-                                                  : RASCAL_E_UNSUPPORTED;
-    if (st_r != RASCAL_OK && st_r != RASCAL_E_UNSUPPORTED) return st_r;
-    clear_error();
-    if (st_r && (st = make_gram(ctx, mode, layout, d_ps, A, &smem, &threads))) return st;
+    size_t smem;
+    int threads;
+    if ((st = make_gram(ctx, fp32 ? kGramSimt : kGramBf16, layout, d_ps, A, &smem, &threads, precision == RASCAL_PS_TF32X3))) return st;
+    if (fp32) return launch_shaped<kGramSimt>(ctx, A, sys->n_atoms, threads, smem);
     // The tensor-core precisions as two launches, coefficients and the spectrum kernel of stored coefficients: 13 440 centres of
     // 25 pairs (12, 9, 4) BF16 564 -> 357 us and TF32x3 698 -> 417, of 2 species (8, 6) 301 -> 119 and 414 -> 125, of 30 pairs (9,
-    // 7, 3) 528 -> 239 and 551 -> 256, 200 centres 24 -> 22 and 27 -> 23; TF32x3 errors 4.8e-7 -> 1.2e-7. The one-launch forms
-    // wait for a chain of barriers and MMAs per l; they serve what the spectrum kernel does not take, and the test hook
-    // that makes their waits run out.
-    if (mode != kGramSimt && !ctx->stall_polls && power_spectrum_fits(ctx, precision, layout)) {
+    // 7, 3) 528 -> 239 and 551 -> 256, 200 centres 24 -> 22 and 27 -> 23; TF32x3 errors 4.8e-7 -> 1.2e-7. The one-launch tcgen05
+    // form waits for a chain of barriers and MMAs per l; it serves the BF16 bases that the spectrum kernel does not take, and the
+    // test hook that makes its wait run out (whose outputs are incomplete in either precision).
+    if (!ctx->stall_polls && power_spectrum_fits(ctx, precision, layout)) {
         if ((st = coefficients(ctx, sys, plain))) return st;
         return power_spectrum_warp(ctx, sys->n_atoms, d_coeffs, precision, layout, d_ps);
     }
-    if (!st_r) return launch_expansion<kGramRTf32>(ctx, R, sys->n_atoms, threads_r, smem_r);
-    if (mode == kGramSimt) return launch_shaped<kGramSimt>(ctx, A, sys->n_atoms, threads, smem);
-    if (mode == kGramBf16) return launch_expansion<kGramBf16>(ctx, A, sys->n_atoms, threads, smem);
-    return launch_expansion<kGramTf32x3>(ctx, A, sys->n_atoms, threads, smem);
+    A = plain;
+    if ((st = make_gram(ctx, kGramBf16, layout, d_ps, A, &smem, &threads))) return st;
+    return launch_expansion<kGramBf16>(ctx, A, sys->n_atoms, threads, smem);
 }
