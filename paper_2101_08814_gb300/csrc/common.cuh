@@ -106,6 +106,14 @@ struct ExpPlan {
     size_t smem;      // dynamic shared memory of the expansion kernel
 };
 
+// One way to launch k_power_spectrum (power_spectrum.cu): l blocks of a staging half, threads, floats of a half and of a row of c,
+// bytes of shared memory
+struct PsPlan {
+    int n_half, threads, half, pitch;
+    size_t smem;
+};
+constexpr int kPsPlans = 9;  // for one to eight centres per SM, and more
+
 }  // namespace rascal
 
 struct rascal_ctx {
@@ -157,6 +165,7 @@ struct rascal_ctx {
     int n_pstasks;
     unsigned* d_psitems;  // Gram items of power_spectrum.cu: warp tiles, then thread tiles PACKED and FULL, each by falling l
     int n_psitems[3];     // of each kind per l
+    rascal::PsPlan ps_plan[3][2][rascal::kPsPlans];  // by precision, layout and centres per SM
 
     // MLP surrogate of the radial integrals (mlp.cu); mlp_params == NULL until parameters are set
     float* mlp_params;   // FP32 master parameters

@@ -26,7 +26,8 @@
 
 namespace rascal {
 
-constexpr int kPsThreads = 256;
+constexpr int kPsThreads = 256;     // of k_power_spectrum_direct, and of k_power_spectrum at first (ps_plan)
+constexpr int kPsMaxThreads = 512;  // of k_power_spectrum (64 registers)
 constexpr int kPsStage = 7168;  // floats of the two staging halves (28 KB: four CTAs per SM at the batch hypers)
 constexpr int kPsOff = 4;       // 8-column blocks left of the diagonal in one item
 
@@ -252,7 +253,7 @@ __device__ __forceinline__ void ps_thread_tile(const float* C, int pitch, int Q,
 }
 
 template <int PREC, bool FULL>
-__global__ void __launch_bounds__(kPsThreads, 4) k_power_spectrum(const PsArgs A) {
+__global__ void __launch_bounds__(kPsMaxThreads, 2) k_power_spectrum(const PsArgs A) {
     extern __shared__ __align__(16) float sm[];
     __shared__ int s_next[kMaxLMax + 1];  // next item of each group
     const int Q = A.Q, L1 = A.l_max + 1, n_lm = L1 * L1, pitch = A.pitch, tid = threadIdx.x, lane = tid & 31, nthr = blockDim.x;
@@ -376,6 +377,8 @@ static int ps_set_attr() {
     return RASCAL_OK;
 }
 
+static void ps_plan(const rascal_ctx* ctx, int precision, int layout, int per_sm, PsPlan& P);
+
 int power_spectrum_setup(rascal_ctx* ctx) {
     const int Q4 = (ctx->Q + 3) / 4;
     std::vector<int> tasks;  // of the fused kernel's Gram
@@ -389,6 +392,9 @@ int power_spectrum_setup(rascal_ctx* ctx) {
         for (int l = ctx->l_max; l >= 0; --l) kind == 0 ? ps_warp_items(ctx->Q, l, items) : ps_thread_items(ctx->Q, l, kind == 2, items);
         ctx->n_psitems[kind] = (int)((items.size() - before) / (ctx->l_max + 1));
     }
+    for (int p = 0; p < 3; ++p)
+        for (int layout = 0; layout < 2; ++layout)
+            for (int k = 0; k < kPsPlans; ++k) ps_plan(ctx, p, layout, k + 1 < kPsPlans ? k + 1 : 64, ctx->ps_plan[p][layout][k]);
     RASCAL_CUDA(cudaMalloc(&ctx->d_pstasks, sizeof(int) * tasks.size()));
     RASCAL_CUDA(cudaMalloc(&ctx->d_psitems, sizeof(unsigned) * items.size()));
     RASCAL_CUDA(cudaMemcpyAsync(ctx->d_pstasks, tasks.data(), sizeof(int) * tasks.size(), cudaMemcpyHostToDevice, ctx->stream));
@@ -400,51 +406,75 @@ int power_spectrum_setup(rascal_ctx* ctx) {
     return RASCAL_OK;
 }
 
-// Sizes of a launch of k_power_spectrum, without its pointers; false where a centre does not fit its shared memory
-static bool ps_plan(const rascal_ctx* ctx, int precision, int layout, PsArgs& A, size_t* smem) {
+// How k_power_spectrum is launched for per_sm centres per SM: kPsStage floats of staging and 256 threads at first. Groups of few
+// items leave an SM half empty in wide bases (one l of Q = 60, PACKED FP32: 72 threads of a CTA) and in small batches, whose
+// single CTA per SM then runs l by l. There the staging grows to the l blocks, and the CTA to the threads, that put most threads
+// to work, in larger batches up to half of the l blocks only (what a group stores has to overlap the next one's tiles: whole
+// centres at once made 4 000 of Q = 36, l_max 8, FULL 72 -> 93 us), and only where fewer than 480 (tensor cores 448) are at
+// work on an SM. Before -> so, 4 000 centres PACKED FP32: (Q 60, l_max 15) 615 -> 342 us, (128, 4) 235 -> 172, (96, 15) 1 212 ->
+// 653; one centre: (64, 12) 31 -> 12, TF32x3 FULL (48, 9) 26 -> 13.
+static void ps_plan(const rascal_ctx* ctx, int precision, int layout, int per_sm, PsPlan& P) {
     const int Q = ctx->Q, L1 = ctx->l_max + 1;
+    const bool full = layout == RASCAL_LAYOUT_FULL, fp32 = precision == RASCAL_PS_FP32;
+    const int per_l = full ? Q * Q : Q * (Q + 1) / 2, pitch = ps_pitch(ctx->n_lm, precision);
+    const int items = ctx->n_psitems[!fp32 ? 0 : (full ? 2 : 1)] * (fp32 ? 1 : 32);  // threads that an l occupies
+    const int rows = fp32 ? (Q + 7) / 8 * 8 : (Q + 15) / 16 * 16;  // of c that edge tiles read
+    auto plan = [&](int n, int threads) {
+        // a staging half: a block of l each, three floats more for a start that matches its target's alignment
+        const int half = (n * per_l + 3 + 3) / 4 * 4;
+        return PsPlan{n, threads, half, pitch, sizeof(float) * ((size_t)2 * half + (size_t)rows * pitch + 32)};
+    };
+    // threads at work: of one CTA, the items of a group over the rounds that they take (FP32: dealt in rounds; else the warps take
+    // them as they come free), and of an SM, on average over the waves of its `centres` CTAs
+    auto fit = [&](const PsPlan& p) { return std::min({(int)(227 * 1024 / (p.smem + 1024)), 1024 / p.threads, 32}); };
+    auto busy = [&](const PsPlan& p, int centres) {
+        const int n = p.n_half * items, one = fp32 ? n / ((n + p.threads - 1) / p.threads) : std::min(n, p.threads);
+        return centres * one / ((centres + fit(p) - 1) / fit(p));
+    };
+    const int n0 = std::max(1, std::min(L1, (kPsStage / 2 - 3) / per_l));
+    P = plan(n0, std::min(kPsThreads, (int)align_up(n0 * items, 32)));
+    if (P.smem > 220 * 1024 || (per_sm > 2 && busy(P, fit(P)) >= (fp32 ? 480 : 448))) return;
+    PsPlan best = P;
+    for (int n = 1; n <= (per_sm > 4 ? std::max(1, L1 / 2) : L1); ++n) {
+        const int rounds = (n * items + kPsMaxThreads - 1) / kPsMaxThreads;
+        const PsPlan p = plan(n, (int)align_up((n * items + rounds - 1) / rounds, 32));
+        if (p.smem <= 220 * 1024 && busy(p, per_sm) > busy(best, per_sm)) best = p;
+    }
+    if (busy(best, per_sm) * 10 > busy(P, per_sm) * 13) P = best;
+}
+
+bool power_spectrum_fits(const rascal_ctx* ctx, int precision, int layout) {
+    return ctx->ps_plan[precision][layout][0].smem <= 220 * 1024;
+}
+
+int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps) {
     const bool full = layout == RASCAL_LAYOUT_FULL;
+    const int Q = ctx->Q, L1 = ctx->l_max + 1;
+    int k = 0;
+    while (k + 1 < kPsPlans && n_centres > (k + 1LL) * ctx->n_sm) ++k;
+    const PsPlan& P = ctx->ps_plan[precision][layout][k];
+    if (P.smem > 220 * 1024) return RASCAL_E_UNSUPPORTED;
+    PsArgs A;
+    A.c = d_coeffs;
+    A.ps = d_ps;
     A.Q = Q;
     A.l_max = ctx->l_max;
     A.per_l = full ? Q * Q : Q * (Q + 1) / 2;
     A.ps_stride = (int64_t)L1 * A.per_l;
     A.ps_norm = ctx->ps_norm;
-    A.pitch = ps_pitch(ctx->n_lm, precision);
+    A.pitch = P.pitch;
     const int kind = precision != RASCAL_PS_FP32 ? 0 : (full ? 2 : 1);
     A.items_per_l = ctx->n_psitems[kind];
     A.items = ctx->d_psitems;
-    for (int k = 0; k < kind; ++k) A.items += (int64_t)ctx->n_psitems[k] * L1;
-    // staging halves: a block of l each at least, three floats more for a start that matches its target's alignment
-    A.n_half = std::max(1, std::min(L1, (kPsStage / 2 - 3) / A.per_l));
-    A.half = (A.n_half * A.per_l + 3 + 3) / 4 * 4;
-    const int rows = std::max((Q + 15) / 16 * 16, (Q + 7) / 8 * 8);
-    *smem = sizeof(float) * ((size_t)2 * A.half + (size_t)rows * A.pitch + 32);
-    return *smem <= 220 * 1024;
-}
-
-bool power_spectrum_fits(const rascal_ctx* ctx, int precision, int layout) {
-    PsArgs A;
-    size_t smem;
-    return ps_plan(ctx, precision, layout, A, &smem);
-}
-
-int power_spectrum_warp(rascal_ctx* ctx, int64_t n_centres, const float* d_coeffs, int precision, int layout, float* d_ps) {
-    const bool full = layout == RASCAL_LAYOUT_FULL;
-    PsArgs A;
-    size_t smem;
-    if (!ps_plan(ctx, precision, layout, A, &smem)) return RASCAL_E_UNSUPPORTED;
-    A.c = d_coeffs;
-    A.ps = d_ps;
-    A.copy16 = A.pitch == ctx->n_lm && A.Q * ctx->n_lm % 4 == 0 && (reinterpret_cast<uintptr_t>(d_coeffs) & 15) == 0;
+    for (int e = 0; e < kind; ++e) A.items += (int64_t)ctx->n_psitems[e] * L1;
+    A.n_half = P.n_half;
+    A.half = P.half;
+    A.copy16 = A.pitch == ctx->n_lm && Q * ctx->n_lm % 4 == 0 && (reinterpret_cast<uintptr_t>(d_coeffs) & 15) == 0;
     auto kernel = precision == RASCAL_PS_BF16 ? (full ? k_power_spectrum<RASCAL_PS_BF16, true> : k_power_spectrum<RASCAL_PS_BF16, false>)
                   : precision == RASCAL_PS_TF32X3
                       ? (full ? k_power_spectrum<RASCAL_PS_TF32X3, true> : k_power_spectrum<RASCAL_PS_TF32X3, false>)
                       : (full ? k_power_spectrum<RASCAL_PS_FP32, true> : k_power_spectrum<RASCAL_PS_FP32, false>);
-    // no more threads than the largest group has tiles for (FP32) or warps than it has items: a small basis leaves the rest of
-    // the SM to other centres (Q = 16, l_max 6, 4 096 centres, FP32: 24 us with 256 threads, 21 us with 64)
-    const int items = A.n_half * A.items_per_l;
-    const int threads = std::min(kPsThreads, precision == RASCAL_PS_FP32 ? (int)align_up(items, 32) : 32 * items);
-    kernel<<<(unsigned)n_centres, threads, smem, ctx->stream>>>(A);
+    kernel<<<(unsigned)n_centres, P.threads, P.smem, ctx->stream>>>(A);
     RASCAL_LAUNCH_CHECK("k_power_spectrum");
     return RASCAL_OK;
 }
