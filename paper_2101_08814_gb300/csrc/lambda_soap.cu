@@ -121,12 +121,14 @@ static void lsoap_pairs(int l_max, int lam, std::vector<int2>& p) {
 // Bound: HBM (the output). 9 001 centres, Q = 48, l_max 9, lambda 1: 1 017 us with 2 x 4 tiles that loaded one value of X
 // per two products (issue-bound, 83 % issue-active); 718 us with 4 x 4 tiles (shared-memory loads 74 % of their rate);
 // 637 us = 3.8 TB/s in this form. Four CTAs of 128 threads per SM hide the barriers better than two of 256
-// (692 against 844 us with runtime pitches).
+// (692 against 844 us with runtime pitches). Where an SM has one or two CTAs at most the pairs follow each other with nothing
+// to hide their latency: there a CTA has 256 threads (G = 1) and asks for a thread's first table entry of the next pair before
+// it makes this one's tiles (kLsoapPrefetch below).
 constexpr int kLsoapThreads = 128, kLsoapCtas = 4;
 constexpr int kLsoapGroups = 36;  // row groups per chunk: X takes 11.5 KB (PX = 20) or 20.7 KB (PX = 36) per buffer
 
-template <bool VEC, int PX, int G>
-__global__ void __launch_bounds__(kLsoapThreads, G == 1 ? 6 : kLsoapCtas) k_lambda_soap(const float* __restrict__ c, int Q, int l_max, int lam,
+template <bool VEC, int PX, int G, int T>
+__global__ void __launch_bounds__(T, T > kLsoapThreads ? 2 : (G == 1 ? 6 : kLsoapCtas)) k_lambda_soap(const float* __restrict__ c, int Q, int l_max, int lam,
                                                                            int chunk, unsigned qt_inv, int n_pairs,
                                                                            const int4* __restrict__ hdr,
                                                                            const float4* __restrict__ R,
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kLsoapThreads, G == 1 ? 6 : kLsoapCtas) k_lamb
     float* C = sm;                           // [QT][gs]
     float* sX = C + QT * gs;                 // two buffers [chunk][4][PX]
     const float* ci = c + i * Q * n_lm;
-    for (int e = tid; e < QT * gs / 4; e += kLsoapThreads) reinterpret_cast<float4*>(C)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int e = tid; e < QT * gs / 4; e += T) reinterpret_cast<float4*>(C)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     auto div_qt = [&](int x) { return QT == 1 ? x : (int)__umulhi((unsigned)x, qt_inv); };  // x / QT, exact for x < 65536
     __syncthreads();
     {
@@ -147,24 +149,31 @@ __global__ void __launch_bounds__(kLsoapThreads, G == 1 ? 6 : kLsoapCtas) k_lamb
             const int l = (int)sqrtf((float)lm);
             float* slot = C + exp_lp(l) + lm - l * l;
 #pragma unroll 4
-            for (int q = warp; q < Q; q += kLsoapThreads / 32) {
+            for (int q = warp; q < Q; q += T / 32) {
                 const int v = VEC ? q & 3 : div_qt(q), g = VEC ? q >> 2 : q - v * QT;
                 slot[g * gs + v * pitch] = __ldg(ci + q * n_lm + lm);
             }
         }
     }
     // output tiling (fixed for the kernel): each thread owns one column group and a stride of row groups
-    const int t_r = div_qt(tid), t_c = tid - t_r * QT, r_step = div_qt(kLsoapThreads);
+    const int t_r = div_qt(tid), t_c = tid - t_r * QT, r_step = div_qt(T);
     const bool t_on = t_r < r_step;
     const int64_t pair_floats = (int64_t)(2 * lam + 1) * Q * Q;
     float* op = out + i * n_pairs * pair_floats + (VEC ? 4 * t_c : t_c);
     const int x_floats = chunk * 4 * PX;
     int cur = 0;  // offset of the X buffer in use
     int4 h = __ldg(hdr);
+    constexpr bool kLsoapPrefetch = T > 128;
+    float4 e0 = make_float4(0.f, 0.f, 0.f, 0.f);  // this thread's first entry of the pair to come
+    auto fetch = [&](const int4& n) {
+        const int d2 = n.w & 63, dp = (d2 + 3) & ~3, r = (tid * (n.w >> 6)) >> 16, col = tid - r * dp;
+        if (col < d2 && r < min(chunk, groups)) e0 = __ldg(R + n.z + col + div_qt(r) * d2);
+    };
+    if (kLsoapPrefetch) fetch(h);
     __syncthreads();
     for (int p = 0; p < n_pairs; ++p, op += pair_floats) {
         const int d2 = h.w & 63, dp = (d2 + 3) & ~3, inv = h.w >> 6;  // inv = ceil(65536 / dp)
-        const int b_r = (tid * inv) >> 16, b_c = tid - b_r * dp, b_s = (kLsoapThreads * inv) >> 16;
+        const int b_r = (tid * inv) >> 16, b_c = tid - b_r * dp, b_s = (T * inv) >> 16;
         const float4* Rp = R + h.z + b_c;
         const float* A = C + h.x;
         const float* Bt = C + h.y + t_c * gs;
@@ -178,7 +187,8 @@ __global__ void __launch_bounds__(kLsoapThreads, G == 1 ? 6 : kLsoapCtas) k_lamb
                     const int u = div_qt(g0 + r);
                     float w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                     if (b_c < d2) {
-                        const float4 e = __ldg(Rp + u * d2);  // the two non-zero m1 of this (mu, m2)
+                        // the two non-zero m1 of this (mu, m2)
+                        const float4 e = kLsoapPrefetch && g0 == 0 && r == b_r ? e0 : __ldg(Rp + u * d2);
                         const float* ag = A + (g0 + r - u * QT) * gs;
                         const float* a0 = ag + __float_as_int(e.z);
                         const float* a1 = ag + __float_as_int(e.w);
@@ -190,6 +200,7 @@ __global__ void __launch_bounds__(kLsoapThreads, G == 1 ? 6 : kLsoapCtas) k_lamb
                     for (int v = 0; v < 4; ++v) x[v * PX] = w[v];
                 }
             }
+            if (kLsoapPrefetch && g0 + chunk >= groups) fetch(h);
             __syncthreads();
             if (!t_on) continue;
             const int half = G == 2 ? (ng + 1) >> 1 : ng;  // a thread's row groups: r and, with G = 2, r + half, if there is one
@@ -263,20 +274,25 @@ static int lsoap_px(int l_max) { return l_max <= 9 ? 20 : 36; }
 // Row groups of a thread's tiles: one where a chunk's 4 x 4 tiles do not exceed the threads (small bases, small ranks), else two;
 // with one, six CTAs per SM (78 registers). Two groups (and 2 x 4 tiles) -> one: 4 000 centres, Q = 15, l_max 9, lambda 0 106
 // (100) -> 72 us; 9 000 centres, Q = 21, l_max 3, lambda 1 90 (167) -> 72 us; 5 000 centres, Q = 12, l_max 4, lambda 0 53 (45) ->
-// 37 us. Past the line two groups win: 3 000 centres, Q = 30, l_max 5, lambda 1 62 against 70 us.
-static bool lsoap_small(int Q, int lam) {
+// 37 us. Past the line two groups win (3 000 centres, Q = 30, l_max 5, lambda 1 62 against 70 us), but for pairs of a few m, which
+// are over before two groups pay (5 000 centres, l_max 1: Q = 60, lambda 1 52 -> 47 us, Q = 36, lambda 2 43 -> 37), and, to l_max 4,
+// for batches that four CTAs per SM leave a few centres of and six do not (700 centres: Q = 20, l_max 4, lambda 4 41 -> 31 us, Q = 60,
+// l_max 2, lambda 2 45 -> 39; l_max 8 loses 7 %).
+static bool lsoap_small(int Q, int l_max, int lam) {
     const int QT = (Q + 3) / 4;
-    return std::min((2 * lam + 1) * QT, kLsoapGroups) * QT <= kLsoapThreads;
+    return l_max <= 1 || std::min((2 * lam + 1) * QT, kLsoapGroups) * QT <= kLsoapThreads;
 }
+enum LsoapForm { kLsoapTwo, kLsoapOne, kLsoapAlone };  // row groups per thread, or the form for one or two CTAs to an SM
 
-template <int G>
+template <int G, int T>
 static auto lsoap_kernel_of(int Q, int l_max) {
     const bool vec = Q % 4 == 0;
-    return lsoap_px(l_max) == 20 ? (vec ? k_lambda_soap<true, 20, G> : k_lambda_soap<false, 20, G>)
-                                 : (vec ? k_lambda_soap<true, 36, G> : k_lambda_soap<false, 36, G>);
+    return lsoap_px(l_max) == 20 ? (vec ? k_lambda_soap<true, 20, G, T> : k_lambda_soap<false, 20, G, T>)
+                                 : (vec ? k_lambda_soap<true, 36, G, T> : k_lambda_soap<false, 36, G, T>);
 }
-static auto lsoap_kernel(int Q, int l_max, int lam) {
-    return lsoap_small(Q, lam) ? lsoap_kernel_of<1>(Q, l_max) : lsoap_kernel_of<2>(Q, l_max);
+static auto lsoap_kernel(int Q, int l_max, LsoapForm form) {
+    return form == kLsoapAlone ? lsoap_kernel_of<1, 2 * kLsoapThreads>(Q, l_max)
+                               : (form == kLsoapOne ? lsoap_kernel_of<1, kLsoapThreads>(Q, l_max) : lsoap_kernel_of<2, kLsoapThreads>(Q, l_max));
 }
 
 int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const float4** R) {
@@ -315,8 +331,10 @@ int lsoap_table(rascal_ctx* ctx, int lam, int* n_pairs, const int4** hdr, const 
         LsoapTable* t = new LsoapTable();
         t->lambda = lam;
         t->n_pairs = (int)P.size();
-        cudaError_t e = cudaFuncSetAttribute(lsoap_kernel(ctx->Q, ctx->l_max, lam), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             227 * 1024);
+        cudaError_t e = cudaSuccess;
+        for (LsoapForm f : {kLsoapTwo, kLsoapOne, kLsoapAlone})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(lsoap_kernel(ctx->Q, ctx->l_max, f), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e == cudaSuccess) e = cudaMalloc(&t->d_hdr, sizeof(int4) * std::max<size_t>(1, h.size()));
         if (e == cudaSuccess) e = cudaMalloc(&t->d_R, sizeof(float4) * std::max<size_t>(1, all.size()));
         if (e == cudaSuccess && !h.empty())
@@ -398,7 +416,14 @@ extern "C" int rascal_lambda_soap(rascal_ctx* ctx, int64_t n_centres, const floa
     int chunk = std::min((2 * lambda + 1) * QT, kLsoapGroups);
     while (chunk > 6 && sizeof(float) * (c_floats + (size_t)2 * 4 * chunk * px) > 227 * 1024) --chunk;
     const size_t smem = sizeof(float) * (c_floats + (size_t)2 * 4 * chunk * px);
-    lsoap_kernel(ctx->Q, ctx->l_max, lambda)<<<(unsigned)n_centres, kLsoapThreads, smem, ctx->stream>>>(
+    const int64_t fit = 228 * 1024 / (smem + 1024), sms = ctx->n_sm;
+    LsoapForm form = lsoap_small(ctx->Q, ctx->l_max, lambda) ? kLsoapOne : kLsoapTwo;
+    if (ctx->l_max <= 4 && n_centres > std::min<int64_t>(fit, kLsoapCtas) * sms && n_centres <= std::min<int64_t>(fit, 6) * sms) form = kLsoapOne;
+    // small batches, bases that leave room for no more CTAs: one centre of Q = 2, l_max 15, lambda 4 68 -> 45 us, Q = 20, lambda 2
+    // 67 -> 43; 1 500 centres of Q = 100, l_max 12, lambda 1 1 257 -> 1 018
+    if (n_centres <= 2 * sms || fit <= 2) form = kLsoapAlone;
+    const int threads = form == kLsoapAlone ? 2 * kLsoapThreads : kLsoapThreads;
+    lsoap_kernel(ctx->Q, ctx->l_max, form)<<<(unsigned)n_centres, threads, smem, ctx->stream>>>(
         d_coeffs, ctx->Q, ctx->l_max, lambda, chunk, (unsigned)((0x100000000ull + QT - 1) / QT), np, hdr, R, d_out);
     RASCAL_LAUNCH_CHECK("k_lambda_soap");
     return RASCAL_OK;
