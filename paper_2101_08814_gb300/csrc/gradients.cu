@@ -187,13 +187,19 @@ struct GradShape {
 
 // Rows of chat_l for l in [l0, l1) from staged packed symmetric blocks (pitch Wp, odd: lanes of different l read different
 // banks): a warp takes R rows q, its lanes the 4-column tiles of the padded rows of C. Whether k lies before, in or past the
-// rows, and with it where W[q][k] sits in the packed block, is the same for the whole warp.
-template <int R, class Shape, class Put>
+// rows, and with it where W[q][k] sits in the packed block, is the same for the whole warp. SPLIT, where the staged l have fewer
+// tiles than lanes (small l_max; wide bases, of which few blocks fit at a time) and the rows are more than one round of the
+// warps: 2^s sets of rows to a warp, as many as leave every warp some (3 000 centres with 24 pairs: (16, 8, 8) 6 489 -> 1 108 us
+// with the larger groups below, (12, 0, 8) 260 -> 78). An instance of its own: beside the plain form it cost that one 2 %.
+template <int R, bool SPLIT, class Shape, class Put>
 __device__ __forceinline__ void adjoint_rows(const Shape& K, const float* s_C, const float* s_W, int Wp, int l0, int l1, int ps_norm,
                                              Put put) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, Q = K.Q, Lq = K.LpAdj;
-    for (int q0 = R * warp; q0 < Q; q0 += R * nwarps) {
-        for (int t = exp_lp(l0) / 4 + lane; t < exp_lp(l1) / 4; t += 32) {
+    int s = 0;
+    while (SPLIT && s < 5 && exp_lp(l1) / 4 - exp_lp(l0) / 4 <= 16 >> s && (R * nwarps << s) < Q) ++s;
+    const int across = 32 >> s;
+    for (int q0 = R * ((warp << s) + lane / across); q0 < Q; q0 += R * nwarps << s) {
+        for (int t = exp_lp(l0) / 4 + lane % across; t < exp_lp(l1) / 4; t += across) {
             int l = l0;
             while (exp_lp(l + 1) <= 4 * t) ++l;
             const float* W = s_W + (l - l0) * Wp;
@@ -257,7 +263,7 @@ __device__ __forceinline__ void adjoint_rows(const Shape& K, const float* s_C, c
 // Per-centre dE/dp: with each l block expanded to a dense matrix in turn, two barriers and 12 to 60 tile tasks per l, the
 // adjoint was 640 us of the kernel's 818 on 8 960 centres (n_max 12, l_max 9, 4 species); all packed blocks staged at once
 // and read as they are, 240 of 557 (0.42 GB of dE/dp: 63 us).
-enum { kLinear = 1, kPerCentre = 2, kPerElement = 4 };
+enum { kLinear = 1, kPerCentre = 2, kPerElement = 4, kSplitRows = 8 };
 template <int SHAPE, int W, class Put>
 __device__ __forceinline__ float adjoint(const GradArgs& A, const GradShape<SHAPE>& K, int i, int a_i, float* s_C, float* s_W, Put put) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -348,10 +354,12 @@ __device__ __forceinline__ float adjoint(const GradArgs& A, const GradShape<SHAP
                     for (int e = tid; e < Qpk; e += blockDim.x) cp_async4(s_W + (l - l0) * Wp + e, Gp + (int64_t)l * Qpk + e);
                 cp_async_wait_all();
                 __syncthreads();
-                if (A.w_rows == 6)
-                    adjoint_rows<6>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
+                if (W & kSplitRows)
+                    adjoint_rows<4, true>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
+                else if (A.w_rows == 6)
+                    adjoint_rows<6, false>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
                 else
-                    adjoint_rows<4>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
+                    adjoint_rows<4, false>(K, s_C, s_W, Wp, l0, l1, A.ps_norm, put);
             }
         }
         return dot;
@@ -945,6 +953,8 @@ static const GradKernel kGradKernels[2][2][5] = {
       k_gradients<3, kPerCentre, 256>, k_gradients<4, kPerCentre, 256>}},
     {{k_gradients<0, kLinear, 128>, nullptr, nullptr, k_gradients<3, kLinear, 128>, nullptr},
      {k_gradients<0, kPerCentre, 128>, nullptr, nullptr, k_gradients<3, kPerCentre, 128>, nullptr}}};
+constexpr int kSplitGrad = kPerCentre | kSplitRows;
+static const GradKernel kSplitKernels[3] = {k_gradients<0, kSplitGrad, 256>, k_gradients<4, kSplitGrad, 256>, k_gradients<0, kSplitGrad, 128>};
 static_assert(kNumExpShapes == 5, "an instance per shape");
 
 int gradients_setup(rascal_ctx* ctx) {
@@ -955,6 +965,8 @@ int gradients_setup(rascal_ctx* ctx) {
         for (int w = 0; w < 2; ++w)
             for (GradKernel k : kGradKernels[t][w])
                 if (k) RASCAL_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    for (GradKernel k : kSplitKernels)
+        RASCAL_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     return RASCAL_OK;
 }
 
@@ -1050,10 +1062,14 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     const int per_sm = d_weights ? 8 : 6;
     const bool small = grad_chain_smem(ctx, 128, true, d_weights ? 0 : L1) <= 226 * 1024 / per_sm - 2 * 1024;
     const int threads = small ? 128 : 256;
-    // a per-centre dE/dp: all its l blocks staged at once where two CTAs per SM still fit, else as many as fit
+    // a per-centre dE/dp: all its l blocks staged at once where two CTAs per SM still fit, else as many as fit (two CTAs, or one
+    // where one block leaves room for no more). Wide bases of a few l read it from global memory (an output per thread): 3 000
+    // centres of Q = 128, l_max 0 181 -> 101 us, l_max 2 486 -> 344.
     A.w_lg = d_weights ? 0 : L1;
-    while (A.w_lg > 1 && grad_chain_smem(ctx, threads, true, A.w_lg) > 112 * 1024) --A.w_lg;
+    const size_t room = (!d_weights && grad_chain_smem(ctx, threads, true, 1) > 112 * 1024 ? 220 : 112) * 1024;
+    while (A.w_lg > 1 && grad_chain_smem(ctx, threads, true, A.w_lg) > room) --A.w_lg;
     if (A.w_lg && grad_chain_smem(ctx, threads, true, A.w_lg) > 220 * 1024) A.w_lg = 0;
+    if (ctx->Q > 96 && ctx->l_max <= 2) A.w_lg = 0;
     size_t smem = grad_chain_smem(ctx, threads, A.wsym || A.w_lg, A.w_lg);
     const bool chains = smem <= 220 * 1024;  // all but the widest bases (about n_species n_max (l_max + 1)^2 > 24 500)
     {  // rows of a warp: the fewest rounds x (loads of a step)
@@ -1100,6 +1116,9 @@ static int gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
     if (chains) {
         GradKernel kernel = kGradKernels[small][d_weights ? 0 : 1][shape];
         if (!kernel) kernel = kGradKernels[small][d_weights ? 0 : 1][0];
+        bool split = false;  // a group of l with fewer tiles than half a warp's lanes
+        for (int l = 0; l < L1 && A.w_lg; l += A.w_lg) split = split || exp_lp(std::min(L1, l + A.w_lg)) - exp_lp(l) <= 4 * 16;
+        if (split && ctx->Q > 4 * threads / 32) kernel = kSplitKernels[small ? 2 : (shape == 4 ? 1 : 0)];
         kernel<<<sys->n_atoms, threads, smem, ctx->stream>>>(A);
     } else {
         k_gradients_wide<<<sys->n_atoms, kGradThreads, smem, ctx->stream>>>(A);

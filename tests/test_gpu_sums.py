@@ -5,6 +5,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 from synth import System  # noqa: E402
+from tests.test_gpu_tiles import test_gradient_chunks as gradient_chunks  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -75,3 +76,11 @@ def test_gpr_energies_repeat(rg, sizes):
     for k in range(n):
         atoms = ea[off[k]:off[k + 1]]
         assert abs(e[k].item() - atoms.sum()) <= len(atoms) * 2.0 ** -53 * np.abs(atoms).sum()
+
+
+# The adjoint of a per-centre dE/dp with several sets of rows to a warp: all l staged at once and groups of three and of one, CTAs of
+# 128 and of 256 threads, the compiled wide shape's neighbours; and wide bases of a few l, which read dE/dp from global memory. The
+# check and its bound are those of the other chunks.
+@pytest.mark.parametrize("n_max,l_max,S", [(16, 0, 3), (5, 3, 4), (9, 6, 4), (12, 2, 8), (12, 4, 8), (16, 8, 8), (16, 2, 8)])
+def test_split_rows(rg, n_max, l_max, S):
+    gradient_chunks(rg, n_max, l_max, S)
