@@ -20,10 +20,11 @@
  *   - c is float32 [n_centres][n_species][n_max][(l_max+1)^2] with lm = l*l + l + m, m = -l..l.
  *   - p PACKED is float32 [n_centres][l_max+1][Q(Q+1)/2], Q = n_species*n_max, pairs q1 <= q2 row-major;
  *     p FULL is float32 [n_centres][l_max+1][Q][Q].
- *   - Every device pointer argument ("d_") is caller-owned device memory; the library only borrows it for the
- *     duration of the call. The context owns the radial table, its scratch arena and the MLP weights.
+ *   - Every device pointer argument ("d_") is caller-owned device memory; the library only borrows it until the
+ *     work that the call enqueued is done. The context owns the radial table, its scratch arena and the MLP weights.
  *   - All work is enqueued on the context's CUDA stream. Calls that must read a count from the device
- *     (rascal_neighbours) synchronise that stream; the others return as soon as the work is enqueued.
+ *     (rascal_neighbours) wait for that count, not for the outputs they enqueue; the others return as soon as the
+ *     work is enqueued.
  *   - Every call returns RASCAL_OK (0) or a negative RASCAL_E_* status; rascal_last_error() then holds a
  *     message for the calling thread. No call aborts the process.
  */
@@ -191,7 +192,7 @@ int rascal_neighbours(rascal_ctx* ctx, const rascal_system* sys, int64_t capacit
  *     than 256 neighbours (rascal_neighbours sorts those in an allocated overflow buffer) is also refused with
  *     RASCAL_E_UNSUPPORTED, but only once the counting pass has run: d_offsets and *n_pairs are then already
  *     written, and this check comes before the capacity check.
- * Synchronises the stream once, like rascal_neighbours. */
+ * Waits for the pair count once, like rascal_neighbours; the fill is enqueued after it, only when the call succeeds. */
 int rascal_neighbours_noalloc(rascal_ctx* ctx, const rascal_system* sys, int64_t capacity, int64_t* d_offsets,
                               int* d_nbr_j, int* d_shift, float* d_rij, int64_t* n_pairs);
 /* Size in bytes of the device array that rascal_neighbours_noalloc uses for scratch. */
@@ -255,6 +256,7 @@ int rascal_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d
 
 /* The linear model from the coefficients alone: forces and virial as rascal_gradients with d_weights, and the energies
  * of rascal_linear_energy as half the product of dE_i/dc_i and c_i (E_i is quadratic in c_i), without a power spectrum.
+ * The two sums of one energy round differently: they agree to FP32 rounding of their terms, not bit for bit.
  *   d_energy [n_structures] float64: overwritten with sum_i w_{a_i} . p_i */
 int rascal_linear_gradients(rascal_ctx* ctx, const rascal_system* sys, const int64_t* d_offsets, const int* d_nbr_j,
                             const float* d_rij, const float* d_coeffs, const float* d_weights, double* d_energy,

@@ -3,7 +3,8 @@
 PowerSpectrumFunction: positions -> PACKED power spectrum p [N, F]; its backward receives dL/dp and returns
 dL/dpositions = -F computed by rascal_gradients (per-pair recomputation, no stored dc/dr).
 LinearSoapEnergy: the additive linear model E_s = sum_{i in s} w_{a_i} . p_i, with forces and virial from the
-backward kernel in one call.
+backward kernel in one call. With forces the energy is summed as half the adjoint times c, without them as w . p: the same
+number up to FP32 rounding, so the last digits of the two differ.
 """
 from __future__ import annotations
 

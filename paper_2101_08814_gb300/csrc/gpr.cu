@@ -154,8 +154,8 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
     constexpr int kParts = kKB / 16;
     constexpr int kMmaWarp = 2 * kGprProducers / 32;
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char* sA = smem;                                        // [stages][8 KB]
-    unsigned char* sB = sA + kGprStages * kGprATile;                 // [stages][COLS * 64 bytes]
+    unsigned char* sA = smem;                                        // [stages][128 rows of kRow bytes]
+    unsigned char* sB = sA + kGprStages * kGprATile;                 // [stages][COLS rows of kRow bytes]
     float* s_x = reinterpret_cast<float*>(sB + kGprStages * kGprB1);  // [COLS]
     float* s_inv = s_x + COLS;                                       // [128]
     float* s_E = s_inv + 128;                                        // [2][128]; [4][128] norm partials before
@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(kGprThreads1, 1) k_gpr_kernel(const __grid_con
 __global__ void __launch_bounds__(kGprThreads2, 2) k_gpr_grad(const __grid_constant__ GprArgs A) {
     constexpr int kKB = 32, kGprATile = 128 * 128;
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char* sA = smem;                                          // [stages][8 KB]
-    unsigned char* sB = sA + kGprStages2 * kGprATile;                  // [stages][8 KB]
+    unsigned char* sA = smem;                                          // [stages][16 KB]
+    unsigned char* sB = sA + kGprStages2 * kGprATile;                  // [stages][32 KB]
     int* s_atom = reinterpret_cast<int*>(sB + kGprStages2 * kGprB2);  // [128]
     float* s_inv = reinterpret_cast<float*>(s_atom + 128);             // [128] 1 / |p|
     float* s_c2 = s_inv + 128;                                         // [128] zeta E / |p|^2
@@ -711,8 +711,9 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// TMA map of a row-major FP32 matrix [rows][pitch] (cols used), boxes of 16 elements (64 bytes) x 64 rows written
-// with 64-byte swizzling (the operand layout of smem_desc_sw64); reads past the last row fill zeros
+// TMA map of a row-major FP32 matrix [rows][pitch] (cols used), in boxes of box_cols x box_rows elements:
+// 16 columns with 64-byte swizzling (the operand layout of smem_desc_sw64), 32 with 128-byte swizzling (smem_desc_sw128); reads
+// past the last row fill zeros
 static int tmap_2d(CUtensorMap* m, const float* base, uint64_t cols, uint64_t rows, uint64_t pitch, uint32_t box_cols, uint32_t box_rows) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
     if (!fn) return set_error(RASCAL_E_CUDA, "cuTensorMapEncodeTiled is not available from the CUDA driver library");

@@ -1,6 +1,6 @@
 // Periodic cell-list neighbour search (Appendix B: every j, including periodic replicas, with r_ji < r_cut).
 //
-// Pipeline (all on the context stream; seven launches and one synchronisation, which reads the pair count):
+// Pipeline (all on the context stream; seven launches, ten from 131 073 atoms on, and one wait of the host, for the pair count):
 //   k_struct_setup  a warp or four lanes per structure: inverse cell, perpendicular widths, bins >= r_cut(1+1e-6) wide per axis; the
 //                   bin counters and the work list are cleared beside it
 //   k_atom_bin      per atom: fractional coordinates, wrap count w, bin, wrapped position p = r - w H split into FP32
@@ -43,7 +43,7 @@ struct StructInfo {
 
 constexpr int kPairWarps = 4;      // warps per block in k_pairs
 constexpr int kPairCap = 128;      // pairs a warp sorts in shared memory; larger segments use global scratch
-constexpr int kNoallocCap = 256;   // the same for rascal_neighbours_noalloc, which has no overflow scratch
+constexpr int kNoallocCap = 256;   // lists of up to as many take a second form; rascal_neighbours_noalloc has no other (no scratch)
 constexpr int kPairChunk = 768;    // candidates staged at a time
 constexpr int kPairEntries = 128;  // stencil bins handled at a time (one per thread)
 constexpr int kPairRec = 160;      // accepted candidates a warp collects before it works out their vectors

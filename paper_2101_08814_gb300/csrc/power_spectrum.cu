@@ -12,7 +12,7 @@
 //                 FMAs, m in order. A tile is made for every t2 mod H >= t1, which meets every unordered pair once.
 //                 Interleaved columns let lanes of neighbouring tiles write neighbouring words.
 // Bound: HBM (c in, p out). 20 000 centres, Q = 48, l_max 9, PACKED: BF16 813 -> 283 us (0.70 of HBM), TF32x3 1 454 -> 372 us
-// (error against 64 bits 6.4e-7 -> 1.9e-7: both parts of the split are rounded), FP32 573 -> 436 us, bit for bit (bound by its
+// (error against 64 bits 6.4e-7 -> 1.9e-7: the high part of the split is rounded, not cut off), FP32 573 -> 436 us, bit for bit (bound by its
 // shared-memory loads, 12 floats for 32 products); FULL: 1 253 -> 465, 2 014 -> 561, 1 391 -> 678 us.
 #include <cuda_bf16.h>
 
