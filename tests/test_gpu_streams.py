@@ -97,3 +97,27 @@ def test_a_captured_stream_takes_no_wait(rg):
     assert torch.equal(out, c)
     calc.neighbours(ds)
     calc.sync()
+
+
+# The no-allocation search's scratch is shared by all contexts of a device: a refused call leaves nothing queued that reads it, so
+# that the next search, on another stream and of another context, meets no fill of the refused one.
+def test_a_refused_search_leaves_nothing_behind(rg):
+    import torch
+
+    s = config_large()
+    other = System(s.positions[:20000] + 0.25, s.species[:20000], s.cells, s.pbc, np.array([0, 20000], np.int32), s.hypers)
+    calcs = [rg.SoapCalculator(**s.hypers) for _ in range(2)]
+    sets = [rg.DeviceSystem.from_numpy(x) for x in (s, other)]
+    ref = [_lists(c.neighbours(x)) for c, x in zip(calcs, sets)]
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(3):
+        st, P, refused = _search(rg, calcs[0], sets[0], a, len(ref[0][1]) - 1, noalloc=True)
+        refused_pairs = [t.clone() for t in refused[1:]]
+        assert st == rg._lib.RASCAL_E_CAPACITY and P == len(ref[0][1]) and a.query()
+        st, P, out = _search(rg, calcs[1], sets[1], b, len(ref[1][1]), noalloc=True)
+        torch.cuda.synchronize()
+        assert st == 0 and P == len(ref[1][1])
+        for o, w in zip(out, ref[1]):
+            assert np.array_equal(o.cpu().numpy(), w)
+        assert all(torch.equal(x.view(torch.uint8), y.view(torch.uint8)) for x, y in zip(refused_pairs, refused[1:]))
